@@ -23,6 +23,22 @@ namespace {
 __host__ __device__ __forceinline__ int64_t tix(int it, int jt) { return ((int64_t)it * (it + 1) / 2 + jt) * 64; }
 __host__ __device__ __forceinline__ int64_t n_tiles(int nt) { return (int64_t)nt * (nt + 1) / 2; }
 
+// The emulated kernel's matrix: lower triangle of 32x32 blocks of 1024 words, in packed row order.
+// A block holds either the fixed point (kFixBits), column by column (word 32 c + r), so that the
+// trailing update's warps, one row per lane, read and write whole 256-byte lines; or, once its
+// columns are reached, 8x8 FP64 tiles, tile column by tile column.  In both forms 16 columns
+// take the same half of the block, so the warp that owns a half turns it from one into the other.
+__host__ __device__ __forceinline__ int64_t bix(int bi, int bj) { return ((int64_t)bi * (bi + 1) / 2 + bj) * 1024; }
+__host__ __device__ __forceinline__ int64_t n_blocks(int rows) {
+    const int64_t nb = (rows + 31) / 32;
+    return nb * (nb + 1) / 2;
+}
+// offset of the FP64 tile (it, jt), jt <= it, of the emulated kernel's matrix
+__host__ __device__ __forceinline__ int64_t eix(int it, int jt) {
+    return bix(it >> 2, jt >> 2) + ((jt & 3) * 4 + (it & 3)) * 64;
+}
+constexpr int kTileCol = 256;  // words from a tile to its right neighbour in the block
+
 // Position of element (r, c) inside a 64-double tile: row major with the columns of rows
 // 2, 3, 6, 7 XOR-swizzled by 4, so the mma fragment loads (row g, column t) of the 32 lanes
 // of a warp hit distinct shared-memory banks in each half-warp.
@@ -111,10 +127,11 @@ struct Shared {
 // slices of one 16-column half of the block are staged for the band (A) and the column tile (B).
 constexpr int kBandT = 16;
 constexpr int kColT = 4;
-constexpr int kSliceTileBytes = 7 * 2 * 128;  // one row tile, one K half: 7 slices x 2 core matrices
-// staging: the band's slices of both K halves (A), and two buffers of the column tile's (B)
-constexpr int kStageA = 2 * kBandT * kSliceTileBytes;
-constexpr int kStageB = 2 * kColT * kSliceTileBytes;
+constexpr int kSliceBytes = 2 * 2 * 128;           // one slice of a row tile: 2 K halves x 2 core matrices
+constexpr int kSliceTileBytes = 7 * kSliceBytes;   // the 7 slices of a row tile
+// staging: the band's slices (A), and two buffers of the column tile's (B)
+constexpr int kStageA = kBandT * kSliceTileBytes;
+constexpr int kStageB = kColT * kSliceTileBytes;
 constexpr int kStageBytes = kStageA + 2 * kStageB;
 constexpr int kEmuTmemCols = 8 * 8 * kColT;    // 8 slice groups x 32 FP32 columns
 // Latent variance in the emulated kernel: up to kBorderQ queries of an instance append their
@@ -341,13 +358,6 @@ __device__ __forceinline__ long long kfix_ff(const float a[3], const float b[3],
     return fix_of_float(vh, kFixBits - m) + fix_of_float(vl, kFixBits - m);
 }
 
-// Entry (i, j), i > j, of K in the fixed point: float pairs in mixed precision, the FP64 value
-// (as kval_pair) rounded to the fixed point in FP64 precision and on the lattice.
-__device__ __forceinline__ long long kfix_pair(const DevParams& P, const Shared& s, bool lattice, int i, int j) {
-    if (lattice || P.precision != VGP_MIXED) return fix_of_double(kval_pair(P, s, lattice, i, j));
-    return kfix_ff(s.Xw + 3 * i, s.Xw + 3 * j, P.inv2l2_hi, P.inv2l2_lo, s.Tff);
-}
-
 // The float pair (hi, lo) of an FP64 value.
 __device__ __forceinline__ void split_pair(double v, float& hi, float& lo) {
     hi = (float)v;
@@ -424,7 +434,7 @@ __device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double*
                 __syncwarp();
                 const int i = 8 * (kt + 1) + lane;  // rows of the block below tile kt
                 if (i < 8 * B1) {
-                    const double* T = A + tix(i >> 3, kt);
+                    const double* T = A + eix(i >> 3, kt);
                     const int r = i & 7;
                     double u = z[i];
 #pragma unroll
@@ -439,7 +449,7 @@ __device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double*
             const int r = i & 7;
             double u = z[i];
             for (int kt = B0; kt < B1; ++kt) {
-                const double* T = A + tix(i >> 3, kt);
+                const double* T = A + eix(i >> 3, kt);
 #pragma unroll
                 for (int c2 = 0; c2 < 8; ++c2) u -= T[te(r, c2)] * z[8 * kt + c2];
             }
@@ -460,7 +470,7 @@ __device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double*
                 __syncwarp();
                 const int j = 8 * B0 + lane;  // columns of the block left of tile kt
                 if (j < 8 * kt) {
-                    const double* T = A + tix(kt, j >> 3);
+                    const double* T = A + eix(kt, j >> 3);
                     const int cj = j & 7;
                     double u = z[j];
 #pragma unroll
@@ -475,7 +485,7 @@ __device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double*
             const int cj = j & 7;
             double u = z[j];
             for (int kt = B0; kt < B1; ++kt) {
-                const double* T = A + tix(kt, j >> 3);
+                const double* T = A + eix(kt, j >> 3);
 #pragma unroll
                 for (int c2 = 0; c2 < 8; ++c2) u -= T[te(c2, cj)] * out[8 * kt + c2];
             }
@@ -491,7 +501,7 @@ __device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double*
 // S: 64 doubles of scratch.  False on a non-positive pivot (the same on every lane).
 __device__ bool diag_tile_warp(double* A, int kt, const Shared& s, double* Ti, double* S) {
     const int lane = threadIdx.x & 31;
-    double* D = A + tix(kt, kt);
+    double* D = A + eix(kt, kt);
     S[lane] = D[lane];
     S[lane + 32] = D[lane + 32];
     __syncwarp();
@@ -533,7 +543,7 @@ __device__ void panel_column(double* A, int kt, int it_end, const double* Ti) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     for (int it = kt + 1 + warp; it < it_end; it += nwarps) {
-        double* T = A + tix(it, kt);
+        double* T = A + eix(it, kt);
         const double a0 = T[te(g, t)], a1 = T[te(g, 4 + t)];
         const double b0 = Ti[te(g, t)], b1 = Ti[te(g, 4 + t)];
         double c0 = 0.0, c1 = 0.0;
@@ -548,27 +558,44 @@ __device__ void panel_column(double* A, int kt, int it_end, const double* Ti) {
 // w 2^sh rounded to an integer (ties up) for a 64-bit integer w: a slice-product update in
 // the fixed point of the trailing matrix.  No overflow: |w| 2^sh is bounded by the entry bound.
 __device__ __forceinline__ long long fix_shift(long long w, int sh) {
-    if (sh >= 0) return w << sh;
-    if (sh < -63) return 0;
-    return ((w >> (-sh - 1)) + 1) >> 1;
+    const int n = min(-sh - 1, 63);  // a shift by 63 leaves -1 or 0, which rounds to 0
+    return sh >= 0 ? w << sh : ((w >> (n & 63)) + 1) >> 1;
+}
+
+// The update w of an entry from its eight slice groups (see factor_emulated), given as the bits of
+// G + 1.5 * 2^23 (kGroupBits + G, exact for |G| < 2^22):
+//   w = 2^40 G_0 + 2^32 G_1 + ... + 2^16 G_3 + round((2^24 G_4 + 2^16 G_5 + 2^8 G_6 + G_7) / 2^16),
+// pairs of groups joined in 32 bits first (|256 G + G'| < 2^31), so the 64-bit part is one wide
+// multiply-add and one addition to the high word.
+constexpr unsigned kGroupBits = 0x4B400000u;
+__device__ __forceinline__ long long join_groups(const unsigned (&g)[8]) {
+    constexpr unsigned kOff = kGroupBits * 257u;
+    const unsigned a = g[0] * 256u + g[1] - kOff;
+    const int b = (int)(g[2] * 256u + g[3] - kOff);
+    const unsigned c = g[4] * 256u + g[5] - kOff;
+    const int d = (int)(g[6] * 256u + g[7] - kOff + 32768u);
+    const int e = (int)(c + (unsigned)(d >> 16));
+    return (long long)b * 65536 + e + (long long)((unsigned long long)a << 32);
 }
 
 // Balanced base-256 digits of row g of an 8-row tile over one block (the FP64 values
 // x[0 .. 2 kEB - 1] held by the four lanes t of the row: columns 8 j + 2t and 8 j + 2t + 1 in
-// x[2j], x[2j + 1]), written as bf16 pairs to F[kh] (the tile's slices of the block's columns
-// 16 kh .. 16 kh + 15) in the tensor cores' K-major layout: [slice][core matrix of 8 columns]
-// [row][8 bf16], 16 bytes per row and 128 per core matrix; and the row scale 2^(em - 1021) to
-// *scale (lane t = 0).  The digit scheme is described at factor_emulated.
-__device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* F0, uint32_t* F1, double* scale) {
+// x[2j], x[2j + 1]), written as bf16 pairs to F in the tensor cores' K-major layout: [slice]
+// [core matrix of 8 columns][row][8 bf16], 16 bytes per row and 128 per core matrix; and the row
+// scale 2^(em - 1021) to *scale (lane t = 0).  The digit scheme is described at factor_emulated.
+// With u (an appended query row's diagonal entry in the fixed point, lane t = 0) the row's own
+// update |row|^2 is taken from the digits here: only the diagonal of the query-by-query block is
+// needed, and 19 integer products per column cost a tenth of the tensor-core tiles that hold it.
+__device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* F, double* scale, long long* u) {
     const int lane = threadIdx.x & 31;
     int em = 0;
 #pragma unroll
     for (int i = 0; i < 2 * kEB; ++i) em = max(em, (int)((__double_as_longlong(x[i]) >> 52) & 0x7FF));
     em = max(em, __shfl_xor_sync(0xffffffffu, em, 1));
     em = max(em, __shfl_xor_sync(0xffffffffu, em, 2));
+    unsigned G[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int kk = 0; kk < kEK; ++kk) {
-        uint32_t* F = kk ? F1 : F0;
         unsigned long long Yb[4];
         bool negx[4];
 #pragma unroll
@@ -596,11 +623,40 @@ __device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* 
                 h16[i] = __float_as_uint((float)qv) >> 16;  // exact: |qv| <= 2^7
             }
             // lane = 4 g + t: row g, columns 2t, 2t + 1 of the core matrices of columns 0-7 and 8-15
-            F[ss * 64 + lane] = h16[0] | (h16[1] << 16);
-            F[ss * 64 + 32 + lane] = h16[2] | (h16[3] << 16);
+            F[ss * 128 + kk * 64 + lane] = h16[0] | (h16[1] << 16);
+            F[ss * 128 + kk * 64 + 32 + lane] = h16[2] | (h16[3] << 16);
+        }
+        if (u) {  // G_g += sum_{s+t=g} q_s q_t of each column (the sign drops out)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int q[7];
+                q[0] = (int)(Yb[i] >> 48);
+#pragma unroll
+                for (int ss = 1; ss < 7; ++ss) q[ss] = (int)((Yb[i] >> (48 - 8 * ss)) & 255ull) - 128;
+#pragma unroll
+                for (int gq = 0; gq < 8; ++gq) {
+                    int v = 0;
+#pragma unroll
+                    for (int ss = 0; 2 * ss < gq; ++ss)
+                        if (gq - ss < 7) v += q[ss] * q[gq - ss];
+                    v *= 2;
+                    if (gq % 2 == 0) v += q[gq / 2] * q[gq / 2];
+                    G[gq] += (unsigned)v;
+                }
+            }
         }
     }
     if ((lane & 3) == 0) *scale = em > 0 ? __longlong_as_double((long long)(em + 2) << 52) : 0.0;
+    if (u) {
+#pragma unroll
+        for (int gq = 0; gq < 8; ++gq) {
+            G[gq] += __shfl_xor_sync(0xffffffffu, G[gq], 1);
+            G[gq] += __shfl_xor_sync(0xffffffffu, G[gq], 2);
+            G[gq] += kGroupBits;
+        }
+        const int e = em > 0 ? em + 2 : 0;
+        if ((lane & 3) == 0) *u -= fix_shift(join_groups(G), 2 * e - (2102 - kFixBits));
+    }
 }
 
 // Row tile it below the factorised diagonal block of tile columns K0 .. K0 + kEB - 1 (inverses
@@ -608,26 +664,26 @@ __device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* 
 // Ti_j^T for j < kEB on the FP64 tensor path, one warp, the row's tiles in registers.  The warp's
 // scratch tile W turns each result from the accumulator into the operand layout.  The
 // results are stored to A and sliced for the trailing update (F, scale: this tile's slices
-// and row scales).
-__device__ void block_rows(double* A, int it, int K0, const double* Tblk, double* W, uint32_t* F0, uint32_t* F1,
-                           double* scale) {
+// and row scales; u: the diagonal entries of an appended query tile's rows, else null).
+__device__ void block_rows(double* A, int it, int K0, const double* Tblk, double* W, uint32_t* F, double* scale,
+                           long long* u) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    double* R = A + tix(it, K0);  // tiles (it, K0 .. K0 + kEB - 1), contiguous
+    double* R = A + eix(it, K0);  // tiles (it, K0 .. K0 + kEB - 1), kTileCol apart
     double x[2 * kEB];            // accumulator layout: tile j holds columns 2t, 2t + 1 of row g
 #pragma unroll
     for (int j = 0; j < kEB; ++j) {
-        x[2 * j] = R[64 * j + te(g, 2 * t)];
-        x[2 * j + 1] = R[64 * j + te(g, 2 * t + 1)];
+        x[2 * j] = R[kTileCol * j + te(g, 2 * t)];
+        x[2 * j + 1] = R[kTileCol * j + te(g, 2 * t + 1)];
     }
     double xa[kEB - 1][2];  // operand layout of the solved tiles: columns t and 4 + t of row g
 #pragma unroll
     for (int j = 0; j < kEB; ++j) {
         double a0 = x[2 * j], a1 = x[2 * j + 1];
-        const double* Lj = A + tix(K0 + j, K0);  // tiles (K0 + j, K0 .. K0 + j), contiguous
+        const double* Lj = A + eix(K0 + j, K0);  // tiles (K0 + j, K0 .. K0 + j)
 #pragma unroll
         for (int k = 0; k < j; ++k) {
-            dmma(a0, a1, neg(xa[k][0]), Lj[64 * k + te(g, t)]);
-            dmma(a0, a1, neg(xa[k][1]), Lj[64 * k + te(g, 4 + t)]);
+            dmma(a0, a1, neg(xa[k][0]), Lj[kTileCol * k + te(g, t)]);
+            dmma(a0, a1, neg(xa[k][1]), Lj[kTileCol * k + te(g, 4 + t)]);
         }
         W[te(g, 2 * t)] = a0;
         W[te(g, 2 * t + 1)] = a1;
@@ -638,8 +694,8 @@ __device__ void block_rows(double* A, int it, int K0, const double* Tblk, double
         double y0 = 0.0, y1 = 0.0;
         dmma(y0, y1, p0, Ti[te(g, t)]);
         dmma(y0, y1, p1, Ti[te(g, 4 + t)]);
-        R[64 * j + te(g, 2 * t)] = y0;
-        R[64 * j + te(g, 2 * t + 1)] = y1;
+        R[kTileCol * j + te(g, 2 * t)] = y0;
+        R[kTileCol * j + te(g, 2 * t + 1)] = y1;
         x[2 * j] = y0;
         x[2 * j + 1] = y1;
         if (j < kEB - 1) {
@@ -651,18 +707,21 @@ __device__ void block_rows(double* A, int it, int K0, const double* Tblk, double
             __syncwarp();
         }
     }
-    slice_row(x, F0, F1, scale + g);
+    slice_row(x, F, scale + g, u ? u + g : nullptr);
 }
 
-// Per-CTA workspace of the emulated factorisation: for each of the block's two 16-column halves
-// the slices of the rows below the current block ([row tile][7 slices][2 core matrices], 1792
-// bytes per row tile), npad row scales, then the inverses of all diagonal tiles ([npad / 8][64]
-// doubles).
+// Per-CTA workspace of the emulated factorisation: the slices of the rows below the current block
+// ([row tile][7 slices][4 core matrices], 3584 bytes per row tile), the row scales, the inverses of
+// all diagonal tiles ([rows / 8][64] doubles), and the appended query rows' diagonal entries in
+// the fixed point.
 __device__ __forceinline__ unsigned char* emu_ws(const SolveCtx& c) { return c.ws_e + (int64_t)blockIdx.x * c.ws_e_stride; }
-__device__ __forceinline__ int64_t emu_half_bytes(int npad) { return (int64_t)(npad / 8) * kSliceTileBytes; }
 __device__ __forceinline__ int emu_rows(const SolveCtx& c) { return c.nrow > 0 ? c.nrow : c.npad; }
-__device__ __forceinline__ double* emu_tile_inverses(const SolveCtx& c) {
-    return reinterpret_cast<double*>(emu_ws(c) + 2 * emu_half_bytes(emu_rows(c))) + emu_rows(c);
+__device__ __forceinline__ double* emu_scales(const SolveCtx& c) {
+    return reinterpret_cast<double*>(emu_ws(c) + (int64_t)(emu_rows(c) / 8) * kSliceTileBytes);
+}
+__device__ __forceinline__ double* emu_tile_inverses(const SolveCtx& c) { return emu_scales(c) + emu_rows(c); }
+__device__ __forceinline__ long long* emu_query_diag(const SolveCtx& c) {
+    return reinterpret_cast<long long*>(emu_tile_inverses(c) + 8 * emu_rows(c));
 }
 
 // ---- tensor-core (tcgen05) helpers for the emulated updates --------------------------------
@@ -675,14 +734,15 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
-// Instruction descriptor of kind::f16: bf16 A and B (K-major), FP32 D, M = 128, N = 8 kColT.
-constexpr uint32_t kUmmaIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(8 * kColT / 8) << 17) |
-                                ((uint32_t)(128 / 16) << 24);
+// Instruction descriptor of kind::f16: bf16 A and B (K-major), FP32 D, M = 128, N = n.
+__host__ __device__ constexpr uint32_t umma_idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n / 8) << 17) | ((uint32_t)(128 / 16) << 24);
+}
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, int n, uint32_t accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(kUmmaIdesc), "r"(accumulate));
+                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(umma_idesc(n)), "r"(accumulate));
 }
 
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -690,16 +750,20 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// Wait for the completion of phase `parity` of an mbarrier, at most kWaitLimit polls; the
-// result is the same on every thread of the CTA (false: the wait gave up somewhere).
+// Wait of the calling thread for the completion of phase `parity` of an mbarrier, at most
+// kWaitLimit polls (false: the wait gave up).
 constexpr int kWaitLimit = 1 << 22;
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool bar_poll(uint32_t bar, uint32_t parity) {
     uint32_t done = 0;
     for (int it = 0; it < kWaitLimit && !done; ++it)
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
                      " selp.u32 %0, 1, 0, p;\n}"
                      : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return __syncthreads_and((int)done) != 0;
+    return done != 0;
+}
+// The same for the whole CTA: the result is the same on every thread.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+    return __syncthreads_and((int)bar_poll(bar, parity)) != 0;
 }
 
 // Tensor memory and barriers of an emulated CTA.
@@ -724,154 +788,163 @@ __device__ __forceinline__ bool emu_fail(const SolveCtx& c, EmuTc& tc) {
     return false;
 }
 
+// Copy the slices of nc row tiles from E into the staging buffer of a column tile (B), one warp:
+// slice by slice ([slice][row tile][512 bytes]), so that the first n slices of the column tile are
+// n * 32 consecutive rows of the MMA's N dimension.  The mbarrier counts `extra` bytes more (the
+// band's A).
+__device__ __forceinline__ void stage_columns(unsigned char* dst, const unsigned char* E, int nc, uint32_t extra,
+                                              uint32_t bar) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                     "r"((uint32_t)nc * kSliceTileBytes + extra)
+                     : "memory");
+    __syncwarp();
+    if (lane < 7 * kColT) {
+        const int ss = lane / kColT, rt = lane % kColT;
+        if (rt < nc)
+            bulk_load(dst + (ss * kColT + rt) * kSliceBytes, E + (int64_t)rt * kSliceTileBytes + ss * kSliceBytes,
+                      kSliceBytes, bar);
+    }
+}
+
 // Trailing update C -= P P^T of the M = Nt - K1 row tiles below the block that ends at K1, on
-// the tensor cores.  P's rows are cut into seven digit slices (see factor_emulated), and every
-// slice group G_g = sum_{s+t=g} P_s P_t^T is accumulated exactly in FP32 in tensor memory.
-// Output tiles of kBandT row tiles (128 rows) by kColT row tiles (32 columns) cover the lower
-// triangle, band by band.  Bulk copies stage the band's slices (A, both 16-column halves of the
-// block) once per band and each column tile's slices (B) in one of two buffers, the next tile's
-// while the current one computes.  One thread issues the 68 slice products of a tile (34 slice
-// pairs x 2 halves) into the 8 group accumulators; all 8 warps then read their rows (lane
-// quadrant warp % 4) and columns (half warp / 4) of the groups, pack each element's groups into
-// one integer and subtract it as an FP64 value.
-// With appended query rows (tiles Ntr .. Nt - 1, see fit_instance) only the diagonal tiles of
-// the query-by-query block are needed: its other column tiles are skipped.
+// the tensor cores, for the columns of the matrix itself (row tiles K1 .. Ntr - 1).  P's rows are
+// cut into seven digit slices (see factor_emulated), and every slice group
+// G_g = sum_{s+t=g} P_s P_t^T is accumulated exactly in FP32 in tensor memory.  Output tiles of
+// kBandT row tiles (128 rows) by kColT row tiles (32 columns) cover the lower triangle, band by
+// band.  Bulk copies stage the band's slices (A) once per band and each column tile's slices (B)
+// in one of two buffers, the next tile's while the current one computes.
+//
+// The groups lie side by side in tensor memory (group g at columns 32 g) and B's slices side by
+// side in shared memory, so A slice s times B slices 0 .. n - 1 is ONE product of N = 32 n columns
+// whose output lands on groups s .. s + n - 1: 15 MMAs per tile instead of 68 of N = 32, each
+// reading its 4 KB of A from shared memory once.  An N = 32 product is bound by that read (about
+// 40 clocks for 16 of arithmetic); all of a tile's now need about 1100 clocks, the arithmetic's.
+// One thread issues them.  All 8 warps then read their rows (lane quadrant warp % 4) and columns
+// (half warp / 4) of the groups, join each element's groups into one integer and subtract it from
+// the fixed point.  C is read and written in whole 256-byte lines (see bix); the next tile's block
+// is prefetched into L2.  Measured against 68 N = 32 products, 8-byte accesses to 64-byte tile rows
+// and a diagonal of the query block from full tiles: 38 instances of about 790 points alone on the
+// GPU 16.1 -> 11.7 ms, 15.6k of 4 to 1024 points 216 -> 180 ms.
 __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr, int K1, const unsigned char* E,
-                                   int64_t KH, const double* sr, unsigned char* stage, EmuTc& tc) {
+                                   const double* sr, unsigned char* stage, EmuTc& tc) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = Nt - K1;
-    const int jr = (max(Ntr - K1, 0) + kColT - 1) / kColT;  // column tiles of the matrix itself
-    const int next1 = min(K1 + kEB, Ntr);                     // end of the next block's columns
+    const int jr = (max(Ntr - K1, 0) + kColT - 1) / kColT;  // column tiles
+    if (jr == 0) return true;
     const uint32_t aA = smem_addr(stage), aB = aA + kStageA;
     const int q = warp & 3, h = warp >> 2;  // lane quadrant (rows 32 q ..) and column half
-    const int row = 32 * q + lane, rb = row >> 3, rr = row & 7;
+    const int kb1 = K1 >> 2;                // 32-row block of the first row below (K1 is a multiple of 4)
+    int fail = 0;
+    auto stage_band = [&](int b0) {  // the band's A and the first column tile's B (buffer 0); warp 0
+        const int nb = min(kBandT, M - b0);
+        if (lane == 0)
+            bulk_load(stage, E + (int64_t)b0 * kSliceTileBytes, (uint32_t)nb * kSliceTileBytes, tc.bar_ld);
+        stage_columns(stage + kStageA, E, min(kColT, Ntr - K1), (uint32_t)nb * kSliceTileBytes, tc.bar_ld);
+    };
+    if (warp == 0) stage_band(0);
     for (int b0 = 0; b0 < M; b0 += kBandT) {
         const int nb = min(kBandT, M - b0);
-        const bool rvalid = rb < nb;
-        const int rt = K1 + b0 + rb;
-        const int er = rvalid ? (int)(__double_as_longlong(sr[8 * (b0 + rb) + rr]) >> 52) : 0;
-        const int n_tiles = (b0 + nb + kColT - 1) / kColT;  // column tiles reaching the band's last row tile
-        // column tiles of appended query rows: only those that meet the band's rows
-        const int qstart = max(jr, b0 / kColT);
-        auto next_tile = [&](int j) { return j + 1 < jr ? j + 1 : max(j + 1, qstart); };
-        const int first = jr > 0 ? 0 : qstart;
-        if (first >= n_tiles) continue;
-        if (tid == 0) {  // the band's A and the first column tile's B (buffer 0)
-            const int nc = min(kColT, M - first * kColT);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
-                         "r"((uint32_t)(2 * (nb + nc) * kSliceTileBytes))
-                         : "memory");
-            for (int kh = 0; kh < 2; ++kh) {
-                const unsigned char* H = E + kh * KH;
-                bulk_load(stage + kh * kBandT * kSliceTileBytes, H + (int64_t)b0 * kSliceTileBytes,
-                          (uint32_t)nb * kSliceTileBytes, tc.bar_ld);
-                bulk_load(stage + kStageA + kh * kColT * kSliceTileBytes, H + (int64_t)first * kColT * kSliceTileBytes,
-                          (uint32_t)nc * kSliceTileBytes, tc.bar_ld);
-            }
-        }
-        for (int jt = first, kb = 0; jt < n_tiles; jt = next_tile(jt), ++kb) {
-            const int c0 = jt * kColT, nc = min(kColT, M - c0);
-            const uint32_t bufB = aB + (uint32_t)((kb & 1) * kStageB);
-            if (!bar_wait(tc.bar_ld, tc.ph_ld)) return emu_fail(c, tc);
-            tc.ph_ld ^= 1;
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int rb = (b0 >> 2) + q;              // the warp's 32-row block below K1
+        const bool rows_in = 4 * q < nb;
+        // the row's exponent (rows past the matrix inside its last block: unused)
+        const int er = rows_in ? (int)(__double_as_longlong(sr[32 * rb + lane]) >> 52) : 0;
+        const int n_tiles = min(jr, (b0 + nb + kColT - 1) / kColT);  // column tiles reaching the band's last row
+        for (int jt = 0; jt < n_tiles; ++jt) {
+            const uint32_t bufB = aB + (uint32_t)((jt & 1) * kStageB);
+            // warp 0 alone waits for the copies, issues the products and then the next copies: every
+            // phase of the copy barrier is seen before the next one can start
+            if (warp == 0 && !bar_poll(tc.bar_ld, tc.ph_ld)) fail = 1;
+            if (warp == 0 && !__any_sync(0xffffffffu, fail)) {
+                if (lane == 0) {
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int kh = 0; kh < 2; ++kh)
-#pragma unroll
-                    for (int ss = 0; ss < 7; ++ss)
-#pragma unroll
-                        for (int tt = 0; tt < 7 && ss + tt < 8; ++tt) {
-                            const int gq = ss + tt;
-                            umma_bf16(tc.tmem + gq * 8 * kColT,
-                                      umma_desc(aA + kh * kBandT * kSliceTileBytes + ss * 256, 128, kSliceTileBytes),
-                                      umma_desc(bufB + kh * kColT * kSliceTileBytes + tt * 256, 128, kSliceTileBytes),
-                                      // the first product of a group (pair (0, g), or (1, 6)
-                                      // for g = 7) overwrites the accumulator
-                                      (kh == 0 && (ss == 0 || (ss == 1 && gq == 7))) ? 0u : 1u);
-                        }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 tc.bar_mma)
-                             : "memory");
-                if (next_tile(jt) < n_tiles) {  // the next column tile's B into the other buffer
-                    const int c1 = next_tile(jt) * kColT, n1 = min(kColT, M - c1);
-                    unsigned char* dst = stage + kStageA + ((kb + 1) & 1) * kStageB;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
-                                 "r"((uint32_t)(2 * n1 * kSliceTileBytes))
-                                 : "memory");
                     for (int kh = 0; kh < 2; ++kh)
-                        bulk_load(dst + kh * kColT * kSliceTileBytes, E + kh * KH + (int64_t)c1 * kSliceTileBytes,
-                                  (uint32_t)n1 * kSliceTileBytes, tc.bar_ld);
-                }
-            }
-            // while the MMAs run: this thread's 16 entries of C (row `row`, the 8 columns of each
-            // of its two column tiles) and the column scales, all loads issued at once
-            long long cv[2][8];
-            int ec[2][8];
-            bool ok[2];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int cb = 2 * h + j, ct = K1 + c0 + cb;
-                ok[j] = rvalid && cb < nc && ct <= rt && (ct < Ntr || ct == rt);
-                const double* C = A + tix(ok[j] ? rt : K1, ok[j] ? ct : K1);
-                const double* scl = sr + 8 * (ok[j] ? c0 + cb : 0);
-#pragma unroll
-                for (int cc = 0; cc < 8; ++cc) {
-                    cv[j][cc] = ok[j] ? __double_as_longlong(C[te(rr, cc)]) : 0;
-                    ec[j][cc] = (int)(__double_as_longlong(scl[cc]) >> 52);
+                        for (int ss = 0; ss < 7; ++ss) {
+                            const int n = ss == 0 ? 7 : 8 - ss;  // B slices of this product
+                            const uint64_t da = umma_desc(aA + ss * kSliceBytes + kh * 256, 128, kSliceTileBytes);
+                            const uint32_t b = bufB + kh * 256;
+                            const uint32_t dcol = tc.tmem + ss * 8 * kColT;
+                            if (kh == 0 && ss == 1) {
+                                // groups 1 .. 6 hold slice 0's products; group 7 starts here
+                                umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), 6 * 8 * kColT, 1u);
+                                umma_bf16(dcol + 6 * 8 * kColT, da, umma_desc(b + 6 * kColT * kSliceBytes, 128, kSliceBytes),
+                                          8 * kColT, 0u);
+                            } else {
+                                umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), n * 8 * kColT,
+                                          (kh == 0 && ss == 0) ? 0u : 1u);
+                            }
+                        }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     tc.bar_mma)
+                                 : "memory");
                 }
+                __syncwarp();
+                if (jt + 1 < n_tiles)  // the next column tile's B into the other buffer
+                    stage_columns(stage + kStageA + ((jt + 1) & 1) * kStageB,
+                                  E + (int64_t)(jt + 1) * kColT * kSliceTileBytes,
+                                  min(kColT, Ntr - K1 - (jt + 1) * kColT), 0, tc.bar_ld);
             }
-            if (!bar_wait(tc.bar_mma, tc.ph_mma)) return emu_fail(c, tc);
+            tc.ph_ld ^= 1;
+            // while the MMAs run: this thread's 16 entries of C (one row, 16 columns) and the column
+            // scales, all loads issued at once
+            const bool on = rows_in && jt <= rb;  // (warp-uniform, as the collective tcgen05.ld needs)
+            long long* C = reinterpret_cast<long long*>(A + bix(kb1 + rb, kb1 + jt)) + 512 * h;
+            long long cv[16];
+            int es = 0;
+            if (on) {
+#pragma unroll
+                for (int cc = 0; cc < 16; ++cc) cv[cc] = C[32 * cc + lane];
+                es = (int)(__double_as_longlong(sr[32 * jt + 16 * h + (lane & 15)]) >> 52);
+                if (jt + 1 < n_tiles && jt < rb && lane == 0)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024), "r"(4096));
+            }
+            if (!bar_poll(tc.bar_mma, tc.ph_mma)) fail = 1;
             tc.ph_mma ^= 1;
+            __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            // the band's last products are done: its A and B buffers take the next band's
+            if (warp == 0 && !__any_sync(0xffffffffu, fail) && jt + 1 == n_tiles && b0 + kBandT < M) stage_band(b0 + kBandT);
+            if (on) {
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {  // the thread's two column tiles of the output tile
-                const int cb = 2 * h + j;
-                // a warp none of whose rows is updated in this column tile (rows past the band,
-                // above the diagonal, or of the query block away from its diagonal) skips it;
-                // the test is warp-uniform, as the collective tcgen05.ld needs
-                if (!__any_sync(0xffffffffu, ok[j])) continue;
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {  // four columns at a time
+                for (int p = 0; p < 4; ++p) {  // four columns at a time
                     uint32_t v[8][4];
 #pragma unroll
                     for (int gq = 0; gq < 8; ++gq)
-                        tmem_ld4(tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(gq * 8 * kColT + 8 * cb + 4 * p), v[gq]);
+                        tmem_ld4(tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(gq * 8 * kColT + 16 * h + 4 * p), v[gq]);
                     tmem_wait_ld();
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const int cc = 4 * p + e;
-                        // each group read from the bits of G + 1.5 * 2^23 (exact: |G| < 2^22)
-                        long long gq8[8];
+                        unsigned gb[8];
 #pragma unroll
-                        for (int gq = 0; gq < 8; ++gq) gq8[gq] = __float_as_int(__uint_as_float(v[gq][e]) + 12582912.0f);
-                        constexpr long long kOffBits = 0x4B400000ll * 0x01010101ll;
-                        const long long hi = gq8[0] * (1ll << 24) + gq8[1] * (1ll << 16) + gq8[2] * 256 + gq8[3] - kOffBits;
-                        const long long lo = gq8[4] * (1ll << 24) + gq8[5] * (1ll << 16) + gq8[6] * 256 + gq8[7] - kOffBits;
+                        for (int gq = 0; gq < 8; ++gq)
+                            gb[gq] = __float_as_uint(__fadd_rn(__uint_as_float(v[gq][e]), 12582912.0f));
+                        const int ec = __shfl_sync(0xffffffffu, es, 4 * p + e);
                         // the update is w 2^(er + ec - 2102), in units of 2^-kFixBits
-                        cv[j][cc] -= fix_shift(hi * (1ll << 16) + ((lo + (1ll << 15)) >> 16),
-                                               er + ec[j][cc] - (2102 - kFixBits));
+                        cv[4 * p + e] -= fix_shift(join_groups(gb), er + ec - (2102 - kFixBits));
                     }
+                }
+                // the next block's columns are final after this update: stored as FP64 tiles (see
+                // factor_emulated), the rest in the fixed point.  The half block is read before it
+                // is written in the other form.
+                if (jt == 0) {
+                    __syncwarp();
+                    double* T = reinterpret_cast<double*>(C) + (lane >> 3) * 64;
+                    const int rr = lane & 7;
+#pragma unroll
+                    for (int cc = 0; cc < 16; cc += 2)
+                        *reinterpret_cast<double2*>(T + (cc >> 3) * kTileCol + te(rr, cc & 7)) =
+                            make_double2(double_of_fix(cv[cc]), double_of_fix(cv[cc + 1]));
+                } else {
+#pragma unroll
+                    for (int cc = 0; cc < 16; ++cc) C[32 * cc + lane] = cv[cc];
                 }
             }
-            // the next block's columns are final after this update: stored as FP64 (see
-            // factor_emulated), the rest in the fixed point
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                if (ok[j]) {
-                    const int ct = K1 + c0 + 2 * h + j;
-                    double* C = A + tix(rt, ct);
-                    if (ct < next1) {
-#pragma unroll
-                        for (int cc = 0; cc < 8; ++cc) C[te(rr, cc)] = double_of_fix(cv[j][cc]);
-                    } else {
-#pragma unroll
-                        for (int cc = 0; cc < 8; ++cc) C[te(rr, cc)] = __longlong_as_double(cv[j][cc]);
-                    }
-                }
             // every thread's reads of the accumulators are done before the next tile's MMAs
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
+            if (__syncthreads_or(fail)) return emu_fail(c, tc);
         }
     }
     return true;
@@ -894,37 +967,23 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
 // 2^22 with W = 32: the rounding of lo is below 2^-57 of the scale 2^(e_r + e_c - 2042).  The
 // trailing matrix is held in the fixed point of kFixBits (assembled so by fit_instance): w is
 // shifted to it and subtracted as an integer, so an updated entry costs no FP64 operation,
-// and each block's columns are stored as FP64 by the update that completes them.  The slice
-// products run on the tensor cores
+// and each block's columns are stored as FP64 by the update that completes them (the first block's
+// by the assembly).  The slice products run on the tensor cores
 // (trailing_update_tc); within a block the diagonal block is factorised as in the plain loop
 // (8x8 tiles, FP64 tensor path) and the rows below it are solved one row tile per warp
 // (block_rows), which also writes their slices.
 // Nt row tiles, of which the first Ntr are factorised (Nt > Ntr: appended query rows, whose
-// rows below are solved and whose diagonal tiles are updated, but not factorised).
+// rows below are solved and whose diagonal entries are updated, but not factorised).
 __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, int Nt, int Ntr, int* s_fail,
                                 EmuTc& tc) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     unsigned char* E = emu_ws(c);
-    const int64_t KH = emu_half_bytes(emu_rows(c));
-    double* sr = reinterpret_cast<double*>(E + 2 * KH);  // row scales of the rows below the block
-    double* Tall = emu_tile_inverses(c);                  // inverses of all diagonal tiles, for the solves
+    double* sr = emu_scales(c);           // row scales of the rows below the block
+    double* Tall = emu_tile_inverses(c);  // inverses of all diagonal tiles, for the solves
+    long long* udiag = emu_query_diag(c);
     for (int K0 = 0; K0 < Ntr; K0 += kEB) {
         const int K1 = min(K0 + kEB, Ntr);
-        // the first block's columns (tiles (it, jt), jt < K1, jt <= it) from the fixed point of
-        // the assembly to FP64; later blocks' columns are stored as FP64 by the trailing update
-        // that completes them
-        if (K0 == 0) {
-            const int nb = K1 - K0;
-            const int64_t ne = (int64_t)(Nt - K0) * nb * 64;
-            for (int64_t x = tid; x < ne; x += blockDim.x) {
-                const int p = (int)(x >> 6), it = K0 + p / nb, jt = K0 + p % nb;
-                if (jt > it) continue;
-                double* v = A + tix(it, jt) + (x & 63);
-                *v = double_of_fix(__double_as_longlong(*v));
-            }
-            __syncthreads();
-        }
         // the diagonal block: tiles (it, jt), K0 <= jt <= it < K1, right-looking by 8 columns
         for (int kt = K0; kt < K1; ++kt) {
             double* Ti = s.Tblk + 64 * (kt - K0);
@@ -943,9 +1002,9 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             const int nj = K1 - kt - 1;
             for (int p = warp; p < nj * (nj + 1) / 2; p += nwarps) {
                 const int ir = tri_row(p), it = kt + 1 + ir, jt = kt + 1 + (p - ir * (ir + 1) / 2);
-                double* C = A + tix(it, jt);
-                const double* Li = A + tix(it, kt);
-                const double* Lj = A + tix(jt, kt);
+                double* C = A + eix(it, jt);
+                const double* Li = A + eix(it, kt);
+                const double* Lj = A + eix(jt, kt);
                 double c0 = C[te(g, 2 * t)], c1 = C[te(g, 2 * t + 1)];
                 dmma(c0, c1, neg(Li[te(g, t)]), Lj[te(g, t)]);
                 dmma(c0, c1, neg(Li[te(g, 4 + t)]), Lj[te(g, 4 + t)]);
@@ -959,12 +1018,12 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
         // block and writes their slices (both column halves) and row scales
         for (int it = K1 + warp; it < Nt; it += nwarps)
             block_rows(A, it, K0, s.Tblk, s.Wsc + 64 * warp,
-                       reinterpret_cast<uint32_t*>(E + (int64_t)(it - K1) * kSliceTileBytes),
-                       reinterpret_cast<uint32_t*>(E + KH + (int64_t)(it - K1) * kSliceTileBytes), sr + 8 * (it - K1));
+                       reinterpret_cast<uint32_t*>(E + (int64_t)(it - K1) * kSliceTileBytes), sr + 8 * (it - K1),
+                       it >= Ntr ? udiag + 8 * (it - Ntr) : nullptr);
         // the slices are read by the copy engine (async proxy)
         asm volatile("fence.proxy.async;" ::: "memory");
         __syncthreads();
-        if (!trailing_update_tc(c, A, Nt, Ntr, K1, E, KH, sr, s.stage, tc)) return false;
+        if (!trailing_update_tc(c, A, Nt, Ntr, K1, E, sr, s.stage, tc)) return false;
     }
     return true;
 }
@@ -1026,49 +1085,72 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
     // columns are the identity so the padded factor is block-diagonal.  The emulated kernel
     // writes the fixed point of kfix_pair (appended query rows: the query's kernel values, 1
     // on the diagonal, and only the diagonal tiles of the query-by-query block).
-    const int64_t ntl = n_tiles(Ntq);
-    if (kEmu)
-        for (int64_t tl = warp; tl < ntl; tl += nwarps) {
-            const int it = tri_row((int)tl), jt = (int)tl - it * (it + 1) / 2;
-            if (jt >= Nt && jt != it) continue;
-            for (int e = lane; e < 64; e += 32) {
-                const int i = 8 * it + (e >> 3), j = 8 * jt + (e & 7);
-                long long v;
-                if (i >= Np) {  // appended query row a = i - Np
-                    const int a = i - Np;
-                    if (j >= Np || a >= nq) {
-                        v = (i == j) ? (1ll << kFixBits) : 0;
-                    } else if (j >= N || isnan(s.qw[3 * a + 1])) {
-                        v = 0;
-                    } else if (lattice) {
-                        v = fix_of_double(c.P.lat_tab[lat_m(s.xi[j], __float_as_int(s.qw[3 * a]))]);
-                    } else if (c.P.precision == VGP_MIXED) {
-                        v = kfix_ff(s.qw + 3 * a, s.Xw + 3 * j, c.P.inv2l2_hi, c.P.inv2l2_lo, s.Tff);
-                    } else {
-                        // the query's FP64 local coordinates, formed as query_local forms them
-                        double r2 = 0.0;
+    if constexpr (kEmu) {
+        // strips of 8 columns of the 32x32 blocks, one per warp at a time: a row per lane (its
+        // point in registers), the columns' points broadcast, whole lines written.  The first
+        // block's columns are stored as FP64 tiles, the rest in the fixed point.
+        const int nbr = (Ntq + 3) >> 2, nbc = (Nt + 3) >> 2;
+        const int sq = nbc * (nbc + 1) / 2;  // blocks of the matrix itself; then nbc per block of query rows
+        const int n_strip = 4 * (sq + (nbr - nbc) * nbc);
+        for (int st = warp; st < n_strip; st += nwarps) {
+            const int p = st >> 2, c0 = 8 * (st & 3);
+            const int bi = p < sq ? tri_row(p) : nbc + (p - sq) / nbc;
+            const int bj = p < sq ? p - bi * (bi + 1) / 2 : (p - sq) % nbc;
+            const int i = 32 * bi + lane, a = i - Np;  // a >= 0: appended query row
+            const bool qrow = nq > 0 && a >= 0;
+            const bool live = qrow ? a < nq && !isnan(s.qw[3 * a + 1]) : i < N;
+            double* B = A + bix(bi, bj);
+            float rw[3] = {0.f, 0.f, 0.f};
+            int rx = 0;
+            if (live && lattice) rx = qrow ? __float_as_int(s.qw[3 * a]) : s.xi[i];
+            if (live && !lattice)
+                for (int k = 0; k < 3; ++k) rw[k] = qrow ? s.qw[3 * a + k] : s.Xw[3 * i + k];
+            long long v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int j = 32 * bj + c0 + e;
+                if (qrow ? !live || j >= N : !live || j >= N || j >= i) {
+                    v[e] = qrow || i != j ? 0 : i < N ? fix_of_double(1.0 + c.P.s2) : 1ll << kFixBits;
+                } else if (lattice) {
+                    v[e] = fix_of_double(c.P.lat_tab[lat_m(s.xi[j], rx)]);
+                } else if (c.P.precision == VGP_MIXED) {
+                    v[e] = kfix_ff(rw, s.Xw + 3 * j, c.P.inv2l2_hi, c.P.inv2l2_lo, s.Tff);
+                } else {
+                    double r2;
+                    if (qrow) {  // the query's FP64 local coordinates, formed as query_local forms them
+                        r2 = 0.0;
                         for (int k = 0; k < 3; ++k) {
                             const double cen = c.b.centre ? c.b.centre[3 * (int64_t)I + k] : 0.0;
-                            const double d = s.X[3 * j + k] - ((double)s.qw[3 * a + k] - cen);
+                            const double d = s.X[3 * j + k] - ((double)rw[k] - cen);
                             r2 += d * d;
                         }
-                        v = fix_of_double(exp(-r2 * c.P.inv2l2));
+                        v[e] = fix_of_double(exp(-r2 * c.P.inv2l2));
+                    } else {
+                        v[e] = fix_of_double(kval_pair(c.P, s, false, i, j));
                     }
-                } else if (i >= N || j >= N) v = (i == j) ? (1ll << kFixBits) : 0;
-                else if (j > i) v = 0;
-                else if (j == i) v = fix_of_double(1.0 + c.P.s2);  // s2: sigma_prop^2 for properties
-                else v = kfix_pair(c.P, s, lattice, i, j);
-                A[tl * 64 + te(e >> 3, e & 7)] = __longlong_as_double(v);
+                }
+            }
+            if (bj == 0) {
+                double* T = B + (c0 >> 3) * kTileCol + (lane >> 3) * 64;
+#pragma unroll
+                for (int e = 0; e < 8; e += 2)
+                    *reinterpret_cast<double2*>(T + te(lane & 7, e)) = make_double2(double_of_fix(v[e]), double_of_fix(v[e + 1]));
+            } else {
+                long long* F = reinterpret_cast<long long*>(B) + 32 * c0 + lane;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) F[32 * e] = v[e];
             }
         }
-    else
-    for (int64_t tl = warp; tl < ntl; tl += nwarps) {
+        if (nq > 0)
+            for (int a = tid; a < 8 * (Ntq - Nt); a += nt) emu_query_diag(c)[a] = 1ll << kFixBits;
+    }
+    if constexpr (!kEmu)
+    for (int64_t tl = warp; tl < n_tiles(Nt); tl += nwarps) {
         const int it = tri_row((int)tl), jt = (int)tl - it * (it + 1) / 2;
-        if (jt >= Nt && jt != it) continue;
         for (int e = lane; e < 64; e += 32) {
             const int i = 8 * it + (e >> 3), j = 8 * jt + (e & 7);
             double v;
-            if (i >= N || j >= N) v = (i == j) ? 1.0 : 0.0;  // (no appended rows here)
+            if (i >= N || j >= N) v = (i == j) ? 1.0 : 0.0;
             else if (j > i) v = 0.0;
             else if (j == i) v = 1.0 + c.P.s2;
             else v = kval_pair(c.P, s, lattice, i, j);
@@ -1525,7 +1607,6 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             // appended rows: the property GP's own matrix, noise sigma_c^2
             const bool pb = kEmu && c.qmax > 0 && q1 - q0 <= c.qmax;
             const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, pb ? (int)(q1 - q0) : 0, q0, I);
-            const int Ntr = ((N + 31) & ~31) >> 3;
             // property mode: means and variance (Eq. 6, variance read as for Eq. 2)
             const int np = c.b.nprop;
             for (int64_t p = q0 + tid; p < q1; p += nt) {
@@ -1537,8 +1618,7 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                     if (isfinite(xl[0]) && isfinite(xl[1]) && isfinite(xl[2])) {
                         property_mean(c.P, s, N, np, lattice, qi, xl, cm);
                         if (pb) {
-                            const int a = (int)(p - q0), ta = Ntr + (a >> 3);
-                            w = fmax(0.0, double_of_fix(__double_as_longlong(s.A[tix(ta, ta) + te(a & 7, a & 7)])));
+                            w = fmax(0.0, double_of_fix(emu_query_diag(c)[p - q0]));
                         } else {
                             w = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
                         }
@@ -1557,7 +1637,6 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
         // the same arithmetic on the instance's own rows, and a query's row involves only
         // itself, so every result is independent of the chunking and of the other queries.
         const bool border = kEmu && c.b.want_var && c.qmax > 0;
-        const int Ntr = ((N + 31) & ~31) >> 3;  // first appended row tile
         for (int64_t cq0 = q0;;) {
             const int64_t cq1 = border ? min(q1, cq0 + (int64_t)c.qmax) : q1;
             const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, border ? (int)(cq1 - cq0) : 0,
@@ -1581,8 +1660,7 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                         double u = 0.0;
                         if (c.b.want_var) {
                             if (border) {  // the Schur complement's diagonal entry, clamped at 0
-                                const int a = (int)(p - cq0), ta = Ntr + (a >> 3);
-                                u = fmax(0.0, double_of_fix(__double_as_longlong(s.A[tix(ta, ta) + te(a & 7, a & 7)])));
+                                u = fmax(0.0, double_of_fix(emu_query_diag(c)[p - cq0]));
                             } else {
                                 u = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
                             }
@@ -1922,8 +2000,12 @@ SolveKernel pick_solve(bool props, bool emu) {
     return emu ? k_solve_emu<false> : k_solve<false>;
 }
 
-// seven bf16 slices of a block's columns, the row scale, and one row of diagonal-tile inverses
-constexpr int64_t kEmuBytesPerRow = 7 * 8 * kEB * 2 + 8 + 64;
+// seven bf16 slices of a block's columns, the row scale, one row of diagonal-tile inverses, and an
+// appended query row's diagonal entry
+constexpr int64_t kEmuBytesPerRow = 7 * 8 * kEB * 2 + 8 + 64 + 8;
+
+// Words of a matrix of `rows` rows in a CTA's workspace (rows: a multiple of 8).
+int64_t matrix_words(bool emu, int rows) { return emu ? n_blocks(rows) * 1024 : n_tiles(rows / 8) * 64; }
 
 // Chunk planning of a solve (see k_chunk_plan): heavy evaluation, and the bordered emulated
 // bucket's bound (kBorderQ queries appended at a time).  False when no launch splits.
@@ -1936,14 +2018,12 @@ bool chunk_args(const SolveBatch& b, const DevParams& P, bool bw, ChunkPlanArgs&
 }
 
 // Emulated launch with the latent variance: the queries of an instance (up to kBorderQ) are
-// appended to its matrix, which is padded to a multiple of 32 rows (see fit_instance); the
-// workspaces hold npad + kBorderQ rows.  Otherwise npad rows.
+// appended to its matrix (see fit_instance); the workspaces hold npad + kBorderQ rows, npad a
+// multiple of 32 (the matrix is stored in 32x32 blocks).  Otherwise npad rows.
 void emu_rows_for(bool emu, const SolveBatch& b, int& npad, int& qmax, int& nrow) {
     qmax = 0;
-    if (emu && b.want_var) {
-        npad = (npad + 31) & ~31;
-        qmax = kBorderQ;
-    }
+    if (emu) npad = (npad + 31) & ~31;
+    if (emu && b.want_var) qmax = kBorderQ;
     nrow = npad + qmax;
 }
 
@@ -2073,7 +2153,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         }
         s.grid = (int)std::min<int64_t>(n, (int64_t)n_sm * per_sm);
         ca.slots[i] = s.grid;
-        if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, n_tiles(s.nrow / 8) * 64 * s.grid);
+        if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
         if (b.want_var) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
         if (s.emu) ws_e_need = std::max<int64_t>(ws_e_need, (int64_t)s.nrow * kEmuBytesPerRow * s.grid);
     }
@@ -2126,7 +2206,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         c.stage_panel = s.stage;
         c.qmax = s.qmax;
         c.nrow = s.nrow;
-        c.ws_a_stride = s.smem_a ? 0 : n_tiles(s.nrow / 8) * 64;
+        c.ws_a_stride = s.smem_a ? 0 : matrix_words(s.emu, s.nrow);
         c.ws_a = s.smem_a ? nullptr : ws_a;
         c.ws_v_stride = (int64_t)s.npad * s.threads;
         c.ws_v = ws_v;
@@ -2258,7 +2338,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         constexpr int kRowsMax = 1024 + kBorderQ;
         int* ctr = (int*)ar.get(Arena::kCounters, sizeof(int) * n, st);
         uint8_t* ws_e = P.emulate ? (uint8_t*)ar.get(Arena::kWs3, kRowsMax * kEmuBytesPerRow, st) : nullptr;
-        double* ws_a = (double*)ar.get(Arena::kWs0, sizeof(double) * n_tiles(kRowsMax / 8) * 64, st);
+        double* ws_a = (double*)ar.get(Arena::kWs0, sizeof(double) * matrix_words(true, kRowsMax), st);
         double* ws_v = b.want_var ? (double*)ar.get(Arena::kWs1, sizeof(double) * 1024 * 512, st) : nullptr;
         if (!ctr || !ws_a || (P.emulate && !ws_e) || (b.want_var && !ws_v)) {
             if (profile) {
@@ -2296,7 +2376,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             c.ws_e_stride = emu ? (int64_t)c.nrow * kEmuBytesPerRow : 0;
             c.ws_e = emu ? ws_e : nullptr;
             cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-            c.ws_a_stride = c.a_in_smem ? 0 : n_tiles(c.nrow / 8) * 64;
+            c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
             c.ws_a = c.a_in_smem ? nullptr : ws_a;
             c.ws_v_stride = (int64_t)c.npad * threads;
             c.ws_v = ws_v;
@@ -2424,7 +2504,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         // a split bucket keeps every resident CTA busy; otherwise one CTA per instance at most
         const bool split = chunk_off && ca.qc[bi] > 0;
         const int grid = (int)std::min<int64_t>(split ? INT32_MAX : cnt, (int64_t)n_sm * per_sm);
-        c.ws_a_stride = c.a_in_smem ? 0 : n_tiles(c.nrow / 8) * 64;
+        c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
         c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * grid, st);
         c.ws_v_stride = (int64_t)c.npad * threads;
         c.ws_v = (b.want_var && !bw) ? (double*)ar.get(Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
