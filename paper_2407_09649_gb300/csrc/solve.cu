@@ -67,6 +67,7 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 constexpr int kEmuThreads = 256;  // CTA size of the emulated-update kernels (two CTAs per SM)
 constexpr int kEB = 4;            // tiles (of 8 columns) per block of the emulated factorisation
 constexpr int kEK = kEB / 2;      // 16-column mma steps per block
+constexpr int kDiagTiles = kEB * (kEB + 1) / 2;
 
 struct SolveCtx {
     SolveBatch b;
@@ -112,12 +113,15 @@ struct Shared {
     double* pa[4];  // property weights per channel (property mode): channels 0 and 1 reuse the
                     // distance alpha and its FP32 copies, which that mode does not use
     double* Tblk;   // [kEB][64] inverses of the diagonal tiles of the current block
+    unsigned* dtab; // [8][32] entries of the diagonal tiles' updates (diag_entry)
+    double* Dblk;   // [kDiagTiles][64] the current block's diagonal tiles (packed lower triangle)
     double* Wsc;    // [warps][64] per-warp tile scratch (layout changes between mma operands)
     unsigned char* stage;  // emulated kernel: slice operands of the tensor-core updates (aliases
                            // X .. alf_lo, which the factorisation does not use; reloaded after it)
     float* qw;             // emulated kernel: [kBorderQ][3] world coordinates of appended queries (FP32;
                            // NaN: not finite); lattice instances: [0] the lattice code's bits, [1] NaN
                            // when not finite
+    double* Dsol;          // emulated kernel: [2][kDiagTiles][64] a group's diagonal tiles in the solves
     float* Xw;             // emulated kernel: [npad][3] world coordinates of the points (FP32, exact)
     float2* Tff;           // emulated kernel: 2^(j/256), j = 0..255, as float pairs
 };
@@ -129,9 +133,11 @@ constexpr int kBandT = 16;
 constexpr int kColT = 4;
 constexpr int kSliceBytes = 2 * 2 * 128;           // one slice of a row tile: 2 K halves x 2 core matrices
 constexpr int kSliceTileBytes = 7 * kSliceBytes;   // the 7 slices of a row tile
-// staging: the band's slices (A), and two buffers of the column tile's (B)
+// Slices in the workspace and of a column tile (B): [group of kColT row tiles][slice][row tile], so a
+// column tile is one contiguous copy.  The band's slices (A) are staged [slice][row tile].
+constexpr int kGroupBytes = kColT * kSliceTileBytes;
 constexpr int kStageA = kBandT * kSliceTileBytes;
-constexpr int kStageB = kColT * kSliceTileBytes;
+constexpr int kStageB = kGroupBytes;
 constexpr int kStageBytes = kStageA + 2 * kStageB;
 constexpr int kEmuTmemCols = 8 * 8 * kColT;    // 8 slice groups x 32 FP32 columns
 // Latent variance in the emulated kernel: up to kBorderQ queries of an instance append their
@@ -145,8 +151,8 @@ constexpr int kEmuCtasPerSm = 512 / kEmuTmemCols;  // CTAs whose tensor memory f
 
 __host__ __device__ __forceinline__ size_t align128(size_t x) { return (x + 127) & ~(size_t)127; }
 __host__ __device__ __forceinline__ size_t emu_fixed_bytes(int npad) {
-    // invd, T256, Tblk, Wsc, Tff
-    return align128((size_t)(npad + 256 + kEB * 64 + 8 * 64 + 256) * sizeof(double));
+    // invd, T256, Tblk, Wsc, Tff, Dblk, dtab
+    return align128((size_t)(npad + 256 + kEB * 64 + 8 * 64 + 256 + kDiagTiles * 64 + 128) * sizeof(double));
 }
 __host__ __device__ __forceinline__ size_t emu_point_bytes(int npad, int nprop, bool lattice) {
     return (size_t)5 * npad * sizeof(double) + (size_t)5 * npad * sizeof(float) +
@@ -190,6 +196,10 @@ __device__ Shared carve_emu(double* sm, int npad, double* ws_a, int nprop, bool 
     s.Xw = lattice ? nullptr : after;
     s.qw = lattice ? after : after + 3 * npad;
     s.Tff = reinterpret_cast<float2*>(s.Wsc + 8 * 64);
+    s.Dblk = s.Wsc + 8 * 64 + 256;
+    s.dtab = reinterpret_cast<unsigned*>(s.Dblk + kDiagTiles * 64);
+    // the solves' diagonal tiles go where the world coordinates were (used by the assembly only)
+    s.Dsol = reinterpret_cast<double*>(after);
     return s;
 }
 
@@ -211,6 +221,9 @@ __device__ Shared carve(double* sm, int npad, int a_in_smem, double* ws_a, int n
     double* end = s.T256 + 256;
     s.Tblk = nullptr;
     s.Wsc = nullptr;
+    s.Dblk = nullptr;
+    s.Dsol = nullptr;
+    s.dtab = nullptr;
     if (a_in_smem) {
         s.A = end;
         end += n_tiles(npad / 8) * 64;
@@ -276,16 +289,10 @@ __device__ __forceinline__ double double_of_fix(long long f) {
 __device__ __forceinline__ long long fix_of_float(float x, int e) {
     const unsigned b = __float_as_uint(x);
     const int ex = (int)((b >> 23) & 255);
-    if (ex == 0) return 0;
-    const long long mant = (long long)((b & 0x7FFFFFu) | 0x800000u);
+    const unsigned mant = ex == 0 ? 0u : (b & 0x7FFFFFu) | 0x800000u;
     const int sh = ex - 150 + e;  // |x| = mant 2^(ex - 150)
-    long long v;
-    if (sh >= 0)
-        v = mant << sh;
-    else if (sh >= -25)
-        v = ((mant >> (-sh - 1)) + 1) >> 1;
-    else
-        v = 0;
+    const long long v = sh >= 0 ? (long long)((unsigned long long)mant << (sh & 63))
+                                : (long long)(((mant >> min(-sh - 1, 31)) + 1) >> 1);
     return (b >> 31) ? -v : v;
 }
 
@@ -332,7 +339,7 @@ __device__ __forceinline__ long long kfix_ff(const float a[3], const float b[3],
     }
     const float yh = __fmul_rn(S, ch);
     const float yl = __fadd_rn(__fmaf_rn(S, ch, -yh), __fmaf_rn(S, cl, __fmul_rn(E, ch)));
-    if (!(yh <= 43.5f)) return 0;
+    // (no branch on yh > 43.5: the entries of a strip then run interleaved)
     const float n = rintf(__fmul_rn(yh, kInvL));
     const int ni = (int)n;
     // r = (n kL0 - yh) + n kL1 - yl + n kL2, the large parts summed error-free
@@ -355,7 +362,8 @@ __device__ __forceinline__ long long kfix_ff(const float a[3], const float b[3],
     const float2 T = tab[(256 - j) & 255];
     const float vh = __fmul_rn(T.x, eh);
     const float vl = __fadd_rn(__fmaf_rn(T.x, eh, -vh), __fmaf_rn(T.x, el, __fmul_rn(T.y, eh)));
-    return fix_of_float(vh, kFixBits - m) + fix_of_float(vl, kFixBits - m);
+    const long long k = fix_of_float(vh, kFixBits - m) + fix_of_float(vl, kFixBits - m);
+    return yh <= 43.5f ? k : 0;
 }
 
 // The float pair (hi, lo) of an FP64 value.
@@ -412,147 +420,219 @@ __device__ void chol_solve(const Shared& s, const double* A, int Nt, double* out
     }
 }
 
-// Solve (L L^T) x = rhs in place on s.z (x written to out) with the inverses of every diagonal
-// tile in Tall ([Nt][64], tile layout); rows >= N of rhs must be zero.  Blocks of four tiles:
-// inside a block warp 0 alone takes each tile (its inverse times the right-hand side, eight
-// lanes) and updates the rest of the block; the rows outside the block are then updated by
-// the whole CTA, two barriers per block and side.
-__device__ void chol_solve_inv(const Shared& s, const double* A, int Nt, double* out, const double* Tall) {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+// Start copying the tiles of the group of tile rows B0 .. B1 - 1 (at most kEB) that a solve takes one
+// after the other into shared memory: the off-diagonal tiles (packed strict lower triangle), then
+// the inverses of the diagonal tiles.  Thread i of n; complete after cp_async_wait and a barrier.
+__device__ __forceinline__ double* solve_inverse(double* D, int k) { return D + (kDiagTiles - kEB + k) * 64; }
+__device__ __forceinline__ double* solve_tile(double* D, int i, int j) { return D + (i * (i - 1) / 2 + j) * 64; }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void load_solve_tiles(double* D, const double* A, const double* Tall, int B0, int B1, int i,
+                                                 int n) {
+    const int nb = B1 - B0;
+    for (int x = i; x < nb * (nb + 1) / 2 * 32; x += n) {
+        const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
+        const double* src = jc < ir ? A + eix(B0 + ir, B0 + jc) : Tall + 64 * (B0 + ir);
+        double* dst = jc < ir ? solve_tile(D, ir, jc) : solve_inverse(D, ir);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + 2 * (x & 31))),
+                     "l"(src + 2 * (x & 31))
+                     : "memory");
+    }
+}
+
+// Solve (L L^T) x = rhs in place on z (x written to out) with the inverses of every diagonal
+// tile in Tall ([Nt][64], tile layout); rows >= N of rhs must be zero.  Groups of four tiles, one
+// barrier per group and side.  A group's own solve is one dependent chain (64 FP64 operations of
+// about 73 clocks, and 32 more for the previous group's part of its rows), so warp 0 does only that,
+// from shared memory and from a row of 32 values loaded a group ahead, while the other warps take
+// the previous group's solution out of the rows beyond and load the next group's tiles.  Every
+// entry's operations keep one order: group by group, tile by tile.
+__device__ __noinline__ void chol_solve_inv(double* z, double* Dsol, const double* A, int Nt, double* out,
+                                            const double* Tall) {
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int Np = Nt * 8;
-    double* z = s.z;
-    for (int B0 = 0; B0 < Nt; B0 += 4) {
-        const int B1 = min(B0 + 4, Nt);
-        if (tid < 32) {
-            for (int kt = B0; kt < B1; ++kt) {
-                const double* Ti = Tall + 64 * kt;
+    double row[4 * 8];  // warp 0: this lane's row (column) of the tiles that meet the previous group
+    load_solve_tiles(Dsol, A, Tall, 0, min(kEB, Nt), tid, nt);
+    cp_async_wait();
+    __syncthreads();
+    for (int B0 = 0, par = 0; B0 < Nt; B0 += kEB, par ^= 1) {  // L y = rhs
+        const int B1 = min(B0 + kEB, Nt);
+        double* D = Dsol + par * kDiagTiles * 64;
+        if (warp == 0) {
+            const int i = 8 * B0 + lane;  // the group's rows less the previous group's part
+            if (B0 > 0 && i < 8 * B1) {
+                double u = z[i];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) u -= row[e] * z[8 * (B0 - kEB) + e];
+                z[i] = u;
+            }
+            const int in = 8 * B1 + lane;
+            if (in < Np) {
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) {
+                    const double2 v = *reinterpret_cast<const double2*>(A + eix(in >> 3, B0 + (e >> 3)) + te(in & 7, e & 7));
+                    row[e] = v.x;
+                    row[e + 1] = v.y;
+                }
+            }
+            __syncwarp();
+            for (int k = 0; k < B1 - B0; ++k) {
+                const double* Ti = solve_inverse(D, k);
+                double* zk = z + 8 * (B0 + k);
                 double v = 0.0;
                 if (lane < 8)
-                    for (int c2 = 0; c2 <= lane; ++c2) v += Ti[te(lane, c2)] * z[8 * kt + c2];
+#pragma unroll
+                    for (int c2 = 0; c2 < 8; ++c2)
+                        if (c2 <= lane) v += Ti[te(lane, c2)] * zk[c2];
                 __syncwarp();
-                if (lane < 8) z[8 * kt + lane] = v;
+                if (lane < 8) zk[lane] = v;
                 __syncwarp();
-                const int i = 8 * (kt + 1) + lane;  // rows of the block below tile kt
-                if (i < 8 * B1) {
-                    const double* T = A + eix(i >> 3, kt);
+                const int il = 8 * (k + 1) + lane;  // rows of the group below tile k
+                if (il < 8 * (B1 - B0)) {
+                    const double* T = solve_tile(D, il >> 3, k);
+                    const int r = il & 7;
+                    double u = z[8 * B0 + il];
+#pragma unroll
+                    for (int c2 = 0; c2 < 8; ++c2) u -= T[te(r, c2)] * zk[c2];
+                    z[8 * B0 + il] = u;
+                }
+                __syncwarp();
+            }
+        } else {
+            if (B1 < Nt)
+                load_solve_tiles(Dsol + (par ^ 1) * kDiagTiles * 64, A, Tall, B1, min(B1 + kEB, Nt), tid - 32, nt - 32);
+            if (B0 > 0)
+                for (int i = 8 * B1 + tid - 32; i < Np; i += nt - 32) {
                     const int r = i & 7;
                     double u = z[i];
 #pragma unroll
-                    for (int c2 = 0; c2 < 8; ++c2) u -= T[te(r, c2)] * z[8 * kt + c2];
+                    for (int k = 0; k < kEB; ++k) {
+                        const double* T = A + eix(i >> 3, B0 - kEB + k);
+                        const double* zk = z + 8 * (B0 - kEB + k);
+#pragma unroll
+                        for (int c2 = 0; c2 < 8; ++c2) u -= T[te(r, c2)] * zk[c2];
+                    }
                     z[i] = u;
                 }
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        for (int i = 8 * B1 + tid; i < Np; i += nt) {
-            const int r = i & 7;
-            double u = z[i];
-            for (int kt = B0; kt < B1; ++kt) {
-                const double* T = A + eix(i >> 3, kt);
-#pragma unroll
-                for (int c2 = 0; c2 < 8; ++c2) u -= T[te(r, c2)] * z[8 * kt + c2];
-            }
-            z[i] = u;
+            cp_async_wait();
         }
         __syncthreads();
     }
-    for (int B1 = Nt; B1 > 0; B1 -= 4) {
-        const int B0 = max(B1 - 4, 0);
-        if (tid < 32) {
-            for (int kt = B1 - 1; kt >= B0; --kt) {
-                const double* Ti = Tall + 64 * kt;
+    // L^T x = y, groups of kEB tiles from the last tile on
+    load_solve_tiles(Dsol, A, Tall, max(Nt - kEB, 0), Nt, tid, nt);
+    cp_async_wait();
+    __syncthreads();
+    for (int B1 = Nt, par = 0; B1 > 0; B1 -= kEB, par ^= 1) {
+        const int B0 = max(B1 - kEB, 0);
+        double* D = Dsol + par * kDiagTiles * 64;
+        if (warp == 0) {
+            const int j = 8 * B0 + lane;  // the group's columns less the next group's part
+            if (B1 < Nt && j < 8 * B1) {
+                double u = z[j];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) u -= row[e] * out[8 * B1 + e];
+                z[j] = u;
+            }
+            // for the group before: the columns of its tiles that meet this (full) group
+            const int P0 = max(B0 - kEB, 0), jn = 8 * P0 + lane;
+            if (jn < 8 * B0) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) row[e] = A[eix(B0 + (e >> 3), jn >> 3) + te(e & 7, jn & 7)];
+            }
+            __syncwarp();
+            for (int k = B1 - B0 - 1; k >= 0; --k) {
+                const double* Ti = solve_inverse(D, k);
+                const int kt = B0 + k;
                 double v = 0.0;
                 if (lane < 8)
-                    for (int r = lane; r < 8; ++r) v += Ti[te(r, lane)] * z[8 * kt + r];
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        if (r >= lane) v += Ti[te(r, lane)] * z[8 * kt + r];
                 __syncwarp();
                 if (lane < 8) out[8 * kt + lane] = v;
                 __syncwarp();
-                const int j = 8 * B0 + lane;  // columns of the block left of tile kt
-                if (j < 8 * kt) {
-                    const double* T = A + eix(kt, j >> 3);
-                    const int cj = j & 7;
-                    double u = z[j];
+                if (lane < 8 * k) {  // columns of the group left of tile k
+                    const double* T = solve_tile(D, k, lane >> 3);
+                    const int cj = lane & 7;
+                    double u = z[8 * B0 + lane];
 #pragma unroll
                     for (int c2 = 0; c2 < 8; ++c2) u -= T[te(c2, cj)] * out[8 * kt + c2];
-                    z[j] = u;
+                    z[8 * B0 + lane] = u;
                 }
                 __syncwarp();
             }
-        }
-        __syncthreads();
-        for (int j = tid; j < 8 * B0; j += nt) {
-            const int cj = j & 7;
-            double u = z[j];
-            for (int kt = B0; kt < B1; ++kt) {
-                const double* T = A + eix(kt, j >> 3);
+        } else {
+            if (B0 > 0)
+                load_solve_tiles(Dsol + (par ^ 1) * kDiagTiles * 64, A, Tall, max(B0 - kEB, 0), B0, tid - 32, nt - 32);
+            if (B1 < Nt)
+                for (int j = tid - 32; j < 8 * B0; j += nt - 32) {
+                    const int cj = j & 7;
+                    double u = z[j];
 #pragma unroll
-                for (int c2 = 0; c2 < 8; ++c2) u -= T[te(c2, cj)] * out[8 * kt + c2];
-            }
-            z[j] = u;
+                    for (int k = 0; k < kEB; ++k) {
+                        const double* T = A + eix(B1 + k, j >> 3);
+                        const double* ok = out + 8 * (B1 + k);
+#pragma unroll
+                        for (int c2 = 0; c2 < 8; ++c2) u -= T[te(c2, cj)] * ok[c2];
+                    }
+                    z[j] = u;
+                }
+            cp_async_wait();
         }
         __syncthreads();
     }
 }
 
-// One warp: the 8x8 Cholesky of diagonal tile kt in place (right-looking, the column scaling
-// and rank-1 updates spread over the lanes, 1 / L_jj from rsqrt), 1 / L_jj into invd and the
-// inverse of the tile's factor into Ti (rows by forward substitution, one lane per column).
-// S: 64 doubles of scratch.  False on a non-positive pivot (the same on every lane).
-__device__ bool diag_tile_warp(double* A, int kt, const Shared& s, double* Ti, double* S) {
+// Which entry of the update of step j (below) a lane takes: tab[32 j + lane] holds its place (bits
+// 0-5; bit 6: in T, else in S), the place of its factor in column j of S (bits 8-13) and that of the
+// other factor (bits 16-21, same array as the entry); bit 31: none.
+__device__ __forceinline__ unsigned diag_entry(int j, int lane) {
+    const int m = 7 - j, nc = m * (m + 1) / 2;  // pairs of rows of S, then rows and columns of T
+    if (lane >= nc + m * (j + 1)) return 1u << 31;
+    if (lane < nc) {
+        const int a = tri_row(lane), r = j + 1 + a, c = j + 1 + lane - a * (a + 1) / 2;
+        return (unsigned)(te(r, c) | te(r, j) << 8 | te(c, j) << 16);
+    }
+    const int q = lane - nc, r = j + 1 + q / (j + 1), c = q % (j + 1);
+    return (unsigned)(te(r, c) | 64 | te(r, j) << 8 | te(j, c) << 16);
+}
+
+// One warp: the 8x8 Cholesky of the diagonal tile S in place (lower part), 1 / L_jj from rsqrt into
+// invd, and the inverse of its factor into T (upper part zero).  One pass over the tile and the
+// identity beside it: step j scales column j of S and row j of T by 1 / L_jj in one operation and
+// takes their products out of the rows below in one more (two where they are over 32).  An FP64
+// operation holds its sub-partition for about 66 clocks however few lanes are on, so what
+// counts is their number: about 8 a step, against 10 and 36 for the inverse after it.  False on a
+// non-positive pivot (the same on every lane).
+__device__ __forceinline__ bool diag_tile_warp(double* S, double* T, double* invd, const unsigned* tab) {
     const int lane = threadIdx.x & 31;
-    double* D = A + eix(kt, kt);
-    S[lane] = D[lane];
-    S[lane + 32] = D[lane + 32];
+    T[lane] = 0.0;
+    T[lane + 32] = 0.0;
     __syncwarp();
+#pragma unroll 1
     for (int j = 0; j < 8; ++j) {
+        const unsigned e = tab[32 * j + lane];
+        double* const M = e & 64 ? T : S;
+        // the lane's entry of the scaling: S_ij for lanes i = j .. 7, T_jc for lanes 8 + c, c <= j
+        double* const xs = lane < 8 ? S + te(lane, j) : T + te(j, lane & 7);
+        const bool on = lane < 8 ? lane >= j : lane <= 8 + j;
         const double v = S[te(j, j)];
+        double x = on ? *xs : 0.0;
+        if (lane == 8 + j) x = 1.0;
         if (!(v > 0.0)) return false;
         const double r = rsqrt(v);
+        const double y = x * r;
         __syncwarp();
-        if (lane > j && lane < 8) S[te(lane, j)] *= r;
-        if (lane == 0) {
-            S[te(j, j)] = v * r;
-            s.invd[8 * kt + j] = r;
-        }
+        if (on) *xs = y;
+        if (lane == 0) invd[j] = r;
         __syncwarp();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {  // entries (rr, cc), j < cc <= rr
-            const int e = lane + 32 * h, rr = e >> 3, cc = e & 7;
-            if (cc > j && rr >= cc) S[te(rr, cc)] -= S[te(rr, j)] * S[te(cc, j)];
-        }
-        __syncwarp();
-    }
-    D[lane] = S[lane];
-    D[lane + 32] = S[lane + 32];
-    // Ti = L^-1: Ti_ii = 1 / L_ii, Ti_ic = -(sum_{c <= k < i} L_ik Ti_kc) / L_ii for c < i
-    for (int i = 0; i < 8; ++i) {
-        if (lane < 8) {
-            double u = lane == i ? 1.0 : 0.0;
-            for (int k = lane; k < i; ++k) u -= S[te(i, k)] * Ti[te(k, lane)];
-            Ti[te(i, lane)] = lane <= i ? u * s.invd[8 * kt + i] : 0.0;
+        if (!(e >> 31)) M[e & 63] -= S[(e >> 8) & 63] * M[(e >> 16) & 63];
+        if (j < 2 && lane < 3 - 2 * j) {  // the entries of T beyond 32: (5 .. 7, 0) and (7, 1)
+            const int r2 = j == 0 ? 5 + lane : 7;
+            T[te(r2, j)] -= S[te(r2, j)] * T[te(j, j)];
         }
         __syncwarp();
     }
     return true;
-}
-
-// Panel column kt: L_it,kt = A_it,kt Ti^T for kt < it < it_end (Ti: inverse of the diagonal
-// tile's factor), one tile per warp.
-__device__ void panel_column(double* A, int kt, int it_end, const double* Ti) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    for (int it = kt + 1 + warp; it < it_end; it += nwarps) {
-        double* T = A + eix(it, kt);
-        const double a0 = T[te(g, t)], a1 = T[te(g, 4 + t)];
-        const double b0 = Ti[te(g, t)], b1 = Ti[te(g, 4 + t)];
-        double c0 = 0.0, c1 = 0.0;
-        dmma(c0, c1, a0, b0);
-        dmma(c0, c1, a1, b1);
-        __syncwarp();
-        T[te(g, 2 * t)] = c0;
-        T[te(g, 2 * t + 1)] = c1;
-    }
 }
 
 // w 2^sh rounded to an integer (ties up) for a 64-bit integer w: a slice-product update in
@@ -580,9 +660,9 @@ __device__ __forceinline__ long long join_groups(const unsigned (&g)[8]) {
 
 // Balanced base-256 digits of row g of an 8-row tile over one block (the FP64 values
 // x[0 .. 2 kEB - 1] held by the four lanes t of the row: columns 8 j + 2t and 8 j + 2t + 1 in
-// x[2j], x[2j + 1]), written as bf16 pairs to F in the tensor cores' K-major layout: [slice]
-// [core matrix of 8 columns][row][8 bf16], 16 bytes per row and 128 per core matrix; and the row
-// scale 2^(em - 1021) to *scale (lane t = 0).  The digit scheme is described at factor_emulated.
+// x[2j], x[2j + 1]), written as bf16 pairs to F (slices kColT kSliceBytes apart) in the tensor cores'
+// K-major layout: [core matrix of 8 columns][row][8 bf16], 16 bytes per row and 128 per core
+// matrix; and the row scale 2^(em - 1021) to *scale (lane t = 0).  The digit scheme is described at factor_emulated.
 // With u (an appended query row's diagonal entry in the fixed point, lane t = 0) the row's own
 // update |row|^2 is taken from the digits here: only the diagonal of the query-by-query block is
 // needed, and 19 integer products per column cost a tenth of the tensor-core tiles that hold it.
@@ -623,8 +703,8 @@ __device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* 
                 h16[i] = __float_as_uint((float)qv) >> 16;  // exact: |qv| <= 2^7
             }
             // lane = 4 g + t: row g, columns 2t, 2t + 1 of the core matrices of columns 0-7 and 8-15
-            F[ss * 128 + kk * 64 + lane] = h16[0] | (h16[1] << 16);
-            F[ss * 128 + kk * 64 + 32 + lane] = h16[2] | (h16[3] << 16);
+            F[ss * (kColT * kSliceBytes / 4) + kk * 64 + lane] = h16[0] | (h16[1] << 16);
+            F[ss * (kColT * kSliceBytes / 4) + kk * 64 + 32 + lane] = h16[2] | (h16[3] << 16);
         }
         if (u) {  // G_g += sum_{s+t=g} q_s q_t of each column (the sign drops out)
 #pragma unroll
@@ -659,14 +739,14 @@ __device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* 
     }
 }
 
-// Row tile it below the factorised diagonal block of tile columns K0 .. K0 + kEB - 1 (inverses
-// of its diagonal tiles in Tblk): L_it,K0+j = (A_it,K0+j - sum_{k<j} L_it,K0+k L_K0+j,K0+k^T)
+// Row tile it below the factorised diagonal block of tile columns K0 .. K0 + kEB - 1 (its tiles in
+// Dblk, the inverses of its diagonal tiles in Tblk): L_it,K0+j = (A_it,K0+j - sum_{k<j} L_it,K0+k L_K0+j,K0+k^T)
 // Ti_j^T for j < kEB on the FP64 tensor path, one warp, the row's tiles in registers.  The warp's
 // scratch tile W turns each result from the accumulator into the operand layout.  The
 // results are stored to A and sliced for the trailing update (F, scale: this tile's slices
 // and row scales; u: the diagonal entries of an appended query tile's rows, else null).
-__device__ void block_rows(double* A, int it, int K0, const double* Tblk, double* W, uint32_t* F, double* scale,
-                           long long* u) {
+__device__ void block_rows(double* A, int it, int K0, const double* Dblk, const double* Tblk, double* W,
+                           uint32_t* F, double* scale, long long* u) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     double* R = A + eix(it, K0);  // tiles (it, K0 .. K0 + kEB - 1), kTileCol apart
     double x[2 * kEB];            // accumulator layout: tile j holds columns 2t, 2t + 1 of row g
@@ -679,11 +759,11 @@ __device__ void block_rows(double* A, int it, int K0, const double* Tblk, double
 #pragma unroll
     for (int j = 0; j < kEB; ++j) {
         double a0 = x[2 * j], a1 = x[2 * j + 1];
-        const double* Lj = A + eix(K0 + j, K0);  // tiles (K0 + j, K0 .. K0 + j)
+        const double* Lj = Dblk + j * (j + 1) / 2 * 64;  // tiles (K0 + j, K0 .. K0 + j)
 #pragma unroll
         for (int k = 0; k < j; ++k) {
-            dmma(a0, a1, neg(xa[k][0]), Lj[kTileCol * k + te(g, t)]);
-            dmma(a0, a1, neg(xa[k][1]), Lj[kTileCol * k + te(g, 4 + t)]);
+            dmma(a0, a1, neg(xa[k][0]), Lj[64 * k + te(g, t)]);
+            dmma(a0, a1, neg(xa[k][1]), Lj[64 * k + te(g, 4 + t)]);
         }
         W[te(g, 2 * t)] = a0;
         W[te(g, 2 * t + 1)] = a1;
@@ -711,7 +791,7 @@ __device__ void block_rows(double* A, int it, int K0, const double* Tblk, double
 }
 
 // Per-CTA workspace of the emulated factorisation: the slices of the rows below the current block
-// ([row tile][7 slices][4 core matrices], 3584 bytes per row tile), the row scales, the inverses of
+// ([group of 4 row tiles][slice][row tile][4 core matrices], 3584 bytes per row tile), the row scales, the inverses of
 // all diagonal tiles ([rows / 8][64] doubles), and the appended query rows' diagonal entries in
 // the fixed point.
 __device__ __forceinline__ unsigned char* emu_ws(const SolveCtx& c) { return c.ws_e + (int64_t)blockIdx.x * c.ws_e_stride; }
@@ -775,37 +855,22 @@ struct EmuTc {
     bool dead;           // a bounded wait gave up: take no more work
 };
 
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&v)[2]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The loaded values pass through the wait, so no use of them is scheduled before it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[8][2]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[2][0]), "+r"(v[2][1]),
+                   "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[5][0]), "+r"(v[5][1]),
+                   "+r"(v[6][0]), "+r"(v[6][1]), "+r"(v[7][0]), "+r"(v[7][1])::"memory");
+}
 
 // A bounded wait gave up: record it; the CTA stops taking work.
 __device__ __forceinline__ bool emu_fail(const SolveCtx& c, EmuTc& tc) {
     if (threadIdx.x == 0) atomicOr(c.err, kErrTimeout);
     tc.dead = true;
     return false;
-}
-
-// Copy the slices of nc row tiles from E into the staging buffer of a column tile (B), one warp:
-// slice by slice ([slice][row tile][512 bytes]), so that the first n slices of the column tile are
-// n * 32 consecutive rows of the MMA's N dimension.  The mbarrier counts `extra` bytes more (the
-// band's A).
-__device__ __forceinline__ void stage_columns(unsigned char* dst, const unsigned char* E, int nc, uint32_t extra,
-                                              uint32_t bar) {
-    const int lane = threadIdx.x & 31;
-    if (lane == 0)
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                     "r"((uint32_t)nc * kSliceTileBytes + extra)
-                     : "memory");
-    __syncwarp();
-    if (lane < 7 * kColT) {
-        const int ss = lane / kColT, rt = lane % kColT;
-        if (rt < nc)
-            bulk_load(dst + (ss * kColT + rt) * kSliceBytes, E + (int64_t)rt * kSliceTileBytes + ss * kSliceBytes,
-                      kSliceBytes, bar);
-    }
 }
 
 // Trailing update C -= P P^T of the M = Nt - K1 row tiles below the block that ends at K1, on
@@ -837,13 +902,23 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
     const int q = warp & 3, h = warp >> 2;  // lane quadrant (rows 32 q ..) and column half
     const int kb1 = K1 >> 2;                // 32-row block of the first row below (K1 is a multiple of 4)
     int fail = 0;
-    auto stage_band = [&](int b0) {  // the band's A and the first column tile's B (buffer 0); warp 0
-        const int nb = min(kBandT, M - b0);
-        if (lane == 0)
-            bulk_load(stage, E + (int64_t)b0 * kSliceTileBytes, (uint32_t)nb * kSliceTileBytes, tc.bar_ld);
-        stage_columns(stage + kStageA, E, min(kColT, Ntr - K1), (uint32_t)nb * kSliceTileBytes, tc.bar_ld);
+    // the band's A (warp w: slice w, a lane per group of 4 row tiles) and the first column tile's B
+    // (buffer 0, warp 7, which also arms the barrier)
+    auto stage_band = [&](int b0) {
+        const int ng = (min(kBandT, M - b0) + kColT - 1) / kColT;
+        const unsigned char* G = E + (int64_t)(b0 / kColT) * kGroupBytes;
+        if (warp < 7) {
+            if (lane < ng)
+                bulk_load(stage + warp * (kStageA / 7) + lane * (kStageB / 7), G + (int64_t)lane * kGroupBytes + warp * (kStageB / 7),
+                          kStageB / 7, tc.bar_ld);
+        } else if (lane == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
+                         "r"((uint32_t)(ng + 1) * kGroupBytes)
+                         : "memory");
+            bulk_load(stage + kStageA, E, kStageB, tc.bar_ld);
+        }
     };
-    if (warp == 0) stage_band(0);
+    stage_band(0);
     for (int b0 = 0; b0 < M; b0 += kBandT) {
         const int nb = min(kBandT, M - b0);
         const int rb = (b0 >> 2) + q;              // the warp's 32-row block below K1
@@ -853,77 +928,83 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
         const int n_tiles = min(jr, (b0 + nb + kColT - 1) / kColT);  // column tiles reaching the band's last row
         for (int jt = 0; jt < n_tiles; ++jt) {
             const uint32_t bufB = aB + (uint32_t)((jt & 1) * kStageB);
-            // warp 0 alone waits for the copies, issues the products and then the next copies: every
-            // phase of the copy barrier is seen before the next one can start
-            if (warp == 0 && !bar_poll(tc.bar_ld, tc.ph_ld)) fail = 1;
-            if (warp == 0 && !__any_sync(0xffffffffu, fail)) {
-                if (lane == 0) {
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-                    for (int kh = 0; kh < 2; ++kh)
-#pragma unroll
-                        for (int ss = 0; ss < 7; ++ss) {
-                            const int n = ss == 0 ? 7 : 8 - ss;  // B slices of this product
-                            const uint64_t da = umma_desc(aA + ss * kSliceBytes + kh * 256, 128, kSliceTileBytes);
-                            const uint32_t b = bufB + kh * 256;
-                            const uint32_t dcol = tc.tmem + ss * 8 * kColT;
-                            if (kh == 0 && ss == 1) {
-                                // groups 1 .. 6 hold slice 0's products; group 7 starts here
-                                umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), 6 * 8 * kColT, 1u);
-                                umma_bf16(dcol + 6 * 8 * kColT, da, umma_desc(b + 6 * kColT * kSliceBytes, 128, kSliceBytes),
-                                          8 * kColT, 0u);
-                            } else {
-                                umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), n * 8 * kColT,
-                                          (kh == 0 && ss == 0) ? 0u : 1u);
-                            }
-                        }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     tc.bar_mma)
-                                 : "memory");
-                }
-                __syncwarp();
-                if (jt + 1 < n_tiles)  // the next column tile's B into the other buffer
-                    stage_columns(stage + kStageA + ((jt + 1) & 1) * kStageB,
-                                  E + (int64_t)(jt + 1) * kColT * kSliceTileBytes,
-                                  min(kColT, Ntr - K1 - (jt + 1) * kColT), 0, tc.bar_ld);
-            }
-            tc.ph_ld ^= 1;
-            // while the MMAs run: this thread's 16 entries of C (one row, 16 columns) and the column
-            // scales, all loads issued at once
+            // this thread's 16 entries of C (one row, 16 columns) and the column scales, all loads
+            // issued at once; they arrive while the MMAs run
             const bool on = rows_in && jt <= rb;  // (warp-uniform, as the collective tcgen05.ld needs)
             long long* C = reinterpret_cast<long long*>(A + bix(kb1 + rb, kb1 + jt)) + 512 * h;
             long long cv[16];
-            int es = 0;
+            double es = 0.0;
             if (on) {
 #pragma unroll
                 for (int cc = 0; cc < 16; ++cc) cv[cc] = C[32 * cc + lane];
-                es = (int)(__double_as_longlong(sr[32 * jt + 16 * h + (lane & 15)]) >> 52);
+                es = sr[32 * jt + 16 * h + (lane & 15)];
                 if (jt + 1 < n_tiles && jt < rb && lane == 0)
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024), "r"(4096));
             }
+            // warp 0 alone waits for the copies, starts the next ones and issues the products: every
+            // phase of the copy barrier is seen before the next one can start
+            if (warp == 0 && !bar_poll(tc.bar_ld, tc.ph_ld)) fail = 1;
+            if (warp == 0 && !__any_sync(0xffffffffu, fail) && lane == 0) {
+                if (jt + 1 < n_tiles) {  // the next column tile's B into the other buffer
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
+                                 "r"((uint32_t)kStageB)
+                                 : "memory");
+                    bulk_load(stage + kStageA + ((jt + 1) & 1) * kStageB, E + (int64_t)(jt + 1) * kGroupBytes, kStageB,
+                              tc.bar_ld);
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+                    for (int ss = 0; ss < 7; ++ss) {
+                        const int n = ss == 0 ? 7 : 8 - ss;  // B slices of this product
+                        const uint64_t da = umma_desc(aA + ss * (kStageA / 7) + kh * 256, 128, kSliceBytes);
+                        const uint32_t b = bufB + kh * 256;
+                        const uint32_t dcol = tc.tmem + ss * 8 * kColT;
+                        if (kh == 0 && ss == 1) {
+                            // groups 1 .. 6 hold slice 0's products; group 7 starts here
+                            umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), 6 * 8 * kColT, 1u);
+                            umma_bf16(dcol + 6 * 8 * kColT, da, umma_desc(b + 6 * kColT * kSliceBytes, 128, kSliceBytes),
+                                      8 * kColT, 0u);
+                        } else {
+                            umma_bf16(dcol, da, umma_desc(b, 128, kSliceBytes), n * 8 * kColT, (kh == 0 && ss == 0) ? 0u : 1u);
+                        }
+                    }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc.bar_mma)
+                             : "memory");
+            }
+            __syncwarp();
+            tc.ph_ld ^= 1;
+            const int ec_lane = (int)(__double_as_longlong(es) >> 52);
             if (!bar_poll(tc.bar_mma, tc.ph_mma)) fail = 1;
             tc.ph_mma ^= 1;
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // the band's last products are done: its A and B buffers take the next band's
-            if (warp == 0 && !__any_sync(0xffffffffu, fail) && jt + 1 == n_tiles && b0 + kBandT < M) stage_band(b0 + kBandT);
+            // the band's last products are done (so warp 0 has seen every copy): its A and B buffers
+            // take the next band's
+            if (!__any_sync(0xffffffffu, fail) && jt + 1 == n_tiles && b0 + kBandT < M) stage_band(b0 + kBandT);
             if (on) {
+                // two columns at a time, the next two read from tensor memory meanwhile
+                uint32_t v[2][8][2];
+                const uint32_t tbase = tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(16 * h);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {  // four columns at a time
-                    uint32_t v[8][4];
+                for (int gq = 0; gq < 8; ++gq) tmem_ld2(tbase + (uint32_t)(gq * 8 * kColT), v[0][gq]);
 #pragma unroll
-                    for (int gq = 0; gq < 8; ++gq)
-                        tmem_ld4(tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(gq * 8 * kColT + 16 * h + 4 * p), v[gq]);
-                    tmem_wait_ld();
+                for (int p = 0; p < 8; ++p) {
+                    tmem_wait_ld(v[p & 1]);
+                    if (p < 7)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
+                        for (int gq = 0; gq < 8; ++gq)
+                            tmem_ld2(tbase + (uint32_t)(gq * 8 * kColT + 2 * p + 2), v[(p + 1) & 1][gq]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
                         unsigned gb[8];
 #pragma unroll
                         for (int gq = 0; gq < 8; ++gq)
-                            gb[gq] = __float_as_uint(__fadd_rn(__uint_as_float(v[gq][e]), 12582912.0f));
-                        const int ec = __shfl_sync(0xffffffffu, es, 4 * p + e);
+                            gb[gq] = __float_as_uint(__fadd_rn(__uint_as_float(v[p & 1][gq][e]), 12582912.0f));
+                        const int ec = __shfl_sync(0xffffffffu, ec_lane, 2 * p + e);
                         // the update is w 2^(er + ec - 2102), in units of 2^-kFixBits
-                        cv[4 * p + e] -= fix_shift(join_groups(gb), er + ec - (2102 - kFixBits));
+                        cv[2 * p + e] -= fix_shift(join_groups(gb), er + ec - (2102 - kFixBits));
                     }
                 }
                 // the next block's columns are final after this update: stored as FP64 tiles (see
@@ -984,41 +1065,74 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
     long long* udiag = emu_query_diag(c);
     for (int K0 = 0; K0 < Ntr; K0 += kEB) {
         const int K1 = min(K0 + kEB, Ntr);
-        // the diagonal block: tiles (it, jt), K0 <= jt <= it < K1, right-looking by 8 columns
-        for (int kt = K0; kt < K1; ++kt) {
-            double* Ti = s.Tblk + 64 * (kt - K0);
+        // the diagonal block: tiles (it, jt), K0 <= jt <= it < K1, in shared memory (packed),
+        // right-looking by 8 columns.  Warp 0 takes the diagonal tiles; its update of the next one
+        // needs no barrier after it.  The other tiles go to warps of the other sub-partitions
+        // (warp 4 shares warp 0's), so the chain of diagonal tiles has its FP64 pipe alone.
+        const int nb = K1 - K0;
+        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
+            const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
+            reinterpret_cast<double2*>(s.Dblk)[x] = reinterpret_cast<const double2*>(A + eix(K0 + ir, K0 + jc))[x & 31];
+        }
+        __syncthreads();
+        auto tile = [&](int ir, int jc) { return s.Dblk + (ir * (ir + 1) / 2 + jc) * 64; };
+        auto update = [&](int ir, int jc, int k) {  // tile (ir, jc) -= tile (ir, k) tile (jc, k)^T
+            double* C = tile(ir, jc);
+            const double* Li = tile(ir, k);
+            const double* Lj = tile(jc, k);
+            double c0 = C[te(g, 2 * t)], c1 = C[te(g, 2 * t + 1)];
+            dmma(c0, c1, neg(Li[te(g, t)]), Lj[te(g, t)]);
+            dmma(c0, c1, neg(Li[te(g, 4 + t)]), Lj[te(g, 4 + t)]);
+            C[te(g, 2 * t)] = c0;
+            C[te(g, 2 * t + 1)] = c1;
+        };
+        for (int k = 0; k < nb; ++k) {
+            const double* Ti = s.Tblk + 64 * k;
             if (warp == 0) {
-                if (diag_tile_warp(A, kt, s, Ti, s.Wsc)) {
-                    Tall[64 * kt + lane] = Ti[lane];
-                    Tall[64 * kt + lane + 32] = Ti[lane + 32];
-                } else if (lane == 0) {
+                if (k > 0) update(k, k, k - 1);
+                __syncwarp();
+                if (!diag_tile_warp(tile(k, k), s.Tblk + 64 * k, s.invd + 8 * (K0 + k), s.dtab) && lane == 0)
                     *s_fail = 1;
+            } else if (k > 0 && (warp & 3) != 0) {
+                // the tiles (ir, jc), k <= jc <= ir, but (k, k): at most 5, one for each of warps 1, 2, 3, 5, 6
+                const int m = nb - k, p = warp - (warp >> 2);
+                if (p < m * (m + 1) / 2) {
+                    const int ir = tri_row(p);
+                    update(k + ir, k + p - ir * (ir + 1) / 2, k - 1);
                 }
             }
             __syncthreads();
             if (*s_fail) return false;
-            panel_column(A, kt, K1, Ti);
-            __syncthreads();
-            const int nj = K1 - kt - 1;
-            for (int p = warp; p < nj * (nj + 1) / 2; p += nwarps) {
-                const int ir = tri_row(p), it = kt + 1 + ir, jt = kt + 1 + (p - ir * (ir + 1) / 2);
-                double* C = A + eix(it, jt);
-                const double* Li = A + eix(it, kt);
-                const double* Lj = A + eix(jt, kt);
-                double c0 = C[te(g, 2 * t)], c1 = C[te(g, 2 * t + 1)];
-                dmma(c0, c1, neg(Li[te(g, t)]), Lj[te(g, t)]);
-                dmma(c0, c1, neg(Li[te(g, 4 + t)]), Lj[te(g, 4 + t)]);
-                C[te(g, 2 * t)] = c0;
-                C[te(g, 2 * t + 1)] = c1;
+            if (k + 1 == nb) break;
+            if (warp >= 1 && warp < nb - k) {  // panel: tile (k + warp, k) Ti^T
+                double* T = tile(k + warp, k);
+                const double a0 = T[te(g, t)], a1 = T[te(g, 4 + t)];
+                const double b0 = Ti[te(g, t)], b1 = Ti[te(g, 4 + t)];
+                double c0 = 0.0, c1 = 0.0;
+                dmma(c0, c1, a0, b0);
+                dmma(c0, c1, a1, b1);
+                __syncwarp();
+                T[te(g, 2 * t)] = c0;
+                T[te(g, 2 * t + 1)] = c1;
             }
             __syncthreads();
+        }
+        // for the solves: the off-diagonal tiles and the inverses
+        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
+            const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
+            if (ir == jc)
+                reinterpret_cast<double2*>(Tall + 64 * (K0 + ir))[x & 31] = reinterpret_cast<const double2*>(s.Tblk + 64 * ir)[x & 31];
+            else
+                reinterpret_cast<double2*>(A + eix(K0 + ir, K0 + jc))[x & 31] = reinterpret_cast<const double2*>(s.Dblk)[x];
         }
         if (K1 >= Nt) break;
         // the rows below: one warp per row tile solves its four tiles against the diagonal
         // block and writes their slices (both column halves) and row scales
         for (int it = K1 + warp; it < Nt; it += nwarps)
-            block_rows(A, it, K0, s.Tblk, s.Wsc + 64 * warp,
-                       reinterpret_cast<uint32_t*>(E + (int64_t)(it - K1) * kSliceTileBytes), sr + 8 * (it - K1),
+            block_rows(A, it, K0, s.Dblk, s.Tblk, s.Wsc + 64 * warp,
+                       reinterpret_cast<uint32_t*>(E + (int64_t)((it - K1) / kColT) * kGroupBytes +
+                                                   (it - K1) % kColT * kSliceBytes),
+                       sr + 8 * (it - K1),
                        it >= Ntr ? udiag + 8 * (it - Ntr) : nullptr);
         // the slices are read by the copy engine (async proxy)
         asm volatile("fence.proxy.async;" ::: "memory");
@@ -1092,6 +1206,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         const int nbr = (Ntq + 3) >> 2, nbc = (Nt + 3) >> 2;
         const int sq = nbc * (nbc + 1) / 2;  // blocks of the matrix itself; then nbc per block of query rows
         const int n_strip = 4 * (sq + (nbr - nbc) * nbc);
+        const long long diag1 = fix_of_double(1.0 + c.P.s2);  // s2: sigma_prop^2 for properties
         for (int st = warp; st < n_strip; st += nwarps) {
             const int p = st >> 2, c0 = 8 * (st & 3);
             const int bi = p < sq ? tri_row(p) : nbc + (p - sq) / nbc;
@@ -1106,29 +1221,33 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
             if (live && !lattice)
                 for (int k = 0; k < 3; ++k) rw[k] = qrow ? s.qw[3 * a + k] : s.Xw[3 * i + k];
             long long v[8];
+            const int j0 = 32 * bj + c0;
+            // (every entry of the strip is computed, without a branch, and replaced where it is not
+            // a kernel value, so that the eight run interleaved)
+            if (lattice) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = live && j0 + e < N ? fix_of_double(c.P.lat_tab[lat_m(s.xi[j0 + e], rx)]) : 0;
+            } else if (c.P.precision == VGP_MIXED) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = kfix_ff(rw, s.Xw + 3 * (j0 + e), c.P.inv2l2_hi, c.P.inv2l2_lo, s.Tff);
+            } else if (qrow) {  // the query's FP64 local coordinates, formed as query_local forms them
+                double xq[3];
+                for (int k = 0; k < 3; ++k) xq[k] = (double)rw[k] - (c.b.centre ? c.b.centre[3 * (int64_t)I + k] : 0.0);
+                for (int e = 0; e < 8; ++e) {
+                    double r2 = 0.0;
+                    for (int k = 0; k < 3; ++k) {
+                        const double d = s.X[3 * (j0 + e) + k] - xq[k];
+                        r2 += d * d;
+                    }
+                    v[e] = fix_of_double(exp(-r2 * c.P.inv2l2));
+                }
+            } else {
+                for (int e = 0; e < 8; ++e) v[e] = j0 + e < i ? fix_of_double(kval_pair(c.P, s, false, i, j0 + e)) : 0;
+            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const int j = 32 * bj + c0 + e;
-                if (qrow ? !live || j >= N : !live || j >= N || j >= i) {
-                    v[e] = qrow || i != j ? 0 : i < N ? fix_of_double(1.0 + c.P.s2) : 1ll << kFixBits;
-                } else if (lattice) {
-                    v[e] = fix_of_double(c.P.lat_tab[lat_m(s.xi[j], rx)]);
-                } else if (c.P.precision == VGP_MIXED) {
-                    v[e] = kfix_ff(rw, s.Xw + 3 * j, c.P.inv2l2_hi, c.P.inv2l2_lo, s.Tff);
-                } else {
-                    double r2;
-                    if (qrow) {  // the query's FP64 local coordinates, formed as query_local forms them
-                        r2 = 0.0;
-                        for (int k = 0; k < 3; ++k) {
-                            const double cen = c.b.centre ? c.b.centre[3 * (int64_t)I + k] : 0.0;
-                            const double d = s.X[3 * j + k] - ((double)rw[k] - cen);
-                            r2 += d * d;
-                        }
-                        v[e] = fix_of_double(exp(-r2 * c.P.inv2l2));
-                    } else {
-                        v[e] = fix_of_double(kval_pair(c.P, s, false, i, j));
-                    }
-                }
+                const int j = j0 + e;
+                if (!live || j >= N || (!qrow && j >= i)) v[e] = qrow || i != j ? 0 : i < N ? diag1 : 1ll << kFixBits;
             }
             if (bj == 0) {
                 double* T = B + (c0 >> 3) * kTileCol + (lane >> 3) * 64;
@@ -1144,8 +1263,8 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         if (nq > 0)
             for (int a = tid; a < 8 * (Ntq - Nt); a += nt) emu_query_diag(c)[a] = 1ll << kFixBits;
     }
-    if constexpr (!kEmu)
-    for (int64_t tl = warp; tl < n_tiles(Nt); tl += nwarps) {
+    const int64_t ntl = kEmu ? 0 : n_tiles(Nt);
+    for (int64_t tl = warp; tl < ntl; tl += nwarps) {
         const int it = tri_row((int)tl), jt = (int)tl - it * (it + 1) / 2;
         for (int e = lane; e < 64; e += 32) {
             const int i = 8 * it + (e >> 3), j = 8 * jt + (e & 7);
@@ -1293,7 +1412,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
             for (int i = tid; i < Ns; i += nt) s.z[i] = i < N ? c.b.yprop[(base + i) * c.b.nprop + ch] : 0.0;
             __syncthreads();
             if (kEmu)
-                chol_solve_inv(s, A, Nts, s.pa[ch], emu_tile_inverses(c));
+                chol_solve_inv(s.z, s.Dsol, A, Nts, s.pa[ch], emu_tile_inverses(c));
             else
                 chol_solve(s, A, Nts, s.pa[ch]);
         }
@@ -1303,7 +1422,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
     for (int i = tid; i < Ns; i += nt) s.z[i] = i < N ? 1.0 : 0.0;
     __syncthreads();
     if (kEmu)
-        chol_solve_inv(s, A, Nts, s.alpha, emu_tile_inverses(c));
+        chol_solve_inv(s.z, s.Dsol, A, Nts, s.alpha, emu_tile_inverses(c));
     else
         chol_solve(s, A, Nts, s.alpha);
     for (int j = tid; j < Ns; j += nt) {
@@ -1537,6 +1656,7 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             float h, l;
             split_pair(c.P.exp_tab[j], h, l);
             s.Tff[j] = make_float2(h, l);
+            s.dtab[j] = diag_entry(j >> 5, j & 31);
         }
     EmuTc tc{};
     if (kEmu) {
@@ -1603,32 +1723,36 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
         const int64_t q0 = qch > 0 ? min(qb, qa + (int64_t)ci * qch) : qa;
         const int64_t q1 = qch > 0 ? min(qb, q0 + qch) : qb;
         if (kProps) {
-            // the variance by bordering too (see below) when the work item's queries fit the
-            // appended rows: the property GP's own matrix, noise sigma_c^2
-            const bool pb = kEmu && c.qmax > 0 && q1 - q0 <= c.qmax;
-            const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, pb ? (int)(q1 - q0) : 0, q0, I);
-            // property mode: means and variance (Eq. 6, variance read as for Eq. 2)
+            // property mode: means and variance (Eq. 6, variance read as for Eq. 2).  The emulated
+            // kernel takes the variance by bordering, chunk by chunk (see below), on the property
+            // GP's own matrix (noise sigma_c^2)
             const int np = c.b.nprop;
-            for (int64_t p = q0 + tid; p < q1; p += nt) {
-                const int64_t qid = c.b.qidx ? c.b.qidx[p] : p;
-                double xl[3], cm[4] = {NAN, NAN, NAN, NAN}, w = INFINITY;
-                int qi = 0;
-                if (ok) {
-                    query_local(c, I, p, qid, xl, &qi);
-                    if (isfinite(xl[0]) && isfinite(xl[1]) && isfinite(xl[2])) {
-                        property_mean(c.P, s, N, np, lattice, qi, xl, cm);
-                        if (pb) {
-                            w = fmax(0.0, double_of_fix(emu_query_diag(c)[p - q0]));
-                        } else {
-                            w = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
+            for (int64_t cq0 = q0;;) {
+                const int64_t cq1 = kEmu ? min(q1, cq0 + (int64_t)c.qmax) : q1;
+                const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, kEmu ? (int)(cq1 - cq0) : 0, cq0, I);
+                const int64_t ce = ok ? cq1 : q1;  // a failed factorisation answers all remaining queries
+                for (int64_t p = cq0 + tid; p < ce; p += nt) {
+                    const int64_t qid = c.b.qidx ? c.b.qidx[p] : p;
+                    double xl[3], cm[4] = {NAN, NAN, NAN, NAN}, w = INFINITY;
+                    int qi = 0;
+                    if (ok) {
+                        query_local(c, I, p, qid, xl, &qi);
+                        if (isfinite(xl[0]) && isfinite(xl[1]) && isfinite(xl[2])) {
+                            property_mean(c.P, s, N, np, lattice, qi, xl, cm);
+                            if constexpr (kEmu)
+                                w = fmax(0.0, double_of_fix(emu_query_diag(c)[p - cq0]));
+                            else
+                                w = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
                         }
                     }
+                    for (int ch = 0; ch < np; ++ch) c.b.pc[qid * np + ch] = cm[ch];
+                    c.b.pw[qid] = w;
                 }
-                for (int ch = 0; ch < np; ++ch) c.b.pc[qid * np + ch] = cm[ch];
-                c.b.pw[qid] = w;
+                if (!ok && N > 0 && tid == 0 && !tc.dead) atomicOr(c.err, kErrFactor);
+                __syncthreads();
+                cq0 = ce;
+                if ((kEmu && tc.dead) || cq0 >= q1) break;
             }
-            if (!ok && N > 0 && tid == 0 && !tc.dead) atomicOr(c.err, kErrFactor);
-            __syncthreads();
             if (kEmu && tc.dead) break;
             continue;
         }
@@ -1636,7 +1760,7 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
         // matrix in chunks of at most qmax, one factorisation per chunk.  Every chunk repeats
         // the same arithmetic on the instance's own rows, and a query's row involves only
         // itself, so every result is independent of the chunking and of the other queries.
-        const bool border = kEmu && c.b.want_var && c.qmax > 0;
+        const bool border = kEmu && c.b.want_var;
         for (int64_t cq0 = q0;;) {
             const int64_t cq1 = border ? min(q1, cq0 + (int64_t)c.qmax) : q1;
             const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, border ? (int)(cq1 - cq0) : 0,
@@ -1659,11 +1783,10 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                         latent_mean(c.P, s, N, lattice, qi, xl, lo, gro);
                         double u = 0.0;
                         if (c.b.want_var) {
-                            if (border) {  // the Schur complement's diagonal entry, clamped at 0
+                            if constexpr (kEmu)  // the Schur complement's diagonal entry, clamped at 0
                                 u = fmax(0.0, double_of_fix(emu_query_diag(c)[p - cq0]));
-                            } else {
+                            else
                                 u = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
-                            }
                         }
                         revert(c.P, lo, gro, u, c.b.want_var != 0, r);
                     }
@@ -2154,7 +2277,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         s.grid = (int)std::min<int64_t>(n, (int64_t)n_sm * per_sm);
         ca.slots[i] = s.grid;
         if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
-        if (b.want_var) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
+        if (b.want_var && !s.emu) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
         if (s.emu) ws_e_need = std::max<int64_t>(ws_e_need, (int64_t)s.nrow * kEmuBytesPerRow * s.grid);
     }
     // every buffer exists before the capture starts (allocation is not captured)
@@ -2507,10 +2630,10 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
         c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * grid, st);
         c.ws_v_stride = (int64_t)c.npad * threads;
-        c.ws_v = (b.want_var && !bw) ? (double*)ar.get(Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
+        c.ws_v = (b.want_var && !bw && !emu) ? (double*)ar.get(Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
         c.ws_e_stride = emu ? (int64_t)c.nrow * kEmuBytesPerRow : 0;
         c.ws_e = emu ? (uint8_t*)ar.get(Arena::kWs3, c.ws_e_stride * grid, st) : nullptr;
-        if ((!c.a_in_smem && !c.ws_a) || (b.want_var && !bw && !c.ws_v) || (emu && !c.ws_e)) {
+        if ((!c.a_in_smem && !c.ws_a) || (b.want_var && !bw && !emu && !c.ws_v) || (emu && !c.ws_e)) {
             if (profile) {
                 cudaEventDestroy(ev0);
                 cudaEventDestroy(ev1);
