@@ -115,7 +115,6 @@ struct Shared {
     double* Tblk;   // [kEB][64] inverses of the diagonal tiles of the current block
     unsigned* dtab; // [8][32] entries of the diagonal tiles' updates (diag_entry)
     double* Dblk;   // [kDiagTiles][64] the current block's diagonal tiles (packed lower triangle)
-    double* Wsc;    // [warps][64] per-warp tile scratch (layout changes between mma operands)
     unsigned char* stage;  // emulated kernel: slice operands of the tensor-core updates (aliases
                            // X .. alf_lo, which the factorisation does not use; reloaded after it)
     float* qw;             // emulated kernel: [kBorderQ][3] world coordinates of appended queries (FP32;
@@ -151,8 +150,8 @@ constexpr int kEmuCtasPerSm = 512 / kEmuTmemCols;  // CTAs whose tensor memory f
 
 __host__ __device__ __forceinline__ size_t align128(size_t x) { return (x + 127) & ~(size_t)127; }
 __host__ __device__ __forceinline__ size_t emu_fixed_bytes(int npad) {
-    // invd, T256, Tblk, Wsc, Tff, Dblk, dtab
-    return align128((size_t)(npad + 256 + kEB * 64 + 8 * 64 + 256 + kDiagTiles * 64 + 128) * sizeof(double));
+    // invd, T256, Tblk, Tff, Dblk, dtab
+    return align128((size_t)(npad + 256 + kEB * 64 + 256 + kDiagTiles * 64 + 128) * sizeof(double));
 }
 __host__ __device__ __forceinline__ size_t emu_point_bytes(int npad, int nprop, bool lattice) {
     return (size_t)5 * npad * sizeof(double) + (size_t)5 * npad * sizeof(float) +
@@ -165,15 +164,14 @@ __host__ __device__ __forceinline__ size_t emu_alias_bytes(int npad, int nprop, 
     return b > (size_t)kStageBytes ? b : (size_t)kStageBytes;
 }
 
-// Emulated kernel: invd, the exp table, the block's tile inverses and the warp scratch first, then
-// (128-byte aligned) the staging buffer of the tensor-core updates, which X, alpha, z, Xf, alf,
-// alf_lo, xi and the property weights alias.
+// Emulated kernel: invd, the exp tables and the diagonal block first, then (128-byte aligned) the
+// staging buffer of the tensor-core updates, which X, alpha, z, Xf, alf, alf_lo, xi and the property
+// weights alias, and so does the warps' scratch of the rows below (kEB tiles each).
 __device__ Shared carve_emu(double* sm, int npad, double* ws_a, int nprop, bool lattice) {
     Shared s;
     s.invd = sm;
     s.T256 = s.invd + npad;
     s.Tblk = s.T256 + 256;
-    s.Wsc = s.Tblk + kEB * 64;
     s.Tinv = nullptr;
     s.w = nullptr;
     s.panel = nullptr;
@@ -195,8 +193,8 @@ __device__ Shared carve_emu(double* sm, int npad, double* ws_a, int nprop, bool 
     float* after = reinterpret_cast<float*>(s.stage + emu_point_bytes(npad, nprop, lattice));
     s.Xw = lattice ? nullptr : after;
     s.qw = lattice ? after : after + 3 * npad;
-    s.Tff = reinterpret_cast<float2*>(s.Wsc + 8 * 64);
-    s.Dblk = s.Wsc + 8 * 64 + 256;
+    s.Tff = reinterpret_cast<float2*>(s.Tblk + kEB * 64);
+    s.Dblk = s.Tblk + kEB * 64 + 256;
     s.dtab = reinterpret_cast<unsigned*>(s.Dblk + kDiagTiles * 64);
     // the solves' diagonal tiles go where the world coordinates were (used by the assembly only)
     s.Dsol = reinterpret_cast<double*>(after);
@@ -220,7 +218,6 @@ __device__ Shared carve(double* sm, int npad, int a_in_smem, double* ws_a, int n
     s.T256 = s.Tinv + 64;
     double* end = s.T256 + 256;
     s.Tblk = nullptr;
-    s.Wsc = nullptr;
     s.Dblk = nullptr;
     s.Dsol = nullptr;
     s.dtab = nullptr;
@@ -739,54 +736,83 @@ __device__ __forceinline__ void slice_row(const double (&x)[2 * kEB], uint32_t* 
     }
 }
 
+// acc_i -= x_0 l_i0 + ... + x_7 l_i7 for the two columns i = c0, c1 of tile L and the row X points at
+// (r: its row in the tile), one operation after the other in that order.
+__device__ __forceinline__ void sub_products(double& acc0, double& acc1, const double* X, int r, const double* L, int c0,
+                                             int c1) {
+#pragma unroll
+    for (int m = 0; m < 8; m += 2) {
+        const double2 x = *reinterpret_cast<const double2*>(X + te(r, m));
+        const double2 u = *reinterpret_cast<const double2*>(L + te(c0, m));
+        const double2 v = *reinterpret_cast<const double2*>(L + te(c1, m));
+        acc0 = fma(-x.x, u.x, acc0);
+        acc1 = fma(-x.x, v.x, acc1);
+        acc0 = fma(-x.y, u.y, acc0);
+        acc1 = fma(-x.y, v.y, acc1);
+    }
+}
+
+// The row r of a tile P times Ti^T, columns c0 <= 3 and c1 (Ti lower triangular, its upper part zero).
+__device__ __forceinline__ void times_inverse(double& y0, double& y1, const double* P, int r, const double* Ti, int c0,
+                                              int c1) {
+    y0 = y1 = 0.0;
+#pragma unroll
+    for (int m = 0; m < 8; m += 2) {
+        const double2 p = *reinterpret_cast<const double2*>(P + te(r, m));
+        const double2 v = *reinterpret_cast<const double2*>(Ti + te(c1, m));
+        if (m < 4) {
+            const double2 u = *reinterpret_cast<const double2*>(Ti + te(c0, m));
+            y0 = fma(p.x, u.x, y0);
+            y0 = fma(p.y, u.y, y0);
+        }
+        y1 = fma(p.x, v.x, y1);
+        y1 = fma(p.y, v.y, y1);
+    }
+}
+
 // Row tile it below the factorised diagonal block of tile columns K0 .. K0 + kEB - 1 (its tiles in
 // Dblk, the inverses of its diagonal tiles in Tblk): L_it,K0+j = (A_it,K0+j - sum_{k<j} L_it,K0+k L_K0+j,K0+k^T)
-// Ti_j^T for j < kEB on the FP64 tensor path, one warp, the row's tiles in registers.  The warp's
-// scratch tile W turns each result from the accumulator into the operand layout.  The
+// Ti_j^T for j < kEB, one warp, lane = 4 g + t: row g, columns t and 7 - t of each tile (so that the
+// zeros of Ti cost the same on every lane).  W: kEB tiles of scratch, the solved tiles.  The
 // results are stored to A and sliced for the trailing update (F, scale: this tile's slices
 // and row scales; u: the diagonal entries of an appended query tile's rows, else null).
+// Bound by the FP64 pipe: 144 operations of 66 clocks.  As 8x8x4 FP64 MMAs (the same chain of fused
+// multiply-adds, bit for bit) it was 20 of 580 clocks, zeros of Ti included.
 __device__ void block_rows(double* A, int it, int K0, const double* Dblk, const double* Tblk, double* W,
                            uint32_t* F, double* scale, long long* u) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     double* R = A + eix(it, K0);  // tiles (it, K0 .. K0 + kEB - 1), kTileCol apart
-    double x[2 * kEB];            // accumulator layout: tile j holds columns 2t, 2t + 1 of row g
+    double a0[kEB], a1[kEB];
 #pragma unroll
     for (int j = 0; j < kEB; ++j) {
-        x[2 * j] = R[kTileCol * j + te(g, 2 * t)];
-        x[2 * j + 1] = R[kTileCol * j + te(g, 2 * t + 1)];
+        a0[j] = R[kTileCol * j + te(g, t)];
+        a1[j] = R[kTileCol * j + te(g, 7 - t)];
     }
-    double xa[kEB - 1][2];  // operand layout of the solved tiles: columns t and 4 + t of row g
 #pragma unroll
     for (int j = 0; j < kEB; ++j) {
-        double a0 = x[2 * j], a1 = x[2 * j + 1];
         const double* Lj = Dblk + j * (j + 1) / 2 * 64;  // tiles (K0 + j, K0 .. K0 + j)
 #pragma unroll
-        for (int k = 0; k < j; ++k) {
-            dmma(a0, a1, neg(xa[k][0]), Lj[64 * k + te(g, t)]);
-            dmma(a0, a1, neg(xa[k][1]), Lj[64 * k + te(g, 4 + t)]);
-        }
-        W[te(g, 2 * t)] = a0;
-        W[te(g, 2 * t + 1)] = a1;
+        for (int k = 0; k < j; ++k) sub_products(a0[j], a1[j], W + 64 * k, g, Lj + 64 * k, t, 7 - t);
+        double* Wj = W + 64 * j;
+        Wj[te(g, t)] = a0[j];
+        Wj[te(g, 7 - t)] = a1[j];
         __syncwarp();
-        const double p0 = W[te(g, t)], p1 = W[te(g, 4 + t)];
+        double y0, y1;
+        times_inverse(y0, y1, Wj, g, Tblk + 64 * j, t, 7 - t);
         __syncwarp();
-        const double* Ti = Tblk + 64 * j;
-        double y0 = 0.0, y1 = 0.0;
-        dmma(y0, y1, p0, Ti[te(g, t)]);
-        dmma(y0, y1, p1, Ti[te(g, 4 + t)]);
-        R[kTileCol * j + te(g, 2 * t)] = y0;
-        R[kTileCol * j + te(g, 2 * t + 1)] = y1;
-        x[2 * j] = y0;
-        x[2 * j + 1] = y1;
-        if (j < kEB - 1) {
-            W[te(g, 2 * t)] = y0;
-            W[te(g, 2 * t + 1)] = y1;
-            __syncwarp();
-            xa[j][0] = W[te(g, t)];
-            xa[j][1] = W[te(g, 4 + t)];
-            __syncwarp();
-        }
+        Wj[te(g, t)] = y0;
+        Wj[te(g, 7 - t)] = y1;
+        __syncwarp();
     }
+    double x[2 * kEB];  // columns 2t, 2t + 1 of each tile
+#pragma unroll
+    for (int j = 0; j < kEB; ++j) {
+        const double2 v = *reinterpret_cast<const double2*>(W + 64 * j + te(g, 2 * t));
+        *reinterpret_cast<double2*>(R + kTileCol * j + te(g, 2 * t)) = v;
+        x[2 * j] = v.x;
+        x[2 * j + 1] = v.y;
+    }
+    __syncwarp();
     slice_row(x, F, scale + g, u ? u + g : nullptr);
 }
 
@@ -1078,13 +1104,10 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
         auto tile = [&](int ir, int jc) { return s.Dblk + (ir * (ir + 1) / 2 + jc) * 64; };
         auto update = [&](int ir, int jc, int k) {  // tile (ir, jc) -= tile (ir, k) tile (jc, k)^T
             double* C = tile(ir, jc);
-            const double* Li = tile(ir, k);
-            const double* Lj = tile(jc, k);
-            double c0 = C[te(g, 2 * t)], c1 = C[te(g, 2 * t + 1)];
-            dmma(c0, c1, neg(Li[te(g, t)]), Lj[te(g, t)]);
-            dmma(c0, c1, neg(Li[te(g, 4 + t)]), Lj[te(g, 4 + t)]);
-            C[te(g, 2 * t)] = c0;
-            C[te(g, 2 * t + 1)] = c1;
+            double c0 = C[te(g, t)], c1 = C[te(g, 7 - t)];
+            sub_products(c0, c1, tile(ir, k), g, tile(jc, k), t, 7 - t);
+            C[te(g, t)] = c0;
+            C[te(g, 7 - t)] = c1;
         };
         for (int k = 0; k < nb; ++k) {
             const double* Ti = s.Tblk + 64 * k;
@@ -1106,14 +1129,11 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             if (k + 1 == nb) break;
             if (warp >= 1 && warp < nb - k) {  // panel: tile (k + warp, k) Ti^T
                 double* T = tile(k + warp, k);
-                const double a0 = T[te(g, t)], a1 = T[te(g, 4 + t)];
-                const double b0 = Ti[te(g, t)], b1 = Ti[te(g, 4 + t)];
-                double c0 = 0.0, c1 = 0.0;
-                dmma(c0, c1, a0, b0);
-                dmma(c0, c1, a1, b1);
+                double c0, c1;
+                times_inverse(c0, c1, T, g, Ti, t, 7 - t);
                 __syncwarp();
-                T[te(g, 2 * t)] = c0;
-                T[te(g, 2 * t + 1)] = c1;
+                T[te(g, t)] = c0;
+                T[te(g, 7 - t)] = c1;
             }
             __syncthreads();
         }
@@ -1129,7 +1149,7 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
         // the rows below: one warp per row tile solves its four tiles against the diagonal
         // block and writes their slices (both column halves) and row scales
         for (int it = K1 + warp; it < Nt; it += nwarps)
-            block_rows(A, it, K0, s.Dblk, s.Tblk, s.Wsc + 64 * warp,
+            block_rows(A, it, K0, s.Dblk, s.Tblk, reinterpret_cast<double*>(s.stage) + kEB * 64 * warp,
                        reinterpret_cast<uint32_t*>(E + (int64_t)((it - K1) / kColT) * kGroupBytes +
                                                    (it - K1) % kColT * kSliceBytes),
                        sr + 8 * (it - K1),
@@ -1263,17 +1283,18 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         if (nq > 0)
             for (int a = tid; a < 8 * (Ntq - Nt); a += nt) emu_query_diag(c)[a] = 1ll << kFixBits;
     }
-    const int64_t ntl = kEmu ? 0 : n_tiles(Nt);
-    for (int64_t tl = warp; tl < ntl; tl += nwarps) {
-        const int it = tri_row((int)tl), jt = (int)tl - it * (it + 1) / 2;
-        for (int e = lane; e < 64; e += 32) {
-            const int i = 8 * it + (e >> 3), j = 8 * jt + (e & 7);
-            double v;
-            if (i >= N || j >= N) v = (i == j) ? 1.0 : 0.0;
-            else if (j > i) v = 0.0;
-            else if (j == i) v = 1.0 + c.P.s2;
-            else v = kval_pair(c.P, s, lattice, i, j);
-            A[tl * 64 + te(e >> 3, e & 7)] = v;
+    if constexpr (!kEmu) {
+        for (int64_t tl = warp; tl < n_tiles(Nt); tl += nwarps) {
+            const int it = tri_row((int)tl), jt = (int)tl - it * (it + 1) / 2;
+            for (int e = lane; e < 64; e += 32) {
+                const int i = 8 * it + (e >> 3), j = 8 * jt + (e & 7);
+                double v;
+                if (i >= N || j >= N) v = (i == j) ? 1.0 : 0.0;
+                else if (j > i) v = 0.0;
+                else if (j == i) v = 1.0 + c.P.s2;
+                else v = kval_pair(c.P, s, lattice, i, j);
+                A[tl * 64 + te(e >> 3, e & 7)] = v;
+            }
         }
     }
     __syncthreads();
