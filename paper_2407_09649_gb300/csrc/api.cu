@@ -1662,6 +1662,7 @@ int vgp_autotune(vgp_map* m, const float* q, int64_t n, vgp_stream stream) {
             cfg.per_sm[i] = cand_p[c][i];
         }
         cfg.stage_panel = cand_s[c];
+        cfg.chosen = true;
         // each candidate twice, the faster run counts
         SolveStats s1, s2;
         TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &s1, nullptr, true, 0, &cfg), "vgp_autotune"));
@@ -1677,6 +1678,7 @@ int vgp_autotune(vgp_map* m, const float* q, int64_t n, vgp_stream stream) {
                 if (i == 0) chosen.stage_panel = cfg.stage_panel;
             }
     }
+    chosen.chosen = true;
     m->cfg = chosen;
     for (int i = 0; i < 5; ++i) {
         m->stats.cfg_threads[i] = chosen.threads[i];
@@ -1700,6 +1702,7 @@ int vgp_set_launch(vgp_map* m, const int32_t* threads, const int32_t* per_sm, in
         m->cfg.per_sm[i] = per_sm[i];
     }
     m->cfg.stage_panel = stage_panel;
+    m->cfg.chosen = true;
     return VGP_OK;
 }
 

@@ -52,18 +52,6 @@ __device__ __forceinline__ int tri_row(int p) {
     return r;
 }
 
-__device__ __forceinline__ double neg(double x) {  // sign flip on the integer pipe
-    return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
-}
-
-// D(8x8) += A(8x4) B(4x8) on the FP64 tensor path.  Fragments: a = A[g][t],
-// b = B[t][g], c = D[g][2t .. 2t+1] with g = lane / 4, t = lane % 4.
-__device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
-                 : "+d"(c0), "+d"(c1)
-                 : "d"(a), "d"(b));
-}
-
 constexpr int kEmuThreads = 256;  // CTA size of the emulated-update kernels (two CTAs per SM)
 constexpr int kEB = 4;            // tiles (of 8 columns) per block of the emulated factorisation
 constexpr int kEK = kEB / 2;      // 16-column mma steps per block
@@ -113,7 +101,8 @@ struct Shared {
     double* pa[4];  // property weights per channel (property mode): channels 0 and 1 reuse the
                     // distance alpha and its FP32 copies, which that mode does not use
     double* Tblk;   // [kEB][64] inverses of the diagonal tiles of the current block
-    unsigned* dtab; // [8][32] entries of the diagonal tiles' updates (diag_entry)
+    uint8_t* dtab;  // [8][32] entries of the diagonal tiles' updates (diag_entry)
+    double* Dsc;    // [64] plain kernel, A in global memory: the current diagonal tile
     double* Dblk;   // [kDiagTiles][64] the current block's diagonal tiles (packed lower triangle)
     unsigned char* stage;  // emulated kernel: slice operands of the tensor-core updates (aliases
                            // X .. alf_lo, which the factorisation does not use; reloaded after it)
@@ -151,7 +140,7 @@ constexpr int kEmuCtasPerSm = 512 / kEmuTmemCols;  // CTAs whose tensor memory f
 __host__ __device__ __forceinline__ size_t align128(size_t x) { return (x + 127) & ~(size_t)127; }
 __host__ __device__ __forceinline__ size_t emu_fixed_bytes(int npad) {
     // invd, T256, Tblk, Tff, Dblk, dtab
-    return align128((size_t)(npad + 256 + kEB * 64 + 256 + kDiagTiles * 64 + 128) * sizeof(double));
+    return align128((size_t)(npad + 256 + kEB * 64 + 256 + kDiagTiles * 64 + 32) * sizeof(double));
 }
 __host__ __device__ __forceinline__ size_t emu_point_bytes(int npad, int nprop, bool lattice) {
     return (size_t)5 * npad * sizeof(double) + (size_t)5 * npad * sizeof(float) +
@@ -195,7 +184,8 @@ __device__ Shared carve_emu(double* sm, int npad, double* ws_a, int nprop, bool 
     s.qw = lattice ? after : after + 3 * npad;
     s.Tff = reinterpret_cast<float2*>(s.Tblk + kEB * 64);
     s.Dblk = s.Tblk + kEB * 64 + 256;
-    s.dtab = reinterpret_cast<unsigned*>(s.Dblk + kDiagTiles * 64);
+    s.dtab = reinterpret_cast<uint8_t*>(s.Dblk + kDiagTiles * 64);
+    s.Dsc = nullptr;
     // the solves' diagonal tiles go where the world coordinates were (used by the assembly only)
     s.Dsol = reinterpret_cast<double*>(after);
     return s;
@@ -216,17 +206,20 @@ __device__ Shared carve(double* sm, int npad, int a_in_smem, double* ws_a, int n
     s.w = with_w ? s.z + npad : nullptr;
     s.Tinv = s.z + (with_w ? 2 : 1) * npad;
     s.T256 = s.Tinv + 64;
-    double* end = s.T256 + 256;
+    s.dtab = reinterpret_cast<uint8_t*>(s.T256 + 256);
+    double* end = s.T256 + 256 + 32;
+    s.Dsc = nullptr;
     s.Tblk = nullptr;
     s.Dblk = nullptr;
     s.Dsol = nullptr;
-    s.dtab = nullptr;
     if (a_in_smem) {
         s.A = end;
         end += n_tiles(npad / 8) * 64;
         s.panel = nullptr;
     } else {
         s.A = ws_a;
+        s.Dsc = end;
+        end += 64;
         s.panel = stage_panel ? end : nullptr;
         if (stage_panel) end += (int64_t)(npad / 8) * 64;
     }
@@ -246,8 +239,8 @@ __device__ Shared carve(double* sm, int npad, int a_in_smem, double* ws_a, int n
 __host__ size_t smem_bytes(int npad, int a_in_smem, int nprop, int stage_panel, bool lattice, bool with_w = false,
                           bool emu = false) {
     if (emu) return emu_fixed_bytes(npad) + emu_alias_bytes(npad, nprop, lattice);
-    size_t d = (size_t)(with_w ? 7 : 6) * npad + 64 + 256 +
-               (a_in_smem ? (size_t)n_tiles(npad / 8) * 64 : (stage_panel ? (size_t)(npad / 8) * 64 : 0));
+    size_t d = (size_t)(with_w ? 7 : 6) * npad + 64 + 256 + 32 +
+               (a_in_smem ? (size_t)n_tiles(npad / 8) * 64 : 64 + (stage_panel ? (size_t)(npad / 8) * 64 : 0));
     return d * sizeof(double) + (size_t)5 * npad * sizeof(float) + (lattice ? (size_t)npad * sizeof(int) : 0) +
            (size_t)std::max(nprop - 2, 0) * npad * sizeof(double);
 }
@@ -372,17 +365,24 @@ __device__ __forceinline__ void split_pair(double v, float& hi, float& lo) {
 // Solve (L L^T) x = rhs in place on s.z (x written to out), L tile-packed; rows >= N of rhs
 // must be zero.  Right-looking by 8-row blocks on each side.
 __device__ void chol_solve(const Shared& s, const double* A, int Nt, double* out) {
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
     const int Np = Nt * 8;
     double* z = s.z;
     for (int kt = 0; kt < Nt; ++kt) {
-        if (tid == 0) {
+        if (warp == (int)((kt + blockIdx.x) % nwarps)) {  // row r final, then out of the rows below it
             const double* D = A + tix(kt, kt);
+            double v = lane < 8 ? z[8 * kt + lane] : 0.0;
+            double d[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) d[r] = D[te(lane & 7, r)];
+            const double inv = s.invd[8 * kt + (lane & 7)];
+#pragma unroll
             for (int r = 0; r < 8; ++r) {
-                double v = z[8 * kt + r];
-                for (int c2 = 0; c2 < r; ++c2) v -= D[te(r, c2)] * z[8 * kt + c2];
-                z[8 * kt + r] = v * s.invd[8 * kt + r];
+                if (lane == r) v *= inv;
+                const double zr = __shfl_sync(0xffffffffu, v, r);
+                if (lane > r) v = fma(-d[r], zr, v);
             }
+            if (lane < 8) z[8 * kt + lane] = v;
         }
         __syncthreads();
         for (int i = 8 * (kt + 1) + tid; i < Np; i += nt) {
@@ -396,10 +396,12 @@ __device__ void chol_solve(const Shared& s, const double* A, int Nt, double* out
         __syncthreads();
     }
     for (int kt = Nt - 1; kt >= 0; --kt) {
-        if (tid == 0) {
+        if (tid == 32 * (int)((kt + blockIdx.x) % nwarps)) {
             const double* D = A + tix(kt, kt);
+#pragma unroll
             for (int r = 7; r >= 0; --r) {
                 double v = z[8 * kt + r];
+#pragma unroll
                 for (int c2 = r + 1; c2 < 8; ++c2) v -= D[te(c2, r)] * out[8 * kt + c2];
                 out[8 * kt + r] = v * s.invd[8 * kt + r];
             }
@@ -579,36 +581,38 @@ __device__ __noinline__ void chol_solve_inv(double* z, double* Dsol, const doubl
     }
 }
 
-// Which entry of the update of step j (below) a lane takes: tab[32 j + lane] holds its place (bits
-// 0-5; bit 6: in T, else in S), the place of its factor in column j of S (bits 8-13) and that of the
-// other factor (bits 16-21, same array as the entry); bit 31: none.
-__device__ __forceinline__ unsigned diag_entry(int j, int lane) {
+// Which entry of the update of step j (below) a lane takes: its place in the tile (bits 0-5; bit 6: in
+// T, else in S), or 128 for none.
+__device__ __forceinline__ uint8_t diag_entry(int j, int lane) {
     const int m = 7 - j, nc = m * (m + 1) / 2;  // pairs of rows of S, then rows and columns of T
-    if (lane >= nc + m * (j + 1)) return 1u << 31;
+    if (lane >= nc + m * (j + 1)) return 128;
     if (lane < nc) {
-        const int a = tri_row(lane), r = j + 1 + a, c = j + 1 + lane - a * (a + 1) / 2;
-        return (unsigned)(te(r, c) | te(r, j) << 8 | te(c, j) << 16);
+        const int a = tri_row(lane);
+        return (uint8_t)te(j + 1 + a, j + 1 + lane - a * (a + 1) / 2);
     }
-    const int q = lane - nc, r = j + 1 + q / (j + 1), c = q % (j + 1);
-    return (unsigned)(te(r, c) | 64 | te(r, j) << 8 | te(j, c) << 16);
+    const int q = lane - nc;
+    return (uint8_t)(te(j + 1 + q / (j + 1), q % (j + 1)) | 64);
 }
 
-// One warp: the 8x8 Cholesky of the diagonal tile S in place (lower part), 1 / L_jj from rsqrt into
-// invd, and the inverse of its factor into T (upper part zero).  One pass over the tile and the
-// identity beside it: step j scales column j of S and row j of T by 1 / L_jj in one operation and
-// takes their products out of the rows below in one more (two where they are over 32).  An FP64
-// operation holds its sub-partition for about 66 clocks however few lanes are on, so what
-// counts is their number: about 8 a step, against 10 and 36 for the inverse after it.  False on a
-// non-positive pivot (the same on every lane).
-__device__ __forceinline__ bool diag_tile_warp(double* S, double* T, double* invd, const unsigned* tab) {
+// One warp: the 8x8 Cholesky of the diagonal tile S in place (lower part), 1 / L_jj into invd, and the
+// inverse of its factor into T (upper part zero).  One pass over the tile and the identity beside
+// it: step j scales column j of S and row j of T by 1 / L_jj in one operation and takes their
+// products out of the rows below in one more (two where they are over 32).  An FP64 operation
+// holds its sub-partition for about 66 clocks however few lanes are on, so what counts is their
+// number: about 8 a step with kRsqrt, 17 without, and none for the inverse by itself.  On one
+// thread, entry by entry, a tile took about 400.  kRsqrt: 1 / L_jj from rsqrt (emulated kernel), else
+// 1 / sqrt.  tab: diag_entry of every step and lane.  False on a non-positive pivot (the same on every lane).
+template <bool kRsqrt>
+__device__ __forceinline__ bool diag_tile_warp(double* S, double* T, double* invd, const uint8_t* tab) {
     const int lane = threadIdx.x & 31;
     T[lane] = 0.0;
     T[lane + 32] = 0.0;
     __syncwarp();
 #pragma unroll 1
     for (int j = 0; j < 8; ++j) {
-        const unsigned e = tab[32 * j + lane];
+        const int e = tab[32 * j + lane], row = (e >> 3) & 7, col = (e & 7) ^ ((row & 2) << 1);
         double* const M = e & 64 ? T : S;
+        const int f1 = te(row, j), f2 = e & 64 ? te(j, col) : te(col, j);
         // the lane's entry of the scaling: S_ij for lanes i = j .. 7, T_jc for lanes 8 + c, c <= j
         double* const xs = lane < 8 ? S + te(lane, j) : T + te(j, lane & 7);
         const bool on = lane < 8 ? lane >= j : lane <= 8 + j;
@@ -616,13 +620,21 @@ __device__ __forceinline__ bool diag_tile_warp(double* S, double* T, double* inv
         double x = on ? *xs : 0.0;
         if (lane == 8 + j) x = 1.0;
         if (!(v > 0.0)) return false;
-        const double r = rsqrt(v);
-        const double y = x * r;
+        double r, y;
+        if (kRsqrt) {
+            r = rsqrt(v);
+            y = x * r;
+        } else {
+            const double d = sqrt(v);
+            r = 1.0 / d;
+            y = x * r;
+            if (lane == j) y = d;
+        }
         __syncwarp();
         if (on) *xs = y;
         if (lane == 0) invd[j] = r;
         __syncwarp();
-        if (!(e >> 31)) M[e & 63] -= S[(e >> 8) & 63] * M[(e >> 16) & 63];
+        if (e < 128) M[e & 63] -= S[f1] * M[f2];
         if (j < 2 && lane < 3 - 2 * j) {  // the entries of T beyond 32: (5 .. 7, 0) and (7, 1)
             const int r2 = j == 0 ? 5 + lane : 7;
             T[te(r2, j)] -= S[te(r2, j)] * T[te(j, j)];
@@ -1114,7 +1126,7 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             if (warp == 0) {
                 if (k > 0) update(k, k, k - 1);
                 __syncwarp();
-                if (!diag_tile_warp(tile(k, k), s.Tblk + 64 * k, s.invd + 8 * (K0 + k), s.dtab) && lane == 0)
+                if (!diag_tile_warp<true>(tile(k, k), s.Tblk + 64 * k, s.invd + 8 * (K0 + k), s.dtab) && lane == 0)
                     *s_fail = 1;
             } else if (k > 0 && (warp & 3) != 0) {
                 // the tiles (ir, jc), k <= jc <= ir, but (k, k): at most 5, one for each of warps 1, 2, 3, 5, 6
@@ -1314,110 +1326,106 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         __syncthreads();
     } else
     for (int kt = 0; kt < Nt; ++kt) {
-        // diagonal tile: 8x8 Cholesky and the inverse of its factor (FP64 pipe)
-        if (tid == 0) {
+        // diagonal tile: 8x8 Cholesky and the inverse of its factor, by one warp, another one for each
+        // tile and CTA so that the resident CTAs' tiles spread over the sub-partitions
+        if (warp == (int)((kt + blockIdx.x) % nwarps)) {
             double* D = A + tix(kt, kt);
-            double* W = s.Tinv;
-            bool bad = false;
-            for (int j = 0; j < 8 && !bad; ++j) {
-                double v = D[te(j, j)];
-                for (int k = 0; k < j; ++k) v -= D[te(j, k)] * D[te(j, k)];
-                if (!(v > 0.0)) {
-                    bad = true;
-                    break;
-                }
-                const double d = sqrt(v), inv = 1.0 / d;
-                D[te(j, j)] = d;
-                s.invd[8 * kt + j] = inv;
-                for (int i = j + 1; i < 8; ++i) {
-                    double u = D[te(i, j)];
-                    for (int k = 0; k < j; ++k) u -= D[te(i, k)] * D[te(j, k)];
-                    D[te(i, j)] = u * inv;
-                }
+            if (s.Dsc) {
+                reinterpret_cast<double2*>(s.Dsc)[lane] = reinterpret_cast<const double2*>(D)[lane];
+                __syncwarp();
             }
-            if (bad) {
-                s_fail = 1;
-            } else {
-                for (int j = 0; j < 8; ++j) {
-                    for (int i = 0; i < j; ++i) W[te(i, j)] = 0.0;
-                    W[te(j, j)] = s.invd[8 * kt + j];
-                    for (int i = j + 1; i < 8; ++i) {
-                        double u = 0.0;
-                        for (int k = j; k < i; ++k) u += D[te(i, k)] * W[te(k, j)];
-                        W[te(i, j)] = -u * s.invd[8 * kt + i];
-                    }
-                }
-            }
+            const bool good = diag_tile_warp<false>(s.Dsc ? s.Dsc : D, s.Tinv, s.invd + 8 * kt, s.dtab);
+            if (s.Dsc) reinterpret_cast<double2*>(D)[lane] = reinterpret_cast<const double2*>(s.Dsc)[lane];
+            if (!good && lane == 0) s_fail = 1;
         }
         __syncthreads();
         if (s_fail) break;
         // panel: L_it,kt = A_it,kt * Tinv^T (kept in shared memory too when A is global)
         for (int it = kt + 1 + warp; it < Nt; it += nwarps) {
             double* T = A + tix(it, kt);
-            const double a0 = T[te(g, t)], a1 = T[te(g, 4 + t)];
-            const double b0 = s.Tinv[te(g, t)], b1 = s.Tinv[te(g, 4 + t)];
-            double c0 = 0.0, c1 = 0.0;
-            dmma(c0, c1, a0, b0);
-            dmma(c0, c1, a1, b1);
+            double c0, c1;
+            times_inverse(c0, c1, T, g, s.Tinv, t, 7 - t);
             __syncwarp();
-            T[te(g, 2 * t)] = c0;
-            T[te(g, 2 * t + 1)] = c1;
+            T[te(g, t)] = c0;
+            T[te(g, 7 - t)] = c1;
             if (s.panel) {
                 double* Pt = s.panel + (it - kt - 1) * 64;
-                Pt[te(g, 2 * t)] = c0;
-                Pt[te(g, 2 * t + 1)] = c1;
+                Pt[te(g, t)] = c0;
+                Pt[te(g, 7 - t)] = c1;
             }
         }
         __syncthreads();
-        // trailing update A_it,jt -= L_it,kt L_jt,kt^T (kt < jt <= it) in 2x2 blocks of tiles:
-        // four independent accumulators per warp, fragments from shared memory
+        // trailing update A_it,jt -= L_it,kt L_jt,kt^T (kt < jt <= it) in 2x2 blocks of tiles per
+        // warp, lane (g, t) row g and columns t, 7 - t of each: eight chains of fused multiply-adds
+        // (the FP64 MMAs' own order and rounding; an 8x8x4 MMA takes 580 clocks for what eight of
+        // these do in 528), six 16-byte operand loads for sixteen of them
         const int M = Nt - kt - 1;
         const int MB = (M + 1) >> 1;
         const int NB = MB * (MB + 1) / 2;
         for (int p = warp; p < NB; p += nwarps) {
             const int bi = tri_row(p), bj = p - bi * (bi + 1) / 2;
-            const int i0 = 2 * bi, j0 = 2 * bj;
-            double na[2][2], bb[2][2];
+            const double *Pi[2], *Pj[2];
+            double* C[2][2];
+            bool valid[2][2];
+            double acc[2][2][2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                const int ii = i0 + r, jj = j0 + r;
-                const double* Pi = s.panel ? s.panel + ii * 64 : A + tix(kt + 1 + ii, kt);
-                const double* Pj = s.panel ? s.panel + jj * 64 : A + tix(kt + 1 + jj, kt);
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    na[r][k] = ii < M ? neg(Pi[te(g, 4 * k + t)]) : 0.0;
-                    bb[r][k] = jj < M ? Pj[te(g, 4 * k + t)] : 0.0;
-                }
+                const int ii = min(2 * bi + r, M - 1), jj = min(2 * bj + r, M - 1);
+                Pi[r] = s.panel ? s.panel + ii * 64 : A + tix(kt + 1 + ii, kt);
+                Pj[r] = s.panel ? s.panel + jj * 64 : A + tix(kt + 1 + jj, kt);
             }
-            double cc[2][2][2];
-            bool valid[2][2];
 #pragma unroll
             for (int r = 0; r < 2; ++r)
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    const int ii = i0 + r, jj = j0 + q;
+                    const int ii = 2 * bi + r, jj = 2 * bj + q;
                     valid[r][q] = ii < M && jj <= ii;
-                    cc[r][q][0] = cc[r][q][1] = 0.0;
-                    if (valid[r][q]) {
-                        const double* C = A + tix(kt + 1 + ii, kt + 1 + jj);
-                        cc[r][q][0] = C[te(g, 2 * t)];
-                        cc[r][q][1] = C[te(g, 2 * t + 1)];
-                    }
+                    C[r][q] = A + (valid[r][q] ? tix(kt + 1 + ii, kt + 1 + jj) : tix(kt + 1 + 2 * bi, kt + 1 + 2 * bj));
+                    acc[r][q][0] = C[r][q][te(g, t)];
+                    acc[r][q][1] = C[r][q][te(g, 7 - t)];
                 }
+            // (a block on the diagonal has no upper right tile, the last row of blocks may have
+            // no lower ones)
+            const bool full = valid[0][1] && valid[1][0];
+            if (full) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
+                for (int m = 0; m < 8; m += 2) {
+                    double2 x[2], u[2], v[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        x[r] = *reinterpret_cast<const double2*>(Pi[r] + te(g, m));
+                        u[r] = *reinterpret_cast<const double2*>(Pj[r] + te(t, m));
+                        v[r] = *reinterpret_cast<const double2*>(Pj[r] + te(7 - t, m));
+                    }
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            acc[r][q][0] = fma(-x[r].x, u[q].x, acc[r][q][0]);
+                            acc[r][q][1] = fma(-x[r].x, v[q].x, acc[r][q][1]);
+                        }
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            acc[r][q][0] = fma(-x[r].y, u[q].y, acc[r][q][0]);
+                            acc[r][q][1] = fma(-x[r].y, v[q].y, acc[r][q][1]);
+                        }
+                }
+            } else {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) dmma(cc[r][q][0], cc[r][q][1], na[r][k], bb[q][k]);
+                    for (int q = 0; q < 2; ++q)
+                        if (valid[r][q]) sub_products(acc[r][q][0], acc[r][q][1], Pi[r], g, Pj[q], t, 7 - t);
+            }
 #pragma unroll
             for (int r = 0; r < 2; ++r)
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
                     if (valid[r][q]) {
-                        double* C = A + tix(kt + 1 + i0 + r, kt + 1 + j0 + q);
-                        C[te(g, 2 * t)] = cc[r][q][0];
-                        C[te(g, 2 * t + 1)] = cc[r][q][1];
+                        C[r][q][te(g, t)] = acc[r][q][0];
+                        C[r][q][te(g, 7 - t)] = acc[r][q][1];
                     }
         }
         __syncthreads();
@@ -1677,8 +1685,8 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             float h, l;
             split_pair(c.P.exp_tab[j], h, l);
             s.Tff[j] = make_float2(h, l);
-            s.dtab[j] = diag_entry(j >> 5, j & 31);
         }
+    for (int j = tid; j < 256; j += nt) s.dtab[j] = diag_entry(j >> 5, j & 31);
     EmuTc tc{};
     if (kEmu) {
         // tensor memory for the 8 slice-group accumulators (held until the CTA exits) and the
@@ -1837,8 +1845,9 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
 // kProps: surface-property mode (Eq. 6); the emulated kernels run the trailing updates of
 // N > 32 instances on the bf16 tensor cores (256 threads, two CTAs per SM).  Separate
 // kernels, so that the plain distance kernel keeps its register budget.
+// (up to 736 threads, the largest shape its registers have allowed)
 template <bool kProps>
-__global__ void k_solve(SolveCtx c) {
+__global__ void __launch_bounds__(736) k_solve(SolveCtx c) {
     solve_body<kProps, false>(c);
 }
 
@@ -1861,7 +1870,11 @@ __global__ void k_backward(SolveCtx c) {
     const double l2 = c.P.l2;
     SolveCtx cc = c;
     cc.P.precision = VGP_FP64;
-    for (int j = tid; j < 256; j += nt) s.T256[j] = c.P.exp_tab[j];
+    for (int j = tid; j < 256; j += nt) {
+        s.T256[j] = c.P.exp_tab[j];
+        s.dtab[j] = diag_entry(j >> 5, j & 31);
+    }
+    __syncthreads();
     for (;;) {
         if (tid == 0) s_w = atomicAdd(c.counter, 1);
         __syncthreads();
@@ -2138,6 +2151,26 @@ int solve_launch_static(const SolveBatch& b, const DevParams& P, int* err_dev, i
 namespace {
 
 using SolveKernel = void (*)(SolveCtx);
+
+// Launch shape of bucket i (cnt instances, `queries` in all) in the plain kernels, unless one was chosen
+// (autotuner, vgp_set_launch):
+// * N > 224, more than eight instances per SM: three CTAs of 256 threads per SM and no panel staging,
+//   so that one's diagonal tiles and barriers overlap the others' updates (2190 instances of
+//   about 400 points: 104 -> 96 ms).  With fewer, the last round of instances costs more than the
+//   overlap gains (677 instances: 51 -> 75 ms), and the default's 512 threads on one instance stay.
+// * 33 to 64 points, heavy evaluation, few instances with 512 queries or more each: 256 threads, so
+//   the chunks are twice as long and fewer of them refit the instance (159 leaves of a frame, 384k
+//   voxels: 5.2 -> 3.9 ms; but 4803 instances with 64 queries each: 3.6 -> 4.0 ms).
+struct BucketShape {
+    int threads, per_sm, stage;
+};
+BucketShape bucket_shape(const SolveConfig& cfg, int i, int64_t cnt, int n_sm, bool heavy, int64_t queries) {
+    BucketShape b{cfg.threads[i], cfg.per_sm[i], cfg.stage_panel};
+    if (cfg.chosen) return b;
+    if (i == 0 && cnt > 8 * n_sm) b = {256, 3, 0};
+    if (i == 3 && heavy && cnt <= 2 * n_sm && queries >= 512 * cnt) b.threads = 256;
+    return b;
+}
 
 SolveKernel pick_solve(bool props, bool emu) {
     if (props) return emu ? k_solve_emu<true> : k_solve<true>;
@@ -2464,14 +2497,12 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     }
     // size buckets, largest first: A in global workspace above 224, in shared memory below
     struct Bucket {
-        int lo, hi, smem_a, threads;
+        int lo, hi, smem_a;
     };
     // with the emulated updates every bucket above 32 points runs the emulated kernel (A in
     // global memory): a single 32-column block leaves it nothing to gain below
     const int emu_mid = P.emulate && !bw ? 0 : 1;
-    const Bucket buckets[] = {{225, 1024, 0, cfg->threads[0]}, {129, 224, emu_mid, cfg->threads[1]},
-                              {65, 128, emu_mid, cfg->threads[2]}, {33, 64, emu_mid, cfg->threads[3]},
-                              {0, 32, 1, cfg->threads[4]}};
+    const Bucket buckets[] = {{225, 1024, 0}, {129, 224, emu_mid}, {65, 128, emu_mid}, {33, 64, emu_mid}, {0, 32, 1}};
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -2554,14 +2585,16 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         }
         return nmax;
     };
-    auto bucket_launch = [&](int i, int nmax) {
+    auto bucket_launch = [&](int i, int nmax, int cnt) {
         const Bucket& bk = buckets[i];
+        const BucketShape bs = bw ? BucketShape{cfg->threads[i], cfg->per_sm[i], cfg->stage_panel}
+                                  : bucket_shape(*cfg, i, cnt, n_sm, heavy, (int64_t)hq[i]);
         Launch L;
         L.npad = std::max((nmax + 7) & ~7, 8);
         L.emu = !bw && !bk.smem_a && P.emulate;
         emu_rows_for(L.emu, b, L.npad, L.qmax, L.nrow);
-        L.threads = L.emu ? kEmuThreads : bk.threads;
-        L.stage = bk.smem_a ? 1 : (L.emu ? 0 : cfg->stage_panel);
+        L.threads = L.emu ? kEmuThreads : bs.threads;
+        L.stage = bk.smem_a ? 1 : (L.emu ? 0 : bs.stage);
         L.shm = smem_bytes(L.npad, bk.smem_a, bw ? 0 : b.nprop, L.stage, b.Xi != nullptr, bw != nullptr, L.emu);
         L.kern = bw ? k_backward : pick_solve(b.nprop > 0, L.emu);
         cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.shm);
@@ -2572,7 +2605,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         } else {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L.per_sm, L.kern, L.threads, L.shm);
             L.per_sm = std::max(L.per_sm, 1);
-            if (cfg->per_sm[i] > 0) L.per_sm = std::min(L.per_sm, cfg->per_sm[i]);
+            if (bs.per_sm > 0) L.per_sm = std::min(L.per_sm, bs.per_sm);
         }
         return L;
     };
@@ -2588,7 +2621,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             ca.off[i] = off;
             ca.cnt[i] = cnt;
             off += cnt;
-            ca.slots[i] = cnt > 0 ? n_sm * bucket_launch(i, nmax).per_sm : 0;
+            ca.slots[i] = cnt > 0 ? n_sm * bucket_launch(i, nmax, cnt).per_sm : 0;
             ca.qc[i] = chunk_size(true, cnt, ca.slots[i], ca.cap[i], (long long)hq[i]);
             chunks = chunks || (cnt > 0 && ca.qc[i] > 0);
         }
@@ -2633,7 +2666,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         c.n_work = cnt;
         c.chunk_off = chunk_off ? chunk_off + done : nullptr;
         c.chunk_q = chunk_q ? chunk_q + bi : nullptr;
-        const Launch L = bucket_launch(bi, nmax);
+        const Launch L = bucket_launch(bi, nmax, cnt);
         c.npad = L.npad;
         c.qmax = L.qmax;
         c.nrow = L.nrow;
