@@ -167,7 +167,8 @@ typedef struct {
     double sum_n3;        /* sum of N^3 over instances */
     double sum_n2;        /* sum of N^2 over instances */
     double t_solve_ms;    /* GP solve kernels (factorise + evaluate), if params.profile */
-    double t_bucket_ms[5];   /* the same per size bucket */
+    double t_bucket_ms[5];   /* the same per launch: N > 224, 129..224, 65..128, 33..64, <= 32 (with
+                                emulate_fp64 the instances above 32 points are one launch, the first) */
     int32_t cfg_threads[5];  /* launch shape used per bucket: threads per CTA ... */
     int32_t cfg_per_sm[5];   /* ... and cap on CTAs per SM (0: occupancy limit) */
     int64_t grid_leaves;  /* leaves in the global grid */

@@ -18,7 +18,7 @@ public:
     enum Slot {
         kScan0, kScan1, kScan2, kHist, kOrder, kTmp0, kTmp1, kTmp2, kTmp3, kTmp4, kTmp5, kTmp6,
         kTmp7, kTmp8, kTmp9, kTmp10, kTmp11, kTmp12, kTmp13, kTmp14, kTmp15, kTmp16, kTmp17,
-        kWs0, kWs1, kWs2, kWs3, kBw0, kBw1, kPair0, kPair1, kPair2, kPair3, kPair4, kPair5, kPair6, kPair7,
+        kWs0, kWs1, kWs2, kWs3, kWs4, kBw0, kBw1, kPair0, kPair1, kPair2, kPair3, kPair4, kPair5, kPair6, kPair7,
         kChunks, kCounters, kNumSlots
     };
     void* get(Slot s, size_t bytes, cudaStream_t st);
@@ -101,8 +101,9 @@ void fill_u64(uint64_t* p, uint64_t v, int64_t n, cudaStream_t st);
 void fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t st);
 void widen_i32(const int32_t* in, int64_t* out, int64_t n, cudaStream_t st);
 
-// CUDA-graph state of a map (launch mode VGP_LAUNCH_GRAPH): a private capture stream, two
-// events joining it to the caller's stream, and one executable graph per solve kind.
+// A map's own stream, two events joining it to the caller's stream, and, for the launch mode
+// VGP_LAUNCH_GRAPH, one executable graph per solve kind.  Direct launches run the smallest size
+// bucket on that stream.
 struct GraphCache {
     cudaStream_t gs = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr, t0 = nullptr, t1 = nullptr;

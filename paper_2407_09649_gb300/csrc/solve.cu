@@ -1963,11 +1963,17 @@ __global__ void k_hist_n(const int64_t* inst_off, int64_t n, int* hist) {
 
 // Queries of each size bucket (N > 224, > 128, > 64, > 32, the rest), for the chunk planning.
 __global__ void k_bucket_queries(const int64_t* inst_off, const int64_t* q_off, int64_t n, unsigned long long* qsum) {
+    __shared__ unsigned long long sum[5];
+    if (threadIdx.x < 5) sum[threadIdx.x] = 0;
+    __syncthreads();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t N = inst_off[i + 1] - inst_off[i];
-    const int bk = N > 224 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
-    atomicAdd(&qsum[bk], (unsigned long long)(q_off[i + 1] - q_off[i]));
+    if (i < n) {
+        const int64_t N = inst_off[i + 1] - inst_off[i];
+        const int bk = N > 224 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
+        atomicAdd(&sum[bk], (unsigned long long)(q_off[i + 1] - q_off[i]));
+    }
+    __syncthreads();
+    if (threadIdx.x < 5 && sum[threadIdx.x]) atomicAdd(&qsum[threadIdx.x], sum[threadIdx.x]);
 }
 
 // order[] sorted by increasing N via the prefix of the histogram
@@ -2001,64 +2007,63 @@ __global__ void k_plan_buckets(const int* hist, int* cursor, int* plan) {
     }
 }
 
-// Work items of the solve launches: where the evaluation is heavy (variance, surface
-// properties), a bucket with few instances is split into chunks of qc queries (chunk_size) so
-// that its queries spread over the GPU; each chunk fits its instance again.  cap[b] > 0
-// bounds qc (the rows a bordered factorisation appends).  chunk_q[b] receives qc (0: no
-// split; taken from a.qc when the host decided); chunk_off[k]
-// the number of work items of the order before instance k, chunk_off[n] the total.  The
-// buckets are contiguous in the order: from the device plan in graph mode, else from a.
+// Work items of the solve launches: a bucket of no more instances than CTAs that can run at once has
+// its queries split into chunks, so that they spread over the GPU; each chunk fits its instance again.
+// Launch b's chunk size qc is the smallest, from qmin[b], that gives no more chunks than the
+// slots[b] CTAs: the refits then run on CTAs that had no work, and the longest chunk is as short as
+// can be.  qmin: what an evaluation has to be worth a fit.  cap[b] > 0 bounds qc (the rows a
+// bordered factorisation appends).  chunk_q[b] receives qc (0: no split); chunk_off[k] the number of
+// work items of the order before instance k, chunk_off[n] the total.  The buckets are contiguous
+// in the order: from the device plan in graph mode, else from a.
 struct ChunkPlanArgs {
-    int off[5], cnt[5], slots[5], cap[5];
-    int heavy;
-    int decided, qc[5];  // decided: the chunk sizes qc were chosen on the host (same rule)
+    int off[5], cnt[5], slots[5], cap[5], qmin[5];
 };
-constexpr int kMinChunk = 64, kMinChunksPer = 8;
-// Queries per work item of a bucket of cnt instances with tq queries in all, launched on slots
-// CTAs; cap > 0 bounds it; 0: no bound (one work item per instance).  A bucket that holds at
-// most half as many instances as CTAs is split into chunks of ceil(tq / slots) queries, at
-// least kMinChunk, when that gives its instances kMinChunksPer chunks on average: for fewer,
-// fitting each chunk again costs more than the spread gains.
-__host__ __device__ inline int chunk_size(bool heavy, int cnt, int slots, int cap, long long tq) {
-    int qc = cap;
-    if (heavy && cnt > 0 && 2 * (long long)cnt <= slots) {
-        long long want = (tq + slots - 1) / slots;
-        if (want < kMinChunk) want = kMinChunk;
-        if (tq >= (long long)kMinChunksPer * want * cnt) {
-            if (qc > 0 && qc < want) want = qc;
-            qc = (int)(want < INT32_MAX ? want : INT32_MAX);
-        }
-    }
-    return qc;
+// Sum over the CTA (all threads call; w: one value per warp of scratch), the same on every thread.
+__device__ long long block_sum(long long v, long long* w) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    v = warp_sum(v);
+    __syncthreads();
+    if (lane == 0) w[warp] = v;
+    __syncthreads();
+    long long t = 0;
+    for (int i = 0; i < nwarp; ++i) t += w[i];
+    return t;
 }
 __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_off, const int64_t* q_off,
                              const int* plan, ChunkPlanArgs a, int* chunk_q, int* chunk_off) {
     __shared__ long long wq[32];
     __shared__ int wsum[32];
-    __shared__ int carry, s_qc;
+    __shared__ int carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
     if (tid == 0) carry = 0;
     for (int bk = 0; bk < 5; ++bk) {
         const int off = plan ? plan[5 + bk] : a.off[bk], cnt = plan ? plan[bk] : a.cnt[bk];
-        // the bucket's queries
-        long long q = 0;
-        for (int k = tid; k < cnt; k += blockDim.x) {
-            const int I = order[off + k];
-            q += q_off[I + 1] - q_off[I];
+        int qc = a.cap[bk];
+        if (cnt > 0 && cnt <= a.slots[bk]) {
+            auto chunks_at = [&](long long q) {  // work items with chunks of q queries
+                long long v = 0;
+                for (int k = tid; k < cnt; k += blockDim.x) {
+                    const int I = order[off + k];
+                    const long long nq = q_off[I + 1] - q_off[I];
+                    v += nq > q ? (nq + q - 1) / q : 1;
+                }
+                return block_sum(v, wq);
+            };
+            long long lo = a.qmin[bk], hi = lo;
+            while (hi < INT32_MAX / 2 && chunks_at(hi) > a.slots[bk]) hi *= 2;
+            if (hi > lo) {
+                lo = hi / 2;  // too many chunks at lo, few enough at hi
+                while (hi - lo > max(1ll, lo / 32)) {
+                    const long long mid = (lo + hi) / 2;
+                    if (chunks_at(mid) > a.slots[bk])
+                        lo = mid;
+                    else
+                        hi = mid;
+                }
+            }
+            qc = qc > 0 ? (int)min((long long)qc, hi) : (int)hi;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-        if (lane == 0) wq[warp] = q;
-        __syncthreads();
-        if (tid == 0) {
-            long long tq = 0;
-            for (int w = 0; w < nwarp; ++w) tq += wq[w];
-            int qc = a.decided ? a.qc[bk] : chunk_size(a.heavy != 0, cnt, a.slots[bk], a.cap[bk], tq);
-            chunk_q[bk] = qc;
-            s_qc = qc;
-        }
-        __syncthreads();
-        const int qc = s_qc;
+        if (tid == 0) chunk_q[bk] = qc;
         // exclusive scan of the chunk counts, continuing the running total
         for (int b0 = 0; b0 < cnt; b0 += blockDim.x) {
             const int k = b0 + tid;
@@ -2184,14 +2189,20 @@ constexpr int64_t kEmuBytesPerRow = 7 * 8 * kEB * 2 + 8 + 64 + 8;
 // Words of a matrix of `rows` rows in a CTA's workspace (rows: a multiple of 8).
 int64_t matrix_words(bool emu, int rows) { return emu ? n_blocks(rows) * 1024 : n_tiles(rows / 8) * 64; }
 
-// Chunk planning of a solve (see k_chunk_plan): heavy evaluation, and the bordered emulated
-// bucket's bound (kBorderQ queries appended at a time).  False when no launch splits.
-bool chunk_args(const SolveBatch& b, const DevParams& P, bool bw, ChunkPlanArgs& a) {
-    a = ChunkPlanArgs{};
-    a.heavy = !bw && (b.want_var || b.nprop > 0);
-    a.cap[0] = (!bw && P.emulate && b.want_var) ? kBorderQ : 0;
-    a.cap[1] = a.cap[2] = a.cap[3] = a.cap[0];  // the emulated buckets
-    return a.heavy != 0;
+// Chunk planning of launch i (cnt instances of up to nmax points, resident CTAs, threads each): the
+// CTAs to spread it over, the bound of an emulated launch that appends query rows, and the
+// shortest chunk worth a fit.
+// * Emulated launches spread over all resident CTAs; 64 queries with variance or properties.
+// * Plain launches with variance run on the FP64 pipe, which one warp per sub-partition nearly fills:
+//   16 warps per SM are enough, and more would only refit; 128 queries.
+// * The mean alone costs about N FP32 values a query: a fit is worth about 64 N of them.
+void chunk_args(const SolveBatch& b, int i, int cnt, int nmax, int n_sm, int per_sm, int threads, bool emu,
+                ChunkPlanArgs& a) {
+    const bool heavy = b.want_var || b.nprop > 0;
+    a.cnt[i] = cnt;
+    a.cap[i] = emu && b.want_var ? kBorderQ : 0;
+    a.slots[i] = n_sm * (emu || !heavy ? per_sm : std::min(per_sm, std::max(1, 512 / threads)));
+    a.qmin[i] = !heavy ? 64 * std::max(nmax, 1) : emu ? 64 : 128;
 }
 
 // Emulated launch with the latent variance: the queries of an instance (up to kBorderQ) are
@@ -2251,6 +2262,18 @@ void graph_cache_destroy(GraphCache& gc) {
 
 namespace {
 
+// The map's own stream and the events that join it to a caller's stream, created on first use.
+bool graph_cache_ready(GraphCache& gc) {
+    if (gc.t1) return true;
+    if ((gc.gs || cudaStreamCreateWithFlags(&gc.gs, cudaStreamNonBlocking) == cudaSuccess) &&
+        (gc.e0 || cudaEventCreateWithFlags(&gc.e0, cudaEventDisableTiming) == cudaSuccess) &&
+        (gc.e1 || cudaEventCreateWithFlags(&gc.e1, cudaEventDisableTiming) == cudaSuccess) &&
+        (gc.t0 || cudaEventCreate(&gc.t0) == cudaSuccess) && cudaEventCreate(&gc.t1) == cudaSuccess)
+        return true;
+    cudaGetLastError();
+    return false;
+}
+
 void add_stats(SolveStats* stats, const std::vector<int>& h) {
     if (!stats) return;
     for (int N = 0; N <= 1024; ++N) {
@@ -2271,13 +2294,7 @@ void add_stats(SolveStats* stats, const std::vector<int>& h) {
 int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStream_t st, Arena& ar,
                       SolveStats* stats, bool profile, const SolveConfig* cfg, GraphCache* gc) {
     const int64_t n = b.n_inst;
-    if (!gc->gs) {
-        if (cudaStreamCreateWithFlags(&gc->gs, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&gc->e0, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&gc->e1, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreate(&gc->t0) != cudaSuccess || cudaEventCreate(&gc->t1) != cudaSuccess)
-            return -1;
-    }
+    if (!graph_cache_ready(*gc)) return -1;
     const bool props = b.nprop > 0;
     const int T = 256;
     int dev = 0, n_sm = 0;
@@ -2314,8 +2331,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         if (cudaFuncSetAttribute(sh[i].kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_max) != cudaSuccess)
             return -1;
     }
-    ChunkPlanArgs ca;
-    const bool chunks = chunk_args(b, P, false, ca);
+    ChunkPlanArgs ca{};
     int64_t ws_a_need = 0, ws_v_need = 0, ws_e_need = 0;
     for (int i = 0; i < 5; ++i) {
         Shape& s = sh[i];
@@ -2328,8 +2344,11 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
             per_sm = std::max(per_sm, 1);
             if (cfg->per_sm[i] > 0) per_sm = std::min(per_sm, cfg->per_sm[i]);
         }
-        s.grid = (int)std::min<int64_t>(n, (int64_t)n_sm * per_sm);
-        ca.slots[i] = s.grid;
+        // (without variance and properties splitting rarely pays: no workspace for it)
+        s.grid = n_sm * per_sm;
+        if (!b.want_var && !props) s.grid = (int)std::min<int64_t>(n, s.grid);
+        chunk_args(b, i, 0, std::min(hi[i], maxn), n_sm, per_sm, s.threads, s.emu, ca);
+        ca.slots[i] = std::min(ca.slots[i], s.grid);
         if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
         if (b.want_var && !s.emu) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
         if (s.emu) ws_e_need = std::max<int64_t>(ws_e_need, (int64_t)s.nrow * kEmuBytesPerRow * s.grid);
@@ -2341,11 +2360,11 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
     double* ws_a = ws_a_need ? (double*)ar.get(Arena::kWs0, sizeof(double) * ws_a_need, st) : nullptr;
     double* ws_v = ws_v_need ? (double*)ar.get(Arena::kWs1, sizeof(double) * ws_v_need, st) : nullptr;
     uint8_t* ws_e = ws_e_need ? (uint8_t*)ar.get(Arena::kWs3, ws_e_need, st) : nullptr;
-    int* chunk_off = chunks ? (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st) : nullptr;
+    int* chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
     if (!hist || !order || !counters || (ws_a_need && !ws_a) || (ws_v_need && !ws_v) || (ws_e_need && !ws_e) ||
-        (chunks && !chunk_off))
+        !chunk_off)
         return alloc_failed(err_dev, st);
-    int* chunk_q = chunk_off ? chunk_off + n + 1 : nullptr;
+    int* chunk_q = chunk_off + n + 1;
     int* cursor = hist + 1025;
     int* plan = counters + 5;
     cudaStream_t gs = gc->gs;
@@ -2359,16 +2378,14 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
     note_launch();
     k_order_n<<<(unsigned)((n + T - 1) / T), T, 0, gs>>>(b.inst_off, n, cursor, order);
     note_launch();
-    if (chunk_off) {
-        k_chunk_plan<<<1, 1024, 0, gs>>>(order, (int)n, b.inst_off, b.q_off, plan, ca, chunk_q, chunk_off);
-        note_launch();
-    }
+    k_chunk_plan<<<1, 1024, 0, gs>>>(order, (int)n, b.inst_off, b.q_off, plan, ca, chunk_q, chunk_off);
+    note_launch();
     for (int i = 0; i < 5; ++i) {
         const Shape& s = sh[i];
         if (!s.live) continue;
         SolveCtx c;
         c.chunk_off = chunk_off;
-        c.chunk_q = chunk_q ? chunk_q + i : nullptr;
+        c.chunk_q = chunk_q + i;
         c.b = b;
         c.P = P;
         c.err = err_dev;
@@ -2456,8 +2473,8 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         return 0;
     }
     // size histogram (and, for chunk planning, each bucket's queries) and decreasing-size order
-    ChunkPlanArgs ca;
-    const bool heavy = chunk_args(b, P, bw != nullptr, ca);
+    const bool heavy = !bw && (b.want_var || b.nprop > 0);
+    ChunkPlanArgs ca{};
     int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * 2 * 1025 + sizeof(unsigned long long) * 5, st);
     if (!hist) return alloc_failed(err_dev, st);
     int* cursor = hist + 1025;
@@ -2467,14 +2484,14 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, n, hist);
     note_launch();
     unsigned long long hq[5] = {0, 0, 0, 0, 0};
-    if (heavy) {
+    if (!bw) {
         cudaMemsetAsync(qsum, 0, sizeof(hq), st);
         k_bucket_queries<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, b.q_off, n, qsum);
         note_launch();
     }
     std::vector<int> h(1025);
     cudaMemcpyAsync(h.data(), hist, sizeof(int) * 1025, cudaMemcpyDeviceToHost, st);
-    if (heavy) cudaMemcpyAsync(hq, qsum, sizeof(hq), cudaMemcpyDeviceToHost, st);
+    if (!bw) cudaMemcpyAsync(hq, qsum, sizeof(hq), cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
     std::vector<int> start(1026, 0);
     for (int i = 0; i < 1025; ++i) start[i + 1] = start[i] + h[i];
@@ -2495,14 +2512,22 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         cudaEventCreate(&ev1);
         cudaEventRecord(ev0, st);
     }
-    // size buckets, largest first: A in global workspace above 224, in shared memory below
+    // size buckets, largest first: A in global workspace above 224, in shared memory below.  With the
+    // emulated updates every instance above 32 points takes the same kernel with the same launch
+    // shape (A in global memory; a single 32-column block leaves it nothing to gain below), so they
+    // share one launch, largest first: four launches one after the other each ended in a nearly
+    // empty last wave (0.6, 1.4, 0.6 ms for a coloured frame's three).
     struct Bucket {
         int lo, hi, smem_a;
     };
-    // with the emulated updates every bucket above 32 points runs the emulated kernel (A in
-    // global memory): a single 32-column block leaves it nothing to gain below
-    const int emu_mid = P.emulate && !bw ? 0 : 1;
-    const Bucket buckets[] = {{225, 1024, 0}, {129, 224, emu_mid}, {65, 128, emu_mid}, {33, 64, emu_mid}, {0, 32, 1}};
+    const Bucket plain_buckets[5] = {{225, 1024, 0}, {129, 224, 1}, {65, 128, 1}, {33, 64, 1}, {0, 32, 1}};
+    const Bucket emu_buckets[5] = {{33, 1024, 0}, {1, 0, 0}, {1, 0, 0}, {1, 0, 0}, {0, 32, 1}};
+    const bool emu_call = P.emulate && !bw;
+    const Bucket* buckets = emu_call ? emu_buckets : plain_buckets;
+    if (emu_call) {
+        hq[0] += hq[1] + hq[2] + hq[3];
+        hq[1] = hq[2] = hq[3] = 0;
+    }
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -2610,22 +2635,21 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         return L;
     };
     int* counters = (int*)ar.get(Arena::kCounters, sizeof(int) * 8, st);
+    // the buckets' ranges of the order, and the CTAs to spread each over; work items are planned
+    // only where some bucket can have more of them than instances
     bool chunks = false;
-    if (heavy) {
-        // the buckets' ranges of the order, their resident CTAs (as the launches below) and
-        // chunk sizes; work items are planned only where some bucket has more than its instances
-        int off = 0;
-        for (int i = 0; i < 5; ++i) {
-            int cnt = 0;
-            const int nmax = bucket_nmax(i, cnt);
-            ca.off[i] = off;
-            ca.cnt[i] = cnt;
-            off += cnt;
-            ca.slots[i] = cnt > 0 ? n_sm * bucket_launch(i, nmax, cnt).per_sm : 0;
-            ca.qc[i] = chunk_size(true, cnt, ca.slots[i], ca.cap[i], (long long)hq[i]);
-            chunks = chunks || (cnt > 0 && ca.qc[i] > 0);
-        }
-        ca.decided = 1;
+    int max_items[5] = {0, 0, 0, 0, 0};
+    for (int i = 0, off = 0; i < 5 && !bw; ++i) {
+        int cnt = 0;
+        const int nmax = bucket_nmax(i, cnt);
+        ca.off[i] = off;
+        off += cnt;
+        if (cnt == 0) continue;
+        const Launch L = bucket_launch(i, nmax, cnt);
+        chunk_args(b, i, cnt, nmax, n_sm, L.per_sm, L.threads, L.emu, ca);
+        const bool split = cnt <= ca.slots[i] && (int64_t)hq[i] > ca.qmin[i];
+        max_items[i] = (int)std::min<int64_t>(INT32_MAX, cnt + (split ? (int64_t)hq[i] / ca.qmin[i] : 0));
+        chunks = chunks || split || (ca.cap[i] > 0 && (int64_t)hq[i] > ca.cap[i]);
     }
     if (chunks) {
         chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
@@ -2643,15 +2667,23 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         return alloc_failed(err_dev, st);
     }
     cudaMemsetAsync(counters, 0, sizeof(int) * 8, st);
+    // the smallest instances run on the map's own stream beside the others, where its CTAs fill the SMs
+    // that the last of those leave (their own variance columns: Arena::kWs4); not while profiling
+    bool beside = false;
+    if (!bw && !profile && gc && graph_cache_ready(*gc)) {
+        int cnt = 0;
+        bucket_nmax(4, cnt);
+        beside = cnt > 0 && cnt < n && cudaEventRecord(gc->e0, st) == cudaSuccess &&
+                 cudaStreamWaitEvent(gc->gs, gc->e0, 0) == cudaSuccess;
+    }
     int done = 0;  // instances already assigned (from the large end)
-    int bi = 0;
-    for (const Bucket& bk : buckets) {
+    for (int bi = 0; bi < 5; ++bi) {
+        const Bucket& bk = buckets[bi];
         int cnt = 0;
         const int nmax = bucket_nmax(bi, cnt);
-        if (cnt == 0) {
-            ++bi;
-            continue;
-        }
+        if (cnt == 0) continue;
+        const bool aside = beside && bi == 4;
+        const cudaStream_t ls = aside ? gc->gs : st;
         SolveCtx c;
         c.plan = nullptr;
         c.bucket = 0;
@@ -2678,13 +2710,11 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         const size_t shm = L.shm;
         auto kern = L.kern;
         const int per_sm = L.per_sm;
-        // a split bucket keeps every resident CTA busy; otherwise one CTA per instance at most
-        const bool split = chunk_off && ca.qc[bi] > 0;
-        const int grid = (int)std::min<int64_t>(split ? INT32_MAX : cnt, (int64_t)n_sm * per_sm);
+        const int grid = (int)std::min<int64_t>(bw ? cnt : max_items[bi], (int64_t)n_sm * per_sm);
         c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
         c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * grid, st);
         c.ws_v_stride = (int64_t)c.npad * threads;
-        c.ws_v = (b.want_var && !bw && !emu) ? (double*)ar.get(Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
+        c.ws_v = (b.want_var && !bw && !emu) ? (double*)ar.get(aside ? Arena::kWs4 : Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
         c.ws_e_stride = emu ? (int64_t)c.nrow * kEmuBytesPerRow : 0;
         c.ws_e = emu ? (uint8_t*)ar.get(Arena::kWs3, c.ws_e_stride * grid, st) : nullptr;
         if ((!c.a_in_smem && !c.ws_a) || (b.want_var && !bw && !emu && !c.ws_v) || (emu && !c.ws_e)) {
@@ -2700,8 +2730,13 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             cudaEventCreate(&b1);
             cudaEventRecord(b0, st);
         }
-        kern<<<grid, threads, shm, st>>>(c);
+        kern<<<grid, threads, shm, ls>>>(c);
         note_launch();
+        if (aside && (cudaEventRecord(gc->e1, gc->gs) != cudaSuccess || cudaStreamWaitEvent(st, gc->e1, 0) != cudaSuccess)) {
+            k_or_err<<<1, 1, 0, st>>>(err_dev, kErrLaunch);
+            note_launch();
+            return -1;
+        }
         if (profile) {
             cudaEventRecord(b1, st);
             cudaEventSynchronize(b1);
@@ -2712,7 +2747,6 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             cudaEventDestroy(b1);
         }
         done += cnt;
-        ++bi;
     }
     if (profile) {
         cudaEventRecord(ev1, st);
