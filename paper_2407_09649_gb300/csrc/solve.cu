@@ -82,6 +82,7 @@ struct SolveCtx {
     const int* chunk_q = nullptr;    // queries of a work item for this launch (0: all of them)
     int qmax = 0;          // emulated kernel with variance: query rows appended to A (0: none)
     int nrow = 0;          // emulated kernel: rows of the workspace matrices (npad + qmax)
+    int ncta = 1;          // emulated kernel: CTAs (a cluster) that work on one instance together
 };
 
 struct Shared {
@@ -828,11 +829,11 @@ __device__ void block_rows(double* A, int it, int K0, const double* Dblk, const 
     slice_row(x, F, scale + g, u ? u + g : nullptr);
 }
 
-// Per-CTA workspace of the emulated factorisation: the slices of the rows below the current block
+// Workspace of the emulated factorisation, per CTA or cluster: the slices of the rows below the current block
 // ([group of 4 row tiles][slice][row tile][4 core matrices], 3584 bytes per row tile), the row scales, the inverses of
 // all diagonal tiles ([rows / 8][64] doubles), and the appended query rows' diagonal entries in
 // the fixed point.
-__device__ __forceinline__ unsigned char* emu_ws(const SolveCtx& c) { return c.ws_e + (int64_t)blockIdx.x * c.ws_e_stride; }
+__device__ __forceinline__ unsigned char* emu_ws(const SolveCtx& c) { return c.ws_e + (int64_t)(blockIdx.x / c.ncta) * c.ws_e_stride; }
 __device__ __forceinline__ int emu_rows(const SolveCtx& c) { return c.nrow > 0 ? c.nrow : c.npad; }
 __device__ __forceinline__ double* emu_scales(const SolveCtx& c) {
     return reinterpret_cast<double*>(emu_ws(c) + (int64_t)(emu_rows(c) / 8) * kSliceTileBytes);
@@ -884,14 +885,58 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
     return __syncthreads_and((int)bar_poll(bar, parity)) != 0;
 }
 
-// Tensor memory and barriers of an emulated CTA.
+// Tensor memory and barriers of an emulated CTA.  kGroup: several CTAs (a cluster) work on one instance
+// together; without it they are one, known to the compiler (1 to 7 % faster for the large batches).
+template <bool kGroup>
 struct EmuTc {
     uint32_t tmem;       // base of kEmuTmemCols columns: slice group g at columns 8 kColT g
     uint32_t bar_ld;     // completion of the staging copies
     uint32_t bar_mma;    // completion of the MMAs
     uint32_t ph_ld, ph_mma;
     bool dead;           // a bounded wait gave up: take no more work
+    // the CTAs that work together: how many, this one's rank, and two sets of shared-memory words,
+    // one for each rank's flag
+    int n_, rank_;
+    int* flags;
+    int set;
+    __device__ __forceinline__ int n() const { return kGroup ? n_ : 1; }
+    __device__ __forceinline__ int rank() const { return kGroup ? rank_ : 0; }
 };
+
+// The shared-memory word of the cluster's CTA `rank` that lies where p does in this one.
+__device__ __forceinline__ uint32_t peer_word(const void* p, int rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void peer_store(const void* p, int rank, int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_word(p, rank)), "r"(v) : "memory");
+}
+
+// Barrier of the CTAs that work together (of this CTA alone without a cluster): what any of them wrote
+// before it is seen by all after it.  Returns whether any thread passed a flag, the same everywhere:
+// each CTA leaves its own in every other's words before it arrives; the two sets alternate, so
+// a word is written again only after everyone has read it.
+template <class Tc>
+__device__ __forceinline__ bool group_sync(Tc& tc, int flag) {
+    const int any = __syncthreads_or(flag);
+    if (tc.n() == 1) return any != 0;
+    int* f = tc.flags + 8 * tc.set;
+    if ((int)threadIdx.x < tc.n()) peer_store(f + tc.rank(), threadIdx.x, any);
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    int all = 0;
+    for (int i = 0; i < tc.n(); ++i) all |= reinterpret_cast<volatile int*>(f)[i];
+    tc.set ^= 1;
+    return all != 0;
+}
+template <class Tc>
+__device__ __forceinline__ void group_barrier(Tc& tc) {
+    if (tc.n() == 1)
+        __syncthreads();
+    else
+        group_sync(tc, 0);
+}
 
 __device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&v)[2]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr) : "memory");
@@ -905,7 +950,8 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[8][2]) {
 }
 
 // A bounded wait gave up: record it; the CTA stops taking work.
-__device__ __forceinline__ bool emu_fail(const SolveCtx& c, EmuTc& tc) {
+template <class Tc>
+__device__ __forceinline__ bool emu_fail(const SolveCtx& c, Tc& tc) {
     if (threadIdx.x == 0) atomicOr(c.err, kErrTimeout);
     tc.dead = true;
     return false;
@@ -930,17 +976,26 @@ __device__ __forceinline__ bool emu_fail(const SolveCtx& c, EmuTc& tc) {
 // is prefetched into L2.  Measured against 68 N = 32 products, 8-byte accesses to 64-byte tile rows
 // and a diagonal of the query block from full tiles: 38 instances of about 790 points alone on the
 // GPU 16.1 -> 11.7 ms, 15.6k of 4 to 1024 points 216 -> 180 ms.
-__device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr, int K1, const unsigned char* E,
-                                   const double* sr, unsigned char* stage, EmuTc& tc) {
+template <class Tc>
+__device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const unsigned char* E,
+                                   const double* sr, unsigned char* stage, Tc& tc) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = Nt - K1;
     const int jr = (max(Ntr - K1, 0) + kColT - 1) / kColT;  // column tiles
-    if (jr == 0) return true;
+    // with a cluster, every n-th column tile of a band, from another rank on for each band
+    auto tiles_of = [&](int b0) { return min(jr, (b0 + min(kBandT, M - b0) + kColT - 1) / kColT); };
+    auto first_of = [&](int b0) { return (tc.rank() + b0 / kBandT) % tc.n(); };
+    auto next_band = [&](int b0) {  // the first band from b0 on that has a tile for this CTA
+        while (b0 < M && first_of(b0) >= tiles_of(b0)) b0 += kBandT;
+        return b0;
+    };
+    int b0 = next_band(0);
+    if (jr == 0 || b0 >= M) return true;
     const uint32_t aA = smem_addr(stage), aB = aA + kStageA;
     const int q = warp & 3, h = warp >> 2;  // lane quadrant (rows 32 q ..) and column half
     const int kb1 = K1 >> 2;                // 32-row block of the first row below (K1 is a multiple of 4)
     int fail = 0;
-    // the band's A (warp w: slice w, a lane per group of 4 row tiles) and the first column tile's B
+    // the band's A (warp w: slice w, a lane per group of 4 row tiles) and its first column tile's B
     // (buffer 0, warp 7, which also arms the barrier)
     auto stage_band = [&](int b0) {
         const int ng = (min(kBandT, M - b0) + kColT - 1) / kColT;
@@ -953,19 +1008,20 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
                          "r"((uint32_t)(ng + 1) * kGroupBytes)
                          : "memory");
-            bulk_load(stage + kStageA, E, kStageB, tc.bar_ld);
+            bulk_load(stage + kStageA, E + (int64_t)first_of(b0) * kGroupBytes, kStageB, tc.bar_ld);
         }
     };
-    stage_band(0);
-    for (int b0 = 0; b0 < M; b0 += kBandT) {
+    stage_band(b0);
+    for (int b1; b0 < M; b0 = b1) {
+        b1 = next_band(b0 + kBandT);
         const int nb = min(kBandT, M - b0);
         const int rb = (b0 >> 2) + q;              // the warp's 32-row block below K1
         const bool rows_in = 4 * q < nb;
         // the row's exponent (rows past the matrix inside its last block: unused)
         const int er = rows_in ? (int)(__double_as_longlong(sr[32 * rb + lane]) >> 52) : 0;
-        const int n_tiles = min(jr, (b0 + nb + kColT - 1) / kColT);  // column tiles reaching the band's last row
-        for (int jt = 0; jt < n_tiles; ++jt) {
-            const uint32_t bufB = aB + (uint32_t)((jt & 1) * kStageB);
+        const int n_tiles = tiles_of(b0);  // column tiles reaching the band's last row
+        for (int jt = first_of(b0), buf = 0; jt < n_tiles; jt += tc.n(), buf ^= 1) {
+            const uint32_t bufB = aB + (uint32_t)(buf * kStageB);
             // this thread's 16 entries of C (one row, 16 columns) and the column scales, all loads
             // issued at once; they arrive while the MMAs run
             const bool on = rows_in && jt <= rb;  // (warp-uniform, as the collective tcgen05.ld needs)
@@ -976,18 +1032,18 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
 #pragma unroll
                 for (int cc = 0; cc < 16; ++cc) cv[cc] = C[32 * cc + lane];
                 es = sr[32 * jt + 16 * h + (lane & 15)];
-                if (jt + 1 < n_tiles && jt < rb && lane == 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024), "r"(4096));
+                if (jt + tc.n() < n_tiles && jt + tc.n() <= rb && lane == 0)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024 * tc.n()), "r"(4096));
             }
             // warp 0 alone waits for the copies, starts the next ones and issues the products: every
             // phase of the copy barrier is seen before the next one can start
             if (warp == 0 && !bar_poll(tc.bar_ld, tc.ph_ld)) fail = 1;
             if (warp == 0 && !__any_sync(0xffffffffu, fail) && lane == 0) {
-                if (jt + 1 < n_tiles) {  // the next column tile's B into the other buffer
+                if (jt + tc.n() < n_tiles) {  // the next column tile's B into the other buffer
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
                                  "r"((uint32_t)kStageB)
                                  : "memory");
-                    bulk_load(stage + kStageA + ((jt + 1) & 1) * kStageB, E + (int64_t)(jt + 1) * kGroupBytes, kStageB,
+                    bulk_load(stage + kStageA + (buf ^ 1) * kStageB, E + (int64_t)(jt + tc.n()) * kGroupBytes, kStageB,
                               tc.bar_ld);
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1020,7 +1076,7 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // the band's last products are done (so warp 0 has seen every copy): its A and B buffers
             // take the next band's
-            if (!__any_sync(0xffffffffu, fail) && jt + 1 == n_tiles && b0 + kBandT < M) stage_band(b0 + kBandT);
+            if (!__any_sync(0xffffffffu, fail) && jt + tc.n() >= n_tiles && b1 < M) stage_band(b1);
             if (on) {
                 // two columns at a time, the next two read from tensor memory meanwhile
                 uint32_t v[2][8][2];
@@ -1063,7 +1119,7 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
             }
             // every thread's reads of the accumulators are done before the next tile's MMAs
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            if (__syncthreads_or(fail)) return emu_fail(c, tc);
+            if (__syncthreads_or(fail)) return false;
         }
     }
     return true;
@@ -1093,8 +1149,8 @@ __device__ bool trailing_update_tc(const SolveCtx& c, double* A, int Nt, int Ntr
 // (block_rows), which also writes their slices.
 // Nt row tiles, of which the first Ntr are factorised (Nt > Ntr: appended query rows, whose
 // rows below are solved and whose diagonal entries are updated, but not factorised).
-__device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, int Nt, int Ntr, int* s_fail,
-                                EmuTc& tc) {
+template <class Tc>
+__device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, int Nt, int Ntr, int* s_fail, Tc& tc) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     unsigned char* E = emu_ws(c);
@@ -1108,7 +1164,7 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
         // needs no barrier after it.  The other tiles go to warps of the other sub-partitions
         // (warp 4 shares warp 0's), so the chain of diagonal tiles has its FP64 pipe alone.
         const int nb = K1 - K0;
-        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
+        for (int x = tid; x < nb * (nb + 1) / 2 * 32 && tc.rank() == 0; x += blockDim.x) {
             const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
             reinterpret_cast<double2*>(s.Dblk)[x] = reinterpret_cast<const double2*>(A + eix(K0 + ir, K0 + jc))[x & 31];
         }
@@ -1121,7 +1177,7 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             C[te(g, t)] = c0;
             C[te(g, 7 - t)] = c1;
         };
-        for (int k = 0; k < nb; ++k) {
+        for (int k = 0; k < nb && tc.rank() == 0; ++k) {
             const double* Ti = s.Tblk + 64 * k;
             if (warp == 0) {
                 if (k > 0) update(k, k, k - 1);
@@ -1137,8 +1193,7 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
                 }
             }
             __syncthreads();
-            if (*s_fail) return false;
-            if (k + 1 == nb) break;
+            if (*s_fail || k + 1 == nb) break;
             if (warp >= 1 && warp < nb - k) {  // panel: tile (k + warp, k) Ti^T
                 double* T = tile(k + warp, k);
                 double c0, c1;
@@ -1149,18 +1204,30 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             }
             __syncthreads();
         }
-        // for the solves: the off-diagonal tiles and the inverses
-        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
-            const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
-            if (ir == jc)
-                reinterpret_cast<double2*>(Tall + 64 * (K0 + ir))[x & 31] = reinterpret_cast<const double2*>(s.Tblk + 64 * ir)[x & 31];
-            else
-                reinterpret_cast<double2*>(A + eix(K0 + ir, K0 + jc))[x & 31] = reinterpret_cast<const double2*>(s.Dblk)[x];
+        // for the solves and the cluster's other CTAs: the off-diagonal tiles and the inverses
+        auto exchange = [&](bool out) {
+            for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
+                const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
+                double2* const g2 = reinterpret_cast<double2*>(ir == jc ? Tall + 64 * (K0 + ir) : A + eix(K0 + ir, K0 + jc));
+                double2* const s2 = reinterpret_cast<double2*>(ir == jc ? s.Tblk + 64 * ir : tile(ir, jc));
+                if (out)
+                    g2[x & 31] = s2[x & 31];
+                else
+                    s2[x & 31] = g2[x & 31];
+            }
+        };
+        if (tc.rank() == 0) exchange(true);
+        if (tc.n() > 1) {
+            if (group_sync(tc, *s_fail)) return false;
+            if (tc.rank() > 0) exchange(false);
+            __syncthreads();
+        } else if (*s_fail) {
+            return false;
         }
         if (K1 >= Nt) break;
         // the rows below: one warp per row tile solves its four tiles against the diagonal
         // block and writes their slices (both column halves) and row scales
-        for (int it = K1 + warp; it < Nt; it += nwarps)
+        for (int it = K1 + warp + nwarps * tc.rank(); it < Nt; it += nwarps * tc.n())
             block_rows(A, it, K0, s.Dblk, s.Tblk, reinterpret_cast<double*>(s.stage) + kEB * 64 * warp,
                        reinterpret_cast<uint32_t*>(E + (int64_t)((it - K1) / kColT) * kGroupBytes +
                                                    (it - K1) % kColT * kSliceBytes),
@@ -1168,10 +1235,28 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
                        it >= Ntr ? udiag + 8 * (it - Ntr) : nullptr);
         // the slices are read by the copy engine (async proxy)
         asm volatile("fence.proxy.async;" ::: "memory");
-        __syncthreads();
-        if (!trailing_update_tc(c, A, Nt, Ntr, K1, E, sr, s.stage, tc)) return false;
+        group_barrier(tc);
+        if (tc.n() > 1) asm volatile("fence.proxy.async;" ::: "memory");
+        const bool ok = trailing_update_tc(A, Nt, Ntr, K1, E, sr, s.stage, tc);
+        // (alone, the update's own last barrier is enough)
+        if (tc.n() > 1 ? group_sync(tc, !ok) : !ok) return emu_fail(c, tc);
     }
     return true;
+}
+
+// The emulated kernel's solve for the right-hand side s.z, by the group's first CTA; the others take
+// the solution from its shared memory.
+template <class Tc>
+__device__ void solve_group(const SolveCtx& c, const Shared& s, const double* A, int Nt, double* out, Tc& tc) {
+    if (tc.rank() == 0) chol_solve_inv(s.z, s.Dsol, A, Nt, out, emu_tile_inverses(c));
+    if (tc.n() == 1) return;
+    group_sync(tc, 0);
+    if (tc.rank() > 0) {
+        const uint32_t from = peer_word(out, 0);
+        for (int j = threadIdx.x; j < 8 * Nt; j += blockDim.x)
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(out[j]) : "r"(from + 8 * j) : "memory");
+    }
+    __syncthreads();
 }
 
 // Assemble A, factorise, solve alpha.  Returns false if a pivot was not positive.
@@ -1185,8 +1270,8 @@ __device__ __forceinline__ void query_local(const SolveCtx& c, int I, int64_t p,
 // columns turns row Nr + a into v_a = L^-1 k_a and leaves the Schur complement, whose diagonal
 // entry is 1 - |v_a|^2 = u_a (Eq. 2).  Each appended row's arithmetic involves only that row and
 // the instance's own rows, so u_a does not depend on the other queries.
-template <bool kProps, bool kEmu = false>
-__device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t base, EmuTc* tc = nullptr, int nq = 0,
+template <bool kProps, bool kEmu = false, class Tc = EmuTc<false>>
+__device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t base, Tc* tc = nullptr, int nq = 0,
                              int64_t q0 = 0, int I = 0) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
@@ -1239,7 +1324,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         const int sq = nbc * (nbc + 1) / 2;  // blocks of the matrix itself; then nbc per block of query rows
         const int n_strip = 4 * (sq + (nbr - nbc) * nbc);
         const long long diag1 = fix_of_double(1.0 + c.P.s2);  // s2: sigma_prop^2 for properties
-        for (int st = warp; st < n_strip; st += nwarps) {
+        for (int st = warp + nwarps * tc->rank(); st < n_strip; st += nwarps * tc->n()) {
             const int p = st >> 2, c0 = 8 * (st & 3);
             const int bi = p < sq ? tri_row(p) : nbc + (p - sq) / nbc;
             const int bj = p < sq ? p - bi * (bi + 1) / 2 : (p - sq) % nbc;
@@ -1293,7 +1378,8 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
             }
         }
         if (nq > 0)
-            for (int a = tid; a < 8 * (Ntq - Nt); a += nt) emu_query_diag(c)[a] = 1ll << kFixBits;
+            for (int a = tid; a < 8 * (Ntq - Nt) && tc->rank() == 0; a += nt) emu_query_diag(c)[a] = 1ll << kFixBits;
+        group_barrier(*tc);
     }
     if constexpr (!kEmu) {
         for (int64_t tl = warp; tl < n_tiles(Nt); tl += nwarps) {
@@ -1440,8 +1526,8 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
         for (int ch = 0; ch < c.b.nprop; ++ch) {
             for (int i = tid; i < Ns; i += nt) s.z[i] = i < N ? c.b.yprop[(base + i) * c.b.nprop + ch] : 0.0;
             __syncthreads();
-            if (kEmu)
-                chol_solve_inv(s.z, s.Dsol, A, Nts, s.pa[ch], emu_tile_inverses(c));
+            if constexpr (kEmu)
+                solve_group(c, s, A, Nts, s.pa[ch], *tc);
             else
                 chol_solve(s, A, Nts, s.pa[ch]);
         }
@@ -1450,8 +1536,8 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
     // alpha = A^-1 1 (Eq. 1)
     for (int i = tid; i < Ns; i += nt) s.z[i] = i < N ? 1.0 : 0.0;
     __syncthreads();
-    if (kEmu)
-        chol_solve_inv(s.z, s.Dsol, A, Nts, s.alpha, emu_tile_inverses(c));
+    if constexpr (kEmu)
+        solve_group(c, s, A, Nts, s.alpha, *tc);
     else
         chol_solve(s, A, Nts, s.alpha);
     for (int j = tid; j < Ns; j += nt) {
@@ -1668,14 +1754,17 @@ __device__ __forceinline__ void invalid(EvalOut& r, int status) {
 }
 
 // The body of the GP solve kernels (see k_solve below).
-template <bool kProps, bool kEmu>
+template <bool kProps, bool kEmu, bool kGroup>
 __device__ __forceinline__ void solve_body(const SolveCtx& c) {
     extern __shared__ __align__(128) double sm[];
     __shared__ int s_item[2];
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_bar[2];
     const int tid = threadIdx.x, nt = blockDim.x;
-    double* ws_a = c.a_in_smem ? nullptr : c.ws_a + (int64_t)blockIdx.x * c.ws_a_stride;
+    __shared__ int s_flags[2 * 8];
+    const int ncta = kGroup ? c.ncta : 1;
+    const int group = (int)blockIdx.x / ncta, n_groups = (int)gridDim.x / ncta;  // CTAs that share work items
+    double* ws_a = c.a_in_smem ? nullptr : c.ws_a + (int64_t)group * c.ws_a_stride;
     Shared s = carve(sm, c.npad, c.a_in_smem, ws_a, c.b.nprop, c.stage_panel, c.b.Xi != nullptr, false, kEmu);
     double* V = c.ws_v ? c.ws_v + (int64_t)blockIdx.x * c.ws_v_stride + tid : nullptr;
     const bool lattice = c.b.Xi != nullptr;
@@ -1687,7 +1776,10 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             s.Tff[j] = make_float2(h, l);
         }
     for (int j = tid; j < 256; j += nt) s.dtab[j] = diag_entry(j >> 5, j & 31);
-    EmuTc tc{};
+    EmuTc<kGroup> tc{};
+    tc.n_ = ncta;
+    tc.rank_ = (int)blockIdx.x % ncta;
+    tc.flags = s_flags;
     if (kEmu) {
         // tensor memory for the 8 slice-group accumulators (held until the CTA exits) and the
         // barriers of the staging copies and of the MMAs
@@ -1709,14 +1801,18 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
         tc.tmem = s_tmem;
         tc.bar_ld = smem_addr(&s_bar[0]);
         tc.bar_mma = smem_addr(&s_bar[1]);
+        if (tc.n() > 1) {  // every CTA of the cluster runs before another one writes to its shared memory
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
     }
     for (bool first = true;; first = false) {
         // the next work item: an instance, or one chunk of its queries (the instance is fitted
         // again for every chunk, so the queries of a large instance spread over the GPU).  CTA i
         // takes item i first (the CTAs of a launch are spread over the SMs in index order, so a
         // grid larger than the work stays balanced), then items from the counter.
-        if (tid == 0) {
-            const int w = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(c.counter, 1);
+        if (tid == 0 && tc.rank() == 0) {
+            const int w = first ? group : n_groups + atomicAdd(c.counter, 1);
             // graph mode: this bucket's count and share of the order, planned on the device
             const int nb = c.plan ? c.plan[c.bucket] : c.n_work;
             const int ob = c.plan ? c.plan[5 + c.bucket] : 0;
@@ -1740,10 +1836,21 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             }
             s_item[0] = w < nw ? (c.order ? c.order[ob + k] : c.inst_base + k) : -1;
             s_item[1] = ci;
+            if constexpr (kEmu)
+                for (int r = 1; r < tc.n(); ++r) {
+                    peer_store(&s_item[0], r, s_item[0]);
+                    peer_store(&s_item[1], r, s_item[1]);
+                }
         }
-        __syncthreads();
+        if constexpr (kEmu)
+            group_barrier(tc);
+        else
+            __syncthreads();
         const int I = s_item[0], ci = s_item[1];
-        __syncthreads();
+        if constexpr (kEmu)
+            group_barrier(tc);
+        else
+            __syncthreads();
         if (I < 0) break;
         const int64_t base = c.b.inst_off[I];
         const int N = (int)(c.b.inst_off[I + 1] - base);
@@ -1760,7 +1867,7 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                 const int64_t cq1 = kEmu ? min(q1, cq0 + (int64_t)c.qmax) : q1;
                 const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, kEmu ? (int)(cq1 - cq0) : 0, cq0, I);
                 const int64_t ce = ok ? cq1 : q1;  // a failed factorisation answers all remaining queries
-                for (int64_t p = cq0 + tid; p < ce; p += nt) {
+                for (int64_t p = cq0 + tid + (int64_t)nt * tc.rank(); p < ce; p += nt * tc.n()) {
                     const int64_t qid = c.b.qidx ? c.b.qidx[p] : p;
                     double xl[3], cm[4] = {NAN, NAN, NAN, NAN}, w = INFINITY;
                     int qi = 0;
@@ -1778,7 +1885,10 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                     c.b.pw[qid] = w;
                 }
                 if (!ok && N > 0 && tid == 0 && !tc.dead) atomicOr(c.err, kErrFactor);
-                __syncthreads();
+                if constexpr (kEmu)
+                    group_barrier(tc);
+                else
+                    __syncthreads();
                 cq0 = ce;
                 if ((kEmu && tc.dead) || cq0 >= q1) break;
             }
@@ -1794,10 +1904,10 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
             const int64_t cq1 = border ? min(q1, cq0 + (int64_t)c.qmax) : q1;
             const bool ok = N > 0 && fit_instance<kProps, kEmu>(c, s, N, base, &tc, border ? (int)(cq1 - cq0) : 0,
                                                                  cq0, I);
-            if (c.b.alpha_out && ci == 0 && cq0 == q0)
+            if (c.b.alpha_out && ci == 0 && cq0 == q0 && tc.rank() == 0)
                 for (int j = tid; j < N; j += nt) c.b.alpha_out[base + j] = ok ? s.alpha[j] : NAN;
             const int64_t ce = ok ? cq1 : q1;  // a failed factorisation answers all remaining queries
-            for (int64_t p = cq0 + tid; p < ce; p += nt) {
+            for (int64_t p = cq0 + tid + (int64_t)nt * tc.rank(); p < ce; p += nt * tc.n()) {
                 const int64_t qid = c.b.qidx ? c.b.qidx[p] : p;
                 EvalOut r;
                 if (!ok) {
@@ -1823,7 +1933,10 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                 write_out(c.b, qid, r);
             }
             if (!ok && N > 0 && tid == 0 && !tc.dead) atomicOr(c.err, kErrFactor);
-            __syncthreads();
+            if constexpr (kEmu)
+                group_barrier(tc);
+            else
+                __syncthreads();
             cq0 = ce;
             if ((kEmu && tc.dead) || cq0 >= q1) break;
         }
@@ -1848,12 +1961,12 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
 // (up to 736 threads, the largest shape its registers have allowed)
 template <bool kProps>
 __global__ void __launch_bounds__(736) k_solve(SolveCtx c) {
-    solve_body<kProps, false>(c);
+    solve_body<kProps, false, false>(c);
 }
 
-template <bool kProps>
+template <bool kProps, bool kGroup>
 __global__ void __launch_bounds__(kEmuThreads, 2) k_solve_emu(SolveCtx c) {
-    solve_body<kProps, true>(c);
+    solve_body<kProps, true, kGroup>(c);
 }
 
 // Backward pass (derived from Eq. 1 and Eq. 3): per instance,
@@ -2177,9 +2290,10 @@ BucketShape bucket_shape(const SolveConfig& cfg, int i, int64_t cnt, int n_sm, b
     return b;
 }
 
-SolveKernel pick_solve(bool props, bool emu) {
-    if (props) return emu ? k_solve_emu<true> : k_solve<true>;
-    return emu ? k_solve_emu<false> : k_solve<false>;
+SolveKernel pick_solve(bool props, bool emu, bool group = false) {
+    if (emu && group) return props ? k_solve_emu<true, true> : k_solve_emu<false, true>;
+    if (props) return emu ? k_solve_emu<true, false> : k_solve<true>;
+    return emu ? k_solve_emu<false, false> : k_solve<false>;
 }
 
 // seven bf16 slices of a block's columns, the row scale, one row of diagonal-tile inverses, and an
@@ -2203,6 +2317,17 @@ void chunk_args(const SolveBatch& b, int i, int cnt, int nmax, int n_sm, int per
     a.cap[i] = emu && b.want_var ? kBorderQ : 0;
     a.slots[i] = n_sm * (emu || !heavy ? per_sm : std::min(per_sm, std::max(1, 512 / threads)));
     a.qmin[i] = !heavy ? 64 * std::max(nmax, 1) : emu ? 64 : 128;
+}
+
+// CTAs that work on an instance together (a cluster) in an emulated launch of at most `items` work
+// items, nmax points at most, on `slots` resident CTAs: as many as keep every item resident, up to 8.
+// K, the rows below and the trailing tiles are shared out, the diagonal blocks and the solves
+// are not, and a block of 32 columns costs three cluster barriers; below 128 points nothing
+// is left to share.
+int group_ctas(int items, int nmax, int slots) {
+    int n = 1;
+    while (n < 8 && nmax > 128 && (int64_t)items * 2 * n <= slots) n *= 2;
+    return n;
 }
 
 // Emulated launch with the latent variance: the queries of an instance (up to kBorderQ) are
@@ -2710,13 +2835,16 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         const size_t shm = L.shm;
         auto kern = L.kern;
         const int per_sm = L.per_sm;
-        const int grid = (int)std::min<int64_t>(bw ? cnt : max_items[bi], (int64_t)n_sm * per_sm);
+        // few emulated work items: clusters of CTAs work on each
+        if (emu) c.ncta = group_ctas(max_items[bi], nmax, n_sm * per_sm);
+        const int groups = (int)std::min<int64_t>(bw ? cnt : max_items[bi], (int64_t)n_sm * per_sm / c.ncta);
+        const int grid = groups * c.ncta;
         c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
-        c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * grid, st);
+        c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * groups, st);
         c.ws_v_stride = (int64_t)c.npad * threads;
         c.ws_v = (b.want_var && !bw && !emu) ? (double*)ar.get(aside ? Arena::kWs4 : Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
         c.ws_e_stride = emu ? (int64_t)c.nrow * kEmuBytesPerRow : 0;
-        c.ws_e = emu ? (uint8_t*)ar.get(Arena::kWs3, c.ws_e_stride * grid, st) : nullptr;
+        c.ws_e = emu ? (uint8_t*)ar.get(Arena::kWs3, c.ws_e_stride * groups, st) : nullptr;
         if ((!c.a_in_smem && !c.ws_a) || (b.want_var && !bw && !emu && !c.ws_v) || (emu && !c.ws_e)) {
             if (profile) {
                 cudaEventDestroy(ev0);
@@ -2730,7 +2858,25 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             cudaEventCreate(&b1);
             cudaEventRecord(b0, st);
         }
-        kern<<<grid, threads, shm, ls>>>(c);
+        if (c.ncta == 1) {
+            kern<<<grid, threads, shm, ls>>>(c);
+        } else {
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = c.ncta;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cudaLaunchConfig_t lc{};
+            lc.gridDim = dim3(grid);
+            lc.blockDim = dim3(threads);
+            lc.dynamicSmemBytes = shm;
+            lc.stream = ls;
+            lc.attrs = &at;
+            lc.numAttrs = 1;
+            kern = pick_solve(b.nprop > 0, true, true);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+            set_emu_carveout(kern);
+            cudaLaunchKernelEx(&lc, kern, c);
+        }
         note_launch();
         if (aside && (cudaEventRecord(gc->e1, gc->gs) != cudaSuccess || cudaStreamWaitEvent(st, gc->e1, 0) != cudaSuccess)) {
             k_or_err<<<1, 1, 0, st>>>(err_dev, kErrLaunch);
