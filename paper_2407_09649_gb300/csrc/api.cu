@@ -1425,13 +1425,14 @@ static int plan_smooth(vgp_map* m, const float* q, int64_t n, int n_nodes, cudaS
     ARENA(nn, uint8_t, kPair1, n);
     ARENA(cnt, int64_t, kTmp15, ni + 1);
     ARENA(q_off, int64_t, kTmp16, ni + 1);
-    ARENA(cursor, int64_t, kTmp17, ni + 1);
+    ARENA(gnode, int32_t, kTmp17, 27 * (int64_t)G.ng);
     ARENA(qidx, int64_t, kPair2, np);
+    ARENA(pair_pos, int32_t, kPair7, np);
     CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * (ni + 1), st));
-    CUDA_TRY(cudaMemsetAsync(cursor, 0, sizeof(int64_t) * (ni + 1), st));
-    smooth_pairs(q, n, G.q_slot, G.slot2group, G.gcen, m->s_tab, it, islot2inst, P, n_nodes, pair_inst, nn, cnt, st);
+    smooth_pairs(q, n, G.q_slot, G.slot2group, G.gcen, G.ng, it, islot2inst, P, n_nodes, gnode, pair_inst, pair_pos, nn,
+                 cnt, st);
     exclusive_scan_i64(cnt, q_off, ni, st, m->ar);
-    smooth_scatter(pair_inst, np, q_off, cursor, qidx, st);
+    smooth_scatter(pair_inst, pair_pos, np, q_off, qidx, st);
     SP.ni = ni;
     SP.T = T;
     SP.ikeys = ikeys;

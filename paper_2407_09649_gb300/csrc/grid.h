@@ -81,10 +81,10 @@ void inst_gather(const uint64_t* ikey, int ni, const Table& s, const int32_t* ss
 // G-GPDF blended per-leaf GPs (Eq. 10)
 void smooth_nodes(const uint64_t* gcen, int ng, const Table& s, const Table& it, int* err, cudaStream_t st);
 void smooth_pairs(const float* q, int64_t n, const int32_t* q_slot, const int32_t* slot2group, const uint64_t* gcen,
-                  const Table& s, const Table& it, const int32_t* islot2inst, const DevParams& P, int Q,
-                  int32_t* pair_inst, uint8_t* n_nodes, int64_t* inst_cnt, cudaStream_t st);
-void smooth_scatter(const int32_t* pair_inst, int64_t npairs, const int64_t* q_off, int64_t* cursor, int64_t* qidx,
-                    cudaStream_t st);
+                  int ng, const Table& it, const int32_t* islot2inst, const DevParams& P, int Q, int32_t* gnode,
+                  int32_t* pair_inst, int32_t* pair_pos, uint8_t* n_nodes, int64_t* inst_cnt, cudaStream_t st);
+void smooth_scatter(const int32_t* pair_inst, const int32_t* pair_pos, int64_t npairs, const int64_t* q_off,
+                    int64_t* qidx, cudaStream_t st);
 void smooth_blend(int64_t n, int Q, const int32_t* q_slot, const uint8_t* n_nodes, const double* pd, const double* pg,
                   const double* pv, const uint8_t* ps, double lambda, const DevParams& P, double* d, double* grad,
                   double* var, uint8_t* status, cudaStream_t st);

@@ -79,7 +79,8 @@ struct SolveCtx {
     BackwardBatch bw;
     const int* chunk_off = nullptr;  // work items (see k_chunk_plan): chunk offsets over the order;
                                      // nullptr: one work item per instance
-    const int* chunk_q = nullptr;    // queries of a work item for this launch (0: all of them)
+    const int* chunk_q = nullptr;    // queries of a work item for this launch (0: all of them; chunk_len)
+    int chunk_qn = 0, chunk_cap = 0;
     int qmax = 0;          // emulated kernel with variance: query rows appended to A (0: none)
     int nrow = 0;          // emulated kernel: rows of the workspace matrices (npad + qmax)
     int ncta = 1;          // emulated kernel: CTAs (a cluster) that work on one instance together
@@ -1549,6 +1550,12 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
     return true;
 }
 
+// Queries of a work item on an instance of N points (see k_chunk_plan).
+__host__ __device__ __forceinline__ long long chunk_len(long long qc, int qn, long long N, int cap) {
+    const long long q = qc > qn * N ? qc : qn * N;
+    return cap > 0 && q > cap ? cap : q;
+}
+
 struct EvalOut {
     double d, g[3], v;
     int status;
@@ -1855,8 +1862,9 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
         const int64_t base = c.b.inst_off[I];
         const int N = (int)(c.b.inst_off[I + 1] - base);
         const int64_t qa = c.b.q_off[I], qb = c.b.q_off[I + 1];
-        const int qch = c.chunk_q ? *c.chunk_q : 0;
-        const int64_t q0 = qch > 0 ? min(qb, qa + (int64_t)ci * qch) : qa;
+        const int qc = c.chunk_q ? *c.chunk_q : 0;
+        const int64_t qch = qc > 0 ? chunk_len(qc, c.chunk_qn, N, c.chunk_cap) : 0;
+        const int64_t q0 = qch > 0 ? min(qb, qa + ci * qch) : qa;
         const int64_t q1 = qch > 0 ? min(qb, q0 + qch) : qb;
         if (kProps) {
             // property mode: means and variance (Eq. 6, variance read as for Eq. 2).  The emulated
@@ -2120,16 +2128,17 @@ __global__ void k_plan_buckets(const int* hist, int* cursor, int* plan) {
     }
 }
 
-// Work items of the solve launches: a bucket of no more instances than CTAs that can run at once has
-// its queries split into chunks, so that they spread over the GPU; each chunk fits its instance again.
-// Launch b's chunk size qc is the smallest, from qmin[b], that gives no more chunks than the
-// slots[b] CTAs: the refits then run on CTAs that had no work, and the longest chunk is as short as
-// can be.  qmin: what an evaluation has to be worth a fit.  cap[b] > 0 bounds qc (the rows a
-// bordered factorisation appends).  chunk_q[b] receives qc (0: no split); chunk_off[k] the number of
-// work items of the order before instance k, chunk_off[n] the total.  The buckets are contiguous
-// in the order: from the device plan in graph mode, else from a.
+// Work items of the solve launches: an instance's queries are split into chunks, so that they spread
+// over the GPU; each chunk fits the instance again.  The chunk size of an instance of N points in
+// launch b is max(qc, qn[b] N), qn N queries being what an evaluation has to be worth a fit
+// (chunk_len).  qc is the smallest, from qmin[b], that gives no more chunks than the slots[b] CTAs
+// that run at once, or slots[b] more than instances where those are more: the refits then run on CTAs
+// that had no work, and the longest chunk, the launch's tail, is as short as can be.  cap[b] > 0
+// bounds qc (the rows a bordered factorisation appends).  chunk_q[b] receives qc (0: no split);
+// chunk_off[k] the number of work items of the order before instance k, chunk_off[n] the total.
+// The buckets are contiguous in the order: from the device plan in graph mode, else from a.
 struct ChunkPlanArgs {
-    int off[5], cnt[5], slots[5], cap[5], qmin[5];
+    int off[5], cnt[5], slots[5], cap[5], qmin[5], qn[5];
 };
 // Sum over the CTA (all threads call; w: one value per warp of scratch), the same on every thread.
 __device__ long long block_sum(long long v, long long* w) {
@@ -2151,24 +2160,42 @@ __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_of
     if (tid == 0) carry = 0;
     for (int bk = 0; bk < 5; ++bk) {
         const int off = plan ? plan[5 + bk] : a.off[bk], cnt = plan ? plan[bk] : a.cnt[bk];
-        int qc = a.cap[bk];
-        if (cnt > 0 && cnt <= a.slots[bk]) {
-            auto chunks_at = [&](long long q) {  // work items with chunks of q queries
-                long long v = 0;
-                for (int k = tid; k < cnt; k += blockDim.x) {
+        const int cap = a.cap[bk], qn = a.qn[bk];
+        int qc = cap;
+        if (cnt > 0 && a.qmin[bk] > 0) {
+            const long long most = (cnt > a.slots[bk] ? (long long)cnt : 0) + a.slots[bk];
+            int n0[4], q0[4];  // this thread's first instances, read once
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int k = tid + r * blockDim.x;
+                n0[r] = q0[r] = 0;
+                if (k < cnt) {
                     const int I = order[off + k];
-                    const long long nq = q_off[I + 1] - q_off[I];
-                    v += nq > q ? (nq + q - 1) / q : 1;
+                    n0[r] = (int)(inst_off[I + 1] - inst_off[I]);
+                    q0[r] = (int)min((long long)INT32_MAX, (long long)(q_off[I + 1] - q_off[I]));
                 }
-                return block_sum(v, wq);
+            }
+            auto chunks_at = [&](long long qs) {  // work items beyond one per instance
+                long long v = 0;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const unsigned q = (unsigned)min((long long)INT32_MAX, chunk_len(qs, qn, n0[r], cap));
+                    if ((unsigned)q0[r] > q) v += ((unsigned)q0[r] - 1) / q;
+                }
+                for (int k = tid + 4 * blockDim.x; k < cnt; k += blockDim.x) {
+                    const int I = order[off + k];
+                    const long long nq = q_off[I + 1] - q_off[I], q = chunk_len(qs, qn, inst_off[I + 1] - inst_off[I], cap);
+                    if (nq > q) v += (nq - 1) / q;
+                }
+                return cnt + block_sum(v, wq);
             };
             long long lo = a.qmin[bk], hi = lo;
-            while (hi < INT32_MAX / 2 && chunks_at(hi) > a.slots[bk]) hi *= 2;
+            while (hi < INT32_MAX / 2 && (cap == 0 || hi < cap) && chunks_at(hi) > most) hi *= 2;
             if (hi > lo) {
                 lo = hi / 2;  // too many chunks at lo, few enough at hi
                 while (hi - lo > max(1ll, lo / 32)) {
                     const long long mid = (lo + hi) / 2;
-                    if (chunks_at(mid) > a.slots[bk])
+                    if (chunks_at(mid) > most)
                         lo = mid;
                     else
                         hi = mid;
@@ -2184,7 +2211,8 @@ __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_of
             if (k < cnt) {
                 const int I = order[off + k];
                 const int64_t nq = q_off[I + 1] - q_off[I];
-                v = qc > 0 ? (int)max((int64_t)1, (nq + qc - 1) / qc) : 1;
+                const long long q = chunk_len(qc, qn, inst_off[I + 1] - inst_off[I], cap);
+                v = qc > 0 ? (int)max(1ll, (nq + q - 1) / q) : 1;
             }
             int x = v;
 #pragma unroll
@@ -2303,20 +2331,20 @@ constexpr int64_t kEmuBytesPerRow = 7 * 8 * kEB * 2 + 8 + 64 + 8;
 // Words of a matrix of `rows` rows in a CTA's workspace (rows: a multiple of 8).
 int64_t matrix_words(bool emu, int rows) { return emu ? n_blocks(rows) * 1024 : n_tiles(rows / 8) * 64; }
 
-// Chunk planning of launch i (cnt instances of up to nmax points, resident CTAs, threads each): the
-// CTAs to spread it over, the bound of an emulated launch that appends query rows, and the
-// shortest chunk worth a fit.
-// * Emulated launches spread over all resident CTAs; 64 queries with variance or properties.
+// Chunk planning of launch i (cnt instances, resident CTAs per SM, threads each): the CTAs to spread it
+// over, the bound of an emulated launch that appends query rows, and the shortest chunk worth a fit.
+// * Emulated launches spread over all resident CTAs; with variance or properties an appended row of
+//   an N-point instance costs about 1 / N of its fit, at least 64 of them.
 // * Plain launches with variance run on the FP64 pipe, which one warp per sub-partition nearly fills:
 //   16 warps per SM are enough, and more would only refit; 128 queries.
 // * The mean alone costs about N FP32 values a query: a fit is worth about 64 N of them.
-void chunk_args(const SolveBatch& b, int i, int cnt, int nmax, int n_sm, int per_sm, int threads, bool emu,
-                ChunkPlanArgs& a) {
+void chunk_args(const SolveBatch& b, int i, int cnt, int n_sm, int per_sm, int threads, bool emu, ChunkPlanArgs& a) {
     const bool heavy = b.want_var || b.nprop > 0;
     a.cnt[i] = cnt;
     a.cap[i] = emu && b.want_var ? kBorderQ : 0;
     a.slots[i] = n_sm * (emu || !heavy ? per_sm : std::min(per_sm, std::max(1, 512 / threads)));
-    a.qmin[i] = !heavy ? 64 * std::max(nmax, 1) : emu ? 64 : 128;
+    a.qmin[i] = heavy && !emu ? 128 : 64;
+    a.qn[i] = !heavy ? 64 : emu ? 1 : 0;
 }
 
 // CTAs that work on an instance together (a cluster) in an emulated launch of at most `items` work
@@ -2472,7 +2500,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         // (without variance and properties splitting rarely pays: no workspace for it)
         s.grid = n_sm * per_sm;
         if (!b.want_var && !props) s.grid = (int)std::min<int64_t>(n, s.grid);
-        chunk_args(b, i, 0, std::min(hi[i], maxn), n_sm, per_sm, s.threads, s.emu, ca);
+        chunk_args(b, i, 0, n_sm, per_sm, s.threads, s.emu, ca);
         ca.slots[i] = std::min(ca.slots[i], s.grid);
         if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
         if (b.want_var && !s.emu) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
@@ -2511,6 +2539,8 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         SolveCtx c;
         c.chunk_off = chunk_off;
         c.chunk_q = chunk_q + i;
+        c.chunk_qn = ca.qn[i];
+        c.chunk_cap = ca.cap[i];
         c.b = b;
         c.P = P;
         c.err = err_dev;
@@ -2771,10 +2801,21 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         off += cnt;
         if (cnt == 0) continue;
         const Launch L = bucket_launch(i, nmax, cnt);
-        chunk_args(b, i, cnt, nmax, n_sm, L.per_sm, L.threads, L.emu, ca);
-        const bool split = cnt <= ca.slots[i] && (int64_t)hq[i] > ca.qmin[i];
-        max_items[i] = (int)std::min<int64_t>(INT32_MAX, cnt + (split ? (int64_t)hq[i] / ca.qmin[i] : 0));
-        chunks = chunks || split || (ca.cap[i] > 0 && (int64_t)hq[i] > ca.cap[i]);
+        chunk_args(b, i, cnt, n_sm, L.per_sm, L.threads, L.emu, ca);
+        int nmin = nmax;
+        for (int N = nmax; N >= buckets[i].lo; --N)
+            if (h[N]) nmin = N;
+        // the shortest chunk any of its instances can have
+        const int64_t len = std::max<int64_t>(1, chunk_len(ca.qmin[i], ca.qn[i], nmin, ca.cap[i]));
+        const int64_t extra = std::min<int64_t>((int64_t)hq[i] / len, ca.cap[i] > 0 ? INT32_MAX : ca.slots[i]);
+        max_items[i] = (int)std::min<int64_t>(INT32_MAX, cnt + extra);
+        // (without a bound, a launch of ten rounds of instances or more has no tail to shorten)
+        if (ca.cap[i] == 0 && cnt > 10 * ca.slots[i]) {
+            ca.qmin[i] = 0;
+            max_items[i] = cnt;
+        } else {
+            chunks = chunks || extra > 0;
+        }
     }
     if (chunks) {
         chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
@@ -2823,6 +2864,8 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         c.n_work = cnt;
         c.chunk_off = chunk_off ? chunk_off + done : nullptr;
         c.chunk_q = chunk_q ? chunk_q + bi : nullptr;
+        c.chunk_qn = ca.qn[bi];
+        c.chunk_cap = ca.cap[bi];
         const Launch L = bucket_launch(bi, nmax, cnt);
         c.npad = L.npad;
         c.qmax = L.qmax;
