@@ -94,7 +94,7 @@ struct vgp_map {
     int device = 0;
     Arena ar;
     int* dev_words = nullptr;  // [0] err, [1] n_valid, [2] count, [3] pool_count, [4] orphan
-    double* tables = nullptr;  // exp_neg table (256) + lattice kernel table (kLatticeTable), FP64
+    double* tables = nullptr;  // exponential table (256 pairs) + lattice kernel table (kLatticeTable), FP64
     float* tables_f = nullptr; // lattice kernel table in FP32
     int* host_words = nullptr; // pinned mirror
     // global grid
@@ -303,14 +303,18 @@ int vgp_create(const vgp_params* p, vgp_map** out) {
     }
     cudaMemset(m->dev_words, 0, sizeof(int) * 8);
     // constant tables, computed on the host in extended precision and rounded once:
-    // 2^(j/256) for the FP64 exponential, exp(-m vs^2 / (2 l^2)) for voxel-lattice distances
-    std::vector<double> tab(256 + kLatticeTable);
+    // 2^(j/256) for the FP64 exponentials (as pairs: all high parts, then all low parts), exp(-m vs^2 / (2 l^2)) for voxel-lattice distances
+    std::vector<double> tab(512 + kLatticeTable);
     std::vector<float> tabf(kLatticeTable);
-    for (int j = 0; j < 256; ++j) tab[j] = (double)exp2l((long double)j / 256.0L);
+    for (int j = 0; j < 256; ++j) {
+        const long double t = exp2l((long double)j / 256.0L);
+        tab[j] = (double)t;
+        tab[256 + j] = (double)(t - (long double)tab[j]);
+    }
     const long double vs = p->voxel_size, l = p->lengthscale;
     for (int m2 = 0; m2 < kLatticeTable; ++m2) {
         const long double v = expl(-(long double)m2 * vs * vs / (2.0L * l * l));
-        tab[256 + m2] = (double)v;
+        tab[512 + m2] = (double)v;
         tabf[m2] = (float)v;
     }
     if (cudaMalloc(&m->tables, sizeof(double) * tab.size()) != cudaSuccess ||
@@ -325,7 +329,8 @@ int vgp_create(const vgp_params* p, vgp_map** out) {
     cudaMemcpy(m->tables, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice);
     cudaMemcpy(m->tables_f, tabf.data(), sizeof(float) * tabf.size(), cudaMemcpyHostToDevice);
     m->P.exp_tab = m->tables;
-    m->P.lat_tab = m->tables + 256;
+    m->P.exp_lo = m->tables + 256;
+    m->P.lat_tab = m->tables + 512;
     m->P.lat_tab_f = m->tables_f;
     std::vector<uint8_t> mc(256 * 17, 0);
     build_mc_table(mc.data(), mc.data() + 256 * 16);

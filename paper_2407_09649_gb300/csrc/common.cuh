@@ -40,7 +40,8 @@ struct DevParams {
     int cap_leaf, cap_group, search_r, fusion, precision, n_props;
     int emulate;        // Cholesky trailing updates of N > 32 instances on the bf16 tensor cores
     double s2p;         // sigma_prop^2 (surface-property GP, Eq. 6)
-    const double* exp_tab;   // 2^(j/256), j = 0..255 (FP64), for exp_neg
+    const double* exp_tab;   // 2^(j/256), j = 0..255 (FP64), for exp_neg and exp_near
+    const double* exp_lo;    // 2^(j/256) - exp_tab[j], rounded
     const double* lat_tab;   // exp(-m vs^2 / (2 l^2)), m = 0..kLatticeTable-1 (FP64)
     const float* lat_tab_f;  // the same in FP32
 };
@@ -51,8 +52,12 @@ constexpr int kLatticeTable = 1024;  // squared integer offsets up to 3 * 15^2 =
 // function in IEEE floating-point arithmetic", 1989): y = (256 m + j) ln2/256 + r with
 // |r| <= ln2/512, e^y = 2^m * 2^(j/256) * e^r, e^r by its degree-4 Taylor polynomial
 // (remainder below 4e-17 relative).  tab[j] = 2^(j/256).  Returns 0 for y < -700.
+__device__ __forceinline__ bool above_700(double y) {  // -700 <= y <= 0, on the integer pipe (false for NaN)
+    const int h = __double2hiint(y) & 0x7fffffff;
+    return h < 0x4085E000 || (h == 0x4085E000 && __double2loint(y) == 0);
+}
 __device__ __forceinline__ double exp_neg(double y, const double* tab) {
-    if (!(y >= -700.0)) return 0.0;
+    if (!above_700(y)) return 0.0;
     const double big = 6755399441055744.0;  // 1.5 * 2^52: y * 256/ln2 rounded to an integer
     const double tm = fma(y, 369.3299304675746, big);
     const int ni = __double2loint(tm);
@@ -64,6 +69,28 @@ __device__ __forceinline__ double exp_neg(double y, const double* tab) {
     p = fma(p, r, 1.0);
     p = fma(p, r, 1.0);
     const double s = tab[ni & 255] * p;
+    return __longlong_as_double(__double_as_longlong(s) + ((long long)(ni >> 8) << 52));
+}
+
+// e^y for y <= 0 in FP64, the same reduction with 2^(j/256) as a pair of doubles: the polynomial's part is
+// added to it last, so the error stays below 0.7 ulp (half an ulp of the final sum, 0.17 of the
+// polynomial's remainder), under the library exp's 1 ulp, in 10 FP64 operations against its 17.
+// For the blend's weights and the backward pass (the forward kernel values keep the library's: a last
+// bit there moves FP64 results by the factorisation's condition number).  tab, lo: exp_tab and
+// exp_lo.  Below -700 the library's.
+__device__ __forceinline__ double exp_near(double y, const double* tab, const double* lo) {
+    if (!above_700(y)) return exp(y);
+    const double big = 6755399441055744.0;
+    const double tm = fma(y, 369.3299304675746, big);
+    const int ni = __double2loint(tm);
+    const double n = tm - big;
+    double r = fma(-n, 0x1.62e42fef80000p-9, y);
+    r = fma(-n, 0x1.1cf79abc9e3b4p-44, r);
+    double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    const double q = fma(r * r, p, r);  // e^r - 1
+    const double T = tab[ni & 255];
+    const double s = T + fma(T, q, lo[ni & 255]);
     return __longlong_as_double(__double_as_longlong(s) + ((long long)(ni >> 8) << 52));
 }
 

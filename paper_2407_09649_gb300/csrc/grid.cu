@@ -1347,7 +1347,7 @@ __global__ void k_smooth_blend(int64_t n, int Q, const int32_t* q_slot, const ui
             for (int t = 0; t < nn; ++t) {
                 const int64_t p = i * Q + t;
                 if (ps[p] != VGP_ST_OK) continue;
-                const double w = exp_neg(-lambda * (pd[p] - dmin), P.exp_tab);
+                const double w = exp_near(-lambda * (pd[p] - dmin), P.exp_tab, P.exp_lo);
                 sw += w;
                 swd += w * pd[p];
                 if (pv) swv += w * pv[p];

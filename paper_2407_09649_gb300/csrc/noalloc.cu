@@ -28,8 +28,8 @@ constexpr int kMaxGrid = 304;            // persistent CTAs (2 per SM on 152 SMs
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kOffWords = 0;                                                  // [0] counter, [1] error
-constexpr size_t kOffTab = 256;                                                  // 2^(j/256), 256 doubles
-constexpr size_t kOffOrder = align256(kOffTab + 256 * sizeof(double));           // int32 per instance
+constexpr size_t kOffTab = 256;                                                  // 2^(j/256), 256 pairs (high, then low parts)
+constexpr size_t kOffOrder = align256(kOffTab + 512 * sizeof(double));           // int32 per instance
 constexpr size_t kOffCentre = align256(kOffOrder + kMaxInst * sizeof(int32_t));  // 3 doubles per instance
 constexpr size_t kOffXl = align256(kOffCentre + 3 * kMaxInst * sizeof(double));  // 3 doubles per point
 constexpr size_t kOffXf = align256(kOffXl + 3 * kMaxPoints * sizeof(double));    // 3 floats per point
@@ -54,9 +54,13 @@ int fail(int code, const char* fmt, ...) {
 // 2^(j/256), j = 0..255, for the FP64 table exponential; written into the scratch array on the
 // caller's stream by every call (stream-ordered, so no stream can read it half written).
 struct ExpTable {
-    double v[256];
+    double v[512];
     ExpTable() {
-        for (int j = 0; j < 256; ++j) v[j] = (double)exp2l((long double)j / 256.0L);
+        for (int j = 0; j < 256; ++j) {
+            const long double t = exp2l((long double)j / 256.0L);
+            v[j] = (double)t;
+            v[256 + j] = (double)(t - (long double)v[j]);
+        }
     }
 };
 const ExpTable g_tab;
@@ -189,6 +193,7 @@ extern "C" int vgp_gp_batch_static(const vgp_params* p, int64_t n_inst, const in
     P.vs_f = (float)p->voxel_size;
     P.precision = p->precision;
     P.exp_tab = (const double*)(base + kOffTab);
+    P.exp_lo = P.exp_tab + 256;
     SolveBatch b;
     b.n_inst = n_inst;
     b.inst_off = inst_off;

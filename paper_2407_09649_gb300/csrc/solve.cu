@@ -1627,79 +1627,93 @@ __device__ __forceinline__ void query_local(const SolveCtx& c, int I, int64_t p,
     for (int a = 0; a < 3; ++a) xl[a] = xg[a] - c.b.centre[3 * (int64_t)I + a];
 }
 
-// Latent mean and gradient at one query; returns lo = log o and gro = grad o / o.
-// qi: biased lattice offsets of the query (lattice instances only).
-__device__ __forceinline__ void latent_mean(const DevParams& P, const Shared& s, int N, bool lattice, int qi,
-                                            const double xl[3], double& lo, double gro[3]) {
-    if (P.precision == VGP_MIXED) {
-        // FP32 kernel values and FP32 accumulation.  Off the lattice, the nearest training point
-        // shifts the exponent (exp(-(r^2 - r0^2) / 2l^2) <= 1, no underflow).  The sum is
-        // compensated: alpha is carried as two floats and the rounding error of every product
-        // and addition is accumulated separately (Neumaier), all on the FP32 pipe.
-        const float qx = (float)xl[0], qy = (float)xl[1], qz = (float)xl[2];
-        float r0 = 0.f;
-        if (!lattice) {
-            r0 = INFINITY;
-            for (int j = 0; j < N; ++j) {
-                float dx = s.Xf[3 * j] - qx, dy = s.Xf[3 * j + 1] - qy, dz = s.Xf[3 * j + 2] - qz;
-                r0 = fminf(r0, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-            }
-        }
-        float sum = 0.f, comp = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+// Mixed precision: latent mean and gradient at one query as sums of kernel values scaled by
+// e^(r0^2 / 2l^2): tot = o times that (FP64 sum of two floats), g = l^2 grad o times it.
+// qi: biased lattice offsets of the query (lattice instances only; r0 = 0 there).
+// FP32 kernel values and FP32 accumulation.  Off the lattice, the nearest training point shifts the
+// exponent (exp(-(r^2 - r0^2) / 2l^2) <= 1, no underflow).  The sum is compensated: alpha is carried
+// as two floats and the rounding error of every product and addition is accumulated separately
+// (Neumaier), all on the FP32 pipe.
+__device__ __forceinline__ void mean_mixed(const DevParams& P, const Shared& s, int N, bool lattice, int qi,
+                                           const double xl[3], float& r0, double& tot, float g[3]) {
+    const float qx = (float)xl[0], qy = (float)xl[1], qz = (float)xl[2];
+    r0 = 0.f;
+    if (!lattice) {
+        r0 = INFINITY;
         for (int j = 0; j < N; ++j) {
             float dx = s.Xf[3 * j] - qx, dy = s.Xf[3 * j + 1] - qy, dz = s.Xf[3 * j + 2] - qz;
-            float e;
-            if (lattice) {
-                e = P.lat_tab_f[lat_m(s.xi[j], qi)];
-            } else {
-                float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                e = exp2f((r0 - r2) * P.inv2l2_log2e);
-            }
-            const float ah = s.alf[j];
-            const float w = ah * e;
-            comp += fmaf(ah, e, -w) + s.alf_lo[j] * e;
-            const float t2 = sum + w;
-            comp += fabsf(sum) >= fabsf(w) ? (sum - t2) + w : (w - t2) + sum;
-            sum = t2;
-            gx = fmaf(w, dx, gx);
-            gy = fmaf(w, dy, gy);
-            gz = fmaf(w, dz, gz);
+            r0 = fminf(r0, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
         }
-        const double tot = (double)sum + (double)comp;
-        if (!(tot > 0.0)) {
-            lo = NAN;
-            gro[0] = gro[1] = gro[2] = 0.0;
-            return;
-        }
-        lo = -(double)r0 * P.inv2l2 + log(tot);
-        const double inv = 1.0 / (tot * P.l2);
-        gro[0] = (double)gx * inv;
-        gro[1] = (double)gy * inv;
-        gro[2] = (double)gz * inv;
-    } else {
-        double o = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-        for (int j = 0; j < N; ++j) {
-            double dx = s.X[3 * j] - xl[0], dy = s.X[3 * j + 1] - xl[1], dz = s.X[3 * j + 2] - xl[2];
-            double k;
-            if (lattice) k = P.lat_tab[lat_m(s.xi[j], qi)];
-            else k = exp(-(dx * dx + dy * dy + dz * dz) * P.inv2l2);
-            const double w = s.alpha[j] * k;
-            o += w;
-            gx += w * dx;
-            gy += w * dy;
-            gz += w * dz;
-        }
-        if (!(o > 0.0)) {
-            lo = NAN;
-            gro[0] = gro[1] = gro[2] = 0.0;
-            return;
-        }
-        lo = log(o);
-        const double inv = 1.0 / (o * P.l2);
-        gro[0] = gx * inv;
-        gro[1] = gy * inv;
-        gro[2] = gz * inv;
     }
+    float sum = 0.f, comp = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+    for (int j = 0; j < N; ++j) {
+        float dx = s.Xf[3 * j] - qx, dy = s.Xf[3 * j + 1] - qy, dz = s.Xf[3 * j + 2] - qz;
+        float e;
+        if (lattice) {
+            e = P.lat_tab_f[lat_m(s.xi[j], qi)];
+        } else {
+            float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            e = exp2f((r0 - r2) * P.inv2l2_log2e);
+        }
+        const float ah = s.alf[j];
+        const float w = ah * e;
+        comp += fmaf(ah, e, -w) + s.alf_lo[j] * e;
+        const float t2 = sum + w;
+        comp += fabsf(sum) >= fabsf(w) ? (sum - t2) + w : (w - t2) + sum;
+        sum = t2;
+        gx = fmaf(w, dx, gx);
+        gy = fmaf(w, dy, gy);
+        gz = fmaf(w, dz, gz);
+    }
+    tot = (double)sum + (double)comp;
+    g[0] = gx;
+    g[1] = gy;
+    g[2] = gz;
+}
+
+// revert() of mean_mixed's sums without the variance: o = tot e^(-r0^2 / 2l^2), grad d = -l^2 grad o /
+// (o d) = -g / (tot d), d exactly as revert() forms it.  An FP64 operation is worth 66 FP32
+// instructions here: one division serves the three components instead of four (about 60 operations a
+// query with the logarithm instead of 95; 4M evaluations of 61 points: 1.49 -> 1.1 ms).
+__device__ __forceinline__ void revert_mixed(const DevParams& P, float r0, double tot, const float g[3], EvalOut& r) {
+    const double lo = tot > 0.0 ? -(double)r0 * P.inv2l2 + log(tot) : NAN;
+    if (!(lo >= P.log_floor) || lo >= 0.0) {
+        const double none[3] = {0.0, 0.0, 0.0};
+        revert(P, lo, none, 0.0, false, r);
+        return;
+    }
+    const double d = sqrt(-2.0 * P.l2 * lo), w = -1.0 / (tot * d);
+    r.status = VGP_ST_OK;
+    r.d = d;
+    for (int a = 0; a < 3; ++a) r.g[a] = w * (double)g[a];
+    r.v = NAN;
+}
+
+// FP64 latent mean and gradient at one query; returns lo = log o and gro = grad o / o.
+__device__ __forceinline__ void latent_mean(const DevParams& P, const Shared& s, int N, bool lattice, int qi,
+                                            const double xl[3], double& lo, double gro[3]) {
+    double o = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    for (int j = 0; j < N; ++j) {
+        double dx = s.X[3 * j] - xl[0], dy = s.X[3 * j + 1] - xl[1], dz = s.X[3 * j + 2] - xl[2];
+        double k;
+        if (lattice) k = P.lat_tab[lat_m(s.xi[j], qi)];
+        else k = exp(-(dx * dx + dy * dy + dz * dz) * P.inv2l2);
+        const double w = s.alpha[j] * k;
+        o += w;
+        gx += w * dx;
+        gy += w * dy;
+        gz += w * dz;
+    }
+    if (!(o > 0.0)) {
+        lo = NAN;
+        gro[0] = gro[1] = gro[2] = 0.0;
+        return;
+    }
+    lo = log(o);
+    const double inv = 1.0 / (o * P.l2);
+    gro[0] = gx * inv;
+    gro[1] = gy * inv;
+    gro[2] = gz * inv;
 }
 
 // u = 1 - |L^-1 k|^2 (Eq. 2) with FP64 kernel values; the thread's own column of V lives in
@@ -1927,7 +1941,6 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                     if (!(isfinite(xl[0]) && isfinite(xl[1]) && isfinite(xl[2]))) {
                         invalid(r, VGP_ST_BAD_INPUT);
                     } else {
-                        latent_mean(c.P, s, N, lattice, qi, xl, lo, gro);
                         double u = 0.0;
                         if (c.b.want_var) {
                             if constexpr (kEmu)  // the Schur complement's diagonal entry, clamped at 0
@@ -1935,7 +1948,22 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
                             else
                                 u = latent_var(c.P, s, N, lattice, qi, xl, V, nt);
                         }
-                        revert(c.P, lo, gro, u, c.b.want_var != 0, r);
+                        if (c.P.precision == VGP_MIXED) {
+                            float r0, g[3];
+                            double tot;
+                            mean_mixed(c.P, s, N, lattice, qi, xl, r0, tot, g);
+                            if (!c.b.want_var) {
+                                revert_mixed(c.P, r0, tot, g, r);
+                            } else {
+                                lo = tot > 0.0 ? -(double)r0 * c.P.inv2l2 + log(tot) : NAN;
+                                const double inv = 1.0 / (tot * c.P.l2);
+                                for (int a = 0; a < 3; ++a) gro[a] = (double)g[a] * inv;
+                                revert(c.P, lo, gro, u, true, r);
+                            }
+                        } else {
+                            latent_mean(c.P, s, N, lattice, qi, xl, lo, gro);
+                            revert(c.P, lo, gro, u, c.b.want_var != 0, r);
+                        }
                     }
                 }
                 write_out(c.b, qid, r);
@@ -1966,9 +1994,9 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
 // kProps: surface-property mode (Eq. 6); the emulated kernels run the trailing updates of
 // N > 32 instances on the bf16 tensor cores (256 threads, two CTAs per SM).  Separate
 // kernels, so that the plain distance kernel keeps its register budget.
-// (up to 736 threads, the largest shape its registers have allowed)
+// (up to 640 threads, five warps per sub-partition, the largest shape its registers have allowed)
 template <bool kProps>
-__global__ void __launch_bounds__(736) k_solve(SolveCtx c) {
+__global__ void __launch_bounds__(640) k_solve(SolveCtx c) {
     solve_body<kProps, false, false>(c);
 }
 
@@ -2041,7 +2069,7 @@ __global__ void k_backward(SolveCtx c) {
                     double xl[3];
                     query_local(cc, I, p, qid, xl);
                     double dx = xl[0] - s.X[3 * j], dy = xl[1] - s.X[3 * j + 1], dz = xl[2] - s.X[3 * j + 2];
-                    double k = exp(-(dx * dx + dy * dy + dz * dz) * c.P.inv2l2);
+                    double k = exp_near(-(dx * dx + dy * dy + dz * dz) * c.P.inv2l2, s.T256, c.P.exp_lo);
                     ab += ob * k;
                     g1[0] += ob * k * dx;
                     g1[1] += ob * k * dy;
@@ -2061,7 +2089,7 @@ __global__ void k_backward(SolveCtx c) {
                     if (i == j) continue;
                     double dx = s.X[3 * i] - s.X[3 * j], dy = s.X[3 * i + 1] - s.X[3 * j + 1],
                            dz = s.X[3 * i + 2] - s.X[3 * j + 2];
-                    double k = exp(-(dx * dx + dy * dy + dz * dz) * c.P.inv2l2);
+                    double k = exp_near(-(dx * dx + dy * dy + dz * dz) * c.P.inv2l2, s.T256, c.P.exp_lo);
                     double cf = (s.w[i] * aj + lj * s.alpha[i]) * k;
                     g2[0] -= cf * dx;
                     g2[1] -= cf * dy;
@@ -2140,20 +2168,17 @@ __global__ void k_plan_buckets(const int* hist, int* cursor, int* plan) {
 struct ChunkPlanArgs {
     int off[5], cnt[5], slots[5], cap[5], qmin[5], qn[5];
 };
-// Sum over the CTA (all threads call; w: one value per warp of scratch), the same on every thread.
-__device__ long long block_sum(long long v, long long* w) {
+// Sum over the CTA (all threads call; w: 32 values of scratch), the same on every thread.
+__device__ int block_sum(int v, int* w) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    v = warp_sum(v);
+    v = __reduce_add_sync(0xffffffffu, v);
     __syncthreads();
     if (lane == 0) w[warp] = v;
     __syncthreads();
-    long long t = 0;
-    for (int i = 0; i < nwarp; ++i) t += w[i];
-    return t;
+    return __reduce_add_sync(0xffffffffu, lane < nwarp ? w[lane] : 0);
 }
 __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_off, const int64_t* q_off,
                              const int* plan, ChunkPlanArgs a, int* chunk_q, int* chunk_off) {
-    __shared__ long long wq[32];
     __shared__ int wsum[32];
     __shared__ int carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
@@ -2176,7 +2201,7 @@ __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_of
                 }
             }
             auto chunks_at = [&](long long qs) {  // work items beyond one per instance
-                long long v = 0;
+                int v = 0;
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const unsigned q = (unsigned)min((long long)INT32_MAX, chunk_len(qs, qn, n0[r], cap));
@@ -2185,15 +2210,15 @@ __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_of
                 for (int k = tid + 4 * blockDim.x; k < cnt; k += blockDim.x) {
                     const int I = order[off + k];
                     const long long nq = q_off[I + 1] - q_off[I], q = chunk_len(qs, qn, inst_off[I + 1] - inst_off[I], cap);
-                    if (nq > q) v += (nq - 1) / q;
+                    if (nq > q) v += (int)((nq - 1) / q);
                 }
-                return cnt + block_sum(v, wq);
+                return cnt + (long long)block_sum(v, wsum);
             };
             long long lo = a.qmin[bk], hi = lo;
             while (hi < INT32_MAX / 2 && (cap == 0 || hi < cap) && chunks_at(hi) > most) hi *= 2;
             if (hi > lo) {
                 lo = hi / 2;  // too many chunks at lo, few enough at hi
-                while (hi - lo > max(1ll, lo / 32)) {
+                while (hi - lo > max(1ll, lo / 16)) {
                     const long long mid = (lo + hi) / 2;
                     if (chunks_at(mid) > most)
                         lo = mid;
