@@ -977,15 +977,22 @@ __device__ __forceinline__ bool emu_fail(const SolveCtx& c, Tc& tc) {
 // is prefetched into L2.  Measured against 68 N = 32 products, 8-byte accesses to 64-byte tile rows
 // and a diagonal of the query block from full tiles: 38 instances of about 790 points alone on the
 // GPU 16.1 -> 11.7 ms, 15.6k of 4 to 1024 points 216 -> 180 ms.
+// With a cluster the call takes the part's tiles r, r + n, .. of each band (r + 1, .. in the next band).
+enum class TilePart { kAll, kFirst, kRest };  // kFirst: the first band's first tile, kRest: all but it
 template <class Tc>
 __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const unsigned char* E,
-                                   const double* sr, unsigned char* stage, Tc& tc) {
+                                   const double* sr, unsigned char* stage, Tc& tc, int r, int n, TilePart part) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = Nt - K1;
     const int jr = (max(Ntr - K1, 0) + kColT - 1) / kColT;  // column tiles
-    // with a cluster, every n-th column tile of a band, from another rank on for each band
-    auto tiles_of = [&](int b0) { return min(jr, (b0 + min(kBandT, M - b0) + kColT - 1) / kColT); };
-    auto first_of = [&](int b0) { return (tc.rank() + b0 / kBandT) % tc.n(); };
+    auto tiles_of = [&](int b0) {
+        if (part == TilePart::kFirst) return b0 == 0 ? 1 : 0;
+        return min(jr, (b0 + min(kBandT, M - b0) + kColT - 1) / kColT);
+    };
+    auto first_of = [&](int b0) {
+        const int f = (r + b0 / kBandT) % n;
+        return part == TilePart::kRest && b0 == 0 && f == 0 ? n : f;
+    };
     auto next_band = [&](int b0) {  // the first band from b0 on that has a tile for this CTA
         while (b0 < M && first_of(b0) >= tiles_of(b0)) b0 += kBandT;
         return b0;
@@ -1021,7 +1028,7 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
         // the row's exponent (rows past the matrix inside its last block: unused)
         const int er = rows_in ? (int)(__double_as_longlong(sr[32 * rb + lane]) >> 52) : 0;
         const int n_tiles = tiles_of(b0);  // column tiles reaching the band's last row
-        for (int jt = first_of(b0), buf = 0; jt < n_tiles; jt += tc.n(), buf ^= 1) {
+        for (int jt = first_of(b0), buf = 0; jt < n_tiles; jt += n, buf ^= 1) {
             const uint32_t bufB = aB + (uint32_t)(buf * kStageB);
             // this thread's 16 entries of C (one row, 16 columns) and the column scales, all loads
             // issued at once; they arrive while the MMAs run
@@ -1033,18 +1040,18 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
 #pragma unroll
                 for (int cc = 0; cc < 16; ++cc) cv[cc] = C[32 * cc + lane];
                 es = sr[32 * jt + 16 * h + (lane & 15)];
-                if (jt + tc.n() < n_tiles && jt + tc.n() <= rb && lane == 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024 * tc.n()), "r"(4096));
+                if (jt + n < n_tiles && jt + n <= rb && lane == 0)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(C + 1024 * n), "r"(4096));
             }
             // warp 0 alone waits for the copies, starts the next ones and issues the products: every
             // phase of the copy barrier is seen before the next one can start
             if (warp == 0 && !bar_poll(tc.bar_ld, tc.ph_ld)) fail = 1;
             if (warp == 0 && !__any_sync(0xffffffffu, fail) && lane == 0) {
-                if (jt + tc.n() < n_tiles) {  // the next column tile's B into the other buffer
+                if (jt + n < n_tiles) {  // the next column tile's B into the other buffer
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc.bar_ld),
                                  "r"((uint32_t)kStageB)
                                  : "memory");
-                    bulk_load(stage + kStageA + (buf ^ 1) * kStageB, E + (int64_t)(jt + tc.n()) * kGroupBytes, kStageB,
+                    bulk_load(stage + kStageA + (buf ^ 1) * kStageB, E + (int64_t)(jt + n) * kGroupBytes, kStageB,
                               tc.bar_ld);
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1077,7 +1084,7 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // the band's last products are done (so warp 0 has seen every copy): its A and B buffers
             // take the next band's
-            if (!__any_sync(0xffffffffu, fail) && jt + tc.n() >= n_tiles && b1 < M) stage_band(b1);
+            if (!__any_sync(0xffffffffu, fail) && jt + n >= n_tiles && b1 < M) stage_band(b1);
             if (on) {
                 // two columns at a time, the next two read from tensor memory meanwhile
                 uint32_t v[2][8][2];
@@ -1158,27 +1165,40 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
     double* sr = emu_scales(c);           // row scales of the rows below the block
     double* Tall = emu_tile_inverses(c);  // inverses of all diagonal tiles, for the solves
     long long* udiag = emu_query_diag(c);
-    for (int K0 = 0; K0 < Ntr; K0 += kEB) {
-        const int K1 = min(K0 + kEB, Ntr);
-        // the diagonal block: tiles (it, jt), K0 <= jt <= it < K1, in shared memory (packed),
-        // right-looking by 8 columns.  Warp 0 takes the diagonal tiles; its update of the next one
-        // needs no barrier after it.  The other tiles go to warps of the other sub-partitions
-        // (warp 4 shares warp 0's), so the chain of diagonal tiles has its FP64 pipe alone.
-        const int nb = K1 - K0;
-        for (int x = tid; x < nb * (nb + 1) / 2 * 32 && tc.rank() == 0; x += blockDim.x) {
+    auto tile = [&](int ir, int jc) { return s.Dblk + (ir * (ir + 1) / 2 + jc) * 64; };
+    auto update = [&](int ir, int jc, int k) {  // tile (ir, jc) -= tile (ir, k) tile (jc, k)^T
+        double* C = tile(ir, jc);
+        double c0 = C[te(g, t)], c1 = C[te(g, 7 - t)];
+        sub_products(c0, c1, tile(ir, k), g, tile(jc, k), t, 7 - t);
+        C[te(g, t)] = c0;
+        C[te(g, 7 - t)] = c1;
+    };
+    // the block's off-diagonal tiles and inverses to the workspace (for the solves and the cluster's
+    // other CTAs) or from it
+    auto exchange = [&](int K0, bool out) {
+        const int nb = min(kEB, Ntr - K0);
+        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
+            const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
+            double2* const g2 = reinterpret_cast<double2*>(ir == jc ? Tall + 64 * (K0 + ir) : A + eix(K0 + ir, K0 + jc));
+            double2* const s2 = reinterpret_cast<double2*>(ir == jc ? s.Tblk + 64 * ir : tile(ir, jc));
+            if (out)
+                g2[x & 31] = s2[x & 31];
+            else
+                s2[x & 31] = g2[x & 31];
+        }
+    };
+    // The diagonal block: tiles (it, jt), K0 <= jt <= it < K0 + kEB, in shared memory (packed),
+    // right-looking by 8 columns.  Warp 0 takes the diagonal tiles; its update of the next one
+    // needs no barrier after it.  The other tiles go to warps of the other sub-partitions
+    // (warp 4 shares warp 0's), so the chain of diagonal tiles has its FP64 pipe alone.
+    auto diagonal_block = [&](int K0) {
+        const int nb = min(kEB, Ntr - K0);
+        for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
             const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
             reinterpret_cast<double2*>(s.Dblk)[x] = reinterpret_cast<const double2*>(A + eix(K0 + ir, K0 + jc))[x & 31];
         }
         __syncthreads();
-        auto tile = [&](int ir, int jc) { return s.Dblk + (ir * (ir + 1) / 2 + jc) * 64; };
-        auto update = [&](int ir, int jc, int k) {  // tile (ir, jc) -= tile (ir, k) tile (jc, k)^T
-            double* C = tile(ir, jc);
-            double c0 = C[te(g, t)], c1 = C[te(g, 7 - t)];
-            sub_products(c0, c1, tile(ir, k), g, tile(jc, k), t, 7 - t);
-            C[te(g, t)] = c0;
-            C[te(g, 7 - t)] = c1;
-        };
-        for (int k = 0; k < nb && tc.rank() == 0; ++k) {
+        for (int k = 0; k < nb; ++k) {
             const double* Ti = s.Tblk + 64 * k;
             if (warp == 0) {
                 if (k > 0) update(k, k, k - 1);
@@ -1205,22 +1225,22 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
             }
             __syncthreads();
         }
-        // for the solves and the cluster's other CTAs: the off-diagonal tiles and the inverses
-        auto exchange = [&](bool out) {
-            for (int x = tid; x < nb * (nb + 1) / 2 * 32; x += blockDim.x) {
-                const int p = x >> 5, ir = tri_row(p), jc = p - ir * (ir + 1) / 2;
-                double2* const g2 = reinterpret_cast<double2*>(ir == jc ? Tall + 64 * (K0 + ir) : A + eix(K0 + ir, K0 + jc));
-                double2* const s2 = reinterpret_cast<double2*>(ir == jc ? s.Tblk + 64 * ir : tile(ir, jc));
-                if (out)
-                    g2[x & 31] = s2[x & 31];
-                else
-                    s2[x & 31] = g2[x & 31];
-            }
-        };
-        if (tc.rank() == 0) exchange(true);
+        exchange(K0, true);
+    };
+    // In a cluster of four or more the first CTA looks ahead: it updates the tile that holds the next
+    // diagonal block first and factorises that while the others take the rest of the update (the
+    // diagonal block's chain of 32 columns, about 31k clocks, is as long as their share of it).
+    const bool ahead = tc.n() >= 4;
+    bool ok = true;
+    for (int K0 = 0; K0 < Ntr; K0 += kEB) {
+        const int K1 = min(K0 + kEB, Ntr);
+        if (tc.rank() == 0 && (K0 == 0 || !ahead)) diagonal_block(K0);
         if (tc.n() > 1) {
-            if (group_sync(tc, *s_fail)) return false;
-            if (tc.rank() > 0) exchange(false);
+            if (group_sync(tc, *s_fail || !ok)) {  // a pivot or, known to all after another barrier, a wait
+                if (group_sync(tc, !ok)) emu_fail(c, tc);
+                return false;
+            }
+            if (tc.rank() > 0) exchange(K0, false);
             __syncthreads();
         } else if (*s_fail) {
             return false;
@@ -1238,9 +1258,19 @@ __device__ bool factor_emulated(const SolveCtx& c, const Shared& s, double* A, i
         asm volatile("fence.proxy.async;" ::: "memory");
         group_barrier(tc);
         if (tc.n() > 1) asm volatile("fence.proxy.async;" ::: "memory");
-        const bool ok = trailing_update_tc(A, Nt, Ntr, K1, E, sr, s.stage, tc);
-        // (alone, the update's own last barrier is enough)
-        if (tc.n() > 1 ? group_sync(tc, !ok) : !ok) return emu_fail(c, tc);
+        const bool first = ahead && tc.rank() == 0;
+        if (!first || K1 < Ntr)
+            ok = trailing_update_tc(A, Nt, Ntr, K1, E, sr, s.stage, tc, first ? 0 : ahead ? tc.rank() - 1 : tc.rank(),
+                                    first ? 1 : ahead ? tc.n() - 1 : tc.n(),
+                                    first ? TilePart::kFirst : ahead ? TilePart::kRest : TilePart::kAll);
+        if (!ahead) {
+            // (alone, the update's own last barrier is enough; together, the next diagonal block needs
+            // every CTA's tiles)
+            if (tc.n() > 1 ? group_sync(tc, !ok) : !ok) return emu_fail(c, tc);
+        } else if (first && K1 < Ntr) {
+            __syncthreads();
+            if (ok) diagonal_block(K1);
+        }
     }
     return true;
 }
