@@ -872,7 +872,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 
 // Wait of the calling thread for the completion of phase `parity` of an mbarrier, at most
 // kWaitLimit polls (false: the wait gave up).
-constexpr int kWaitLimit = 1 << 22;
+constexpr int kWaitLimit = 1 << 18;
 __device__ __forceinline__ bool bar_poll(uint32_t bar, uint32_t parity) {
     uint32_t done = 0;
     for (int it = 0; it < kWaitLimit && !done; ++it)
@@ -939,15 +939,20 @@ __device__ __forceinline__ void group_barrier(Tc& tc) {
         group_sync(tc, 0);
 }
 
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&v)[2]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr) : "memory");
+// columns a tensor-memory load reads for each lane (four, with nothing else in flight: 154.8 ms for the
+// city step; two at a time with the next two in flight 157.0, eight 154.8 with more spills)
+constexpr int kLdCols = 4;
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[kLdCols]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
 }
 // The loaded values pass through the wait, so no use of them is scheduled before it.
-__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[8][2]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[2][0]), "+r"(v[2][1]),
-                   "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[4][0]), "+r"(v[4][1]), "+r"(v[5][0]), "+r"(v[5][1]),
-                   "+r"(v[6][0]), "+r"(v[6][1]), "+r"(v[7][0]), "+r"(v[7][1])::"memory");
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[8][kLdCols]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : : : "memory");
+#pragma unroll
+    for (int g = 0; g < 8; ++g)
+#pragma unroll
+        for (int e = 0; e < kLdCols; ++e) asm volatile("" : "+r"(v[g][e]));
 }
 
 // A bounded wait gave up: record it; the CTA stops taking work.
@@ -1086,27 +1091,22 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
             // take the next band's
             if (!__any_sync(0xffffffffu, fail) && jt + n >= n_tiles && b1 < M) stage_band(b1);
             if (on) {
-                // two columns at a time, the next two read from tensor memory meanwhile
-                uint32_t v[2][8][2];
                 const uint32_t tbase = tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(16 * h);
 #pragma unroll
-                for (int gq = 0; gq < 8; ++gq) tmem_ld2(tbase + (uint32_t)(gq * 8 * kColT), v[0][gq]);
+                for (int p = 0; p < 16 / kLdCols; ++p) {
+                    uint32_t v[8][kLdCols];
 #pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    tmem_wait_ld(v[p & 1]);
-                    if (p < 7)
+                    for (int gq = 0; gq < 8; ++gq) tmem_ld(tbase + (uint32_t)(gq * 8 * kColT + kLdCols * p), v[gq]);
+                    tmem_wait_ld(v);
 #pragma unroll
-                        for (int gq = 0; gq < 8; ++gq)
-                            tmem_ld2(tbase + (uint32_t)(gq * 8 * kColT + 2 * p + 2), v[(p + 1) & 1][gq]);
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
+                    for (int e = 0; e < kLdCols; ++e) {
                         unsigned gb[8];
 #pragma unroll
                         for (int gq = 0; gq < 8; ++gq)
-                            gb[gq] = __float_as_uint(__fadd_rn(__uint_as_float(v[p & 1][gq][e]), 12582912.0f));
-                        const int ec = __shfl_sync(0xffffffffu, ec_lane, 2 * p + e);
+                            gb[gq] = __float_as_uint(__fadd_rn(__uint_as_float(v[gq][e]), 12582912.0f));
+                        const int ec = __shfl_sync(0xffffffffu, ec_lane, kLdCols * p + e);
                         // the update is w 2^(er + ec - 2102), in units of 2^-kFixBits
-                        cv[2 * p + e] -= fix_shift(join_groups(gb), er + ec - (2102 - kFixBits));
+                        cv[kLdCols * p + e] -= fix_shift(join_groups(gb), er + ec - (2102 - kFixBits));
                     }
                 }
                 // the next block's columns are final after this update: stored as FP64 tiles (see
