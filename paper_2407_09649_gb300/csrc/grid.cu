@@ -498,18 +498,58 @@ __device__ void jacobi3_rn(double a[3][3], double v[3][3]) {
     }
 }
 
-// Thread per surface voxel.
+// Integer 3D Bresenham line from the origin's voxel to the surface voxel sv (excluded): the voxels the
+// grid already knows.
+__device__ void walk_ray(const int sv[3], const uint64_t* gkeys, uint32_t gmask, const int32_t* g_slot2pool,
+                         const unsigned long long* g_known, int ovx, int ovy, int ovz, uint64_t* tkeys, uint32_t tmask,
+                         unsigned* tflags, int* err) {
+    const int a0[3] = {ovx, ovy, ovz};
+    long long d[3], st[3], pcur[3] = {a0[0], a0[1], a0[2]};
+    for (int k = 0; k < 3; ++k) {
+        d[k] = sv[k] > a0[k] ? (long long)sv[k] - a0[k] : (long long)a0[k] - sv[k];
+        st[k] = sv[k] > a0[k] ? 1 : -1;
+    }
+    int m = 0;
+    if (d[1] > d[m]) m = 1;
+    if (d[2] > d[m]) m = 2;
+    const int u = (m + 1) % 3, w = (m + 2) % 3;
+    long long eu = 2 * d[u] - d[m], ew = 2 * d[w] - d[m];
+    for (long long step = 0; step < d[m]; ++step) {
+        if (grid_known(gkeys, gmask, g_slot2pool, g_known, (int)pcur[0], (int)pcur[1], (int)pcur[2]))
+            add_test(tkeys, tmask, tflags, (int)pcur[0], (int)pcur[1], (int)pcur[2], 1, err);
+        if (eu > 0) {
+            pcur[u] += st[u];
+            eu -= 2 * d[m];
+        }
+        if (ew > 0) {
+            pcur[w] += st[w];
+            ew -= 2 * d[m];
+        }
+        eu += 2 * d[u];
+        ew += 2 * d[w];
+        pcur[m] += st[m];
+    }
+}
+
+// Thread per surface voxel, even CTAs for its normal and the voxels along it (a chain of some 4000 FP64
+// operations), odd ones for its ray (a chain of hash probes), so that the two run beside each
+// other; one after the other in a thread they took 280 us for a 400 x 250 frame.
 __global__ void k_raycast_tests(const uint64_t* svox, int64_t ns, const uint64_t* fkeys, uint32_t fmask,
                                 const unsigned long long* fmasks, const uint64_t* gkeys, uint32_t gmask,
                                 const int32_t* g_slot2pool, const unsigned long long* g_known, double ox, double oy,
                                 double oz, int have_o, int ovx, int ovy, int ovz, double vs, int K, uint64_t* tkeys,
                                 uint32_t tmask, unsigned* tflags, int* err) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t)(blockIdx.x >> 1) * blockDim.x + threadIdx.x;
+    const bool ray = blockIdx.x & 1;
     if (i >= ns) return;
     int sv[3];
     unpack_key(svox[i], sv[0], sv[1], sv[2]);
-    add_test(tkeys, tmask, tflags, sv[0], sv[1], sv[2], 1, err);
+    if (!ray) add_test(tkeys, tmask, tflags, sv[0], sv[1], sv[2], 1, err);
     if (!have_o) return;
+    if (ray) {
+        walk_ray(sv, gkeys, gmask, g_slot2pool, g_known, ovx, ovy, ovz, tkeys, tmask, tflags, err);
+        return;
+    }
     // normal from the exact integer scatter of the occupied 3x3x3 block
     long long cnt = 0, S1[3] = {0, 0, 0}, S2[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     for (int dz = -1; dz <= 1; ++dz)
@@ -546,33 +586,6 @@ __global__ void k_raycast_tests(const uint64_t* svox, int64_t ns, const uint64_t
             for (int a = 0; a < 3; ++a) v[a] = sv[a] + (int)floor(__dadd_rn(__dmul_rn((double)kk, nrm[a]), 0.5));
             add_test(tkeys, tmask, tflags, v[0], v[1], v[2], kk > 0 ? 1 : -1, err);
         }
-    }
-    // integer 3D Bresenham from the origin's voxel to the surface voxel (excluded)
-    const int a0[3] = {ovx, ovy, ovz};
-    long long d[3], st[3], pcur[3] = {a0[0], a0[1], a0[2]};
-    for (int k = 0; k < 3; ++k) {
-        d[k] = sv[k] > a0[k] ? (long long)sv[k] - a0[k] : (long long)a0[k] - sv[k];
-        st[k] = sv[k] > a0[k] ? 1 : -1;
-    }
-    int m = 0;
-    if (d[1] > d[m]) m = 1;
-    if (d[2] > d[m]) m = 2;
-    const int u = (m + 1) % 3, w = (m + 2) % 3;
-    long long eu = 2 * d[u] - d[m], ew = 2 * d[w] - d[m];
-    for (long long step = 0; step < d[m]; ++step) {
-        if (grid_known(gkeys, gmask, g_slot2pool, g_known, (int)pcur[0], (int)pcur[1], (int)pcur[2]))
-            add_test(tkeys, tmask, tflags, (int)pcur[0], (int)pcur[1], (int)pcur[2], 1, err);
-        if (eu > 0) {
-            pcur[u] += st[u];
-            eu -= 2 * d[m];
-        }
-        if (ew > 0) {
-            pcur[w] += st[w];
-            ew -= 2 * d[m];
-        }
-        eu += 2 * d[u];
-        ew += 2 * d[w];
-        pcur[m] += st[m];
     }
 }
 
@@ -702,7 +715,7 @@ void frame_raycast_tests(const uint64_t* svox, int64_t ns, const Table& ft, cons
                          const double origin[3], int have_o, const int ov[3], double vs, int K, const Table& tt,
                          unsigned* tflags, int* err, cudaStream_t st) {
     if (ns > 0) {
-        k_raycast_tests<<<nblk(ns, 128), 128, 0, st>>>(svox, ns, ft.keys, ft.mask, fmasks, g.keys, g.mask, g_slot2pool,
+        k_raycast_tests<<<2 * nblk(ns, 128), 128, 0, st>>>(svox, ns, ft.keys, ft.mask, fmasks, g.keys, g.mask, g_slot2pool,
                                                        g_known, origin[0], origin[1], origin[2], have_o, ov[0], ov[1],
                                                        ov[2], vs, K, tt.keys, tt.mask, tflags, err);
         note_launch();
@@ -1433,21 +1446,28 @@ __global__ void k_fuse_insert(const uint64_t* vkey, const double* d, const doubl
 __global__ void k_fuse_alloc(int32_t* slot2pool, int64_t cap, int* pool_count, int pool_cap,
                              unsigned long long* known, int32_t* flags, int* err, PropGrid pg) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= cap || slot2pool[s] != -2) return;
-    int p = atomicAdd(pool_count, 1);
-    if (p >= pool_cap) {
-        atomicOr(err, kErrCapacity);
-        slot2pool[s] = -1;
-        return;
-    }
-    slot2pool[s] = p;
-    for (int w = 0; w < 8; ++w) known[(int64_t)p * 8 + w] = 0ull;
-    flags[p] = 0;
-    if (pg.nc > 0)
-        for (int e = 0; e < 512; ++e) {
-            pg.W[(int64_t)p * 512 + e] = __longlong_as_double(0x7ff8000000000000ll);
-            for (int ch = 0; ch < pg.nc; ++ch) pg.C[((int64_t)p * 512 + e) * pg.nc + ch] = __longlong_as_double(0x7ff8000000000000ll);
+    int p = -1;
+    if (s < cap && slot2pool[s] == -2) {
+        p = atomicAdd(pool_count, 1);
+        if (p >= pool_cap) {
+            atomicOr(err, kErrCapacity);
+            p = -1;
         }
+        slot2pool[s] = p;
+    }
+    if (p >= 0) {
+        for (int w = 0; w < 8; ++w) known[(int64_t)p * 8 + w] = 0ull;
+        flags[p] = 0;
+    }
+    if (pg.nc == 0) return;
+    // a new leaf's properties are NaN, written by the whole warp (by its own thread, 512 voxels one
+    // after the other, a frame's new leaves took 160 us)
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    for (unsigned todo = __ballot_sync(0xffffffffu, p >= 0); todo; todo &= todo - 1) {
+        const int64_t q = __shfl_sync(0xffffffffu, p, __ffs(todo) - 1);
+        for (int e = threadIdx.x & 31; e < 512; e += 32) pg.W[q * 512 + e] = nan;
+        for (int e = threadIdx.x & 31; e < 512 * pg.nc; e += 32) pg.C[q * 512 * pg.nc + e] = nan;
+    }
 }
 
 // Surface-property fusion: the rules of the distance fusion (Eqs. 8-9) applied to every
