@@ -1,0 +1,152 @@
+"""The solve's routes: clusters of CTAs on one instance, chunked queries, launch shapes chosen by the
+number of instances and queries, and the smallest instances on a stream of their own.
+
+Which of them answers a query depends on what else is in the batch and must not show in the
+result, so the routes are compared bit for bit; the plain FP64 kernels at the edges of their tiles
+and buckets are compared with the oracle at the FP64 contract (|dd| <= 1e-4 m, gradient
+angle <= 0.1 deg, variance 1e-5 relative).
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("d", "grad", "var", "status")
+
+
+@pytest.fixture(scope="module")
+def vg():
+    import paper_2407_09649_gb300 as P
+    P.build()
+    from paper_2407_09649_gb300 import api
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    return api
+
+
+def _instances(sizes, nq, seed):
+    """Points at a density that keeps |K| well conditioned, nq queries around each instance."""
+    rng = np.random.default_rng(seed)
+    X, Q = [], []
+    for N in sizes:
+        c = rng.uniform(-20, 20, 3)
+        X.append((c + rng.uniform(-0.05, 0.05, (N, 3)) * np.sqrt(N)).astype(np.float32))
+        Q.append((c + rng.uniform(-1, 1, (nq, 3))).astype(np.float32))
+    return X, Q
+
+
+def _solve(m, X, Q, var):
+    io = np.concatenate([[0], np.cumsum([len(x) for x in X])])
+    qo = np.concatenate([[0], np.cumsum([len(q) for q in Q])])
+    out = m.gp_batch(io, np.vstack(X), qo, np.vstack(Q), var=var)
+    out = {k: out[k].cpu().numpy() for k in KEYS if out[k] is not None}
+    return [{k: v[a:b] for k, v in out.items()} for a, b in zip(qo, qo[1:])]
+
+
+def _same(a, b):
+    for k in a:
+        x, y = (np.ascontiguousarray(t[k]).view(np.uint8) for t in (a, b))
+        assert np.array_equal(x, y), k
+
+
+@pytest.mark.parametrize("var", [False, True])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_clusters_do_not_show(vg, precision, var):
+    """Eight, four, two CTAs per instance and one: 1, 40, 100 and 400 instances at the edges of the
+    32-column blocks and 128-row bands, among them the largest size and one bad query."""
+    sizes = [129, 160, 161, 225, 256, 257, 1000, 1024]
+    X, Q = _instances(sizes, 5, 51)
+    Q[3][2] = np.nan
+    m = vg.Map(precision=precision, emulate_fp64=1)
+    small, qs = _instances([130] * 392, 1, 52)
+    ref = _solve(m, X + small, Q + qs, var)[:len(sizes)]
+    assert (ref[3]["status"] == 3).tolist() == [False, False, True, False, False]
+    for n in (0, 32, 92):
+        for a, b in zip(_solve(m, X + small[:n], Q + qs[:n], var), ref):
+            _same(a, b)
+    for x, q, r in zip(X, Q, ref):
+        _same(_solve(m, [x], [q], var)[0], r)
+
+
+@pytest.mark.parametrize("emulate,sizes,n_fill", [(1, [33, 40, 300], 0), (0, [20, 33, 64, 65], 0), (0, [225, 231, 260], 1300)])
+@pytest.mark.parametrize("var", [False, True])
+def test_chunks_and_shapes_do_not_show(vg, emulate, sizes, n_fill, var):
+    """Instances with 3000 queries, which are split over work items, against 24 of the same
+    queries on their own; and few large instances against the same ones in a batch of more than
+    eight per SM (three smaller CTAs per SM)."""
+    X, Q = _instances(sizes, 3000, 53)
+    fill, qf = _instances([226] * n_fill, 1, 54)
+    for precision in ("fp64", "mixed"):
+        m = vg.Map(precision=precision, emulate_fp64=emulate)
+        full = _solve(m, X + fill, Q + qf, var)
+        part = _solve(m, X, [q[::125] for q in Q], var)
+        for f, p in zip(full, part):
+            _same({k: v[::125] for k, v in f.items()}, p)
+
+
+def test_smallest_instances_follow_their_stream(vg):
+    """Instances of at most 32 points run beside the others on a stream of the map's own: inputs that
+    the caller's stream writes late are seen, and what it does next sees the results."""
+    X, Q = _instances([8] * 50 + [150] * 50, 40, 55)
+    m = vg.Map(precision="fp64")
+    ref = _solve(m, X, Q, True)
+    io = torch.from_numpy(np.concatenate([[0], np.cumsum([len(x) for x in X])])).cuda()
+    qo = torch.arange(len(Q) + 1, dtype=torch.int64, device="cuda") * 40
+    xs, qs = (torch.from_numpy(np.vstack(a)).cuda() for a in (X, Q))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        busy = torch.zeros((8192, 8192), device="cuda")
+        x, q = torch.zeros_like(xs), torch.zeros_like(qs)
+        for _ in range(4):
+            busy = busy @ busy
+        x.copy_(xs)
+        q.copy_(qs)
+        out = m.gp_batch(io, x, qo, q, var=True)
+        got = {k: out[k].clone() for k in KEYS}
+        for t in [x, q] + [out[k] for k in KEYS]:
+            t.zero_()
+    s.synchronize()
+    want = {k: np.concatenate([r[k] for r in ref]) for k in KEYS}
+    _same({k: v.cpu().numpy() for k, v in got.items()}, want)
+
+
+def test_plain_kernels_at_tile_edges(vg, orc):
+    sizes = [1, 7, 8, 9, 16, 17, 32, 33, 64, 65, 128, 129, 224, 225, 232, 233]
+    X, Q = _instances(sizes, 30, 56)
+    io = np.concatenate([[0], np.cumsum(sizes)])
+    qo = np.arange(len(sizes) + 1) * 30
+    ref = orc.gp_batch(io, np.vstack(X).astype(np.float64), qo, np.vstack(Q).astype(np.float64), orc.params())
+    out = _solve(vg.Map(precision="fp64", emulate_fp64=0), X, Q, True)
+    d, g, v, s = (np.concatenate([o[k] for o in out]) for k in KEYS)
+    assert np.array_equal(s, ref.status)
+    ok = ref.status == 0
+    assert np.abs(d[ok] - ref.d[ok]).max() <= 1e-4
+    na, nb = np.linalg.norm(g, axis=1), np.linalg.norm(ref.grad, axis=1)
+    big = ok & (nb > 0.1)
+    cos = np.sum(g * ref.grad, 1)[big] / (na * nb)[big]
+    assert np.degrees(np.arccos(np.clip(cos, -1, 1))).max() <= 0.1
+    fin = ok & np.isfinite(ref.var)
+    np.testing.assert_allclose(v[fin], ref.var[fin], rtol=1e-5, atol=1e-12)
+
+
+@pytest.mark.parametrize("n_nodes,lam", [(1, 100.0), (27, 2000.0), (27, 1e-3)])
+def test_blend_weights_at_their_range(vg, orc, n_nodes, lam):
+    """Blend weights exp(-lambda (d - d_min)) from underflow to all but equal, one node and every
+    node of the neighbourhood, queries at leaf corners (ties between nodes) among them."""
+    from paper_2407_09649_gb300 import scenes
+    rng = np.random.default_rng(57)
+    surf = scenes.sphere_plane_frame(4, n_sphere=2000, n_plane=2000).astype(np.float32)
+    q = (surf[rng.integers(0, len(surf), 600)] + rng.normal(0, 0.1, (600, 3))).astype(np.float32)
+    P = orc.params()
+    q[:100] = np.round(q[:100] / 0.8) * 0.8
+    ref = orc.Surface(surf, P).query_smooth(q, n_nodes=n_nodes, lam=lam, want_var=False)
+    m = vg.Map(precision="fp64")
+    m.set_surface(torch.from_numpy(surf).cuda())
+    out = {k: v.cpu().numpy() for k, v in m.query_smooth(torch.from_numpy(q).cuda(), n_nodes=n_nodes, lam=lam).items()
+           if v is not None}
+    assert np.array_equal(out["status"], ref["status"])
+    ok = ref["status"] == 0
+    assert ok.sum() > 100
+    assert np.abs(out["d"][ok] - ref["d"][ok]).max() <= 1e-4
