@@ -109,7 +109,7 @@ enum {
  *                    report their time in vgp_stats.t_solve_ms (adds one stream sync per call).
  *   normal_steps     K in [0, 16] (default 3): with a sensor origin, vgp_build_frame also tests
  *                    the voxels round(s + k n), k = +-1..+-K, along each surface voxel's normal.
- *   emulate_fp64     1: instances with N > 32 (A in global memory) are factorised in blocks of
+ *   emulate_fp64     1: instances with N > 32 are factorised in blocks of
  *                    32 columns whose trailing updates run on the bf16 tensor cores to FP64
  *                    accuracy: each row of the block is cut into seven balanced base-256 digit
  *                    slices (55 bits under a power-of-two row scale), the slice products
@@ -120,15 +120,16 @@ enum {
  *                    below 2^-45 k (1 + r^2 / 2l^2)), and off-lattice distance instances take
  *                    the latent variance from the Schur complement of the matrix with up to
  *                    1024 query rows appended.  Same results up to rounding; 0 keeps every
- *                    update on the FP64 tensor path.  Uses a per-CTA workspace of about
- *                    0.5 KB per matrix row and 8 bytes per lower-triangle entry.
+ *                    update on the FP64 pipe.  Uses a per-CTA workspace of about 0.5 KB per
+ *                    matrix row and 8 bytes per lower-triangle entry.  Few instances are worked
+ *                    on by clusters of up to 8 CTAs each, with the same bits as by one.
  *   launch           VGP_LAUNCH_BATCHED (default): all GP instances of a call run in a few
  *                    persistent launches, one per size bucket, largest first.
  *                    VGP_LAUNCH_PER_INSTANCE: one kernel launch per instance, in instance
  *                    order (the plain comparison form; same arithmetic, no batching).
  *                    VGP_LAUNCH_GRAPH: the batched form with the size histogram, bucket
  *                    plan and ordering computed on the device, so that the whole solve of a
- *                    call (eight kernels) is captured as a CUDA graph on a stream the map
+ *                    call (plan and bucket launches) is captured as a CUDA graph on a stream the map
  *                    owns and replayed through a cached executable graph, updated in place
  *                    from call to call; the launch shapes are sized for the largest
  *                    instance the call can hold (max_pts_leaf for frames, max_pts_group for

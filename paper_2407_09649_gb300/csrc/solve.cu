@@ -2,13 +2,14 @@
 // evaluation of every query of the instance (latent mean Eq. 1, variance Eq. 2, gradient
 // Eq. 5, reverting Eq. 3 and distance variance Eq. 4), plus the backward pass.
 //
-// One CTA owns one instance at a time and pulls instances from a list sorted by decreasing
-// size (a persistent launch per size bucket, longest first).  A = K + sigma^2 I is stored as
-// the lower triangle of 8x8 tiles (64 contiguous doubles per tile, tiles in packed row
-// order), in shared memory when it fits, else in a per-CTA global workspace.  The Cholesky
-// factorisation is right-looking by 8-column panels; the panel solve and the trailing
-// update run on the FP64 tensor path (mma.sync m8n8k4 f64), the 8x8 diagonal blocks on the
-// FP64 pipe.
+// A CTA (or a cluster of them, see group_ctas) works on one instance at a time and takes instances
+// from a list sorted by decreasing size (a persistent launch per size bucket, longest first).
+// Plain kernel: A = K + sigma^2 I is stored as the lower triangle of 8x8 tiles (64 contiguous
+// doubles per tile, tiles in packed row order), in shared memory when it fits, else in a per-CTA
+// global workspace; the Cholesky factorisation is right-looking by 8-column panels, all on the
+// FP64 pipe.  FP64 mma.sync (m8n8k4) is not used: it runs at the same FP64 rate and its results are
+// those of the ascending fma chain, but one holds a sub-partition's pipe for 580 clocks, against
+// 66 for an FMA, so every chain beside it waits.  Emulated kernel: see factor_emulated.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
@@ -40,8 +41,8 @@ __host__ __device__ __forceinline__ int64_t eix(int it, int jt) {
 constexpr int kTileCol = 256;  // words from a tile to its right neighbour in the block
 
 // Position of element (r, c) inside a 64-double tile: row major with the columns of rows
-// 2, 3, 6, 7 XOR-swizzled by 4, so the mma fragment loads (row g, column t) of the 32 lanes
-// of a warp hit distinct shared-memory banks in each half-warp.
+// 2, 3, 6, 7 XOR-swizzled by 4, so the loads of a warp's 32 lanes at (row lane / 4, column
+// lane % 4) hit distinct shared-memory banks in each half-warp.
 __host__ __device__ __forceinline__ int te(int r, int c) { return r * 8 + (c ^ ((r & 2) << 1)); }
 
 // row index of packed-triangle entry p (0 <= col <= row)
@@ -288,13 +289,58 @@ __device__ __forceinline__ long long fix_of_float(float x, int e) {
     return (b >> 31) ? -v : v;
 }
 
+// The same for a positive normal x.
+__device__ __forceinline__ long long fix_of_positive(float x, int e) {
+    const unsigned b = __float_as_uint(x), mant = (b & 0x7FFFFFu) | 0x800000u;
+    const int sh = (int)(b >> 23) - 150 + e;
+    return sh >= 0 ? (long long)((unsigned long long)mant << (sh & 63))
+                   : (long long)(((mant >> min(-sh - 1, 31)) + 1) >> 1);
+}
+
 // Float pairs: a value is hi + lo, |lo| near 2^-24 |hi| at most.  Knuth's two-sum and the
-// FMA product error are error-free; every operation is an _rn intrinsic, so nothing is
+// FMA product error are error-free; every operation is rounded by itself (_rn), so nothing is
 // contracted or reassociated.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float bv = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
+// Two floats in one register pair: packed FP32 operations, the IEEE result in both halves for one issue
+// slot.
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 pair2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ F2 pair2(float x) { return pair2(x, x); }
+__device__ __forceinline__ float lo2(F2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float hi2(F2 a) { return __uint_as_float((unsigned)(a >> 32)); }
+__device__ __forceinline__ F2 neg2(F2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ void two_sum2(F2 a, F2 b, F2& s, F2& e) {
+    s = add2(a, b);
+    const F2 bv = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bv)), sub2(b, bv));
+}
+// The same where |a| >= |b| (Dekker's): half the operations.
+__device__ __forceinline__ void fast_two_sum2(F2 a, F2 b, F2& s, F2& e) {
+    s = add2(a, b);
+    e = sub2(b, sub2(s, a));
 }
 
 // ln2/256 = kL0 + kL1 + kL2 (kL0 with 10 significant bits, so n kL0 is exact for n < 2^14;
@@ -313,49 +359,63 @@ constexpr float kInvL = 369.32993046757464f;
 //   Taylor terms to r^4 (the next term is below 2^-54), 2^(i/256) from the float-pair table;
 //   the float-pair result scaled by 2^(61 - m) into a 64-bit integer.
 // The error stays below 2^-45 k (1 + y) + 2 units of 2^-61, about 2^-47 at most in k, at the
-// level of the Cholesky's own backward error; 0 where y > 43.5 (k < 2^-62).
-__device__ __forceinline__ long long kfix_ff(const float a[3], const float b[3], float ch, float cl,
-                                             const float2* tab) {
-    float S = 0.f, E = 0.f;
+// level of the Cholesky's own backward error; 0 where y > 43.5 (k < 2^-62).  Bound by issue slots
+// (about 110 FP32 and 40 integer operations an entry): two entries (b, b + 3) at once in packed FP32, and no
+// error term where a sum is exact or ordered (2.5M queries of a city: 154.8 -> 150.9 ms in all,
+// 152.2 of it without the packing).
+__device__ __forceinline__ void kfix_ff2(const F2 (&a)[3], const float* b, F2 ch, F2 cl, const float2* tab,
+                                         long long& k0, long long& k1) {
+    F2 S, E;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float dh, dl;
-        two_sum(a[k], -b[k], dh, dl);  // a - b = dh + dl exactly
-        const float p = __fmul_rn(dh, dh), pe = __fmaf_rn(dh, dh, -p);
-        float t, te;
-        two_sum(S, p, t, te);
+        const F2 nb = neg2(pair2(b[k], b[3 + k]));
+        F2 dh, dl;
+        two_sum2(a[k], nb, dh, dl);  // a - b = dh + dl exactly
+        const F2 p = mul2(dh, dh), pe = fma2(dh, dh, neg2(p));
         // (dh + dl)^2 = p + pe + dl (2 dh + dl); then renormalise (S, E)
-        E = __fadd_rn(E, __fadd_rn(te, __fmaf_rn(dl, __fmaf_rn(2.f, dh, dl), pe)));
-        S = __fadd_rn(t, E);
-        E = __fsub_rn(E, __fsub_rn(S, t));
+        const F2 rest = fma2(dl, fma2(pair2(2.f), dh, dl), pe);
+        F2 t = p;
+        if (k == 0) {
+            E = rest;
+        } else {
+            F2 te;
+            two_sum2(S, p, t, te);
+            E = add2(E, add2(te, rest));
+        }
+        fast_two_sum2(t, E, S, E);
     }
-    const float yh = __fmul_rn(S, ch);
-    const float yl = __fadd_rn(__fmaf_rn(S, ch, -yh), __fmaf_rn(S, cl, __fmul_rn(E, ch)));
+    const F2 yh = mul2(S, ch);
+    const F2 yl = add2(fma2(S, ch, neg2(yh)), fma2(S, cl, mul2(E, ch)));
     // (no branch on yh > 43.5: the entries of a strip then run interleaved)
-    const float n = rintf(__fmul_rn(yh, kInvL));
-    const int ni = (int)n;
-    // r = (n kL0 - yh) + n kL1 - yl + n kL2, the large parts summed error-free
-    float a0, ae, b0, be, rh, ce;
-    two_sum(__fmul_rn(n, kL0), -yh, a0, ae);
-    const float p2 = __fmul_rn(n, kL1), p2e = __fmaf_rn(n, kL1, -p2);
-    two_sum(a0, p2, b0, be);
-    two_sum(b0, -yl, rh, ce);
-    const float rl = __fadd_rn(__fadd_rn(__fadd_rn(ae, be), ce), __fmaf_rn(n, kL2, p2e));
+    const F2 yn = mul2(yh, pair2(kInvL));
+    const float n0 = rintf(lo2(yn)), n1 = rintf(hi2(yn));
+    const F2 n = pair2(n0, n1);
+    // r = (n kL0 - yh) + n kL1 - yl + n kL2, the large parts summed error-free.  n kL0 - yh is exact:
+    // within a factor of two of each other from n = 2 (Sterbenz), and for n = 1 a multiple of 2^-33
+    // below 2^-9.
+    F2 b0, be, rh, ce;
+    const F2 a0 = sub2(mul2(n, pair2(kL0)), yh);
+    const F2 p2 = mul2(n, pair2(kL1)), p2e = fma2(n, pair2(kL1), neg2(p2));
+    two_sum2(a0, p2, b0, be);
+    two_sum2(b0, neg2(yl), rh, ce);
+    const F2 rl = add2(add2(be, ce), fma2(n, pair2(kL2), p2e));
     // e^r - 1 = rh + rh^2/2 + [rl + rh rl + rh^3/6 + rh^4/24 + (rh^2 error)/2]
-    const float q = __fmul_rn(rh, rh), qe = __fmaf_rn(rh, rh, -q);
-    const float c34 = __fmul_rn(__fmul_rn(q, rh), __fmaf_rn(rh, 1.f / 24.f, 1.f / 6.f));
-    const float small = __fadd_rn(__fmaf_rn(0.5f, qe, rl), __fmaf_rn(rh, rl, c34));
-    float u, ue, eh, e4;
-    two_sum(rh, __fmul_rn(0.5f, q), u, ue);
-    two_sum(1.f, u, eh, e4);
-    const float el = __fadd_rn(e4, __fadd_rn(ue, small));
+    const F2 q = mul2(rh, rh), qe = fma2(rh, rh, neg2(q));
+    const F2 c34 = mul2(mul2(q, rh), fma2(rh, pair2(1.f / 24.f), pair2(1.f / 6.f)));
+    const F2 small = add2(fma2(pair2(0.5f), qe, rl), fma2(rh, rl, c34));
+    F2 u, ue, eh, e4;
+    fast_two_sum2(rh, mul2(pair2(0.5f), q), u, ue);
+    fast_two_sum2(pair2(1.f), u, eh, e4);
+    const F2 el = add2(e4, add2(ue, small));
     // 2^(-n/256) = 2^-m 2^(i/256) with m = ceil(n / 256) and i = (-n) mod 256
-    const int j = ni & 255, m = (ni >> 8) + (j != 0);
-    const float2 T = tab[(256 - j) & 255];
-    const float vh = __fmul_rn(T.x, eh);
-    const float vl = __fadd_rn(__fmaf_rn(T.x, eh, -vh), __fmaf_rn(T.x, el, __fmul_rn(T.y, eh)));
-    const long long k = fix_of_float(vh, kFixBits - m) + fix_of_float(vl, kFixBits - m);
-    return yh <= 43.5f ? k : 0;
+    const int i0 = (int)n0, i1 = (int)n1;
+    const int m0 = (i0 + 255) >> 8, m1 = (i1 + 255) >> 8;
+    const float2 T0 = tab[-i0 & 255], T1 = tab[-i1 & 255];
+    const F2 Tx = pair2(T0.x, T1.x), Ty = pair2(T0.y, T1.y);
+    const F2 vh = mul2(Tx, eh);
+    const F2 vl = add2(fma2(Tx, eh, neg2(vh)), fma2(Tx, el, mul2(Ty, eh)));
+    k0 = lo2(yh) <= 43.5f ? fix_of_positive(lo2(vh), kFixBits - m0) + fix_of_float(lo2(vl), kFixBits - m0) : 0;
+    k1 = hi2(yh) <= 43.5f ? fix_of_positive(hi2(vh), kFixBits - m1) + fix_of_float(hi2(vl), kFixBits - m1) : 0;
 }
 
 // The float pair (hi, lo) of an FP64 value.
@@ -1152,9 +1212,9 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
 // shifted to it and subtracted as an integer, so an updated entry costs no FP64 operation,
 // and each block's columns are stored as FP64 by the update that completes them (the first block's
 // by the assembly).  The slice products run on the tensor cores
-// (trailing_update_tc); within a block the diagonal block is factorised as in the plain loop
-// (8x8 tiles, FP64 tensor path) and the rows below it are solved one row tile per warp
-// (block_rows), which also writes their slices.
+// (trailing_update_tc); within a block the diagonal block is factorised in 8x8 tiles in shared
+// memory and the rows below it are solved one row tile per warp (block_rows, FP64 pipe), which
+// also writes their slices.
 // Nt row tiles, of which the first Ntr are factorised (Nt > Ntr: appended query rows, whose
 // rows below are solved and whose diagonal entries are updated, but not factorised).
 template <class Tc>
@@ -1345,7 +1405,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
     double* A = s.A;
     // A = K + sigma^2 I in 8x8 tiles (Sec. III-A kernel, Eq. 1 noise term); padding rows and
     // columns are the identity so the padded factor is block-diagonal.  The emulated kernel
-    // writes the fixed point of kfix_pair (appended query rows: the query's kernel values, 1
+    // writes the fixed point of kfix_ff2 (appended query rows: the query's kernel values, 1
     // on the diagonal, and only the diagonal tiles of the query-by-query block).
     if constexpr (kEmu) {
         // strips of 8 columns of the 32x32 blocks, one per warp at a time: a row per lane (its
@@ -1376,8 +1436,10 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[e] = live && j0 + e < N ? fix_of_double(c.P.lat_tab[lat_m(s.xi[j0 + e], rx)]) : 0;
             } else if (c.P.precision == VGP_MIXED) {
+                const F2 rw2[3] = {pair2(rw[0]), pair2(rw[1]), pair2(rw[2])};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = kfix_ff(rw, s.Xw + 3 * (j0 + e), c.P.inv2l2_hi, c.P.inv2l2_lo, s.Tff);
+                for (int e = 0; e < 8; e += 2)
+                    kfix_ff2(rw2, s.Xw + 3 * (j0 + e), pair2(c.P.inv2l2_hi), pair2(c.P.inv2l2_lo), s.Tff, v[e], v[e + 1]);
             } else if (qrow) {  // the query's FP64 local coordinates, formed as query_local forms them
                 double xq[3];
                 for (int k = 0; k < 3; ++k) xq[k] = (double)rw[k] - (c.b.centre ? c.b.centre[3 * (int64_t)I + k] : 0.0);
@@ -3017,9 +3079,10 @@ __global__ void k_kfix_probe(const float* xa, const float* xb, long long* out, i
     __syncthreads();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float a[3] = {xa[3 * i], xa[3 * i + 1], xa[3 * i + 2]};
-    const float b[3] = {xb[3 * i], xb[3 * i + 1], xb[3 * i + 2]};
-    out[i] = kfix_ff(a, b, P.inv2l2_hi, P.inv2l2_lo, tab);
+    const F2 a[3] = {pair2(xa[3 * i]), pair2(xa[3 * i + 1]), pair2(xa[3 * i + 2])};
+    const float b[6] = {xb[3 * i], xb[3 * i + 1], xb[3 * i + 2], xb[3 * i], xb[3 * i + 1], xb[3 * i + 2]};
+    long long k1;
+    kfix_ff2(a, b, pair2(P.inv2l2_hi), pair2(P.inv2l2_lo), tab, out[i], k1);
 }
 }  // namespace
 
