@@ -340,6 +340,7 @@ int vgp_create(const vgp_params* p, vgp_map** out) {
         return fail(VGP_ERR_OOM, "vgp_create: table allocation failed");
     }
     cudaMemcpy(m->mc_tab, mc.data(), mc.size(), cudaMemcpyHostToDevice);
+    graph_cache_ready(m->gcache);  // the map's own stream (if it fails, a call that wants one tries again)
     *out = m;
     return VGP_OK;
 }

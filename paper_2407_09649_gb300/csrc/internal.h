@@ -111,6 +111,7 @@ struct GraphCache {
     int64_t replays = 0, instantiations = 0;
 };
 void graph_cache_destroy(GraphCache& gc);
+bool graph_cache_ready(GraphCache& gc);  // its stream and events; false if they cannot be created
 
 // Solve every instance of the batch (factorise, alpha, evaluate its queries).  Returns
 // error bits through *err_dev.  Synchronises once to read the size histogram (in graph mode

@@ -2530,9 +2530,8 @@ void graph_cache_destroy(GraphCache& gc) {
     gc = GraphCache{};
 }
 
-namespace {
-
-// The map's own stream and the events that join it to a caller's stream, created on first use.
+// The map's own stream and the events that join it to a caller's stream, created with the map (or, if
+// that failed, by the first call that wants them).
 bool graph_cache_ready(GraphCache& gc) {
     if (gc.t1) return true;
     if ((gc.gs || cudaStreamCreateWithFlags(&gc.gs, cudaStreamNonBlocking) == cudaSuccess) &&
@@ -2543,6 +2542,8 @@ bool graph_cache_ready(GraphCache& gc) {
     cudaGetLastError();
     return false;
 }
+
+namespace {
 
 void add_stats(SolveStats* stats, const std::vector<int>& h) {
     if (!stats) return;
