@@ -41,10 +41,10 @@ WORKLOAD = "city G-GPDF: 2M surface pts, 10M queries (70% free space, 30% <=0.5 
 # by the ratio of the two launches' algorithmic work (sum of N^3/3 + 2 N^2: 2.854e12 against
 # 1.851e12 flop, x1.542; an earlier kernel's small and full-size captures had that ratio).
 # None when the kernel has changed since.
-K_SOLVE_TRAFFIC = 1.0921e12
-K_SOLVE_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the N > 224 launch (k_solve_emu) on "
+K_SOLVE_TRAFFIC = 1.2163e12
+K_SOLVE_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the N > 32 launch (k_solve_emu) on "
                           "the 100k-query city case, scaled to the full step by its algorithmic work; "
-                          "smaller buckets not included")
+                          "instances of at most 32 points not included")
 
 # Algorithmic DRAM bytes of the HBM-bound steps (what each step must move at least):
 #   bin (S1): read the point (12 B) and write its leaf slot (4 B); the leaf table and its
@@ -141,7 +141,7 @@ def bf16_peak_tflops(pk):
     return float(pk.get("bf16_tflops") or 1900.0)
 
 
-# FP64 tensor path (mma.sync m8n8k4 f64) peak: the measured bf16 dense peak times the nominal
+# FP64 peak (pipe and tensor path alike): the measured bf16 dense peak times the nominal
 # FP64 / bf16 ratio of GB300 (1.25 / 2250 TFLOP/s).
 def fp64_tensor_peak_tflops(pk):
     return bf16_peak_tflops(pk) * 1.25 / 2250.0
@@ -427,11 +427,11 @@ def comparisons(S, Q, S_h, Q_h, args):
 
 
 def city_lines(S, Q, args):
-    """On the city workload: the all-FP64 tensor path, variance on (full size), the precision
+    """On the city workload: every update in FP64, variance on (full size), the precision
     subset, the blended Eq. 10 G-GPDF, and the plain FP64 per-instance form."""
     from paper_2407_09649_gb300.api import Map
     out = {}
-    # the headline workload with every Cholesky update on the FP64 tensor path (no emulation)
+    # the headline workload with every Cholesky update on the FP64 pipe (no emulation)
     mpl = Map(precision="mixed", profile=1)
     mpl.set_surface(S)
     mpl.autotune(Q[: min(Q.shape[0], args.n_tune)].contiguous())

@@ -303,7 +303,8 @@ int vgp_create(const vgp_params* p, vgp_map** out) {
     }
     cudaMemset(m->dev_words, 0, sizeof(int) * 8);
     // constant tables, computed on the host in extended precision and rounded once:
-    // 2^(j/256) for the FP64 exponentials (as pairs: all high parts, then all low parts), exp(-m vs^2 / (2 l^2)) for voxel-lattice distances
+    // 2^(j/256) for the FP64 exponentials (as pairs: all high parts, then all low parts),
+    // exp(-m vs^2 / (2 l^2)) for voxel-lattice distances
     std::vector<double> tab(512 + kLatticeTable);
     std::vector<float> tabf(kLatticeTable);
     for (int j = 0; j < 256; ++j) {
