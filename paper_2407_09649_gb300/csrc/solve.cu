@@ -2867,28 +2867,25 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         }
         return 0;
     }
-    // a bucket's launch: shapes, kernel and resident CTAs per SM
+    // a bucket's launch: shapes, kernel, resident CTAs per SM, clusters and workspaces
     struct Launch {
-        int npad, qmax, nrow, threads, stage, per_sm;
+        int nmax, cnt, npad, qmax, nrow, threads, stage, per_sm, ncta, groups;
         size_t shm;
+        int64_t ws_a, ws_v, ws_e;  // strides, per group of CTAs (ws_v: per CTA)
         bool emu;
         SolveKernel kern;
     };
-    auto bucket_nmax = [&](int i, int& cnt) {
-        int nmax = 0;
-        cnt = 0;
-        for (int N = buckets[i].lo; N <= buckets[i].hi; ++N) {
-            cnt += h[N];
-            if (h[N]) nmax = N;
-        }
-        return nmax;
-    };
-    auto bucket_launch = [&](int i, int nmax, int cnt) {
+    auto bucket_launch = [&](int i) {
         const Bucket& bk = buckets[i];
+        Launch L{};
+        for (int N = bk.lo; N <= bk.hi; ++N) {
+            L.cnt += h[N];
+            if (h[N]) L.nmax = N;
+        }
+        if (L.cnt == 0) return L;
         const BucketShape bs = bw ? BucketShape{cfg->threads[i], cfg->per_sm[i], cfg->stage_panel}
-                                  : bucket_shape(*cfg, i, cnt, n_sm, heavy, (int64_t)hq[i]);
-        Launch L;
-        L.npad = std::max((nmax + 7) & ~7, 8);
+                                  : bucket_shape(*cfg, i, L.cnt, n_sm, heavy, (int64_t)hq[i]);
+        L.npad = std::max((L.nmax + 7) & ~7, 8);
         L.emu = !bw && !bk.smem_a && P.emulate;
         emu_rows_for(L.emu, b, L.npad, L.qmax, L.nrow);
         L.threads = L.emu ? kEmuThreads : bs.threads;
@@ -2896,76 +2893,88 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         L.shm = smem_bytes(L.npad, bk.smem_a, bw ? 0 : b.nprop, L.stage, b.Xi != nullptr, bw != nullptr, L.emu);
         L.kern = bw ? k_backward : pick_solve(b.nprop > 0, L.emu);
         cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.shm);
-        if (L.emu) set_emu_carveout(L.kern);
-        L.per_sm = 0;
         if (L.emu) {
+            set_emu_carveout(L.kern);
             L.per_sm = emu_ctas_per_sm(L.kern, L.threads, L.shm);
         } else {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L.per_sm, L.kern, L.threads, L.shm);
             L.per_sm = std::max(L.per_sm, 1);
             if (bs.per_sm > 0) L.per_sm = std::min(L.per_sm, bs.per_sm);
         }
+        L.ws_a = bk.smem_a ? 0 : matrix_words(L.emu, L.nrow);
+        L.ws_v = b.want_var && !bw && !L.emu ? (int64_t)L.npad * L.threads : 0;
+        L.ws_e = L.emu ? (int64_t)L.nrow * kEmuBytesPerRow : 0;
         return L;
     };
-    int* counters = (int*)ar.get(Arena::kCounters, sizeof(int) * 8, st);
-    // the buckets' ranges of the order, and the CTAs to spread each over; work items are planned
-    // only where some bucket can have more of them than instances
+    // the launches, the buckets' ranges of the order and the CTAs to spread each over; work items are
+    // planned only where some bucket can have more of them than instances
+    Launch launches[5];
     bool chunks = false;
-    int max_items[5] = {0, 0, 0, 0, 0};
-    for (int i = 0, off = 0; i < 5 && !bw; ++i) {
-        int cnt = 0;
-        const int nmax = bucket_nmax(i, cnt);
+    int64_t need_a = 0, need_v = 0, need_v_aside = 0, need_e = 0;
+    // the smallest instances run on the map's own stream beside the others, where its CTAs fill the SMs
+    // that the last of those leave; not while profiling
+    bool beside = false;
+    for (int i = 0, off = 0; i < 5; ++i) {
+        Launch& L = launches[i];
+        L = bucket_launch(i);
         ca.off[i] = off;
-        off += cnt;
-        if (cnt == 0) continue;
-        const Launch L = bucket_launch(i, nmax, cnt);
-        chunk_args(b, i, cnt, n_sm, L.per_sm, L.threads, L.emu, ca);
-        int nmin = nmax;
-        for (int N = nmax; N >= buckets[i].lo; --N)
-            if (h[N]) nmin = N;
-        // the shortest chunk any of its instances can have
-        const int64_t len = std::max<int64_t>(1, chunk_len(ca.qmin[i], ca.qn[i], nmin, ca.cap[i]));
-        const int64_t extra = std::min<int64_t>((int64_t)hq[i] / len, ca.cap[i] > 0 ? INT32_MAX : ca.slots[i]);
-        max_items[i] = (int)std::min<int64_t>(INT32_MAX, cnt + extra);
-        // (without a bound, a launch of ten rounds of instances or more has no tail to shorten)
-        if (ca.cap[i] == 0 && cnt > 10 * ca.slots[i]) {
-            ca.qmin[i] = 0;
-            max_items[i] = cnt;
-        } else {
-            chunks = chunks || extra > 0;
+        off += L.cnt;
+        if (L.cnt == 0) continue;
+        int items = L.cnt;  // an upper bound of the launch's work items
+        if (!bw) {
+            chunk_args(b, i, L.cnt, n_sm, L.per_sm, L.threads, L.emu, ca);
+            int nmin = L.nmax;
+            for (int N = L.nmax; N >= buckets[i].lo; --N)
+                if (h[N]) nmin = N;
+            // the shortest chunk any of its instances can have
+            const int64_t len = std::max<int64_t>(1, chunk_len(ca.qmin[i], ca.qn[i], nmin, ca.cap[i]));
+            const int64_t extra = std::min<int64_t>((int64_t)hq[i] / len, ca.cap[i] > 0 ? INT32_MAX : ca.slots[i]);
+            // (without a bound, a launch of ten rounds of instances or more has no tail to shorten)
+            if (ca.cap[i] == 0 && L.cnt > 10 * ca.slots[i]) {
+                ca.qmin[i] = 0;
+            } else {
+                chunks = chunks || extra > 0;
+                items = (int)std::min<int64_t>(INT32_MAX, L.cnt + extra);
+            }
         }
+        // few emulated work items: clusters of CTAs work on each
+        L.ncta = L.emu ? group_ctas(items, L.nmax, n_sm * L.per_sm) : 1;
+        L.groups = (int)std::min<int64_t>(items, (int64_t)n_sm * L.per_sm / L.ncta);
+        if (i == 4) beside = !bw && !profile && L.cnt < n && gc && graph_cache_ready(*gc);
+        need_a = std::max(need_a, L.ws_a * L.groups);
+        int64_t& nv = i == 4 && beside ? need_v_aside : need_v;
+        nv = std::max(nv, L.ws_v * L.groups);
+        need_e = std::max(need_e, L.ws_e * L.groups);
     }
-    if (chunks) {
-        chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
-        if (chunk_off) {
-            chunk_q = chunk_off + n + 1;
-            k_chunk_plan<<<1, 1024, 0, st>>>(order, (int)n, b.inst_off, b.q_off, nullptr, ca, chunk_q, chunk_off);
-            note_launch();
-        }
-    }
-    if (!counters || (chunks && !chunk_off)) {
+    // Every workspace is obtained before the first launch and before e0: a slot that grew between two
+    // launches would give its block back behind the first one's kernel, in the order of st alone, and
+    // the allocator may hand that block to a launch on the map's own stream, which waits for
+    // nothing after e0.
+    int* counters = (int*)ar.get(Arena::kCounters, sizeof(int) * 8, st);
+    double* ws_a = need_a ? (double*)ar.get(Arena::kWs0, sizeof(double) * need_a, st) : nullptr;
+    double* ws_v = need_v ? (double*)ar.get(Arena::kWs1, sizeof(double) * need_v, st) : nullptr;
+    double* ws_v_aside = need_v_aside ? (double*)ar.get(Arena::kWs4, sizeof(double) * need_v_aside, st) : nullptr;
+    uint8_t* ws_e = need_e ? (uint8_t*)ar.get(Arena::kWs3, need_e, st) : nullptr;
+    if (chunks) chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
+    if (!counters || (need_a && !ws_a) || (need_v && !ws_v) || (need_v_aside && !ws_v_aside) || (need_e && !ws_e) ||
+        (chunks && !chunk_off)) {
         if (profile) {
             cudaEventDestroy(ev0);
             cudaEventDestroy(ev1);
         }
         return alloc_failed(err_dev, st);
     }
-    cudaMemsetAsync(counters, 0, sizeof(int) * 8, st);
-    // the smallest instances run on the map's own stream beside the others, where its CTAs fill the SMs
-    // that the last of those leave (their own variance columns: Arena::kWs4); not while profiling
-    bool beside = false;
-    if (!bw && !profile && gc && graph_cache_ready(*gc)) {
-        int cnt = 0;
-        bucket_nmax(4, cnt);
-        beside = cnt > 0 && cnt < n && cudaEventRecord(gc->e0, st) == cudaSuccess &&
-                 cudaStreamWaitEvent(gc->gs, gc->e0, 0) == cudaSuccess;
+    if (chunks) {
+        chunk_q = chunk_off + n + 1;
+        k_chunk_plan<<<1, 1024, 0, st>>>(order, (int)n, b.inst_off, b.q_off, nullptr, ca, chunk_q, chunk_off);
+        note_launch();
     }
+    cudaMemsetAsync(counters, 0, sizeof(int) * 8, st);
+    beside = beside && cudaEventRecord(gc->e0, st) == cudaSuccess && cudaStreamWaitEvent(gc->gs, gc->e0, 0) == cudaSuccess;
     int done = 0;  // instances already assigned (from the large end)
     for (int bi = 0; bi < 5; ++bi) {
-        const Bucket& bk = buckets[bi];
-        int cnt = 0;
-        const int nmax = bucket_nmax(bi, cnt);
-        if (cnt == 0) continue;
+        const Launch& L = launches[bi];
+        if (L.cnt == 0) continue;
         const bool aside = beside && bi == 4;
         const cudaStream_t ls = aside ? gc->gs : st;
         SolveCtx c;
@@ -2979,40 +2988,28 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         c.counter = counters + bi;
         c.order = order + done;
         c.inst_base = 0;
-        c.n_work = cnt;
+        c.n_work = L.cnt;
         c.chunk_off = chunk_off ? chunk_off + done : nullptr;
         c.chunk_q = chunk_q ? chunk_q + bi : nullptr;
         c.chunk_qn = ca.qn[bi];
         c.chunk_cap = ca.cap[bi];
-        const Launch L = bucket_launch(bi, nmax, cnt);
         c.npad = L.npad;
         c.qmax = L.qmax;
         c.nrow = L.nrow;
-        c.a_in_smem = bk.smem_a;
-        const bool emu = L.emu;
-        const int threads = L.threads;
+        c.a_in_smem = buckets[bi].smem_a;
         c.stage_panel = L.stage;
         if (bw) c.bw = *bw;
-        const size_t shm = L.shm;
-        auto kern = L.kern;
-        const int per_sm = L.per_sm;
-        // few emulated work items: clusters of CTAs work on each
-        if (emu) c.ncta = group_ctas(max_items[bi], nmax, n_sm * per_sm);
-        const int groups = (int)std::min<int64_t>(bw ? cnt : max_items[bi], (int64_t)n_sm * per_sm / c.ncta);
-        const int grid = groups * c.ncta;
-        c.ws_a_stride = c.a_in_smem ? 0 : matrix_words(emu, c.nrow);
-        c.ws_a = c.a_in_smem ? nullptr : (double*)ar.get(Arena::kWs0, sizeof(double) * c.ws_a_stride * groups, st);
-        c.ws_v_stride = (int64_t)c.npad * threads;
-        c.ws_v = (b.want_var && !bw && !emu) ? (double*)ar.get(aside ? Arena::kWs4 : Arena::kWs1, sizeof(double) * c.ws_v_stride * grid, st) : nullptr;
-        c.ws_e_stride = emu ? (int64_t)c.nrow * kEmuBytesPerRow : 0;
-        c.ws_e = emu ? (uint8_t*)ar.get(Arena::kWs3, c.ws_e_stride * groups, st) : nullptr;
-        if ((!c.a_in_smem && !c.ws_a) || (b.want_var && !bw && !emu && !c.ws_v) || (emu && !c.ws_e)) {
-            if (profile) {
-                cudaEventDestroy(ev0);
-                cudaEventDestroy(ev1);
-            }
-            return alloc_failed(err_dev, st);
-        }
+        c.ncta = L.ncta;
+        const int grid = L.groups * L.ncta;
+        c.ws_a_stride = L.ws_a;
+        c.ws_a = L.ws_a ? ws_a : nullptr;
+        c.ws_v_stride = L.ws_v;
+        c.ws_v = !L.ws_v ? nullptr : bi == 4 && need_v_aside ? ws_v_aside : ws_v;
+        c.ws_e_stride = L.ws_e;
+        c.ws_e = L.ws_e ? ws_e : nullptr;
+        // (buckets share kernels, whose limit is that of the bucket shaped last)
+        auto kern = L.ncta > 1 ? pick_solve(b.nprop > 0, true, true) : L.kern;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.shm);
         cudaEvent_t b0 = nullptr, b1 = nullptr;
         if (profile) {
             cudaEventCreate(&b0);
@@ -3020,7 +3017,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             cudaEventRecord(b0, st);
         }
         if (c.ncta == 1) {
-            kern<<<grid, threads, shm, ls>>>(c);
+            kern<<<grid, L.threads, L.shm, ls>>>(c);
         } else {
             cudaLaunchAttribute at{};
             at.id = cudaLaunchAttributeClusterDimension;
@@ -3028,13 +3025,11 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             at.val.clusterDim.y = at.val.clusterDim.z = 1;
             cudaLaunchConfig_t lc{};
             lc.gridDim = dim3(grid);
-            lc.blockDim = dim3(threads);
-            lc.dynamicSmemBytes = shm;
+            lc.blockDim = dim3(L.threads);
+            lc.dynamicSmemBytes = L.shm;
             lc.stream = ls;
             lc.attrs = &at;
             lc.numAttrs = 1;
-            kern = pick_solve(b.nprop > 0, true, true);
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
             set_emu_carveout(kern);
             cudaLaunchKernelEx(&lc, kern, c);
         }
@@ -3053,7 +3048,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             cudaEventDestroy(b0);
             cudaEventDestroy(b1);
         }
-        done += cnt;
+        done += L.cnt;
     }
     if (profile) {
         cudaEventRecord(ev1, st);

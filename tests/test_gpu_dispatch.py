@@ -150,3 +150,41 @@ def test_blend_weights_at_their_range(vg, orc, n_nodes, lam):
     ok = ref["status"] == 0
     assert ok.sum() > 100
     assert np.abs(out["d"][ok] - ref["d"][ok]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("sizes,nq", [([240] + [100] * 200 + [20] * 40, [4000] + [40] * 240),
+                                      ([1000] * 2 + [200] * 2000 + [8] * 100, [300] * 2 + [24] * 2000 + [300] * 100)])
+def test_workspaces_grow_beside_the_smallest(vg, sizes, nq):
+    """The first call of a map whose few large instances need less workspace than the many of the next
+    size, with instances of at most 32 points on the map's stream beside them: no launch may be
+    given memory that another one still uses."""
+    X, Q = _instances(sizes, max(nq), 58)
+    Q = [q[:k] for q, k in zip(Q, nq)]
+    ref = vg.Map(precision="fp64", emulate_fp64=0)
+    want = []
+    for n in sorted(set(sizes), reverse=True):  # one size at a time: one launch, nothing beside it
+        pick = [i for i, s in enumerate(sizes) if s == n]
+        want += _solve(ref, [X[i] for i in pick], [Q[i] for i in pick], True)
+    for _ in range(3):
+        for a, b in zip(_solve(vg.Map(precision="fp64", emulate_fp64=0), X, Q, True), want):
+            _same(a, b)
+
+
+def test_caller_waits_for_the_smallest(vg):
+    """The smallest instances take far longer than the one beside them, on a map that has run nothing
+    before: what the caller's stream does next sees their results."""
+    sizes = [40] + [32] * 6000
+    X, Q = _instances(sizes, 200, 59)
+    io = torch.from_numpy(np.concatenate([[0], np.cumsum(sizes)])).cuda()
+    qo = torch.arange(len(Q) + 1, dtype=torch.int64, device="cuda") * 200
+    x, q = (torch.from_numpy(np.vstack(a)).cuda() for a in (X, Q))
+    ref = vg.Map(precision="fp64", emulate_fp64=0)
+    want = [_solve(ref, X[a:b], Q[a:b], True) for a, b in ((0, 1), (1, len(sizes)))]
+    want = {k: np.concatenate([r[k] for part in want for r in part]) for k in KEYS}
+    for m in (vg.Map(precision="fp64", emulate_fp64=0), ref):
+        out = m.gp_batch(io, x, qo, q, var=True)
+        got = {k: out[k].clone() for k in KEYS}
+        for k in KEYS:
+            out[k].zero_()
+        torch.cuda.synchronize()
+        _same({k: v.cpu().numpy() for k, v in got.items()}, want)
