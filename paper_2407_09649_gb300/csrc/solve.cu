@@ -2260,14 +2260,16 @@ __global__ void k_plan_buckets(const int* hist, int* cursor, int* plan) {
 struct ChunkPlanArgs {
     int off[5], cnt[5], slots[5], cap[5], qmin[5], qn[5];
 };
-// Sum over the CTA (all threads call; w: 32 values of scratch), the same on every thread.
+// Sum over the CTA (all threads call; w: 32 values of scratch, the caller's again on return), the same on
+// every thread.
 __device__ int block_sum(int v, int* w) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     v = __reduce_add_sync(0xffffffffu, v);
-    __syncthreads();
     if (lane == 0) w[warp] = v;
     __syncthreads();
-    return __reduce_add_sync(0xffffffffu, lane < nwarp ? w[lane] : 0);
+    const int x = lane < nwarp ? w[lane] : 0;
+    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, x);
 }
 __global__ void k_chunk_plan(const int32_t* order, int n, const int64_t* inst_off, const int64_t* q_off,
                              const int* plan, ChunkPlanArgs a, int* chunk_q, int* chunk_off) {

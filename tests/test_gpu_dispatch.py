@@ -188,3 +188,19 @@ def test_caller_waits_for_the_smallest(vg):
             out[k].zero_()
         torch.cuda.synchronize()
         _same({k: v.cpu().numpy() for k, v in got.items()}, want)
+
+
+def test_work_items_of_many_instances(vg):
+    """More instances than the planning CTA has threads, with none to 3000 queries each: every query is
+    answered, call after call, as in batches that are planned in one pass."""
+    rng = np.random.default_rng(60)
+    sizes = rng.integers(33, 65, 2500)
+    X, Q = _instances(sizes, 0, 60)
+    nq = np.where(rng.random(2500) < 0.02, 3000, rng.integers(0, 60, 2500))
+    Q = [(x[0] + rng.uniform(-1, 1, (k, 3))).astype(np.float32) for x, k in zip(X, nq)]
+    for emulate in (0, 1):
+        m = vg.Map(precision="mixed", emulate_fp64=emulate)
+        want = [r for a in range(0, 2500, 500) for r in _solve(m, X[a:a + 500], Q[a:a + 500], True)]
+        for _ in range(3):
+            for a, b in zip(_solve(m, X, Q, True), want):
+                _same(a, b)
