@@ -984,6 +984,7 @@ __device__ __forceinline__ bool group_sync(Tc& tc, int flag) {
     if (tc.n() == 1) return any != 0;
     int* f = tc.flags + 8 * tc.set;
     if ((int)threadIdx.x < tc.n()) peer_store(f + tc.rank(), threadIdx.x, any);
+    __syncwarp();  // (the aligned barrier wants the whole warp, and only its first lanes stored)
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     int all = 0;
@@ -1149,7 +1150,10 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // the band's last products are done (so warp 0 has seen every copy): its A and B buffers
             // take the next band's
-            if (!__any_sync(0xffffffffu, fail) && jt + n >= n_tiles && b1 < M) stage_band(b1);
+            if (!__any_sync(0xffffffffu, fail) && jt + n >= n_tiles && b1 < M) {
+                stage_band(b1);
+                __syncwarp();  // (some lanes copied; the aligned tensor-memory loads want the whole warp)
+            }
             if (on) {
                 const uint32_t tbase = tc.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(16 * h);
 #pragma unroll
