@@ -204,3 +204,46 @@ def test_work_items_of_many_instances(vg):
         for _ in range(3):
             for a, b in zip(_solve(m, X, Q, True), want):
                 _same(a, b)
+
+
+@pytest.mark.parametrize("precision,nc,raycast", [("fp64", 4, False), ("mixed", 3, True), ("mixed", 1, False)])
+def test_voxel_frames_with_properties_in_clusters(vg, orc, precision, nc, raycast):
+    """Frames of one to five leaves of 129 to 512 points, whose distance and property GPs clusters of CTAs
+    work on: the oracle's values, and the same bits as in a frame of so many other leaves that each
+    instance has one CTA."""
+    rng = np.random.default_rng(61)
+    leaves = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [6, 0, 0], [0, -6, 2]])
+    keep = [512, 129, 256, 300, 161]
+    origin = np.array([0.4, 0.4, 3.0]) if raycast else None
+    vox = [8 * L + np.stack(np.unravel_index(rng.permutation(512)[:k], (8, 8, 8)), 1) for L, k in zip(leaves, keep)]
+    far = np.array([[8 * (20 + 4 * i), 8 * 4 * j, 0] for i in range(12) for j in range(12)])
+    far = (far[:, None] + np.stack(np.meshgrid(np.arange(8), np.arange(8), [3, 4]), -1).reshape(1, -1, 3)).reshape(-1, 3)
+    pr = lambda v: (0.5 + 0.4 * np.sin(0.13 * v @ np.array([[1.0, 2, 3, 1], [2, 1, 0, 3], [0, 3, 1, 2]]))[:, :nc]).astype(np.float32)
+
+    def frame(v):
+        m = vg.Map(precision=precision, max_pts_leaf=512, n_props=nc, emulate_fp64=1)
+        pts = torch.from_numpy((v * 0.1).astype(np.float32)).cuda()
+        f = m.build_frame(pts, origin=origin, props=torch.from_numpy(pr(v)).cuda())
+        r = {k: t.cpu().numpy() for k, t in f.results().items()}
+        c, w = (t.cpu().numpy() for t in f.props())
+        return {int(k): i for i, k in enumerate(r["keys"])}, (r["d"], r["v"], r["grad"], c, w)
+
+    for n in (1, 2, 5):
+        v = np.concatenate(vox[:n])
+        at, val = frame(v)
+        if n < 5 and not raycast:  # eight and two CTAs each (rays to the far leaves would add voxels here)
+            many, ref = frame(np.concatenate([v, far]))
+            pick = [many[k] for k in at]
+            for a, b in zip(val, ref):
+                assert np.array_equal(np.ascontiguousarray(a).view(np.uint8), np.ascontiguousarray(b[pick]).view(np.uint8))
+        want = orc.frame((v * 0.1).astype(np.float32), orc.params(max_pts_leaf=512, n_props=nc), origin=origin, props=pr(v))
+        assert len(at) == len(want.test_key)
+        pick = [at[int(k)] for k in want.test_key]
+        fin = np.isfinite(want.w)
+        assert fin.any() and np.array_equal(np.isfinite(val[4][pick]), fin)
+        # (property values as in the property tests: linear in the data, solved in FP64 on both sides)
+        assert np.abs(val[3][pick][fin] - want.c[fin]).max() <= 1e-8
+        assert np.abs(val[4][pick][fin] - want.w[fin]).max() <= 1e-8
+        if precision == "fp64":
+            ok = want.status == 0
+            assert np.abs(val[0][pick][ok] - want.d[ok]).max() <= 1e-4
