@@ -435,7 +435,8 @@ int vgp_autotune(vgp_map* m, const float* q_dev, int64_t n, vgp_stream stream);
  * the size buckets N > 224, 129..224, 65..128, 33..64, <= 32 (multiples of 32 in [32, 1024]),
  * per_sm[5] caps on CTAs per SM (0: the occupancy limit), stage_panel 1 or 0 for the N > 224
  * bucket (panel column staged in shared memory, or read through L1/L2 with room for two
- * CTAs per SM).  VGP_ERR_ARG on a bad value.  Results do not depend on the shapes.
+ * CTAs per SM).  CTAs of more than 640 threads run with 640, the kernels' limit.
+ * VGP_ERR_ARG on a bad value.  Results do not depend on the shapes.
  */
 int vgp_set_launch(vgp_map* m, const int32_t* threads, const int32_t* per_sm, int32_t stage_panel);
 

@@ -54,6 +54,10 @@ __device__ __forceinline__ int tri_row(int p) {
 }
 
 constexpr int kEmuThreads = 256;  // CTA size of the emulated-update kernels (two CTAs per SM)
+// Largest CTA of the plain kernels: five warps per sub-partition leave each thread 96 registers (k_solve is
+// bounded to them; k_backward takes 86, and 96 with spills when bounded).  A chosen shape of more
+// threads runs with this many.
+constexpr int kPlainThreads = 640;
 constexpr int kEB = 4;            // tiles (of 8 columns) per block of the emulated factorisation
 constexpr int kEK = kEB / 2;      // 16-column mma steps per block
 constexpr int kDiagTiles = kEB * (kEB + 1) / 2;
@@ -2090,9 +2094,8 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
 // kProps: surface-property mode (Eq. 6); the emulated kernels run the trailing updates of
 // N > 32 instances on the bf16 tensor cores (256 threads, two CTAs per SM).  Separate
 // kernels, so that the plain distance kernel keeps its register budget.
-// (up to 640 threads, five warps per sub-partition, the largest shape its registers have allowed)
 template <bool kProps>
-__global__ void __launch_bounds__(640) k_solve(SolveCtx c) {
+__global__ void __launch_bounds__(kPlainThreads) k_solve(SolveCtx c) {
     solve_body<kProps, false, false>(c);
 }
 
@@ -2593,7 +2596,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         s.emu = !s.smem_a && P.emulate;
         emu_rows_for(s.emu, b, s.npad, s.qmax, s.nrow);
         s.stage = s.smem_a ? 1 : (s.emu ? 0 : cfg->stage_panel);
-        s.threads = s.emu ? kEmuThreads : cfg->threads[i];
+        s.threads = s.emu ? kEmuThreads : std::min(cfg->threads[i], kPlainThreads);
         s.shm = smem_bytes(s.npad, s.smem_a, b.nprop, s.stage, b.Xi != nullptr, false, s.emu);
         s.kern = pick_solve(props, s.emu);
     }
@@ -2894,7 +2897,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         L.npad = std::max((L.nmax + 7) & ~7, 8);
         L.emu = !bw && !bk.smem_a && P.emulate;
         emu_rows_for(L.emu, b, L.npad, L.qmax, L.nrow);
-        L.threads = L.emu ? kEmuThreads : bs.threads;
+        L.threads = L.emu ? kEmuThreads : std::min(bs.threads, kPlainThreads);
         L.stage = bk.smem_a ? 1 : (L.emu ? 0 : bs.stage);
         L.shm = smem_bytes(L.npad, bk.smem_a, bw ? 0 : b.nprop, L.stage, b.Xi != nullptr, bw != nullptr, L.emu);
         L.kern = bw ? k_backward : pick_solve(b.nprop > 0, L.emu);

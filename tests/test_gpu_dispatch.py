@@ -247,3 +247,37 @@ def test_voxel_frames_with_properties_in_clusters(vg, orc, precision, nc, raycas
         if precision == "fp64":
             ok = want.status == 0
             assert np.abs(val[0][pick][ok] - want.d[ok]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("threads", [640, 672, 768, 1024])
+def test_largest_launch_shapes(vg, threads):
+    """Every shape that vgp_set_launch takes runs, in each kernel and launch mode that uses it."""
+    rng = np.random.default_rng(62)
+    surf = rng.uniform(-1, 1, (9000, 3)).astype(np.float32) * [1, 1, 0.4]
+    q = torch.from_numpy(rng.uniform(-1, 1, (600, 3)).astype(np.float32)).cuda()
+    surf = torch.from_numpy(surf.astype(np.float32)).cuda()
+    gd = torch.from_numpy(rng.uniform(-1, 1, 600)).cuda()
+    X, Q = _instances([9, 40, 100, 200, 300], 30, 62)
+    ref = None
+    for launch, chosen in (("batched", None), ("batched", threads), ("graph", threads)):
+        m = vg.Map(precision="fp64", launch=launch, max_pts_leaf=256, n_props=1)
+        if chosen:
+            m.set_launch([threads] * 5, [0] * 5, 1)
+        m.set_surface(surf)
+        out = [v.cpu().numpy() for v in m.query(q, grad=True, var=True).values()]
+        dq, dX = m.query_backward(q, gd)
+        out += [dq.cpu().numpy()] + [v for r in _solve(m, X, Q, True) for v in r.values()]
+        f = m.build_frame(surf, props=surf[:, :1].contiguous())
+        out += [v.cpu().numpy() for v in f.results().values()] + [v.cpu().numpy() for v in f.props()]
+        if ref is None:
+            ref, ref_x = out, dX
+            continue
+        for a, b in zip(out[:-7], ref[:-7]):
+            assert np.array_equal(np.ascontiguousarray(a).view(np.uint8), np.ascontiguousarray(b).view(np.uint8))
+        # testing voxels come in an order of their own
+        oa, ob = (np.argsort(o[-7], kind="stable") for o in (out, ref))
+        for a, b in zip(out[-7:], ref[-7:]):
+            assert np.array_equal(np.ascontiguousarray(a[oa]).view(np.uint8), np.ascontiguousarray(b[ob]).view(np.uint8))
+        # (each point's sum of two parts per instance, by atomics in any order: 54 terms at most, which
+        # may exceed their sum by 1e4)
+        assert (dX - ref_x).abs().max().item() <= 1e-9 * ref_x.abs().max().item()
