@@ -170,7 +170,8 @@ typedef struct {
     double t_solve_ms;    /* GP solve kernels (factorise + evaluate), if params.profile */
     double t_bucket_ms[5];   /* the same per launch: N > 224, 129..224, 65..128, 33..64, <= 32 (with
                                 emulate_fp64 the instances above 32 points are one launch, the first) */
-    int32_t cfg_threads[5];  /* launch shape used per bucket: threads per CTA ... */
+    int32_t cfg_threads[5];  /* launch shape used per bucket (those of t_bucket_ms; the one set or chosen
+                                where nothing was launched): threads per CTA ... */
     int32_t cfg_per_sm[5];   /* ... and cap on CTAs per SM (0: occupancy limit) */
     int64_t grid_leaves;  /* leaves in the global grid */
     int64_t grid_capacity_leaves;

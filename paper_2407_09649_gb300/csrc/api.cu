@@ -585,6 +585,7 @@ int vgp_build_frame_props(vgp_map* m, const float* pts, const float* props, int6
     b.alpha_out = f->alpha;
     b.want_var = 1;
     SolveStats ss;
+    ss.cfg = m->cfg;
     b.max_n = P.cap_leaf;
     if (solve_batch(b, P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0, m->prm.launch, &m->cfg,
                     &m->gcache) == -2)
@@ -644,10 +645,10 @@ int vgp_build_frame_props(vgp_map* m, const float* pts, const float* props, int6
     S.t_solve_ms = ss.t_solve_ms;
     for (int i = 0; i < 5; ++i) {
         S.t_bucket_ms[i] = ss.t_bucket_ms[i];
-        S.cfg_threads[i] = m->cfg.threads[i];
-        S.cfg_per_sm[i] = m->cfg.per_sm[i];
+        S.cfg_threads[i] = ss.cfg.threads[i];
+        S.cfg_per_sm[i] = ss.cfg.per_sm[i];
     }
-    S.cfg_stage_panel = m->cfg.stage_panel;
+    S.cfg_stage_panel = ss.cfg.stage_panel;
     S.graph_replays = m->gcache.replays;
     S.graph_instantiations = m->gcache.instantiations;
     S.grid_leaves = m->g_leaves;
@@ -1492,6 +1493,7 @@ int vgp_query_distance_gradient(vgp_map* m, const float* q, int64_t n, double* d
     b.status = status;
     b.want_var = var != nullptr;
     SolveStats ss;
+    ss.cfg = m->cfg;
     b.max_n = m->P.cap_group;
     TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0,
                                  m->prm.launch, &m->cfg, &m->gcache),
@@ -1512,10 +1514,10 @@ int vgp_query_distance_gradient(vgp_map* m, const float* q, int64_t n, double* d
     S.t_solve_ms = ss.t_solve_ms;
     for (int i = 0; i < 5; ++i) {
         S.t_bucket_ms[i] = ss.t_bucket_ms[i];
-        S.cfg_threads[i] = m->cfg.threads[i];
-        S.cfg_per_sm[i] = m->cfg.per_sm[i];
+        S.cfg_threads[i] = ss.cfg.threads[i];
+        S.cfg_per_sm[i] = ss.cfg.per_sm[i];
     }
-    S.cfg_stage_panel = m->cfg.stage_panel;
+    S.cfg_stage_panel = ss.cfg.stage_panel;
     S.graph_replays = m->gcache.replays;
     S.graph_instantiations = m->gcache.instantiations;
     S.grid_leaves = m->g_leaves;
@@ -1565,6 +1567,7 @@ int vgp_query_smooth(vgp_map* m, const float* q, int64_t n, int32_t n_nodes, dou
     b.status = ps;
     b.want_var = var != nullptr;
     SolveStats ss;
+    ss.cfg = m->cfg;
     b.max_n = P.cap_leaf;
     TRY(solve_status(solve_batch(b, P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0, m->prm.launch,
                                  &m->cfg, &m->gcache),
@@ -1581,10 +1584,10 @@ int vgp_query_smooth(vgp_map* m, const float* q, int64_t n, int32_t n_nodes, dou
     for (int i = 0; i < 5; ++i) {
         S.bucket_count[i] = ss.bucket_count[i];
         S.t_bucket_ms[i] = ss.t_bucket_ms[i];
-        S.cfg_threads[i] = m->cfg.threads[i];
-        S.cfg_per_sm[i] = m->cfg.per_sm[i];
+        S.cfg_threads[i] = ss.cfg.threads[i];
+        S.cfg_per_sm[i] = ss.cfg.per_sm[i];
     }
-    S.cfg_stage_panel = m->cfg.stage_panel;
+    S.cfg_stage_panel = ss.cfg.stage_panel;
     S.graph_replays = m->gcache.replays;
     S.graph_instantiations = m->gcache.instantiations;
     S.sum_n3 = ss.sum_n3;
@@ -1852,6 +1855,7 @@ extern "C" int vgp_gp_batch(vgp_map* m, int64_t n_inst, const int64_t* inst_off,
     b.status = status;
     b.want_var = var != nullptr;
     SolveStats ss;
+    ss.cfg = m->cfg;
     TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0,
                                  m->prm.launch, &m->cfg, &m->gcache),
                      "vgp_gp_batch"));
@@ -1866,10 +1870,10 @@ extern "C" int vgp_gp_batch(vgp_map* m, int64_t n_inst, const int64_t* inst_off,
     S.t_solve_ms = ss.t_solve_ms;
     for (int i = 0; i < 5; ++i) {
         S.t_bucket_ms[i] = ss.t_bucket_ms[i];
-        S.cfg_threads[i] = m->cfg.threads[i];
-        S.cfg_per_sm[i] = m->cfg.per_sm[i];
+        S.cfg_threads[i] = ss.cfg.threads[i];
+        S.cfg_per_sm[i] = ss.cfg.per_sm[i];
     }
-    S.cfg_stage_panel = m->cfg.stage_panel;
+    S.cfg_stage_panel = ss.cfg.stage_panel;
     S.graph_replays = m->gcache.replays;
     S.graph_instantiations = m->gcache.instantiations;
     m->stats = S;

@@ -89,6 +89,7 @@ struct SolveStats {
     double sum_n3 = 0;
     double sum_n2 = 0;
     double t_solve_ms = 0;  // filled when profiling
+    SolveConfig cfg;        // the shapes launched; of buckets without a launch, the configured ones
 };
 
 // Process-wide count of kernel launches (each launch site calls this once).

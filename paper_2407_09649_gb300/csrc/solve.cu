@@ -2436,6 +2436,13 @@ using SolveKernel = void (*)(SolveCtx);
 struct BucketShape {
     int threads, per_sm, stage;
 };
+// Bucket i was launched with this shape (per_sm: the cap on CTAs per SM, 0: none).
+void note_shape(SolveStats* stats, int i, int threads, int per_sm, int stage) {
+    if (!stats) return;
+    stats->cfg.threads[i] = threads;
+    stats->cfg.per_sm[i] = per_sm;
+    if (i == 0) stats->cfg.stage_panel = stage;
+}
 BucketShape bucket_shape(const SolveConfig& cfg, int i, int64_t cnt, int n_sm, bool heavy, int64_t queries) {
     BucketShape b{cfg.threads[i], cfg.per_sm[i], cfg.stage_panel};
     if (cfg.chosen) return b;
@@ -2624,6 +2631,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
             per_sm = std::max(per_sm, 1);
             if (cfg->per_sm[i] > 0) per_sm = std::min(per_sm, cfg->per_sm[i]);
         }
+        note_shape(stats, i, s.threads, s.emu ? 0 : cfg->per_sm[i], s.stage);
         // (without variance and properties splitting rarely pays: no workspace for it)
         s.grid = n_sm * per_sm;
         if (!b.want_var && !props) s.grid = (int)std::min<int64_t>(n, s.grid);
@@ -2736,6 +2744,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     const SolveConfig dflt;
     if (!cfg) cfg = &dflt;
     const int64_t n = b.n_inst;
+    if (stats) stats->cfg = *cfg;
     if (n <= 0) return 0;
     if (launch == VGP_LAUNCH_GRAPH && !bw && gc) {
         const int rc = solve_batch_graph(b, P, err_dev, st, ar, stats, profile, cfg, gc);
@@ -2816,7 +2825,9 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     if (launch == VGP_LAUNCH_PER_INSTANCE && !bw) {
         // the plain comparison form: one launch per instance, in instance order, one CTA each
         // workspaces sized for the largest instance (N <= 1024, at most 512 threads, appended
-        // query rows of the emulated kernel)
+        // query rows of the emulated kernel); the default shapes, whichever were chosen
+        if (stats) stats->cfg = dflt;
+        if (P.emulate) note_shape(stats, 0, kEmuThreads, 0, 0);
         constexpr int kRowsMax = 1024 + kBorderQ;
         int* ctr = (int*)ar.get(Arena::kCounters, sizeof(int) * n, st);
         uint8_t* ws_e = P.emulate ? (uint8_t*)ar.get(Arena::kWs3, kRowsMax * kEmuBytesPerRow, st) : nullptr;
@@ -2910,6 +2921,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             L.per_sm = std::max(L.per_sm, 1);
             if (bs.per_sm > 0) L.per_sm = std::min(L.per_sm, bs.per_sm);
         }
+        note_shape(stats, i, L.threads, L.emu ? 0 : bs.per_sm, L.stage);
         L.ws_a = bk.smem_a ? 0 : matrix_words(L.emu, L.nrow);
         L.ws_v = b.want_var && !bw && !L.emu ? (int64_t)L.npad * L.threads : 0;
         L.ws_e = L.emu ? (int64_t)L.nrow * kEmuBytesPerRow : 0;

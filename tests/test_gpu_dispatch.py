@@ -281,3 +281,30 @@ def test_largest_launch_shapes(vg, threads):
         # (each point's sum of two parts per instance, by atomics in any order: 54 terms at most, which
         # may exceed their sum by 1e4)
         assert (dX - ref_x).abs().max().item() <= 1e-9 * ref_x.abs().max().item()
+
+
+@pytest.mark.parametrize("launch", ["batched", "graph", "per_instance"])
+def test_stats_tell_the_shapes_launched(vg, launch):
+    """Defaults, shapes that follow from the batch, pinned shapes, the emulated kernel's own."""
+    def shapes(m, sizes, nq, var):
+        _solve(m, *_instances(sizes, nq, 63), var)
+        st = m.stats()
+        return st["cfg_threads"], st["cfg_per_sm"], st["cfg_stage_panel"]
+
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    dflt = [512, 512, 256, 128, 64]
+    follow = launch == "batched"  # (only these launches know their counts)
+    m = vg.Map(precision="fp64", launch=launch)
+    assert shapes(m, [300, 40, 8], 4, True) == (dflt, [1, 0, 0, 0, 0], 1)
+    many = [226] * (8 * n_sm + 1)
+    want = ([256] + dflt[1:], [3, 0, 0, 0, 0], 0)
+    assert shapes(m, many, 1, False) == (want if follow else (dflt, [1, 0, 0, 0, 0], 1))
+    want = (dflt[:3] + [256, 64], [1, 0, 0, 0, 0], 1)
+    assert shapes(m, [40], 600, True) == (want if follow else (dflt, [1, 0, 0, 0, 0], 1))
+    if launch == "per_instance":
+        return
+    m.set_launch([384, 1024, 96, 32, 128], [2, 0, 1, 0, 3], 0)
+    assert shapes(m, [300, 200, 100, 40, 8], 4, True) == ([384, 640, 96, 32, 128], [2, 0, 1, 0, 3], 0)
+    e = vg.Map(precision="fp64", launch=launch, emulate_fp64=1)
+    got = shapes(e, [300], 4, True)
+    assert got[0][0] == 256 and got[1][0] == 0 and got[2] == 0
