@@ -2480,15 +2480,55 @@ void chunk_args(const SolveBatch& b, int i, int cnt, int n_sm, int per_sm, int t
     a.qn[i] = !heavy ? 64 : emu ? 1 : 0;
 }
 
+// The emulated kernel's shared memory (about 100 KB at N = 1024) fits twice per SM only in the
+// largest shared-memory configuration; ask for it (a preference, so a failure is harmless).
+template <class Kernel>
+void set_emu_carveout(Kernel k) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared) !=
+        cudaSuccess)
+        cudaGetLastError();
+}
+
+// Stands in for the emulated kernel in resident_clusters.
+__global__ void k_no_tensor_memory() {}
+
+// Clusters of n CTAs that run at once, an emulated CTA's shared memory each: fewer than the SMs' CTAs over n,
+// for a cluster stays within a part of the GPU (38 would fill 152 SMs at n = 8, 36 run; 74 of 76 at
+// n = 4).  0 where no such cluster can run.  The calculator counts one CTA per SM for a kernel with tensor
+// memory (see emu_ctas_per_sm), so it is asked about one without; shared memory allows two of
+// either.
+int resident_clusters(int n, int threads, size_t shm) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = n;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(n);
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = shm;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    int clusters = 0;
+    set_emu_carveout(k_no_tensor_memory);
+    if (cudaFuncSetAttribute(k_no_tensor_memory, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_no_tensor_memory, &lc) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return clusters;
+}
+
 // CTAs that work on an instance together (a cluster) in an emulated launch of at most `items` work
 // items, nmax points at most, on `slots` resident CTAs: as many as keep every item resident, up to 8.
 // K, the rows below and the trailing tiles are shared out, the diagonal blocks and the solves
 // are not, and a block of 32 columns costs three cluster barriers; below 128 points nothing
-// is left to share.
-int group_ctas(int items, int nmax, int slots) {
-    int n = 1;
-    while (n < 8 && nmax > 128 && (int64_t)items * 2 * n <= slots) n *= 2;
-    return n;
+// is left to share.  Items that wait for a cluster to end cost more than the larger one gains: 38
+// instances of 130 points take 0.61 ms by eights, 0.41 ms by fours and 0.47 ms by one CTA each.
+int group_ctas(int items, int nmax, int slots, int threads, size_t shm) {
+    if (nmax <= 128) return 1;
+    for (int n = 8; n > 1; n /= 2)
+        if ((int64_t)items * n <= slots && resident_clusters(n, threads, shm) >= items) return n;
+    return 1;
 }
 
 // Emulated launch with the latent variance: the queries of an instance (up to kBorderQ) are
@@ -2499,14 +2539,6 @@ void emu_rows_for(bool emu, const SolveBatch& b, int& npad, int& qmax, int& nrow
     if (emu) npad = (npad + 31) & ~31;
     if (emu && b.want_var) qmax = kBorderQ;
     nrow = npad + qmax;
-}
-
-// The emulated kernel's shared memory (about 100 KB at N = 1024) fits twice per SM only in the
-// largest shared-memory configuration; ask for it (a preference, so a failure is harmless).
-void set_emu_carveout(SolveKernel k) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared) !=
-        cudaSuccess)
-        cudaGetLastError();
 }
 
 // Resident CTAs per SM of the emulated kernel.  The occupancy calculator reports one CTA per SM
@@ -2959,7 +2991,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             }
         }
         // few emulated work items: clusters of CTAs work on each
-        L.ncta = L.emu ? group_ctas(items, L.nmax, n_sm * L.per_sm) : 1;
+        L.ncta = L.emu ? group_ctas(items, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
         L.groups = (int)std::min<int64_t>(items, (int64_t)n_sm * L.per_sm / L.ncta);
         if (i == 4) beside = !bw && !profile && L.cnt < n && gc && graph_cache_ready(*gc);
         need_a = std::max(need_a, L.ws_a * L.groups);

@@ -308,3 +308,30 @@ def test_stats_tell_the_shapes_launched(vg, launch):
     e = vg.Map(precision="fp64", launch=launch, emulate_fp64=1)
     got = shapes(e, [300], 4, True)
     assert got[0][0] == 256 and got[1][0] == 0 and got[2] == 0
+
+
+@pytest.mark.parametrize("per_sm", [4, 2])
+def test_clusters_all_run_at_once(vg, per_sm):
+    """As many instances as clusters of eight (four) would fill the GPU's CTAs with: not all of those
+    clusters run at once, and a second round must not make the call slower than one more instance does,
+    with smaller clusters (1.5 times as slow, had it one)."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count // per_sm
+    m = vg.Map(precision="mixed", emulate_fp64=1)
+
+    def best(count):
+        X, Q = _instances([130] * count, 5, 64)
+        io = torch.arange(count + 1, dtype=torch.int64, device="cuda") * 130
+        qo = torch.arange(count + 1, dtype=torch.int64, device="cuda") * 5
+        x, q = (torch.from_numpy(np.vstack(a)).cuda() for a in (X, Q))
+        ms = []
+        for _ in range(40):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            m.gp_batch(io, x, qo, q, var=False)
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    full = best(n)
+    assert full <= 1.2 * best(n + 1)
