@@ -1673,7 +1673,7 @@ int vgp_autotune(vgp_map* m, const float* q, int64_t n, vgp_stream stream) {
             cfg.per_sm[i] = cand_p[c][i];
         }
         cfg.stage_panel = cand_s[c];
-        cfg.chosen = true;
+        std::fill(cfg.chosen, cfg.chosen + 5, true);
         // each candidate twice, the faster run counts
         SolveStats s1, s2;
         TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &s1, nullptr, true, 0, &cfg), "vgp_autotune"));
@@ -1682,14 +1682,15 @@ int vgp_autotune(vgp_map* m, const float* q, int64_t n, vgp_stream stream) {
         SolveStats ss = s1;
         for (int i = 0; i < 5; ++i) ss.t_bucket_ms[i] = std::min(s1.t_bucket_ms[i], s2.t_bucket_ms[i]);
         for (int i = 0; i < 5; ++i)
-            if (ss.bucket_count[i] > 0 && ss.t_bucket_ms[i] < best[i]) {
+            if (ss.t_bucket_ms[i] > 0 && ss.t_bucket_ms[i] < best[i]) {  // (no time: no launch)
                 best[i] = ss.t_bucket_ms[i];
+                if (m->P.emulate && i < 4) continue;  // the emulated kernel has one shape
                 chosen.threads[i] = cfg.threads[i];
                 chosen.per_sm[i] = cfg.per_sm[i];
+                chosen.chosen[i] = true;
                 if (i == 0) chosen.stage_panel = cfg.stage_panel;
             }
     }
-    chosen.chosen = true;
     m->cfg = chosen;
     for (int i = 0; i < 5; ++i) {
         m->stats.cfg_threads[i] = chosen.threads[i];
@@ -1713,7 +1714,7 @@ int vgp_set_launch(vgp_map* m, const int32_t* threads, const int32_t* per_sm, in
         m->cfg.per_sm[i] = per_sm[i];
     }
     m->cfg.stage_panel = stage_panel;
-    m->cfg.chosen = true;
+    std::fill(m->cfg.chosen, m->cfg.chosen + 5, true);
     return VGP_OK;
 }
 

@@ -79,8 +79,9 @@ struct SolveConfig {
     // read it from the global tile-packed matrix through L1/L2 (0), which leaves room for two
     // CTAs per SM
     int stage_panel = 1;
-    bool chosen = false;  // by vgp_autotune or vgp_set_launch; else two buckets' shapes go by their
-                          // numbers of instances and queries (see bucket_shape)
+    // by vgp_autotune or vgp_set_launch; else two buckets' shapes go by their numbers of instances and
+    // queries (see bucket_shape)
+    bool chosen[5] = {false, false, false, false, false};
 };
 
 struct SolveStats {

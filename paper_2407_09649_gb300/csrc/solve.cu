@@ -2445,7 +2445,7 @@ void note_shape(SolveStats* stats, int i, int threads, int per_sm, int stage) {
 }
 BucketShape bucket_shape(const SolveConfig& cfg, int i, int64_t cnt, int n_sm, bool heavy, int64_t queries) {
     BucketShape b{cfg.threads[i], cfg.per_sm[i], cfg.stage_panel};
-    if (cfg.chosen) return b;
+    if (cfg.chosen[i]) return b;
     if (i == 0 && cnt > 8 * n_sm) b = {256, 3, 0};
     if (i == 3 && heavy && cnt <= 2 * n_sm && queries >= 512 * cnt) b.threads = 256;
     return b;

@@ -335,3 +335,26 @@ def test_clusters_all_run_at_once(vg, per_sm):
 
     full = best(n)
     assert full <= 1.2 * best(n + 1)
+
+
+def test_autotuner_chooses_for_the_buckets_it_timed(vg):
+    """Neighbourhoods above 224 points only: that bucket is timed and chosen, the others keep the rules
+    that follow the batch, and an emulated map, whose kernel has one shape there, keeps the defaults."""
+    rng = np.random.default_rng(65)
+    surf = torch.from_numpy((rng.uniform(-1, 1, (40000, 3)) * [2, 2, 0.2]).astype(np.float32)).cuda()
+    q = (torch.from_numpy((rng.uniform(-1, 1, (2000, 3)) * [1.5, 1.5, 0.2]).astype(np.float32))).cuda()
+    dflt = [512, 512, 256, 128, 64]
+    for emulate in (0, 1):
+        m = vg.Map(precision="mixed", emulate_fp64=emulate)
+        m.set_surface(surf)
+        m.query(q)
+        assert m.stats()["bucket_count"][:3] == [0, 0, 0]
+        cfg = m.autotune(q)
+        assert cfg["bucket_ms"][0] > 0 and cfg["bucket_ms"][1:] == [0, 0, 0, 0]
+        assert cfg["threads"][1:] == dflt[1:] and (not emulate or cfg["threads"][0] == dflt[0])
+        if not emulate:
+            _solve(m, *_instances([40], 600, 65), True)
+            assert m.stats()["cfg_threads"][3] == 256
+            assert (m.stats()["cfg_threads"][0], m.stats()["cfg_stage_panel"]) == (cfg["threads"][0], cfg["stage_panel"])
+            _solve(m, *_instances([226] * 1300, 1, 65), False)
+            assert m.stats()["cfg_threads"][0] == cfg["threads"][0]
