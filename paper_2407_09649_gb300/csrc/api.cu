@@ -587,6 +587,7 @@ int vgp_build_frame_props(vgp_map* m, const float* pts, const float* props, int6
     SolveStats ss;
     ss.cfg = m->cfg;
     b.max_n = P.cap_leaf;
+    b.max_pos = f->ntest;
     if (solve_batch(b, P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0, m->prm.launch, &m->cfg,
                     &m->gcache) == -2)
         return bail(VGP_ERR_OOM, "device allocation of a solve workspace failed");
@@ -1495,6 +1496,7 @@ int vgp_query_distance_gradient(vgp_map* m, const float* q, int64_t n, double* d
     SolveStats ss;
     ss.cfg = m->cfg;
     b.max_n = m->P.cap_group;
+    b.max_pos = n;
     TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0,
                                  m->prm.launch, &m->cfg, &m->gcache),
                      "query"));
@@ -1569,6 +1571,7 @@ int vgp_query_smooth(vgp_map* m, const float* q, int64_t n, int32_t n_nodes, dou
     SolveStats ss;
     ss.cfg = m->cfg;
     b.max_n = P.cap_leaf;
+    b.max_pos = np;
     TRY(solve_status(solve_batch(b, P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0, m->prm.launch,
                                  &m->cfg, &m->gcache),
                      "vgp_query_smooth"));
@@ -1857,6 +1860,7 @@ extern "C" int vgp_gp_batch(vgp_map* m, int64_t n_inst, const int64_t* inst_off,
     b.want_var = var != nullptr;
     SolveStats ss;
     ss.cfg = m->cfg;
+    b.max_pos = NQ;
     TRY(solve_status(solve_batch(b, m->P, m->dev_words, st, m->ar, &ss, nullptr, m->prm.profile != 0,
                                  m->prm.launch, &m->cfg, &m->gcache),
                      "vgp_gp_batch"));

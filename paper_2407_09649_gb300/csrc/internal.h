@@ -53,7 +53,8 @@ struct SolveBatch {
     // surface-property mode (Eq. 6): nprop > 0 replaces the right-hand side 1 by the nprop
     // columns of yprop and writes property means / variances instead of distances
     int nprop = 0;
-    int max_n = 1024;                   // largest N the batch can hold (sizes graph-mode buffers)
+    int max_n = 1024;                   // largest N the batch can hold, and
+    int64_t max_pos = INT64_MAX / 2;    // most positions in the list (they size graph-mode buffers)
     const double* yprop = nullptr;      // [T][nprop]
     double* pc = nullptr;               // [n_queries][nprop] by query id
     double* pw = nullptr;               // [n_queries] by query id

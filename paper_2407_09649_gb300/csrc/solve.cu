@@ -2664,10 +2664,13 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
             if (cfg->per_sm[i] > 0) per_sm = std::min(per_sm, cfg->per_sm[i]);
         }
         note_shape(stats, i, s.threads, s.emu ? 0 : cfg->per_sm[i], s.stage);
-        // (without variance and properties splitting rarely pays: no workspace for it)
-        s.grid = n_sm * per_sm;
-        if (!b.want_var && !props) s.grid = (int)std::min<int64_t>(n, s.grid);
+        // no more CTAs, and workspaces, than the batch can have work items in this bucket: its instances
+        // and every shortest chunk (without variance and properties splitting rarely pays: no
+        // workspace for it)
         chunk_args(b, i, 0, n_sm, per_sm, s.threads, s.emu, ca);
+        const int64_t len = chunk_len(ca.qmin[i], ca.qn[i], std::max(lo[i], 1), ca.cap[i]);
+        const int64_t items = n + (b.want_var || props ? b.max_pos / len : 0);
+        s.grid = (int)std::min<int64_t>(items, (int64_t)n_sm * per_sm);
         ca.slots[i] = std::min(ca.slots[i], s.grid);
         if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
         if (b.want_var && !s.emu) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);

@@ -358,3 +358,22 @@ def test_autotuner_chooses_for_the_buckets_it_timed(vg):
             assert (m.stats()["cfg_threads"][0], m.stats()["cfg_stage_panel"]) == (cfg["threads"][0], cfg["stage_panel"])
             _solve(m, *_instances([226] * 1300, 1, 65), False)
             assert m.stats()["cfg_threads"][0] == cfg["threads"][0]
+
+
+def test_graph_workspaces_follow_the_batch(vg):
+    """Graph launches size their CTAs and workspaces before the counts are known, but not beyond the
+    batch: three instances with variance took 5 GB; later calls of more give the direct launches' bits."""
+    m = vg.Map(precision="mixed", emulate_fp64=1, launch="graph")
+    direct = vg.Map(precision="mixed", emulate_fp64=1)
+    sizes, nq = [300, 40, 8], 5
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(2):
+        X, Q = _instances(sizes, nq, 66)
+        out = _solve(m, X, Q, True)
+        torch.cuda.synchronize()
+        if nq == 5:  # a CTA's rows are 1024 and the variance's 1024: 17 MB, and 8 of them at most
+            assert free - torch.cuda.mem_get_info()[0] < 1 << 29
+        for a, b in zip(out, _solve(direct, X, Q, True)):
+            _same(a, b)
+        sizes, nq = [33, 65, 129, 225, 300, 1024] * 20, 700
