@@ -12,6 +12,7 @@
 // 66 for an FMA, so every chain beside it waits.  Emulated kernel: see factor_emulated.
 #include <algorithm>
 #include <cstdio>
+#include <cstring>
 #include <vector>
 
 #include "internal.h"
@@ -2202,26 +2203,21 @@ __global__ void k_backward(SolveCtx c) {
     }
 }
 
-__global__ void k_hist_n(const int64_t* inst_off, int64_t n, int* hist) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int N = (int)(inst_off[i + 1] - inst_off[i]);
-    atomicAdd(&hist[min(N, 1024)], 1);
-}
-
-// Queries of each size bucket (N > 224, > 128, > 64, > 32, the rest), for the chunk planning.
-__global__ void k_bucket_queries(const int64_t* inst_off, const int64_t* q_off, int64_t n, unsigned long long* qsum) {
+// Instances of each size, and with qsum the queries of each size bucket (N > 224, > 128, > 64, > 32, the
+// rest) for the chunk planning.
+__global__ void k_hist_n(const int64_t* inst_off, const int64_t* q_off, int64_t n, int* hist, unsigned long long* qsum) {
     __shared__ unsigned long long sum[5];
     if (threadIdx.x < 5) sum[threadIdx.x] = 0;
     __syncthreads();
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) {
-        const int64_t N = inst_off[i + 1] - inst_off[i];
+        const int N = (int)(inst_off[i + 1] - inst_off[i]);
+        atomicAdd(&hist[min(N, 1024)], 1);
         const int bk = N > 224 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
-        atomicAdd(&sum[bk], (unsigned long long)(q_off[i + 1] - q_off[i]));
+        if (qsum) atomicAdd(&sum[bk], (unsigned long long)(q_off[i + 1] - q_off[i]));
     }
     __syncthreads();
-    if (threadIdx.x < 5 && sum[threadIdx.x]) atomicAdd(&qsum[threadIdx.x], sum[threadIdx.x]);
+    if (qsum && threadIdx.x < 5 && sum[threadIdx.x]) atomicAdd(&qsum[threadIdx.x], sum[threadIdx.x]);
 }
 
 // order[] sorted by increasing N via the prefix of the histogram
@@ -2695,7 +2691,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
     if (cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return -1;
     fill_i32(hist, 0, 1025, gs);
     fill_i32(counters, 0, 5, gs);
-    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, gs>>>(b.inst_off, n, hist);
+    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, gs>>>(b.inst_off, b.q_off, n, hist, nullptr);
     note_launch();
     k_plan_buckets<<<1, 32, 0, gs>>>(hist, cursor, plan);
     note_launch();
@@ -2801,24 +2797,20 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     // size histogram (and, for chunk planning, each bucket's queries) and decreasing-size order
     const bool heavy = !bw && (b.want_var || b.nprop > 0);
     ChunkPlanArgs ca{};
-    int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * 2 * 1025 + sizeof(unsigned long long) * 5, st);
+    constexpr int kHistWords = 1026 + 2 * 5;  // sizes (and a word of padding), the buckets' queries in 64 bits
+    int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * (kHistWords + 1025), st);
     if (!hist) return alloc_failed(err_dev, st);
-    int* cursor = hist + 1025;
-    unsigned long long* qsum = reinterpret_cast<unsigned long long*>(hist + 2 * 1025);
-    cudaMemsetAsync(hist, 0, sizeof(int) * 1025, st);
+    int* cursor = hist + kHistWords;
+    cudaMemsetAsync(hist, 0, sizeof(int) * kHistWords, st);
     const int T = 256;
-    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, n, hist);
+    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, b.q_off, n, hist,
+                                                        bw ? nullptr : reinterpret_cast<unsigned long long*>(hist + 1026));
     note_launch();
-    unsigned long long hq[5] = {0, 0, 0, 0, 0};
-    if (!bw) {
-        cudaMemsetAsync(qsum, 0, sizeof(hq), st);
-        k_bucket_queries<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, b.q_off, n, qsum);
-        note_launch();
-    }
-    std::vector<int> h(1025);
-    cudaMemcpyAsync(h.data(), hist, sizeof(int) * 1025, cudaMemcpyDeviceToHost, st);
-    if (!bw) cudaMemcpyAsync(hq, qsum, sizeof(hq), cudaMemcpyDeviceToHost, st);
+    std::vector<int> h(kHistWords);
+    cudaMemcpyAsync(h.data(), hist, sizeof(int) * kHistWords, cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
+    unsigned long long hq[5];
+    std::memcpy(hq, h.data() + 1026, sizeof(hq));
     std::vector<int> start(1026, 0);
     for (int i = 0; i < 1025; ++i) start[i + 1] = start[i] + h[i];
     cudaMemcpyAsync(cursor, start.data(), sizeof(int) * 1025, cudaMemcpyHostToDevice, st);

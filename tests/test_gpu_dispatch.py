@@ -377,3 +377,17 @@ def test_graph_workspaces_follow_the_batch(vg):
         for a, b in zip(out, _solve(direct, X, Q, True)):
             _same(a, b)
         sizes, nq = [33, 65, 129, 225, 300, 1024] * 20, 700
+
+
+@pytest.mark.parametrize("emulate,sizes", [(0, [8]), (1, [8]), (0, [300, 40, 8])])
+def test_kernels_of_a_small_call(vg, emulate, sizes):
+    """A mean-only call of a few small instances plans no work items, so it is four kernels (points and
+    centres, sizes, two for the order) and a launch for each bucket."""
+    from paper_2407_09649_gb300 import _lib
+    lib = _lib.load()
+    m = vg.Map(precision="mixed", emulate_fp64=emulate)
+    X, Q = _instances(sizes, 8, 67)
+    _solve(m, X, Q, False)
+    n0 = lib.vgp_launch_count()
+    _solve(m, X, Q, False)
+    assert lib.vgp_launch_count() - n0 == 4 + len(sizes)
