@@ -147,8 +147,8 @@ constexpr int kEmuCtasPerSm = 512 / kEmuTmemCols;  // CTAs whose tensor memory f
 
 __host__ __device__ __forceinline__ size_t align128(size_t x) { return (x + 127) & ~(size_t)127; }
 __host__ __device__ __forceinline__ size_t emu_fixed_bytes(int npad) {
-    // invd, T256, Tblk, Tff, Dblk, dtab
-    return align128((size_t)(npad + 256 + kEB * 64 + 256 + kDiagTiles * 64 + 32) * sizeof(double));
+    // invd, Tblk, Tff, Dblk, dtab
+    return align128((size_t)(npad + kEB * 64 + 256 + kDiagTiles * 64 + 32) * sizeof(double));
 }
 __host__ __device__ __forceinline__ size_t emu_point_bytes(int npad, int nprop, bool lattice) {
     return (size_t)5 * npad * sizeof(double) + (size_t)5 * npad * sizeof(float) +
@@ -161,14 +161,14 @@ __host__ __device__ __forceinline__ size_t emu_alias_bytes(int npad, int nprop, 
     return b > (size_t)kStageBytes ? b : (size_t)kStageBytes;
 }
 
-// Emulated kernel: invd, the exp tables and the diagonal block first, then (128-byte aligned) the
+// Emulated kernel: invd, the exp table and the diagonal block first, then (128-byte aligned) the
 // staging buffer of the tensor-core updates, which X, alpha, z, Xf, alf, alf_lo, xi and the property
 // weights alias, and so does the warps' scratch of the rows below (kEB tiles each).
 __device__ Shared carve_emu(double* sm, int npad, double* ws_a, int nprop, bool lattice) {
     Shared s;
     s.invd = sm;
-    s.T256 = s.invd + npad;
-    s.Tblk = s.T256 + 256;
+    s.Tblk = s.invd + npad;
+    s.T256 = nullptr;  // (mixed values come from Tff, FP64 ones from exp)
     s.Tinv = nullptr;
     s.w = nullptr;
     s.panel = nullptr;
@@ -259,11 +259,14 @@ __device__ __forceinline__ int lat_m(int a, int b) {
 }
 
 // SE kernel value of a pair of training points (Sec. III-A), FP64: from the exact lattice
-// table for voxel-centre instances, else exp_neg (mixed) or the library exp (plain).
+// table for voxel-centre instances, else exp_neg (mixed) or the library exp (plain) of kval_arg.
+__device__ __forceinline__ double kval_arg(const DevParams& P, const Shared& s, int i, int j) {
+    double dx = s.X[3 * i] - s.X[3 * j], dy = s.X[3 * i + 1] - s.X[3 * j + 1], dz = s.X[3 * i + 2] - s.X[3 * j + 2];
+    return -(dx * dx + dy * dy + dz * dz) * P.inv2l2;
+}
 __device__ __forceinline__ double kval_pair(const DevParams& P, const Shared& s, bool lattice, int i, int j) {
     if (lattice) return P.lat_tab[lat_m(s.xi[i], s.xi[j])];
-    double dx = s.X[3 * i] - s.X[3 * j], dy = s.X[3 * i + 1] - s.X[3 * j + 1], dz = s.X[3 * i + 2] - s.X[3 * j + 2];
-    const double y = -(dx * dx + dy * dy + dz * dz) * P.inv2l2;
+    const double y = kval_arg(P, s, i, j);
     return P.precision == VGP_MIXED ? exp_neg(y, s.T256) : exp(y);
 }
 
@@ -724,6 +727,7 @@ __device__ __forceinline__ long long fix_shift(long long w, int sh) {
 // pairs of groups joined in 32 bits first (|256 G + G'| < 2^31), so the 64-bit part is one wide
 // multiply-add and one addition to the high word.
 constexpr unsigned kGroupBits = 0x4B400000u;
+static_assert(7 * 8 * kEB * 128 * 128 < 1 << 22, "a slice group of a block's columns exceeds 22 bits");
 __device__ __forceinline__ long long join_groups(const unsigned (&g)[8]) {
     constexpr unsigned kOff = kGroupBits * 257u;
     const unsigned a = g[0] * 256u + g[1] - kOff;
@@ -1209,15 +1213,15 @@ __device__ bool trailing_update_tc(double* A, int Nt, int Ntr, int K1, const uns
 // from the bits of its FP64 values aligned to the row's largest biased exponent e_r (rounded
 // to nearest at 2^-55 of the row maximum): a 55-bit integer per value, cut into seven
 // balanced base-256 digits (the lower six in [-128, 127], the top one in [0, 128]), each
-// exact in bf16.  A slice product Q_s Q_t^T sums W <= 64 products of at most 2^14, so every
-// group G_g = sum_{s+t=g} Q_s Q_t^T with g <= 9 (at most 7 terms) is an integer below 2^23
+// exact in bf16.  A slice product Q_s Q_t^T sums W = 32 products of at most 2^14, so every
+// group G_g = sum_{s+t=g} Q_s Q_t^T with g <= 9 (at most 7 terms) is an integer below 2^22
 // and accumulates exactly in FP32; groups g >= 10 are below 2^-64 relative and dropped.  The
 // FP64 update is
 //     C_rc -= 2^(e_r + e_c - 2042) sum_g 2^(-8 g) G_g,rc.
-// The groups are packed exactly into two 64-bit integers, hi (g = 2..5) and lo (g = 6..9),
-// and joined as w = 2^16 hi + round(lo / 2^16), below 2^63 because every group stays below
-// 2^22 with W = 32: the rounding of lo is below 2^-57 of the scale 2^(e_r + e_c - 2042).  The
-// trailing matrix is held in the fixed point of kFixBits (assembled so by fit_instance): w is
+// The eight groups are joined into one 64-bit integer w (join_groups, where they are counted from 0),
+// pairs of them in 32 bits first; the lower four are rounded, by less than 2^-57 of the scale
+// 2^(e_r + e_c - 2042).  The trailing matrix is held in the fixed point of kFixBits (assembled so
+// by fit_instance): w is
 // shifted to it and subtracted as an integer, so an updated entry costs no FP64 operation,
 // and each block's columns are stored as FP64 by the update that completes them (the first block's
 // by the assembly).  The slice products run on the tensor cores
@@ -1461,7 +1465,7 @@ __device__ bool fit_instance(const SolveCtx& c, const Shared& s, int N, int64_t 
                     v[e] = fix_of_double(exp(-r2 * c.P.inv2l2));
                 }
             } else {
-                for (int e = 0; e < 8; ++e) v[e] = j0 + e < i ? fix_of_double(kval_pair(c.P, s, false, i, j0 + e)) : 0;
+                for (int e = 0; e < 8; ++e) v[e] = j0 + e < i ? fix_of_double(exp(kval_arg(c.P, s, i, j0 + e))) : 0;
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1890,13 +1894,15 @@ __device__ __forceinline__ void solve_body(const SolveCtx& c) {
     Shared s = carve(sm, c.npad, c.a_in_smem, ws_a, c.b.nprop, c.stage_panel, c.b.Xi != nullptr, false, kEmu);
     double* V = c.ws_v ? c.ws_v + (int64_t)blockIdx.x * c.ws_v_stride + tid : nullptr;
     const bool lattice = c.b.Xi != nullptr;
-    for (int j = tid; j < 256; j += nt) s.T256[j] = c.P.exp_tab[j];
-    if (kEmu)
-        for (int j = tid; j < 256; j += nt) {
+    for (int j = tid; j < 256; j += nt) {
+        if constexpr (kEmu) {
             float h, l;
             split_pair(c.P.exp_tab[j], h, l);
             s.Tff[j] = make_float2(h, l);
+        } else {
+            s.T256[j] = c.P.exp_tab[j];
         }
+    }
     for (int j = tid; j < 256; j += nt) s.dtab[j] = diag_entry(j >> 5, j & 31);
     EmuTc<kGroup> tc{};
     tc.n_ = ncta;
