@@ -106,7 +106,9 @@ enum {
  *                    cannot underflow); Cholesky, triangular solves, variance and the
  *                    reverting log in FP64.
  *   profile          0 (default) or 1: record CUDA events around the GP solve kernels and
- *                    report their time in vgp_stats.t_solve_ms (adds one stream sync per call).
+ *                    report their time in vgp_stats.t_solve_ms (adds one stream sync per call;
+ *                    the size buckets then run one after the other, where the smallest otherwise
+ *                    runs beside the rest).
  *   normal_steps     K in [0, 16] (default 3): with a sensor origin, vgp_build_frame also tests
  *                    the voxels round(s + k n), k = +-1..+-K, along each surface voxel's normal.
  *   emulate_fp64     1: instances with N > 32 are factorised in blocks of
@@ -117,16 +119,19 @@ enum {
  *                    integer and added to the not yet factorised matrix, held as 64-bit
  *                    integers round(v 2^61) (error of the order of the FP64 rounding of the
  *                    update).  In mixed precision their K entries are float-pair values (error
- *                    below 2^-45 k (1 + r^2 / 2l^2)), and off-lattice distance instances take
- *                    the latent variance from the Schur complement of the matrix with up to
+ *                    below 2^-45 k (1 + r^2 / 2l^2)).  The variance is read from the Schur
+ *                    complement of the matrix with up to
  *                    1024 query rows appended.  Same results up to rounding; 0 keeps every
  *                    update on the FP64 pipe.  Uses a per-CTA workspace of about 0.5 KB per
  *                    matrix row and 8 bytes per lower-triangle entry.  Few instances are worked
  *                    on by clusters of up to 8 CTAs each, with the same bits as by one.
+ *                    VGP_LAUNCH_PER_INSTANCE factorises instances of at most 224 points on the
+ *                    FP64 pipe all the same.
  *   launch           VGP_LAUNCH_BATCHED (default): all GP instances of a call run in a few
  *                    persistent launches, one per size bucket, largest first.
  *                    VGP_LAUNCH_PER_INSTANCE: one kernel launch per instance, in instance
- *                    order (the plain comparison form; same arithmetic, no batching).
+ *                    order (the plain comparison form; same arithmetic but for emulate_fp64, see
+ *                    there, and no batching).
  *                    VGP_LAUNCH_GRAPH: the batched form with the size histogram, bucket
  *                    plan and ordering computed on the device, so that the whole solve of a
  *                    call (plan and bucket launches) is captured as a CUDA graph on a stream the map
