@@ -544,6 +544,9 @@ int vgp_get_stats(const vgp_map* m, vgp_stats* out);
  */
 int vgp_debug_exp_neg(const vgp_map* m, const double* y_dev, double* out_dev, int64_t n, vgp_stream stream);
 
+/* The same of the exponential of Eq. 10's weights and of the backward pass (below 0.85 ulp). */
+int vgp_debug_exp_near(const vgp_map* m, const double* y_dev, double* out_dev, int64_t n, vgp_stream stream);
+
 /*
  * Diagnostic: out_dev[i] = round(k 2^61), k = exp(-|a_i - b_i|^2 / (2 l^2)), as the emulated
  * factorisation (emulate_fp64 = 1) assembles its mixed-precision kernel matrix (Sec. III-A

@@ -1800,16 +1800,25 @@ __global__ void k_batch_prep(const int64_t* inst_off, int64_t n_inst, const floa
 }  // namespace
 
 namespace {
-__global__ void k_exp_probe(const double* y, double* out, int64_t n, const double* tab) {
+__global__ void k_exp_probe(const double* y, double* out, int64_t n, const double* tab, const double* lo) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = exp_neg(y[i], tab);
+    if (i < n) out[i] = lo ? exp_near(y[i], tab, lo) : exp_neg(y[i], tab);
 }
 }  // namespace
 
 extern "C" int vgp_debug_exp_neg(const vgp_map* m, const double* y, double* out, int64_t n, vgp_stream stream) {
     if (!m || n < 0 || (n > 0 && (!y || !out))) return fail(VGP_ERR_ARG, "vgp_debug_exp_neg: bad argument");
     if (n == 0) return VGP_OK;
-    k_exp_probe<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(y, out, n, m->P.exp_tab);
+    k_exp_probe<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(y, out, n, m->P.exp_tab, nullptr);
+    note_launch();
+    CUDA_TRY(cudaGetLastError());
+    return VGP_OK;
+}
+
+extern "C" int vgp_debug_exp_near(const vgp_map* m, const double* y, double* out, int64_t n, vgp_stream stream) {
+    if (!m || n < 0 || (n > 0 && (!y || !out))) return fail(VGP_ERR_ARG, "vgp_debug_exp_near: bad argument");
+    if (n == 0) return VGP_OK;
+    k_exp_probe<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(y, out, n, m->P.exp_tab, m->P.exp_lo);
     note_launch();
     CUDA_TRY(cudaGetLastError());
     return VGP_OK;

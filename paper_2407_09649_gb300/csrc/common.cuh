@@ -73,8 +73,9 @@ __device__ __forceinline__ double exp_neg(double y, const double* tab) {
 }
 
 // e^y for y <= 0 in FP64, the same reduction with 2^(j/256) as a pair of doubles: the polynomial's part is
-// added to it last, so the error stays below 0.7 ulp (half an ulp of the final sum, 0.17 of the
-// polynomial's remainder), under the library exp's 1 ulp, in 10 FP64 operations against its 17.
+// added to it last, so the error stays below 0.85 ulp (half an ulp of the final sum, up to 0.342 of the
+// polynomial's remainder, the reduction's rest), in 10 FP64 operations against the library exp's 17.
+// Over 4M values in [-700, 0] it is 0.832 at most and 0.256 on average, the library's 0.863 and 0.258.
 // For the blend's weights and the backward pass (the forward kernel values keep the library's: a last
 // bit there moves FP64 results by the factorisation's condition number).  tab, lo: exp_tab and
 // exp_lo.  Below -700 the library's.

@@ -1,0 +1,49 @@
+"""Device arithmetic at the edges of its range: the paired exponential, both halves of the packed
+float-pair kernel values, the sign test of zero crossings."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def vg():
+    import paper_2407_09649_gb300 as P
+    P.build()
+    return P
+
+
+def _ptr(t):
+    return C.c_void_p(t.data_ptr())
+
+
+def _stream():
+    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+
+def test_paired_exp_below_its_bound(vg):
+    """The exponential of Eq. 10's weights and of the backward pass: below 0.85 ulp (half an ulp of the
+    last sum, r^5 / 120 <= 0.342 ulp for |r| <= ln2 / 512, the reduction's 0.006), the library's
+    values below -700."""
+    from paper_2407_09649_gb300 import _lib
+    m = vg.Map()
+    rng = np.random.default_rng(70)
+    mid = -(np.arange(1, 5000) + 0.5) * np.log(2) / 256  # |r| at its largest
+    y = np.concatenate([-rng.uniform(0, 40, 1000000), -rng.uniform(0, 700, 300000), mid, np.nextafter(mid, 0),
+                        [-0.0, 0.0, -5e-324, -1e-300, -1e-17, -699.999, -700.0]])
+    yt = torch.from_numpy(y).cuda()
+    out = torch.empty_like(yt)
+    _lib.check(_lib.load().vgp_debug_exp_near(m._h, _ptr(yt), _ptr(out), len(y), _stream()))
+    got = out.cpu().numpy()
+    ref = np.exp(y.astype(np.longdouble))
+    err = np.abs(got.astype(np.longdouble) - ref) / np.spacing(ref.astype(np.float64))
+    assert float(err.max()) <= 0.85
+    assert np.all(got[y == 0.0] == 1.0)
+    far = torch.tensor([-np.nextafter(700.0, 800.0), -740.0, -800.0, -np.inf, np.nan], device="cuda", dtype=torch.float64)
+    out = torch.empty_like(far)
+    _lib.check(_lib.load().vgp_debug_exp_near(m._h, _ptr(far), _ptr(out), len(far), _stream()))
+    assert torch.equal(out[:4], torch.exp(far[:4])) and torch.isnan(out[4])
