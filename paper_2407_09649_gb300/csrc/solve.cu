@@ -3117,8 +3117,8 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
 }
 
 namespace {
-// One pair of FP32 world coordinates per thread: the emulated kernel's mixed-precision kernel
-// value in the fixed point.
+// Two pairs of FP32 world coordinates per thread, one in each half of the packed operations (even pairs
+// in the lower): the emulated kernel's mixed-precision kernel values in the fixed point.
 __global__ void k_kfix_probe(const float* xa, const float* xb, long long* out, int64_t n, DevParams P) {
     __shared__ float2 tab[256];
     for (int j = threadIdx.x; j < 256; j += blockDim.x) {
@@ -3127,19 +3127,26 @@ __global__ void k_kfix_probe(const float* xa, const float* xb, long long* out, i
         tab[j] = make_float2(h, l);
     }
     __syncthreads();
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i1 = i + 1 < n ? i + 1 : i;
     if (i >= n) return;
-    const F2 a[3] = {pair2(xa[3 * i]), pair2(xa[3 * i + 1]), pair2(xa[3 * i + 2])};
-    const float b[6] = {xb[3 * i], xb[3 * i + 1], xb[3 * i + 2], xb[3 * i], xb[3 * i + 1], xb[3 * i + 2]};
-    long long k1;
-    kfix_ff2(a, b, pair2(P.inv2l2_hi), pair2(P.inv2l2_lo), tab, out[i], k1);
+    F2 a[3];
+    float b[6];
+    for (int k = 0; k < 3; ++k) {
+        a[k] = pair2(xa[3 * i + k], xa[3 * i1 + k]);
+        b[k] = xb[3 * i + k];
+        b[3 + k] = xb[3 * i1 + k];
+    }
+    long long k0, k1;
+    kfix_ff2(a, b, pair2(P.inv2l2_hi), pair2(P.inv2l2_lo), tab, k0, k1);
+    out[i] = k0;
+    if (i1 > i) out[i1] = k1;
 }
 }  // namespace
 
 int debug_kernel_fix(const DevParams& P, const float* xa, const float* xb, int64_t n, long long* out,
                      cudaStream_t st) {
     if (n <= 0) return 0;
-    k_kfix_probe<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(xa, xb, out, n, P);
+    k_kfix_probe<<<(unsigned)((n + 511) / 512), 256, 0, st>>>(xa, xb, out, n, P);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

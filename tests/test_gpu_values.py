@@ -47,3 +47,29 @@ def test_paired_exp_below_its_bound(vg):
     out = torch.empty_like(far)
     _lib.check(_lib.load().vgp_debug_exp_near(m._h, _ptr(far), _ptr(out), len(far), _stream()))
     assert torch.equal(out[:4], torch.exp(far[:4])) and torch.isnan(out[4])
+
+
+def test_both_halves_of_packed_kernel_values(vg):
+    """An entry's bits do not depend on the half it is computed in nor on the other half's entry, from
+    coincident points to values beyond the fixed point's range."""
+    from paper_2407_09649_gb300 import _lib
+    m = vg.Map(precision="mixed", emulate_fp64=1)
+    rng = np.random.default_rng(71)
+    n = 100001
+    xa = (np.array([103.7, -45.3, 12.9]) + rng.uniform(-1.5, 1.5, (n, 3))).astype(np.float32)
+    xb = (xa + rng.normal(size=(n, 3)) * 10.0 ** rng.uniform(-6, 1.5, (n, 1))).astype(np.float32)
+    xb[::7] = xa[::7]
+
+    def run(a, b):
+        ta, tb = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+        out = torch.empty(len(a), dtype=torch.int64, device="cuda")
+        _lib.check(_lib.load().vgp_debug_kernel_fix(m._h, _ptr(ta), _ptr(tb), len(a), _ptr(out), _stream()))
+        return out.cpu().numpy()
+
+    got = run(xa, xb)
+    assert np.all(got[::7] == 2**61) and np.any(got == 0)
+    assert np.array_equal(run(xa[1:].copy(), xb[1:].copy()), got[1:])  # every entry in the other half
+    L = np.longdouble
+    y = np.sum((xa.astype(L) - xb.astype(L)) ** 2, axis=1) / (2 * L(0.3) * L(0.3))
+    exact = np.exp(-y) * L(2.0) ** 61
+    assert np.all(np.abs(got.astype(L) - exact) <= exact * (1 + y) * L(2.0) ** -45 + 2)
