@@ -73,3 +73,37 @@ def test_both_halves_of_packed_kernel_values(vg):
     y = np.sum((xa.astype(L) - xb.astype(L)) ** 2, axis=1) / (2 * L(0.3) * L(0.3))
     exact = np.exp(-y) * L(2.0) ** 61
     assert np.all(np.abs(got.astype(L) - exact) <= exact * (1 + y) * L(2.0) ** -45 + 2)
+
+
+def test_crossings_of_special_values(vg, orc):
+    """Zero crossings (inside is D < 0) between voxels that hold zeros of both signs, subnormals, the
+    largest finite values, infinities and NaN, against the rule written out."""
+    rng = np.random.default_rng(72)
+    vs = 0.1
+    vals = np.array([0.0, -0.0, 5e-324, -5e-324, 1e-310, -1e-310, 0.3, -0.3, 0.02, -0.07, 1.7e308, -1.7e308, np.inf,
+                     -np.inf, np.nan, np.copysign(np.nan, -1.0)])
+    ijk = np.stack(np.meshgrid(np.arange(-8, 16), np.arange(-8, 8), np.arange(0, 8), indexing="ij"), -1).reshape(-1, 3)
+    D = vals[rng.integers(0, len(vals), len(ijk))]
+    m = vg.Map(precision="fp64", voxel_size=vs)
+    m.import_grid(orc.pack_key(ijk), D, np.ones(len(D)), np.ones(len(D), np.uint8))
+    x, o, s = (t.cpu().numpy() for t in m.extract_mesh(triangles=False)["crossings"])
+    at = {tuple(v): d for v, d in zip(ijk.tolist(), D)}
+    want = {}
+    with np.errstate(all="ignore"):
+        for v, da in at.items():
+            for axis in range(3):
+                w = tuple(c + (k == axis) for k, c in enumerate(v))
+                if w not in at or (da < 0) == (at[w] < 0):
+                    continue
+                t = np.float64(da) / (np.float64(da) - np.float64(at[w]))
+                p = np.array([np.float32((c + (t if k == axis else 0.0)) * vs) for k, c in enumerate(v)])
+                if not np.all(np.isfinite(p)):
+                    continue
+                own = tuple(np.floor(p.astype(np.float64) / vs + 0.5).astype(int))
+                for u, slot in ((v, 2 * axis + 1), (w, 2 * axis)):
+                    if own == u:
+                        want[(int(orc.pack_key(np.array([u]))[0]), slot)] = p
+    got = {(int(k), int(c)): p for k, c, p in zip(o, s, x)}
+    assert len(got) == len(x) and got.keys() == want.keys() and len(got) > 1000
+    for k, p in got.items():
+        assert np.array_equal(p.view(np.uint32), want[k].view(np.uint32))
