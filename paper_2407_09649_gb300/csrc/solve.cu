@@ -2521,15 +2521,33 @@ int resident_clusters(int n, int threads, size_t shm) {
 }
 
 // CTAs that work on an instance together (a cluster) in an emulated launch of at most `items` work
-// items, nmax points at most, on `slots` resident CTAs: as many as keep every item resident, up to 8.
+// items, on `slots` resident CTAs, up to 8: as many as have all items resident or, where items are
+// instances (h: how many of each size, nmax the largest), as end no later by eights (fours) in two rounds
+// than by fours (twos) in one.
 // K, the rows below and the trailing tiles are shared out, the diagonal blocks and the solves
 // are not, and a block of 32 columns costs three cluster barriers; below 128 points nothing
-// is left to share.  Items that wait for a cluster to end cost more than the larger one gains: 38
-// instances of 130 points take 0.61 ms by eights, 0.41 ms by fours and 0.47 ms by one CTA each.
-int group_ctas(int items, int nmax, int slots, int threads, size_t shm) {
+// is left to share.  Two rounds: the items beyond the resident clusters follow the smallest of the first
+// round (largest first).  An instance's time goes as N (N + 700) (0.26, 0.41, 0.82, 1.43 and 3.45 ms
+// by eights at 130, 224, 400, 640 and 1024 points), and half as many CTAs take 1.0, 1.1, 1.26 and 1.35
+// times as long at 400, 500, 640 and 800 points by fours, 1.1 to 1.25 from 500 by twos.  38 instances of
+// 130 points: 0.61 ms by eights, 0.41 by fours, 0.47 by one CTA each; of 1024 down to 420: 3.0
+// by eights, 4.2 by fours.
+int group_ctas(int items, const std::vector<int>& h, int nmax, int slots, int threads, size_t shm) {
     if (nmax <= 128) return 1;
-    for (int n = 8; n > 1; n /= 2)
-        if ((int64_t)items * n <= slots && resident_clusters(n, threads, shm) >= items) return n;
+    for (int n = 8; n > 1; n /= 2) {
+        if ((int64_t)items * n > slots) continue;
+        const int fit = resident_clusters(n, threads, shm);
+        if (fit >= items) return n;
+        if (n == 2 || 2 * fit < items) continue;
+        std::vector<int> sizes;  // decreasing
+        for (int N = nmax; N > 32; --N) sizes.insert(sizes.end(), h[N], N);
+        if ((int)sizes.size() != items) continue;
+        auto cost = [](double N) { return N * (N + 700.0); };
+        const double most = cost(nmax) * (1.0 + std::min(n == 8 ? 0.35 : 0.15, std::max(0.0, (nmax - 400) / 1000.0)));
+        bool two = true;
+        for (int k = 0; fit + k < items; ++k) two = two && cost(sizes[fit - 1 - k]) + cost(sizes[fit + k]) <= most;
+        if (two) return n;
+    }
     return 1;
 }
 
@@ -2992,7 +3010,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             }
         }
         // few emulated work items: clusters of CTAs work on each
-        L.ncta = L.emu ? group_ctas(items, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
+        L.ncta = L.emu ? group_ctas(items, h, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
         L.groups = (int)std::min<int64_t>(items, (int64_t)n_sm * L.per_sm / L.ncta);
         if (i == 4) beside = !bw && !profile && L.cnt < n && gc && graph_cache_ready(*gc);
         need_a = std::max(need_a, L.ws_a * L.groups);

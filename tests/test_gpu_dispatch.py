@@ -310,6 +310,22 @@ def test_stats_tell_the_shapes_launched(vg, launch):
     assert got[0][0] == 256 and got[1][0] == 0 and got[2] == 0
 
 
+def _best_ms(m, sizes):
+    X, Q = _instances(sizes, 5, 64)
+    io = torch.from_numpy(np.concatenate([[0], np.cumsum(sizes)])).cuda()
+    qo = torch.arange(len(sizes) + 1, dtype=torch.int64, device="cuda") * 5
+    x, q = (torch.from_numpy(np.vstack(a)).cuda() for a in (X, Q))
+    ms = []
+    for _ in range(40):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        m.gp_batch(io, x, qo, q, var=False)
+        b.record()
+        b.synchronize()
+        ms.append(a.elapsed_time(b))
+    return min(ms)
+
+
 @pytest.mark.parametrize("per_sm", [4, 2])
 def test_clusters_all_run_at_once(vg, per_sm):
     """As many instances as clusters of eight (four) would fill the GPU's CTAs with: not all of those
@@ -317,24 +333,15 @@ def test_clusters_all_run_at_once(vg, per_sm):
     with smaller clusters (1.5 times as slow, had it one)."""
     n = torch.cuda.get_device_properties(0).multi_processor_count // per_sm
     m = vg.Map(precision="mixed", emulate_fp64=1)
+    assert _best_ms(m, [130] * n) <= 1.2 * _best_ms(m, [130] * (n + 1))
 
-    def best(count):
-        X, Q = _instances([130] * count, 5, 64)
-        io = torch.arange(count + 1, dtype=torch.int64, device="cuda") * 130
-        qo = torch.arange(count + 1, dtype=torch.int64, device="cuda") * 5
-        x, q = (torch.from_numpy(np.vstack(a)).cuda() for a in (X, Q))
-        ms = []
-        for _ in range(40):
-            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            a.record()
-            m.gp_batch(io, x, qo, q, var=False)
-            b.record()
-            b.synchronize()
-            ms.append(a.elapsed_time(b))
-        return min(ms)
 
-    full = best(n)
-    assert full <= 1.2 * best(n + 1)
+def test_small_instances_follow_in_a_second_round(vg):
+    """The same number with a few large ones: the small ones beyond the clusters of eight that run at once
+    end before the large ones do, which smaller clusters would make 1.4 times as long."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count // 4
+    m = vg.Map(precision="mixed", emulate_fp64=1)
+    assert _best_ms(m, [1024] * 4 + [300] * (n - 4)) <= 1.15 * _best_ms(m, [1024] * 4 + [300] * (n - 8))
 
 
 def test_autotuner_chooses_for_the_buckets_it_timed(vg):
