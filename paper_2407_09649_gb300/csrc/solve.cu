@@ -1661,6 +1661,19 @@ __host__ __device__ __forceinline__ long long chunk_len(long long qc, int qn, lo
     return cap > 0 && q > cap ? cap : q;
 }
 
+// The shortest work item worth a fit, chunk_len(qmin, qn, N, cap) queries, in the plain kernel or the
+// emulated one:
+// * Emulated launches with variance or properties: an appended row of an N-point instance costs about
+//   1 / N of its fit; at least 64 of them, and at most what a factorisation appends.
+// * Plain launches with variance run on the FP64 pipe; 128 queries.
+// * The mean alone costs about N FP32 values a query: a fit is worth about 64 N of them.
+struct ChunkRule {
+    int qmin, qn, cap;
+};
+__host__ __device__ __forceinline__ ChunkRule chunk_rule(bool heavy, bool var, bool emu) {
+    return {heavy && !emu ? 128 : 64, !heavy ? 64 : emu ? 1 : 0, emu && var ? kBorderQ : 0};
+}
+
 struct EvalOut {
     double d, g[3], v;
     int status;
@@ -2209,9 +2222,12 @@ __global__ void k_backward(SolveCtx c) {
     }
 }
 
-// Instances of each size, and with qsum the queries of each size bucket (N > 224, > 128, > 64, > 32, the
-// rest) for the chunk planning.
-__global__ void k_hist_n(const int64_t* inst_off, const int64_t* q_off, int64_t n, int* hist, unsigned long long* qsum) {
+// Instances of each size.  With more (1025 words, then five of 64 bits, 8-byte aligned): the work items
+// beyond one per instance of each size, were every chunk the shortest (chunk_rule), and the
+// queries of each size bucket (N > 224, > 128, > 64, > 32, the rest).
+constexpr int kHistWords = 1026;  // (a word of padding)
+__global__ void k_hist_n(const int64_t* inst_off, const int64_t* q_off, int64_t n, int* hist, int* more, bool heavy,
+                         bool var, bool emulate) {
     __shared__ unsigned long long sum[5];
     if (threadIdx.x < 5) sum[threadIdx.x] = 0;
     __syncthreads();
@@ -2219,11 +2235,18 @@ __global__ void k_hist_n(const int64_t* inst_off, const int64_t* q_off, int64_t 
     if (i < n) {
         const int N = (int)(inst_off[i + 1] - inst_off[i]);
         atomicAdd(&hist[min(N, 1024)], 1);
-        const int bk = N > 224 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
-        if (qsum) atomicAdd(&sum[bk], (unsigned long long)(q_off[i + 1] - q_off[i]));
+        if (more) {
+            const int64_t nq = q_off[i + 1] - q_off[i];
+            const int bk = N > 224 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
+            atomicAdd(&sum[bk], (unsigned long long)nq);
+            const ChunkRule r = chunk_rule(heavy, var, emulate && N > 32);
+            const long long len = chunk_len(r.qmin, r.qn, N, r.cap);
+            if (nq > len) atomicAdd(&more[min(N, 1024)], (int)((nq - 1) / len));
+        }
     }
     __syncthreads();
-    if (qsum && threadIdx.x < 5 && sum[threadIdx.x]) atomicAdd(&qsum[threadIdx.x], sum[threadIdx.x]);
+    if (more && threadIdx.x < 5 && sum[threadIdx.x])
+        atomicAdd(reinterpret_cast<unsigned long long*>(more + kHistWords) + threadIdx.x, sum[threadIdx.x]);
 }
 
 // order[] sorted by increasing N via the prefix of the histogram
@@ -2466,20 +2489,17 @@ constexpr int64_t kEmuBytesPerRow = 7 * 8 * kEB * 2 + 8 + 64 + 8;
 // Words of a matrix of `rows` rows in a CTA's workspace (rows: a multiple of 8).
 int64_t matrix_words(bool emu, int rows) { return emu ? n_blocks(rows) * 1024 : n_tiles(rows / 8) * 64; }
 
-// Chunk planning of launch i (cnt instances, resident CTAs per SM, threads each): the CTAs to spread it
-// over, the bound of an emulated launch that appends query rows, and the shortest chunk worth a fit.
-// * Emulated launches spread over all resident CTAs; with variance or properties an appended row of
-//   an N-point instance costs about 1 / N of its fit, at least 64 of them.
-// * Plain launches with variance run on the FP64 pipe, which one warp per sub-partition nearly fills:
-//   16 warps per SM are enough, and more would only refit; 128 queries.
-// * The mean alone costs about N FP32 values a query: a fit is worth about 64 N of them.
+// Chunk planning of launch i (cnt instances, resident CTAs per SM, threads each): the rule for its chunks
+// and the CTAs to spread it over, all resident ones, but for plain launches with variance, whose FP64 pipe one
+// warp per sub-partition nearly fills: 16 warps per SM are enough, and more would only refit.
 void chunk_args(const SolveBatch& b, int i, int cnt, int n_sm, int per_sm, int threads, bool emu, ChunkPlanArgs& a) {
     const bool heavy = b.want_var || b.nprop > 0;
+    const ChunkRule r = chunk_rule(heavy, b.want_var, emu);
     a.cnt[i] = cnt;
-    a.cap[i] = emu && b.want_var ? kBorderQ : 0;
+    a.cap[i] = r.cap;
     a.slots[i] = n_sm * (emu || !heavy ? per_sm : std::min(per_sm, std::max(1, 512 / threads)));
-    a.qmin[i] = heavy && !emu ? 128 : 64;
-    a.qn[i] = !heavy ? 64 : emu ? 1 : 0;
+    a.qmin[i] = r.qmin;
+    a.qn[i] = r.qn;
 }
 
 // The emulated kernel's shared memory (about 100 KB at N = 1024) fits twice per SM only in the
@@ -2521,9 +2541,9 @@ int resident_clusters(int n, int threads, size_t shm) {
 }
 
 // CTAs that work on an instance together (a cluster) in an emulated launch of at most `items` work
-// items, on `slots` resident CTAs, up to 8: as many as have all items resident or, where items are
-// instances (h: how many of each size, nmax the largest), as end no later by eights (fours) in two rounds
-// than by fours (twos) in one.
+// items (h[N] + more[N] on instances of N points, nmax the largest), on `slots` resident CTAs, up to 8: as
+// many as have all items resident, or as end no later by eights (fours) in two rounds than by fours
+// (twos) in one.
 // K, the rows below and the trailing tiles are shared out, the diagonal blocks and the solves
 // are not, and a block of 32 columns costs three cluster barriers; below 128 points nothing
 // is left to share.  Two rounds: the items beyond the resident clusters follow the smallest of the first
@@ -2532,7 +2552,7 @@ int resident_clusters(int n, int threads, size_t shm) {
 // times as long at 400, 500, 640 and 800 points by fours, 1.1 to 1.25 from 500 by twos.  38 instances of
 // 130 points: 0.61 ms by eights, 0.41 by fours, 0.47 by one CTA each; of 1024 down to 420: 3.0
 // by eights, 4.2 by fours.
-int group_ctas(int items, const std::vector<int>& h, int nmax, int slots, int threads, size_t shm) {
+int group_ctas(int items, const int* h, const int* more, int nmax, int slots, int threads, size_t shm) {
     if (nmax <= 128) return 1;
     for (int n = 8; n > 1; n /= 2) {
         if ((int64_t)items * n > slots) continue;
@@ -2540,8 +2560,7 @@ int group_ctas(int items, const std::vector<int>& h, int nmax, int slots, int th
         if (fit >= items) return n;
         if (n == 2 || 2 * fit < items) continue;
         std::vector<int> sizes;  // decreasing
-        for (int N = nmax; N > 32; --N) sizes.insert(sizes.end(), h[N], N);
-        if ((int)sizes.size() != items) continue;
+        for (int N = nmax; N > 32; --N) sizes.insert(sizes.end(), h[N] + more[N], N);
         auto cost = [](double N) { return N * (N + 700.0); };
         const double most = cost(nmax) * (1.0 + std::min(n == 8 ? 0.35 : 0.15, std::max(0.0, (nmax - 400) / 1000.0)));
         bool two = true;
@@ -2715,7 +2734,7 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
     if (cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return -1;
     fill_i32(hist, 0, 1025, gs);
     fill_i32(counters, 0, 5, gs);
-    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, gs>>>(b.inst_off, b.q_off, n, hist, nullptr);
+    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, gs>>>(b.inst_off, b.q_off, n, hist, nullptr, false, false, false);
     note_launch();
     k_plan_buckets<<<1, 32, 0, gs>>>(hist, cursor, plan);
     note_launch();
@@ -2821,20 +2840,21 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     // size histogram (and, for chunk planning, each bucket's queries) and decreasing-size order
     const bool heavy = !bw && (b.want_var || b.nprop > 0);
     ChunkPlanArgs ca{};
-    constexpr int kHistWords = 1026 + 2 * 5;  // sizes (and a word of padding), the buckets' queries in 64 bits
-    int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * (kHistWords + 1025), st);
+    const int words = bw ? kHistWords : 2 * kHistWords + 2 * 5;
+    int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * (words + 1025), st);
     if (!hist) return alloc_failed(err_dev, st);
-    int* cursor = hist + kHistWords;
-    cudaMemsetAsync(hist, 0, sizeof(int) * kHistWords, st);
+    int* cursor = hist + words;
+    cudaMemsetAsync(hist, 0, sizeof(int) * words, st);
     const int T = 256;
-    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, b.q_off, n, hist,
-                                                        bw ? nullptr : reinterpret_cast<unsigned long long*>(hist + 1026));
+    k_hist_n<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(b.inst_off, b.q_off, n, hist, bw ? nullptr : hist + kHistWords,
+                                                        heavy, b.want_var, P.emulate);
     note_launch();
-    std::vector<int> h(kHistWords);
-    cudaMemcpyAsync(h.data(), hist, sizeof(int) * kHistWords, cudaMemcpyDeviceToHost, st);
+    std::vector<int> h(words);
+    cudaMemcpyAsync(h.data(), hist, sizeof(int) * words, cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
-    unsigned long long hq[5];
-    std::memcpy(hq, h.data() + 1026, sizeof(hq));
+    const int* more = h.data() + (bw ? 0 : kHistWords);
+    unsigned long long hq[5] = {0, 0, 0, 0, 0};
+    if (!bw) std::memcpy(hq, more + kHistWords, sizeof(hq));
     std::vector<int> start(1026, 0);
     for (int i = 0; i < 1025; ++i) start[i + 1] = start[i] + h[i];
     cudaMemcpyAsync(cursor, start.data(), sizeof(int) * 1025, cudaMemcpyHostToDevice, st);
@@ -2995,12 +3015,9 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         int items = L.cnt;  // an upper bound of the launch's work items
         if (!bw) {
             chunk_args(b, i, L.cnt, n_sm, L.per_sm, L.threads, L.emu, ca);
-            int nmin = L.nmax;
-            for (int N = L.nmax; N >= buckets[i].lo; --N)
-                if (h[N]) nmin = N;
-            // the shortest chunk any of its instances can have
-            const int64_t len = std::max<int64_t>(1, chunk_len(ca.qmin[i], ca.qn[i], nmin, ca.cap[i]));
-            const int64_t extra = std::min<int64_t>((int64_t)hq[i] / len, ca.cap[i] > 0 ? INT32_MAX : ca.slots[i]);
+            int64_t extra = 0;
+            for (int N = buckets[i].lo; N <= buckets[i].hi; ++N) extra += more[N];
+            if (ca.cap[i] == 0) extra = std::min<int64_t>(extra, ca.slots[i]);
             // (without a bound, a launch of ten rounds of instances or more has no tail to shorten)
             if (ca.cap[i] == 0 && L.cnt > 10 * ca.slots[i]) {
                 ca.qmin[i] = 0;
@@ -3010,7 +3027,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
             }
         }
         // few emulated work items: clusters of CTAs work on each
-        L.ncta = L.emu ? group_ctas(items, h, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
+        L.ncta = L.emu ? group_ctas(items, h.data(), more, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
         L.groups = (int)std::min<int64_t>(items, (int64_t)n_sm * L.per_sm / L.ncta);
         if (i == 4) beside = !bw && !profile && L.cnt < n && gc && graph_cache_ready(*gc);
         need_a = std::max(need_a, L.ws_a * L.groups);

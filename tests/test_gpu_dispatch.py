@@ -398,3 +398,19 @@ def test_kernels_of_a_small_call(vg, emulate, sizes):
     n0 = lib.vgp_launch_count()
     _solve(m, X, Q, False)
     assert lib.vgp_launch_count() - n0 == 4 + len(sizes)
+
+
+def test_work_items_are_counted_by_instance(vg):
+    """Queries that no instance has enough of for two work items are not planned as such, however many they
+    are together: no planning kernel."""
+    from paper_2407_09649_gb300 import _lib
+    lib = _lib.load()
+    m = vg.Map(precision="mixed", emulate_fp64=1)
+    X, Q = _instances([130] * 75, 100, 68)
+    _solve(m, X, Q, True)
+    n0 = lib.vgp_launch_count()
+    _solve(m, X, Q, True)
+    assert lib.vgp_launch_count() - n0 == 5
+    n0 = lib.vgp_launch_count()
+    _solve(m, X, Q[:74] + [np.concatenate([Q[74]] * 2)], True)  # 200 queries: two items of 130 at most
+    assert lib.vgp_launch_count() - n0 == 6
