@@ -55,6 +55,7 @@ void* Arena::get(Slot s, size_t bytes, cudaStream_t st) {
     if (cudaMallocAsync(&p, want, st) != cudaSuccess) {
         cudaGetLastError();
         if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
+            cudaGetLastError();
             ptr_[s] = nullptr;
             size_[s] = 0;
             return nullptr;

@@ -2690,7 +2690,6 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
             return -1;
     }
     ChunkPlanArgs ca{};
-    int64_t ws_a_need = 0, ws_v_need = 0, ws_e_need = 0;
     for (int i = 0; i < 5; ++i) {
         Shape& s = sh[i];
         if (!s.live) continue;
@@ -2710,22 +2709,36 @@ int solve_batch_graph(const SolveBatch& b, const DevParams& P, int* err_dev, cud
         const int64_t len = chunk_len(ca.qmin[i], ca.qn[i], std::max(lo[i], 1), ca.cap[i]);
         const int64_t items = n + (b.want_var || props ? b.max_pos / len : 0);
         s.grid = (int)std::min<int64_t>(items, (int64_t)n_sm * per_sm);
-        ca.slots[i] = std::min(ca.slots[i], s.grid);
-        if (!s.smem_a) ws_a_need = std::max<int64_t>(ws_a_need, matrix_words(s.emu, s.nrow) * s.grid);
-        if (b.want_var && !s.emu) ws_v_need = std::max<int64_t>(ws_v_need, (int64_t)s.npad * s.threads * s.grid);
-        if (s.emu) ws_e_need = std::max<int64_t>(ws_e_need, (int64_t)s.nrow * kEmuBytesPerRow * s.grid);
     }
-    // every buffer exists before the capture starts (allocation is not captured)
+    // every buffer exists before the capture starts (allocation is not captured); where memory is short,
+    // fewer CTAs share the work
     int* hist = (int*)ar.get(Arena::kHist, sizeof(int) * 2 * 1025, st);
     int32_t* order = (int32_t*)ar.get(Arena::kOrder, sizeof(int32_t) * n, st);
     int* counters = (int*)ar.get(Arena::kCounters, sizeof(int) * 16, st);
-    double* ws_a = ws_a_need ? (double*)ar.get(Arena::kWs0, sizeof(double) * ws_a_need, st) : nullptr;
-    double* ws_v = ws_v_need ? (double*)ar.get(Arena::kWs1, sizeof(double) * ws_v_need, st) : nullptr;
-    uint8_t* ws_e = ws_e_need ? (uint8_t*)ar.get(Arena::kWs3, ws_e_need, st) : nullptr;
     int* chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
-    if (!hist || !order || !counters || (ws_a_need && !ws_a) || (ws_v_need && !ws_v) || (ws_e_need && !ws_e) ||
-        !chunk_off)
-        return alloc_failed(err_dev, st);
+    if (!hist || !order || !counters || !chunk_off) return alloc_failed(err_dev, st);
+    double *ws_a = nullptr, *ws_v = nullptr;
+    uint8_t* ws_e = nullptr;
+    for (;;) {
+        int64_t need_a = 0, need_v = 0, need_e = 0;
+        int grid = 0;
+        for (const Shape& s : sh) {
+            if (!s.live) continue;
+            if (!s.smem_a || b.want_var) grid = std::max(grid, s.grid);
+            if (!s.smem_a) need_a = std::max<int64_t>(need_a, matrix_words(s.emu, s.nrow) * s.grid);
+            if (b.want_var && !s.emu) need_v = std::max<int64_t>(need_v, (int64_t)s.npad * s.threads * s.grid);
+            if (s.emu) need_e = std::max<int64_t>(need_e, (int64_t)s.nrow * kEmuBytesPerRow * s.grid);
+        }
+        ws_a = need_a ? (double*)ar.get(Arena::kWs0, sizeof(double) * need_a, st) : nullptr;
+        ws_v = need_v ? (double*)ar.get(Arena::kWs1, sizeof(double) * need_v, st) : nullptr;
+        ws_e = need_e ? (uint8_t*)ar.get(Arena::kWs3, need_e, st) : nullptr;
+        if (!(need_a && !ws_a) && !(need_v && !ws_v) && !(need_e && !ws_e)) break;
+        if (grid <= 1) return alloc_failed(err_dev, st);
+        for (Shape& s : sh)
+            if (s.live && (!s.smem_a || b.want_var)) s.grid = (s.grid + 1) / 2;
+    }
+    for (int i = 0; i < 5; ++i)
+        if (sh[i].live) ca.slots[i] = std::min(ca.slots[i], sh[i].grid);
     int* chunk_q = chunk_off + n + 1;
     int* cursor = hist + 1025;
     int* plan = counters + 5;
@@ -3002,7 +3015,6 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
     // planned only where some bucket can have more of them than instances
     Launch launches[5];
     bool chunks = false;
-    int64_t need_a = 0, need_v = 0, need_v_aside = 0, need_e = 0;
     // the smallest instances run on the map's own stream beside the others, where its CTAs fill the SMs
     // that the last of those leave; not while profiling
     bool beside = false;
@@ -3030,23 +3042,39 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         L.ncta = L.emu ? group_ctas(items, h.data(), more, L.nmax, n_sm * L.per_sm, L.threads, L.shm) : 1;
         L.groups = (int)std::min<int64_t>(items, (int64_t)n_sm * L.per_sm / L.ncta);
         if (i == 4) beside = !bw && !profile && L.cnt < n && gc && graph_cache_ready(*gc);
-        need_a = std::max(need_a, L.ws_a * L.groups);
-        int64_t& nv = i == 4 && beside ? need_v_aside : need_v;
-        nv = std::max(nv, L.ws_v * L.groups);
-        need_e = std::max(need_e, L.ws_e * L.groups);
     }
     // Every workspace is obtained before the first launch and before e0: a slot that grew between two
     // launches would give its block back behind the first one's kernel, in the order of st alone, and
     // the allocator may hand that block to a launch on the map's own stream, which waits for
     // nothing after e0.
+    // Where memory is short, fewer CTAs share the work.
     int* counters = (int*)ar.get(Arena::kCounters, sizeof(int) * 8, st);
-    double* ws_a = need_a ? (double*)ar.get(Arena::kWs0, sizeof(double) * need_a, st) : nullptr;
-    double* ws_v = need_v ? (double*)ar.get(Arena::kWs1, sizeof(double) * need_v, st) : nullptr;
-    double* ws_v_aside = need_v_aside ? (double*)ar.get(Arena::kWs4, sizeof(double) * need_v_aside, st) : nullptr;
-    uint8_t* ws_e = need_e ? (uint8_t*)ar.get(Arena::kWs3, need_e, st) : nullptr;
     if (chunks) chunk_off = (int*)ar.get(Arena::kChunks, sizeof(int) * (n + 1 + 5), st);
-    if (!counters || (need_a && !ws_a) || (need_v && !ws_v) || (need_v_aside && !ws_v_aside) || (need_e && !ws_e) ||
-        (chunks && !chunk_off)) {
+    double *ws_a = nullptr, *ws_v = nullptr, *ws_v_aside = nullptr;
+    uint8_t* ws_e = nullptr;
+    bool got = counters && (!chunks || chunk_off);
+    while (got) {
+        int64_t need_a = 0, need_v = 0, need_v_aside = 0, need_e = 0;
+        int groups = 0;
+        for (int i = 0; i < 5; ++i) {
+            const Launch& L = launches[i];
+            if (L.ws_a || L.ws_v) groups = std::max(groups, L.groups);
+            need_a = std::max(need_a, L.ws_a * L.groups);
+            int64_t& nv = i == 4 && beside ? need_v_aside : need_v;
+            nv = std::max(nv, L.ws_v * L.groups);
+            need_e = std::max(need_e, L.ws_e * L.groups);
+        }
+        ws_a = need_a ? (double*)ar.get(Arena::kWs0, sizeof(double) * need_a, st) : nullptr;
+        ws_v = need_v ? (double*)ar.get(Arena::kWs1, sizeof(double) * need_v, st) : nullptr;
+        ws_v_aside = need_v_aside ? (double*)ar.get(Arena::kWs4, sizeof(double) * need_v_aside, st) : nullptr;
+        ws_e = need_e ? (uint8_t*)ar.get(Arena::kWs3, need_e, st) : nullptr;
+        got = !(need_a && !ws_a) && !(need_v && !ws_v) && !(need_v_aside && !ws_v_aside) && !(need_e && !ws_e);
+        if (got || groups <= 1) break;
+        for (Launch& L : launches)
+            if (L.ws_a || L.ws_v) L.groups = (L.groups + 1) / 2;
+        got = true;
+    }
+    if (!got) {
         if (profile) {
             cudaEventDestroy(ev0);
             cudaEventDestroy(ev1);
@@ -3093,7 +3121,7 @@ int solve_batch(const SolveBatch& b, const DevParams& P, int* err_dev, cudaStrea
         c.ws_a_stride = L.ws_a;
         c.ws_a = L.ws_a ? ws_a : nullptr;
         c.ws_v_stride = L.ws_v;
-        c.ws_v = !L.ws_v ? nullptr : bi == 4 && need_v_aside ? ws_v_aside : ws_v;
+        c.ws_v = !L.ws_v ? nullptr : bi == 4 && ws_v_aside ? ws_v_aside : ws_v;
         c.ws_e_stride = L.ws_e;
         c.ws_e = L.ws_e ? ws_e : nullptr;
         // (buckets share kernels, whose limit is that of the bucket shaped last)

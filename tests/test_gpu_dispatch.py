@@ -414,3 +414,23 @@ def test_work_items_are_counted_by_instance(vg):
     n0 = lib.vgp_launch_count()
     _solve(m, X, Q[:74] + [np.concatenate([Q[74]] * 2)], True)  # 200 queries: two items of 130 at most
     assert lib.vgp_launch_count() - n0 == 6
+
+
+@pytest.mark.parametrize("launch", ["batched", "graph"])
+@pytest.mark.parametrize("sizes,nq", [([1000] + [40] * 300, 5), ([1000] * 8, 20000)])
+def test_short_memory_takes_fewer_workspaces(vg, launch, sizes, nq):
+    """A workspace for every CTA of the GPU would take 5 GB; with 1.5 GB left fewer CTAs share the work, as
+    they did when each size had its own launch, and the bits are the same."""
+    import gc
+    X, Q = _instances(sizes, nq, 69)
+    want = _solve(vg.Map(precision="mixed", emulate_fp64=1, launch=launch), X, Q, True)
+    gc.collect()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    m = vg.Map(precision="mixed", emulate_fp64=1, launch=launch)
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (3 << 29), dtype=torch.uint8, device="cuda")
+    got = _solve(m, X, Q, True)
+    del fill
+    torch.cuda.empty_cache()
+    for a, b in zip(got, want):
+        _same(a, b)
