@@ -354,7 +354,7 @@ def solve_roofline(prof, fp64_peak, bf16_peak):
     bf16_flop = float(_emu_mma_table()[big].sum())
     bf16_achieved = bf16_flop / (prof["emu_ms"] / 1e3) / 1e12 if prof["emu_ms"] > 0 else None
     return {"kernel": ("k_solve_emu (N > 32: FP64-accurate Cholesky, trailing updates as bf16 slice products) + "
-                       "k_solve (N <= 32: FP64 tile Cholesky on mma.sync f64); alpha, fused eval"),
+                       "k_solve (N <= 32: FP64 tile Cholesky on the FP64 pipe); alpha, fused eval"),
             "bound": "tensor", "dtype": "fp64 (FP64-equivalent work)", "achieved": achieved, "peak": fp64_peak,
             "unit": "TFLOP/s", "frac": achieved / fp64_peak,
             "frac_note": ("achieved counts the FP64 Cholesky flops the method needs; the emulated updates run "

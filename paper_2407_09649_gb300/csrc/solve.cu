@@ -2453,11 +2453,16 @@ using SolveKernel = void (*)(SolveCtx);
 // (autotuner, vgp_set_launch):
 // * N > 224, more than eight instances per SM: three CTAs of 256 threads per SM and no panel staging,
 //   so that one's diagonal tiles and barriers overlap the others' updates (2190 instances of
-//   about 400 points: 104 -> 96 ms).  With fewer, the last round of instances costs more than the
+//   about 400 points: 104 -> 96 ms).  With fewer, the last round of instances can cost more than the
 //   overlap gains (677 instances: 51 -> 75 ms), and the default's 512 threads on one instance stay.
+//   Measured on 152 SMs, mean only: sizes spread over 225..1024, 608 instances 71 -> 80 ms, 912 104 -> 99,
+//   1217 130 -> 125, 3000 337 -> 319; equal sizes gain 2 (1000 points) to 26 % (230) from 304 to 3000
+//   instances, at 1217 and above 3 to 26.
 // * 33 to 64 points, heavy evaluation, few instances with 512 queries or more each: 256 threads, so
 //   the chunks are twice as long and fewer of them refit the instance (159 leaves of a frame, 384k
-//   voxels: 5.2 -> 3.9 ms; but 4803 instances with 64 queries each: 3.6 -> 4.0 ms).
+//   voxels: 5.2 -> 3.9 ms; but 4803 instances with 64 queries each: 3.6 -> 4.0 ms).  Measured at 36 and 64
+//   points with variance: from 512 to 2500 queries each, 20 to 304 instances take 0.76 to 1.02 of
+//   the time; at 128, 456 take 1.1.
 struct BucketShape {
     int threads, per_sm, stage;
 };
